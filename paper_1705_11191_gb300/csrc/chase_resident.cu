@@ -1,0 +1,384 @@
+// Band -> tridiagonal bulge chase with the band held on chip (arXiv:1705.11191 Eq. 11,
+// second line; the same reflectors and the same order as chase_kernel in sb2st.cu).
+//
+// What bounds it: the chase is one chain. Step t of sweep j + 1 needs step t + 1 of sweep
+// j, which needs step t of sweep j, so n sweeps cost n times (two steps + two hand-overs),
+// whatever the number of SMs. With a CTA per sweep every step loads a 2b x b window of the
+// band from L2, stores it again and hands over through a fence and a flag: 7.4 us a step
+// in binary32 and 17 us in binary64 (b = 64).
+//
+// Layout: a CTA per step position t instead. Its window (X = A[r .. r+b-1, r-b .. r-1] and
+// D = A[r .. r+b-1]^2, r = j + 1 + t b) moves by one row and column per sweep; row and column
+// g of the matrix live in slot g mod b, so a sweep replaces one slot and moves nothing:
+// thread (row slot i, column slots c0 ..) keeps its elements of X and D in registers for
+// the whole reduction, and the column that leaves D enters X inside the same thread. What
+// two positions exchange per sweep is a reflector (t -> t + 1: b + 1 values) and one row
+// (t + 1 -> t: b + 1 values), as packets of value and sweep number in one 64-bit word: the
+// reader polls the data itself, so a hand-over is one store and one load through L2 with
+// no fence and no separate flag. A position's first step after its reflector is known
+// sends it on before updating its own D.
+//
+// Per step, with v_p, tau_p the previous position's reflector (X0 before the step):
+//   y = tau_p X0 v_p, x = X0[:, first] - y, v = house(x), p = tau v^T (X0 - y v_p^T),
+//   q = tau D v, w = q - (1/2) tau (v.q) v,
+//   X = X0 - y v_p^T - v p^T,  D = D - v w^T - w v^T.
+// The column sums x^T X0 and D x are taken with the unscaled x (x_first apart), so that
+// three block barriers serve a whole step.
+//
+// Measured, b = 64, against the kernel of sb2st.cu: binary32 n = 777 10.6 -> 3.0 ms,
+// n = 4096 60.3 -> 17.3 ms, n = 16384 245 -> 76 ms (14.7 -> 4.2 - 4.7 us a sweep, two block
+// barriers' worth of arithmetic and two L2 hand-overs); binary64 n = 512 15.2 -> 11.0 ms,
+// n = 1531 51.3 -> 35.7 ms (a step's 28 000 FMAs at two a clock bound it).
+#include "common.cuh"
+#include "kernels.h"
+
+namespace egb {
+namespace sys {
+
+typedef unsigned long long u64;
+
+struct Args {
+    int n, ldb, S;      // S positions = grid size; also the stride of the reflector slots
+    u64 *vmsg, *rmsg;   // reflector / row packets, one record of kWords<T> * (B + 2) words each
+    int *status;
+    long long spin_limit;
+};
+
+template <typename T> constexpr int kWords = (int)(sizeof(T) / 4);  // packet words per value
+
+__device__ __forceinline__ void st_relaxed(u64 *p, u64 v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ u64 ld_relaxed(const u64 *p)
+{
+    u64 v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Packet word: 32 bits of the value, the sequence number (never 0) above them.
+__device__ __forceinline__ void put(u64 *p, float v, unsigned seq)
+{
+    st_relaxed(p, ((u64)seq << 32) | __float_as_uint(v));
+}
+__device__ __forceinline__ void put(u64 *p, double v, unsigned seq)
+{
+    const u64 u = (u64)__double_as_longlong(v);
+    st_relaxed(p, ((u64)seq << 32) | (u & 0xFFFFFFFFull));
+    st_relaxed(p + 1, ((u64)seq << 32) | (u >> 32));
+}
+__device__ __forceinline__ bool try_get(const u64 *p, unsigned seq, float &v)
+{
+    const u64 a = ld_relaxed(p);
+    v = __uint_as_float((unsigned)a);
+    return (unsigned)(a >> 32) == seq;
+}
+__device__ __forceinline__ bool try_get(const u64 *p, unsigned seq, double &v)
+{
+    const u64 a = ld_relaxed(p), b = ld_relaxed(p + 1);
+    v = __longlong_as_double((long long)((a & 0xFFFFFFFFull) | (b << 32)));
+    return (unsigned)(a >> 32) == seq && (unsigned)(b >> 32) == seq;
+}
+// Bounded wait for a packet; false when the limit is reached or another CTA has failed.
+template <typename T>
+__device__ __forceinline__ bool get(const u64 *p, unsigned seq, T &v, const Args &a)
+{
+    long long it = 0;
+    while (!try_get(p, seq, v)) {
+        if (++it > a.spin_limit) {
+            report_error(a.status, ELSI_ERR_TIMEOUT, (int)seq);
+            return false;
+        }
+        if ((it & 255) == 0 && *(volatile int *)(a.status + ST_CODE) != 0) return false;
+    }
+    return true;
+}
+
+template <typename T> __device__ __forceinline__ T rsq(T x);
+template <> __device__ __forceinline__ float rsq(float x) { return 1.0f / sqrtf(x); }
+template <> __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+
+// a[q] for a run-time q without indexing registers
+template <typename T, int N>
+__device__ __forceinline__ T pick(const T (&a)[N], int q)
+{
+    T v = a[0];
+#pragma unroll
+    for (int k = 1; k < N; ++k) v = (k == q) ? a[k] : v;
+    return v;
+}
+
+template <typename T, int B>
+__global__ void __launch_bounds__(4 * B, 512 / (4 * B))
+chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, double *eout, const Args a)
+{
+    constexpr int CPT = B / 4;       // columns of a row per thread (four threads per row)
+    constexpr int NW = 4 * B / 32;   // warps
+    constexpr int PH = CPT / 8;      // columns per lane after the in-warp column sums
+    __shared__ __align__(16) T vps[2][B];      // v_p by slot (double buffered: see the end)
+    __shared__ __align__(16) T rows_[2][B];    // row message by slot
+    __shared__ T msc[2][2];                    // tau_p, d of the row message
+    __shared__ __align__(16) T xs[B], xrow[B], ps[B], qs[B], vs[B];
+    __shared__ __align__(16) T upart[NW][B];
+    __shared__ T red[3][NW], ysl[2];           // partial sums; x and y at the first row
+    __shared__ int failed;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int i = tid >> 2, part = tid & 3, c0 = part * CPT, quad = lane & ~3;
+    const int t = blockIdx.x, n = a.n, ldb = a.ldb;
+    const int nsweep = n - 2;
+    constexpr int REC = kWords<T> * (B + 2);
+    u64 *vin = a.vmsg + (size_t)(t > 0 ? t - 1 : 0) * REC, *vout = a.vmsg + (size_t)t * REC;
+    u64 *rin = a.rmsg + (size_t)t * REC, *rout = a.rmsg + (size_t)(t > 0 ? t - 1 : 0) * REC;
+
+    if (t == 0)  // defined values should a wait run out below
+        for (int q = tid; q < n; q += 4 * B) {
+            dout[q] = (q == 0) ? (double)band[0] : 0.0;
+            if (q + 1 < n) eout[q] = 0.0;
+        }
+    if (tid == 0) failed = *(volatile int *)(a.status + ST_CODE) != 0;
+
+    // ---- windows of sweep 0
+    T X[CPT], D[CPT], x0 = T(0);
+    {
+        const int r = 1 + t * B, rs = r % B;
+        const int gi = r + (i - rs + B) % B;
+#pragma unroll
+        for (int q = 0; q < CPT; ++q) {
+            const int c = c0 + q, gj = r + (c - rs + B) % B, gc = gj - B;
+            const int lo = min(gi, gj), hi = max(gi, gj);
+            D[q] = (hi < n) ? band[(size_t)(hi - lo) + (size_t)lo * ldb] : T(0);
+            X[q] = (t > 0 && gi < n) ? band[(size_t)(gi - gc) + (size_t)gc * ldb] : T(0);
+        }
+        if (t == 0 && gi < n) x0 = band[gi];  // column 0, rows 1 .. B
+    }
+    __syncthreads();
+    if (failed) return;
+
+    int rs = 1 % B;      // slot of the first row (and, for t > 0, of the first column of X)
+    for (int j = 0; j < nsweep; ++j) {
+        const int r = j + 1 + t * B;
+        if (r > n - 1) break;
+        const int par = j & 1;
+        const int pr = rs == 0 ? B - 1 : rs - 1;           // slot that leaves / enters
+        const bool have_row = j > 0 && r - 1 + B <= n - 1;  // position t + 1 had a step in sweep j - 1
+        const bool have_next = r + B <= n - 1;              // position t + 1 has one in this sweep
+        // ---- what this step waits for
+        {
+            bool ok = true;
+            if (tid < B) {
+                if (t > 0) ok = get(vin + tid * kWords<T>, (unsigned)j + 1, vps[par][tid], a);
+            } else if (tid < 2 * B) {
+                const int c = tid - B;
+                T v = T(0);
+                if (have_row) ok = get(rin + c * kWords<T>, (unsigned)j, v, a);
+                rows_[par][c] = v;
+            } else if (tid == 2 * B) {
+                if (t > 0) ok = get(vin + B * kWords<T>, (unsigned)j + 1, msc[par][0], a);
+            } else if (tid == 2 * B + 32) {
+                T v = T(0);
+                if (have_row) ok = get(rin + B * kWords<T>, (unsigned)j, v, a);
+                msc[par][1] = v;
+            }
+            if (!ok) failed = 1;
+        }
+        __syncthreads();
+        if (failed) return;
+        // ---- the window moves: slot pr takes the new row and column
+        if (j > 0) {
+            const T dold = __shfl_sync(0xffffffffu, pick(D, pr % CPT), quad | (pr / CPT));
+            if (i == pr) {
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) {
+                    const int c = c0 + q;
+                    X[q] = (c == pr) ? rows_[par][c] : T(0);
+                    D[q] = (c == pr) ? msc[par][1] : rows_[par][c];
+                }
+                x0 = rows_[par][pr];
+            } else {
+                if (part == pr / CPT) {
+                    const T ri = rows_[par][i];
+#pragma unroll
+                    for (int q = 0; q < CPT; ++q)
+                        if (q == pr % CPT) { X[q] = D[q]; D[q] = ri; }
+                }
+                x0 = dold;
+            }
+        }
+        // ---- y, x and the partial sums over rows
+        const bool first = i == rs;
+        T y = T(0), x = x0;
+        if (t > 0) {
+#pragma unroll
+            for (int q = 0; q < CPT; ++q) y = fma(X[q], vps[par][c0 + q], y);
+            y += __shfl_xor_sync(0xffffffffu, y, 1);
+            y += __shfl_xor_sync(0xffffffffu, y, 2);
+            y *= msc[par][0];
+            x = __shfl_sync(0xffffffffu, pick(X, rs % CPT), quad | (rs / CPT)) - y;
+        }
+        const T xz = first ? T(0) : x;
+        if (part == 0) {
+            xs[i] = xz;
+            if (first) { ysl[0] = x; ysl[1] = y; }
+        }
+        {
+            T ss = xz * xz, xy = xz * y;
+            if (t > 0) {
+                // column sums of xz X0 over the warp's eight rows: exchange halves so that each
+                // lane ends with PH columns
+                T u[CPT];
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) u[q] = xz * X[q];
+                if (first)
+#pragma unroll
+                    for (int q = 0; q < CPT; ++q) xrow[c0 + q] = X[q];
+                int base = 0;
+#pragma unroll
+                for (int s = 0; s < 3; ++s) {
+                    const int o = 16 >> s;
+                    const int half = CPT >> (s + 1);
+                    const bool up = (lane & o) != 0;
+#pragma unroll
+                    for (int q = 0; q < half; ++q) {
+                        const T keep = up ? u[q + half] : u[q], give = up ? u[q] : u[q + half];
+                        u[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+                    base += up ? half : 0;
+                }
+#pragma unroll
+                for (int q = 0; q < PH; ++q) upart[warp][c0 + base + q] = u[q];
+            }
+#pragma unroll
+            for (int o = 16; o >= 4; o >>= 1) {
+                ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                if (t > 0) xy += __shfl_xor_sync(0xffffffffu, xy, o);
+            }
+            if (lane == 0) { red[0][warp] = ss; red[1][warp] = xy; }
+        }
+        __syncthreads();
+        // ---- the reflector (every thread computes the same scalars) and q = tau D v
+        const T alpha = ysl[0];
+        T ss = T(0), xy = T(0);
+#pragma unroll
+        for (int w = 0; w < NW; ++w) { ss += red[0][w]; xy += red[1][w]; }
+        T tau = T(0), beta = alpha, scl = T(0);
+        if (ss != T(0)) {
+            const T s2 = fma(alpha, alpha, ss), rn = rsq<T>(s2), nrm = s2 * rn;
+            beta = (alpha >= T(0)) ? -nrm : nrm;
+            tau = fma(fabs(alpha), rn, T(1));                 // (beta - alpha) / beta
+            scl = T(1) / (alpha - beta);
+        }
+        const T v = first ? T(1) : xz * scl;
+        if (part == 0) {
+            if (have_next) put(vout + i * kWords<T>, v, (unsigned)j + 1);
+            if (i == 0 && have_next) put(vout + B * kWords<T>, tau, (unsigned)j + 1);
+            vs[i] = v;
+        } else if (part == 1) {
+            const size_t slot = (size_t)j * a.S + t;
+            v2[slot * B + (i >= rs ? i - rs : i - rs + B)] = v;
+            if (i == 0) tau2[slot] = tau;
+        }
+        T qd;
+        {
+            T g = T(0);
+#pragma unroll
+            for (int q = 0; q < CPT; ++q) g = fma(D[q], xs[c0 + q], g);
+            g += __shfl_xor_sync(0xffffffffu, g, 1);
+            g += __shfl_xor_sync(0xffffffffu, g, 2);
+            const T dc = __shfl_sync(0xffffffffu, pick(D, rs % CPT), quad | (rs / CPT));
+            qd = tau * fma(scl, g, dc);
+        }
+        if (t > 0 && tid < B) {
+            T s = T(0);
+#pragma unroll
+            for (int w = 0; w < NW; ++w) s += upart[w][tid];
+            ps[tid] = tau * (fma(scl, s, xrow[tid]) - fma(scl, xy, ysl[1]) * vps[par][tid]);
+        }
+        if (part == 0) qs[i] = qd;
+        {
+            T kp = v * qd;
+#pragma unroll
+            for (int o = 16; o >= 4; o >>= 1) kp += __shfl_xor_sync(0xffffffffu, kp, o);
+            if (lane == 0) red[2][warp] = kp;
+        }
+        __syncthreads();
+        // ---- updates
+        T K = T(0);
+#pragma unroll
+        for (int w = 0; w < NW; ++w) K += red[2][w];
+        K *= T(0.5) * tau;
+        const T wi = fma(-K, v, qd);
+#pragma unroll
+        for (int q = 0; q < CPT; ++q) {
+            const int c = c0 + q;
+            const T vc = vs[c], wc = fma(-K, vc, qs[c]);
+            D[q] = fma(-v, wc, fma(-wi, vc, D[q]));
+        }
+        if (t > 0) {
+#pragma unroll
+            for (int q = 0; q < CPT; ++q) {
+                const int c = c0 + q;
+                X[q] = fma(-v, ps[c], fma(-y, vps[par][c], X[q]));
+            }
+            if (first) {  // the row that position t - 1 takes in at its next sweep
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) {
+                    const int c = c0 + q;
+                    put(rout + c * kWords<T>, c == rs ? beta : X[q], (unsigned)j + 1);
+                }
+                if (part == rs / CPT) put(rout + B * kWords<T>, pick(D, rs % CPT), (unsigned)j + 1);
+            }
+        } else {
+            if (first && part == rs / CPT) {
+                dout[j + 1] = (double)pick(D, rs % CPT);
+                eout[j] = (double)beta;
+            }
+            if (j == nsweep - 1 && i == (n - 1) % B) {
+                if (part == i / CPT) dout[n - 1] = (double)pick(D, i % CPT);
+                if (part == rs / CPT) eout[n - 2] = (double)pick(D, rs % CPT);
+            }
+        }
+        // The next step's packets go to the other buffer of vps, rows_ and msc while slower
+        // threads still read this one; every other shared array is written again only after
+        // the next step's first barrier.
+        rs = rs + 1 == B ? 0 : rs + 1;
+    }
+}
+
+template <typename T, int B>
+cudaError_t launch(cudaStream_t st, int n, const T *band, int ldb, double *d, double *e, T *v2, T *tau2,
+                   int *status, unsigned *sync, size_t sync_words, int num_sms)
+{
+    const int S = sb2st_steps(n, B);
+    int per_sm = 0;
+    cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chase_resident_kernel<T, B>, 4 * B, 0);
+    if (err != cudaSuccess) return err;
+    const size_t words = (size_t)S * kWords<T> * (B + 2);
+    if (S > per_sm * num_sms || 64 + 4 * words > sync_words) return cudaErrorNotSupported;
+    Args a;
+    a.n = n; a.ldb = ldb; a.S = S; a.status = status; a.spin_limit = spin_limit();
+    a.vmsg = reinterpret_cast<u64 *>(sync + 64);
+    a.rmsg = a.vmsg + words;
+    if ((err = cudaMemsetAsync(a.vmsg, 0, 2 * words * sizeof(u64), st)) != cudaSuccess) return err;
+    void *args[] = {&band, &v2, &tau2, &d, &e, &a};
+    EGB_COUNT_LAUNCH();
+    return cudaLaunchCooperativeKernel((void *)chase_resident_kernel<T, B>, dim3(S), dim3(4 * B), args, 0, st);
+}
+
+}  // namespace sys
+
+template <typename T>
+cudaError_t chase_resident(cudaStream_t st, int n, int b, const T *band, int ldb, double *d, double *e,
+                           T *v2, T *tau2, int *status, unsigned *sync, size_t sync_words, int num_sms)
+{
+    if (n < 3) return cudaErrorNotSupported;
+    if (b == 64) return sys::launch<T, 64>(st, n, band, ldb, d, e, v2, tau2, status, sync, sync_words, num_sms);
+    if (b == 32) return sys::launch<T, 32>(st, n, band, ldb, d, e, v2, tau2, status, sync, sync_words, num_sms);
+    return cudaErrorNotSupported;
+}
+template cudaError_t chase_resident<double>(cudaStream_t, int, int, const double *, int, double *, double *,
+                                            double *, double *, int *, unsigned *, size_t, int);
+template cudaError_t chase_resident<float>(cudaStream_t, int, int, const float *, int, double *, double *,
+                                           float *, float *, int *, unsigned *, size_t, int);
+
+}  // namespace egb

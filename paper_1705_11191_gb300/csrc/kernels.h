@@ -94,6 +94,10 @@ template <typename T>
 cudaError_t trsm_left_lower(cudaStream_t st, int trans, int n, int ncol, const T *L, int ldl,
                             const T *inv_diag, T *B, int ldb, T *work);
 
+// Words of the sync scratch of the cooperative kernels (grid barriers, exchanged partials,
+// packets of the bulge chase).
+constexpr size_t kSyncWords = 64 + 2 * (1024 + 64 + 1024 * 64 + 1024 * 64 * 64);
+
 // ---- full -> band (Eq. 11, first line) ----
 template <typename T>
 cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T *work,
@@ -107,6 +111,11 @@ int sb2st_steps(int n, int b);
 template <typename T>
 cudaError_t sb2st(cudaStream_t st, int n, int b, T *band, int ldb, double *d, double *e,
                   T *v2, T *tau2, int *status, unsigned *sync, int num_sms);
+// The chase with the band held on chip (b = 32 or 64, all step positions co-resident); else
+// cudaErrorNotSupported. Writes d and e itself. sync: kSyncWords words of scratch.
+template <typename T>
+cudaError_t chase_resident(cudaStream_t st, int n, int b, const T *band, int ldb, double *d, double *e,
+                           T *v2, T *tau2, int *status, unsigned *sync, size_t sync_words, int num_sms);
 template <typename T>
 cudaError_t extract_band(cudaStream_t st, int n, int b, const T *a, int lda, T *band, int ldb);
 

@@ -72,7 +72,7 @@ int ensure_workspace(elsi_gb_handle_s *h, int kz)
     } else {
         ENSURE(stein, double, 3 * n * kz + kz + 64);
     }
-    ENSURE(sync, unsigned, 64 + 2 * (1024 + 64 + 1024 * 64 + 1024 * 64 * 64));
+    ENSURE(sync, unsigned, kSyncWords);
     ENSURE(status, int, ST_WORDS);
     if (h->precision == ELSI_PREC_FP32_REFINE) {
         const size_t k = h->n_state;
