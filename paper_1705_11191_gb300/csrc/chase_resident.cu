@@ -31,11 +31,12 @@
 // n = 1531 51.3 -> 35.7 ms (a step's 28 000 FMAs at two a clock bound it).
 #include "common.cuh"
 #include "kernels.h"
+#include "packets.cuh"
 
 namespace egb {
 namespace sys {
 
-typedef unsigned long long u64;
+using namespace pkt;
 
 struct Args {
     int n, ldb, S;      // S positions = grid size; also the stride of the reflector slots
@@ -43,71 +44,6 @@ struct Args {
     int *status;
     long long spin_limit;
 };
-
-template <typename T> constexpr int kWords = (int)(sizeof(T) / 4);  // packet words per value
-
-__device__ __forceinline__ void st_relaxed(u64 *p, u64 v)
-{
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ u64 ld_relaxed(const u64 *p)
-{
-    u64 v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Packet word: 32 bits of the value, the sequence number (never 0) above them.
-__device__ __forceinline__ void put(u64 *p, float v, unsigned seq)
-{
-    st_relaxed(p, ((u64)seq << 32) | __float_as_uint(v));
-}
-__device__ __forceinline__ void put(u64 *p, double v, unsigned seq)
-{
-    const u64 u = (u64)__double_as_longlong(v);
-    st_relaxed(p, ((u64)seq << 32) | (u & 0xFFFFFFFFull));
-    st_relaxed(p + 1, ((u64)seq << 32) | (u >> 32));
-}
-__device__ __forceinline__ bool try_get(const u64 *p, unsigned seq, float &v)
-{
-    const u64 a = ld_relaxed(p);
-    v = __uint_as_float((unsigned)a);
-    return (unsigned)(a >> 32) == seq;
-}
-__device__ __forceinline__ bool try_get(const u64 *p, unsigned seq, double &v)
-{
-    const u64 a = ld_relaxed(p), b = ld_relaxed(p + 1);
-    v = __longlong_as_double((long long)((a & 0xFFFFFFFFull) | (b << 32)));
-    return (unsigned)(a >> 32) == seq && (unsigned)(b >> 32) == seq;
-}
-// Bounded wait for a packet; false when the limit is reached or another CTA has failed.
-template <typename T>
-__device__ __forceinline__ bool get(const u64 *p, unsigned seq, T &v, const Args &a)
-{
-    long long it = 0;
-    while (!try_get(p, seq, v)) {
-        if (++it > a.spin_limit) {
-            report_error(a.status, ELSI_ERR_TIMEOUT, (int)seq);
-            return false;
-        }
-        if ((it & 255) == 0 && *(volatile int *)(a.status + ST_CODE) != 0) return false;
-    }
-    return true;
-}
-
-template <typename T> __device__ __forceinline__ T rsq(T x);
-template <> __device__ __forceinline__ float rsq(float x) { return 1.0f / sqrtf(x); }
-template <> __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
-
-// a[q] for a run-time q without indexing registers
-template <typename T, int N>
-__device__ __forceinline__ T pick(const T (&a)[N], int q)
-{
-    T v = a[0];
-#pragma unroll
-    for (int k = 1; k < N; ++k) v = (k == q) ? a[k] : v;
-    return v;
-}
 
 template <typename T, int B>
 __global__ void __launch_bounds__(4 * B, 512 / (4 * B))
@@ -167,17 +103,21 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         {
             bool ok = true;
             if (tid < B) {
-                if (t > 0) ok = get(vin + tid * kWords<T>, (unsigned)j + 1, vps[par][tid], a);
+                T v = T(0);
+                if (t > 0) ok = get(vin + tid * kWords<T>, (unsigned)j + 1, v, a.spin_limit, a.status);
+                vps[par][tid] = v;
             } else if (tid < 2 * B) {
                 const int c = tid - B;
                 T v = T(0);
-                if (have_row) ok = get(rin + c * kWords<T>, (unsigned)j, v, a);
+                if (have_row) ok = get(rin + c * kWords<T>, (unsigned)j, v, a.spin_limit, a.status);
                 rows_[par][c] = v;
             } else if (tid == 2 * B) {
-                if (t > 0) ok = get(vin + B * kWords<T>, (unsigned)j + 1, msc[par][0], a);
+                T v = T(0);
+                if (t > 0) ok = get(vin + B * kWords<T>, (unsigned)j + 1, v, a.spin_limit, a.status);
+                msc[par][0] = v;
             } else if (tid == 2 * B + 32) {
                 T v = T(0);
-                if (have_row) ok = get(rin + B * kWords<T>, (unsigned)j, v, a);
+                if (have_row) ok = get(rin + B * kWords<T>, (unsigned)j, v, a.spin_limit, a.status);
                 msc[par][1] = v;
             }
             if (!ok) failed = 1;
@@ -261,13 +201,8 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         T ss = T(0), xy = T(0);
 #pragma unroll
         for (int w = 0; w < NW; ++w) { ss += red[0][w]; xy += red[1][w]; }
-        T tau = T(0), beta = alpha, scl = T(0);
-        if (ss != T(0)) {
-            const T s2 = fma(alpha, alpha, ss), rn = rsq<T>(s2), nrm = s2 * rn;
-            beta = (alpha >= T(0)) ? -nrm : nrm;
-            tau = fma(fabs(alpha), rn, T(1));                 // (beta - alpha) / beta
-            scl = T(1) / (alpha - beta);
-        }
+        T beta, tau, scl;
+        reflector<T>(alpha, ss, beta, tau, scl);
         const T v = first ? T(1) : xz * scl;
         if (part == 0) {
             if (have_next) put(vout + i * kWords<T>, v, (unsigned)j + 1);

@@ -28,45 +28,14 @@ __device__ __forceinline__ void report_error(int *status, int code, int aux)
     if (atomicCAS(status + ST_CODE, 0, code) == 0) status[ST_AUX] = aux;
 }
 
-// Default iteration limit of the SIMT spin waits of this library (the grid barrier of the
-// cooperative kernels and the progress flags of the bulge chase). Each iteration backs off
-// for 32-64 ns and reads a word from L2, so the limit is reached after seconds, far longer
+// Default iteration limit of the SIMT spin waits of this library (the packets of the panel
+// factorisation and the bulge chase, the progress flags of the general chase). Each
+// iteration reads a word from L2, so the limit is reached after seconds, far longer
 // than any legitimate wait; on expiry the waiting kernel records ELSI_ERR_TIMEOUT and
 // returns. The limit in force is read on the host at each launch (spin_limit()) and passed
 // to the kernel, so that a test can make a wait run out (elsi_gb_set_spin_limit).
 constexpr long long kSpinLimit = 1ll << 26;
 long long spin_limit();
-
-// Grid-wide barrier for cooperative launches (all CTAs co-resident by construction).
-// *count lives in global memory, is zero before the launch and only grows: every CTA
-// adds one at each barrier, so barrier number k (k = 1, 2, ...) is passed once the count
-// reaches k * nblocks. Nobody resets the count, which saves the round trips of a
-// generation word. A CTA that has polled the count more than `limit` times records
-// ELSI_ERR_TIMEOUT. Returns false if the wait timed out or another CTA reported an error;
-// the caller must then return.
-__device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, int *status,
-                                             long long limit)
-{
-    __shared__ int ok_flag;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        __threadfence();
-        atomicAdd(count, 1u);
-        volatile unsigned *vc = count;
-        volatile int *vst = status;
-        long long it = 0;
-        while (*vc < target) {
-            if (++it > limit) { report_error(status, ELSI_ERR_TIMEOUT, 0); ok = 0; break; }
-            if ((it & 255) == 0 && vst[ST_CODE] != 0) { ok = 0; break; }
-            __nanosleep(32);
-        }
-        __threadfence();
-        ok_flag = ok;
-    }
-    __syncthreads();
-    return ok_flag != 0;
-}
 
 template <typename T> __device__ __forceinline__ T dsqrt(T x);
 template <> __device__ __forceinline__ double dsqrt<double>(double x) { return sqrt(x); }

@@ -1,0 +1,114 @@
+// Values handed from one CTA to another of the same launch through global memory (L2): each
+// 64-bit word carries 32 bits of a value and, above them, a sequence number that is never 0
+// and is used once per word and launch. The reader polls the word itself, so a hand-over is
+// one store and one load: no fence, no separate flag. A binary64 value (or a pair of
+// binary32 values) is two words. The words are zeroed before they are used.
+#pragma once
+
+#include "common.cuh"
+
+namespace egb {
+namespace pkt {
+
+typedef unsigned long long u64;
+
+template <typename T> constexpr int kWords = (int)(sizeof(T) / 4);  // words per value
+
+__device__ __forceinline__ void st_relaxed(u64 *p, u64 v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ u64 ld_relaxed(const u64 *p)
+{
+    u64 v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ u64 word(unsigned v, unsigned seq) { return ((u64)seq << 32) | v; }
+__device__ __forceinline__ unsigned seq_of(u64 w) { return (unsigned)(w >> 32); }
+
+__device__ __forceinline__ void put(u64 *p, float v, unsigned seq) { st_relaxed(p, word(__float_as_uint(v), seq)); }
+__device__ __forceinline__ void put(u64 *p, double v, unsigned seq)
+{
+    st_relaxed(p, word((unsigned)__double2loint(v), seq));
+    st_relaxed(p + 1, word((unsigned)__double2hiint(v), seq));
+}
+__device__ __forceinline__ bool try_get(const u64 *p, unsigned seq, float &v)
+{
+    const u64 a = ld_relaxed(p);
+    v = __uint_as_float((unsigned)a);
+    return seq_of(a) == seq;
+}
+__device__ __forceinline__ bool try_get(const u64 *p, unsigned seq, double &v)
+{
+    const u64 a = ld_relaxed(p), b = ld_relaxed(p + 1);
+    v = __hiloint2double((int)(unsigned)b, (int)(unsigned)a);
+    return seq_of(a) == seq && seq_of(b) == seq;
+}
+
+// One failed poll: counts it, false when the wait has to be given up (the limit is reached,
+// which is recorded, or another CTA has recorded an error).
+__device__ __forceinline__ bool poll_again(long long &it, long long limit, int *status, int aux)
+{
+    if (++it > limit) {
+        report_error(status, ELSI_ERR_TIMEOUT, aux);
+        return false;
+    }
+    return (it & 255) != 0 || *(volatile int *)(status + ST_CODE) == 0;
+}
+
+// Bounded wait for a value.
+template <typename T>
+__device__ __forceinline__ bool get(const u64 *p, unsigned seq, T &v, long long limit, int *status)
+{
+    long long it = 0;
+    while (!try_get(p, seq, v))
+        if (!poll_again(it, limit, status, (int)seq)) return false;
+    return true;
+}
+
+}  // namespace pkt
+
+// 1 / sqrt(x): in binary64 the division and the square root are long sequences on the chip's
+// few binary64 units, the reciprocal square root a shorter one.
+template <typename T> __device__ __forceinline__ T rsq(T x);
+template <> __device__ __forceinline__ float rsq(float x) { return 1.0f / sqrtf(x); }
+template <> __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+
+// Householder scalars of x = (alpha, tail) with |tail|^2 = ss: v = (1, scl tail), H = I - tau
+// v v^T, H x = beta e_1.
+template <typename T>
+__device__ __forceinline__ void reflector(T alpha, T ss, T &beta, T &tau, T &scl)
+{
+    beta = alpha;
+    tau = scl = T(0);
+    if (ss != T(0)) {
+        const T s2 = fma(alpha, alpha, ss), rn = rsq<T>(s2), nrm = s2 * rn;
+        beta = (alpha >= T(0)) ? -nrm : nrm;
+        tau = fma(fabs(alpha), rn, T(1));  // (beta - alpha) / beta
+        scl = T(1) / (alpha - beta);
+    }
+}
+
+// v = a where q == k: a predicated move that the compiler cannot turn into an indexed access
+// (which would put the array that a comes from into local memory).
+__device__ __forceinline__ void move_if(float &v, float a, int q, int k)
+{
+    asm("{\n .reg .pred p;\n setp.eq.s32 p, %2, %3;\n @p mov.b32 %0, %1;\n}\n" : "+f"(v) : "f"(a), "r"(q), "r"(k));
+}
+__device__ __forceinline__ void move_if(double &v, double a, int q, int k)
+{
+    asm("{\n .reg .pred p;\n setp.eq.s32 p, %2, %3;\n @p mov.b64 %0, %1;\n}\n" : "+d"(v) : "d"(a), "r"(q), "r"(k));
+}
+
+// a[q] for a run-time q without indexing registers
+template <typename T, int N>
+__device__ __forceinline__ T pick(const T (&a)[N], int q)
+{
+    T v = a[0];
+#pragma unroll
+    for (int k = 1; k < N; ++k) move_if(v, a[k], q, k);
+    return v;
+}
+
+}  // namespace egb

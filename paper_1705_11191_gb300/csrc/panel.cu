@@ -1,0 +1,348 @@
+// QR factorisation of one panel (m x bw, bw <= 64) of the full -> band reduction: Householder
+// reflectors column by column and the compact-WY factor T (Q = I - V T V^T).
+//
+// What bounds it: bw columns one after the other, each with a sum over all rows between the
+// column and the update, so the time is bw times the latency of one all-to-all exchange plus
+// the arithmetic of the CTA with the most rows. With the panel in shared memory, a grid
+// barrier per column and the partial sums read after it, a column took 12.5 us in binary32
+// and 18 us in binary64.
+//
+// Layout: lane l of warp w holds columns l and l + 32 of RW consecutive rows in registers for
+// the whole factorisation, so the column sums and the rank-1 update need no exchange between
+// lanes; the current column reaches the other lanes through one broadcast from shared memory.
+// A CTA publishes its 64 column sums as packets (packets.cuh) and every CTA polls the packets
+// of all others directly: one store and one load through L2 per column, no barrier between
+// CTAs. The sums x_j . P_c over the rows below j serve three uses at once: c = j is the
+// column's squared norm, c > j gives the update and c < j, where the storage already holds
+// the reflectors, the Gram column for T. T itself is formed by one extra CTA that reads the
+// same packets and is never waited for.
+//
+// Sums over CTAs are kept to more than the panel's precision: binary32 partial sums are added
+// with their rounding errors (Knuth's two-sum), since binary64 additions are scarce here.
+//
+// Measured per 64-column panel, before -> now: binary32 n = 777 0.73 -> 0.21 ms, n = 4096 0.82
+// -> 0.24 ms, n = 16384 0.85 -> 0.29 ms; binary64 n = 512 1.09 -> 0.40 ms, n = 5000 1.24 ->
+// 0.51 ms. What is left is one L2 exchange a column (about 1.5 us) and, in binary64, the
+// 2 x 64 x 64 FMAs of a CTA's rows at two a clock.
+#include "common.cuh"
+#include "kernels.h"
+#include "packets.cuh"
+
+namespace egb {
+namespace pan {
+
+using namespace pkt;
+
+struct Args {
+    int m, bw, lda, ldv, G, gs;  // G row CTAs (one more forms T); gs >= G the packet stride
+    unsigned seq0;               // the packets of column j carry seq0 + j + 1
+    u64 *dpk;                    // [64][gs][64][2]: column sums
+    u64 *rpk;                    // [64][64][2]: row j of the panel
+    int *status;
+    long long spin_limit;
+};
+
+// A sum with at least the precision of binary64 accumulation of binary32 terms, or a plain
+// binary64 one; two packet words either way.
+template <typename T> struct Sum;
+template <> struct Sum<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ void add(const Sum &o) { v += o.v; }
+    __device__ __forceinline__ double value() const { return v; }
+    __device__ __forceinline__ unsigned w0() const { return (unsigned)__double2loint(v); }
+    __device__ __forceinline__ unsigned w1() const { return (unsigned)__double2hiint(v); }
+    __device__ __forceinline__ static Sum from(unsigned a, unsigned b) { Sum s; s.v = __hiloint2double((int)b, (int)a); return s; }
+    __device__ __forceinline__ Sum other(int o) const { Sum s; s.v = __shfl_xor_sync(0xffffffffu, v, o); return s; }
+};
+template <> struct Sum<float> {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float s = h + x, b = s - h;
+        l += (h - (s - b)) + (x - b);
+        h = s;
+    }
+    __device__ __forceinline__ void add(const Sum &o) { add(o.h); l += o.l; }
+    __device__ __forceinline__ float value() const { return h + l; }
+    __device__ __forceinline__ unsigned w0() const { return __float_as_uint(h); }
+    __device__ __forceinline__ unsigned w1() const { return __float_as_uint(l); }
+    __device__ __forceinline__ static Sum from(unsigned a, unsigned b) { Sum s; s.h = __uint_as_float(a); s.l = __uint_as_float(b); return s; }
+    __device__ __forceinline__ Sum other(int o) const
+    {
+        Sum s;
+        s.h = __shfl_xor_sync(0xffffffffu, h, o);
+        s.l = __shfl_xor_sync(0xffffffffu, l, o);
+        return s;
+    }
+};
+
+__device__ __forceinline__ void ld2_relaxed(const u64 *p, u64 &a, u64 &b)
+{
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+
+// RW rows per warp, CPL columns per lane (bw <= 32 CPL), NW warps.
+template <typename T, int RW, int CPL, int NW>
+constexpr size_t smem_bytes()
+{
+    const size_t tile = (size_t)NW * 32 * CPL * (RW + 1) * sizeof(T);
+    const size_t tm = (size_t)64 * 65 * sizeof(double);
+    return tile > tm ? tile : tm;
+}
+
+template <typename T, int RW, int CPL, int NW>
+__global__ void __launch_bounds__(32 * NW, 512 / (32 * NW))
+panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
+{
+    constexpr int NC = 32 * CPL;       // columns held (zero beyond bw)
+    constexpr int LPC = 32 * NW / NC;  // threads per column in the exchange
+    constexpr int RPL = 32 / RW;       // columns of a warp's rows moved by one access
+    constexpr int FLY = 8;             // packets of a thread in flight
+    static_assert(LPC >= 4 && LPC <= 16 && NW % LPC == 0 && RW <= 32, "layout");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(16) T xbuf[NW][RW];
+    __shared__ T partw[NW][NC];
+    __shared__ T rowown[NC], dsum[NC], rowj[NC], scal[3];
+    __shared__ int failed;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int g = blockIdx.x, G = a.G, bw = a.bw;
+    const int row0 = (g * NW + warp) * RW;  // first row of the warp
+    T *tile = reinterpret_cast<T *>(smem_raw) + (size_t)warp * NC * (RW + 1);
+    double(*Ts)[65] = reinterpret_cast<double(*)[65]>(smem_raw);  // CTA G
+    const int nref = min(bw, a.m);
+    const int rl = lane % RW, cl = lane / RW;  // row and column of a lane in the copies
+
+    T p[CPL][RW];
+    if (tid == 0) failed = 0;
+    if (g < G) {
+#pragma unroll 8
+        for (int c = cl; c < NC; c += RPL)
+            tile[c * (RW + 1) + rl] =
+                (row0 + rl < a.m && c < bw) ? P[(size_t)(row0 + rl) + (size_t)c * a.lda] : T(0);
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < CPL; ++h)
+#pragma unroll
+            for (int i = 0; i < RW; ++i) p[h][i] = tile[(h * 32 + lane) * (RW + 1) + i];
+    } else {
+        for (int e = tid; e < 64 * 65; e += 32 * NW) Ts[0][e] = 0.0;
+    }
+    __syncthreads();
+
+    const int xc = tid / LPC, xg = tid % LPC;  // column and share of this thread in the exchange
+    for (int j = 0; j < nref; ++j) {
+        const unsigned seq = a.seq0 + (unsigned)j + 1;
+        Sum<T> tot;
+        if (g < G) {
+            // ---- column sums of x P over the rows below j
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < RW; ++i) {
+                T x = p[0][i];
+                if (CPL == 2 && j >= 32) x = p[CPL - 1][i];
+                if (lane == (j & 31)) xbuf[warp][i] = (row0 + i > j) ? x : T(0);
+            }
+            __syncwarp();
+            T s[CPL][2] = {};
+#pragma unroll
+            for (int i = 0; i < RW; i += 2)
+#pragma unroll
+                for (int c = 0; c < CPL; ++c) {
+                    s[c][0] = fma(xbuf[warp][i], p[c][i], s[c][0]);
+                    s[c][1] = fma(xbuf[warp][i + 1], p[c][i + 1], s[c][1]);
+                }
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) partw[warp][c * 32 + lane] = s[c][0] + s[c][1];
+            if (g == 0 && warp == j / RW)
+#pragma unroll
+                for (int c = 0; c < CPL; ++c) {
+                    const T x = pick(p[c], j % RW);
+                    rowown[c * 32 + lane] = x;
+                    put(a.rpk + (size_t)(j * 64 + c * 32 + lane) * 2, x, seq);
+                }
+            __syncthreads();
+            Sum<T> sm;
+#pragma unroll
+            for (int w = 0; w < NW / LPC; ++w) sm.add(partw[xg * (NW / LPC) + w][xc]);
+#pragma unroll
+            for (int o = 1; o < LPC; o <<= 1) sm.add(sm.other(o));
+            if (xg == 0) {
+                u64 *d = a.dpk + ((size_t)(j * a.gs + g) * 64 + xc) * 2;
+                st_relaxed(d, word(sm.w0(), seq));
+                st_relaxed(d + 1, word(sm.w1(), seq));
+            }
+            tot = sm;
+        }
+        // ---- the sums of all CTAs, and row j
+        bool ok = true;
+        T row = T(0);
+        if (G > 1 || g == G) {
+            tot = Sum<T>();
+            for (int q0 = xg; q0 < G && ok; q0 += LPC * FLY) {
+                u64 w0[FLY], w1[FLY];
+                long long it = 0;
+                for (;;) {
+                    bool ready = true;
+#pragma unroll
+                    for (int u = 0; u < FLY; ++u) {
+                        const int q = q0 + LPC * u;
+                        if (q < G) ld2_relaxed(a.dpk + ((size_t)(j * a.gs + q) * 64 + xc) * 2, w0[u], w1[u]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < FLY; ++u)
+                        if (q0 + LPC * u < G) ready = ready && seq_of(w0[u]) == seq && seq_of(w1[u]) == seq;
+                    if (ready) break;
+                    if (!poll_again(it, a.spin_limit, a.status, j)) { ok = false; break; }
+                }
+#pragma unroll
+                for (int u = 0; u < FLY; ++u)
+                    if (ok && q0 + LPC * u < G) tot.add(Sum<T>::from((unsigned)w0[u], (unsigned)w1[u]));
+            }
+            __syncwarp();
+#pragma unroll
+            for (int o = 1; o < LPC; o <<= 1) tot.add(tot.other(o));
+        }
+        if (xg == 0) {
+            if (g == 0) row = rowown[xc];
+            else ok = get(a.rpk + (size_t)(j * 64 + xc) * 2, seq, row, a.spin_limit, a.status) && ok;
+            const T d = tot.value();
+            dsum[xc] = d;
+            rowj[xc] = row;
+            if (xc == j) {
+                T beta, tau, scl;
+                reflector<T>(row, d, beta, tau, scl);
+                scal[0] = beta; scal[1] = tau; scal[2] = scl;
+            }
+        }
+        if (!ok) failed = 1;
+        __syncthreads();
+        if (failed) return;
+        const T beta = scal[0], tau = scal[1], scl = scal[2];
+        if (g < G) {
+            // ---- P_c -= v (tau v . P_c), c > j; column j becomes the reflector
+            T wv[CPL];
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+                const int col = c * 32 + lane;
+                wv[c] = col > j ? tau * fma(scl, dsum[col], rowj[col]) : T(0);
+            }
+#pragma unroll
+            for (int i = 0; i < RW; ++i) {
+                const T v = xbuf[warp][i] * scl;
+#pragma unroll
+                for (int c = 0; c < CPL; ++c) {
+                    p[c][i] = fma(-v, wv[c], p[c][i]);
+                    if (c * 32 + lane == j && row0 + i > j) p[c][i] = v;
+                }
+            }
+            if (g == 0 && warp == j / RW) {
+#pragma unroll
+                for (int i = 0; i < RW; ++i)
+#pragma unroll
+                    for (int c = 0; c < CPL; ++c)
+                        move_if(p[c][i], c * 32 + lane == j ? beta : p[c][i] - wv[c], j % RW, i);
+            }
+        } else {
+            // ---- T[0:j, j] = -tau T[0:j, 0:j] (v_c . v_j), forward recurrence
+            double acc = 0.0;
+            if (xc < j)
+                for (int q = xc + xg; q < j; q += LPC) acc += Ts[xc][q] * ((double)scl * (double)dsum[q] + (double)rowj[q]);
+            __syncwarp();
+#pragma unroll
+            for (int o = 1; o < LPC; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (xg == 0 && xc <= j) Ts[xc][j] = xc < j ? -(double)tau * acc : (double)tau;
+            __syncthreads();
+        }
+    }
+    __syncthreads();
+    if (g == G) {
+        for (int e = tid; e < bw * bw; e += 32 * NW) {
+            const int r = e % bw, c = e / bw;
+            Tm[(size_t)r + (size_t)c * ldt] = (T)Ts[r][c];
+        }
+        return;
+    }
+    // ---- the panel (R on and above the diagonal, reflector tails below) and the explicit V
+    //      (unit diagonal, zero above) for the products of the update
+#pragma unroll
+    for (int h = 0; h < CPL; ++h)
+#pragma unroll
+        for (int i = 0; i < RW; ++i) tile[(h * 32 + lane) * (RW + 1) + i] = p[h][i];
+    __syncwarp();
+    const int gi = row0 + rl;
+    if (gi < a.m)
+#pragma unroll 4
+        for (int c = cl; c < bw; c += RPL) {
+            const T pv = tile[c * (RW + 1) + rl];
+            P[(size_t)gi + (size_t)c * a.lda] = pv;
+            V[(size_t)gi + (size_t)c * a.ldv] = (c >= nref || gi < c) ? T(0) : (gi == c ? T(1) : pv);
+        }
+}
+
+template <typename T, int RW, int CPL, int NW>
+cudaError_t launch(cudaStream_t st, T *P, T *V, T *Tm, int ldt, Args a, int num_sms, bool *fits)
+{
+    constexpr size_t smem = smem_bytes<T, RW, CPL, NW>();
+    static PerDeviceOnce attr;  // per instantiation
+    cudaError_t e = once_per_device(attr, [] {
+        return cudaFuncSetAttribute(panel_kernel<T, RW, CPL, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    });
+    if (e != cudaSuccess) return e;
+    a.G = ceil_div(a.m, RW * NW);
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, panel_kernel<T, RW, CPL, NW>, 32 * NW, smem);
+    if (e != cudaSuccess) return e;
+    *fits = a.G + 1 <= per_sm * num_sms && a.G <= a.gs;
+    if (!*fits) return cudaSuccess;
+    void *args[] = {&P, &V, &Tm, &ldt, &a};
+    EGB_COUNT_LAUNCH();
+    return cudaLaunchCooperativeKernel((void *)panel_kernel<T, RW, CPL, NW>, dim3(a.G + 1), dim3(32 * NW), args, smem, st);
+}
+
+template <typename T, int CPL>
+cudaError_t choose(cudaStream_t st, T *P, T *V, T *Tm, int ldt, const Args &a, int num_sms)
+{
+    // Rows per CTA. Binary32: the exchange costs more than the arithmetic, so 256, and 512 once
+    // that gives more than 32 CTAs (one round of packets in flight). Binary64: two FMAs a clock
+    // make the arithmetic of a CTA's rows the larger part, so 64 where the CTAs fit.
+    bool fits = false;
+    cudaError_t e = cudaSuccess;
+    if constexpr (sizeof(T) == 4) {
+        if (a.m <= 32 * 256) e = launch<T, 32, CPL, 8>(st, P, V, Tm, ldt, a, num_sms, &fits);
+        if (e == cudaSuccess && !fits) e = launch<T, 32, CPL, 16>(st, P, V, Tm, ldt, a, num_sms, &fits);
+    } else {
+        e = launch<T, 8, CPL, 8>(st, P, V, Tm, ldt, a, num_sms, &fits);
+        if (e == cudaSuccess && !fits) e = launch<T, 16, CPL, 16>(st, P, V, Tm, ldt, a, num_sms, &fits);
+    }
+    if (e != cudaSuccess) return e;
+    return fits ? cudaSuccess : cudaErrorInvalidConfiguration;
+}
+
+}  // namespace pan
+
+size_t panel_packet_words(int m, int elem)
+{
+    const int gs = ceil_div(m, elem == 4 ? 256 : 64);
+    return (size_t)64 * 64 * 2 * (gs + 1);
+}
+
+template <typename T>
+cudaError_t panel_qr(cudaStream_t st, int m, int m_first, int bw, T *P, int lda, T *V, int ldv, T *Tm, int ldt,
+                     unsigned seq0, unsigned long long *packets, int *status, int num_sms)
+{
+    if (bw < 1 || bw > 64) return cudaErrorInvalidValue;
+    pan::Args a;
+    a.m = m; a.bw = bw; a.lda = lda; a.ldv = ldv; a.G = 0;
+    a.gs = ceil_div(m_first, sizeof(T) == 4 ? 256 : 64);
+    a.seq0 = seq0; a.rpk = packets; a.dpk = packets + 64 * 64 * 2;
+    a.status = status; a.spin_limit = spin_limit();
+    return bw <= 32 ? pan::choose<T, 1>(st, P, V, Tm, ldt, a, num_sms)
+                    : pan::choose<T, 2>(st, P, V, Tm, ldt, a, num_sms);
+}
+template cudaError_t panel_qr<double>(cudaStream_t, int, int, int, double *, int, double *, int, double *, int,
+                                      unsigned, unsigned long long *, int *, int);
+template cudaError_t panel_qr<float>(cudaStream_t, int, int, int, float *, int, float *, int, float *, int,
+                                     unsigned, unsigned long long *, int *, int);
+
+}  // namespace egb

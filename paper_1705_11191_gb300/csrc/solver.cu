@@ -72,7 +72,7 @@ int ensure_workspace(elsi_gb_handle_s *h, int kz)
     } else {
         ENSURE(stein, double, 3 * n * kz + kz + 64);
     }
-    ENSURE(sync, unsigned, kSyncWords);
+    ENSURE(sync, unsigned, sync_words(h->n, (int)eb));
     ENSURE(status, int, ST_WORDS);
     if (h->precision == ELSI_PREC_FP32_REFINE) {
         const size_t k = h->n_state;

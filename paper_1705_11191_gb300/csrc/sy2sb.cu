@@ -6,267 +6,11 @@
 // two-sided update A22 <- Q_p^T A22 Q_p = A22 - V W^T - W V^T with
 // X = A22 V T and W = X - (1/2) V (T^T (V^T X)).
 //
-// The panel QR is one cooperative launch: the m x b panel is split by rows over G CTAs,
-// each holding its rows in shared memory; one grid barrier per column exchanges the
-// partial norm and the partial products of the column with the remaining columns. The
-// trailing update is GEMM work.
-#include <cooperative_groups.h>
-
+// The panel QR is one cooperative launch (panel.cu); the trailing update is GEMM work.
 #include "common.cuh"
 #include "kernels.h"
 
 namespace egb {
-
-struct PanelArgs {
-    int m, bw, rows_per_cta;
-    int lda, ldv;
-    unsigned *count;         // grid barrier counter (zeroed before the launch)
-    double *part;            // 2 x gstride partial norms (by column parity)
-    double *alpha;           // 2 x 64: row j of the panel (by column parity)
-    double *wpart;           // 2 x gstride x 64 partial dot products (by column parity)
-    int gstride;             // >= G
-    double *gram;            // scratch of the W kernels (not used by the panel kernel)
-    int *status;
-    long long spin_limit;    // polls of a grid-barrier wait before ELSI_ERR_TIMEOUT
-};
-
-template <typename T>
-__global__ void __launch_bounds__(256) panel_qr_kernel(T *P, T *V, T *Tm, int ldt, PanelArgs a)
-{
-    extern __shared__ unsigned char smem_raw[];
-    const int bw = a.bw, bwp = bw + 1;
-    const int R = a.rows_per_cta;
-    T *Ploc = reinterpret_cast<T *>(smem_raw);          // R x bwp, row-major
-    __shared__ double red[32];
-    __shared__ double tau_s[64];
-    __shared__ double wsum[64];
-    __shared__ double colpart[4][64];
-    __shared__ double prow_s[64];  // row j of the panel (published by the CTA holding it)
-    __shared__ double refl[3];  // beta, tau, 1 / (alpha - beta) of the current column
-    const int g = blockIdx.x, G = gridDim.x;
-    const int tid = threadIdx.x;
-    const int row0 = g * R;
-    const int nrow = max(0, min(a.m - row0, R));
-    const int tc = tid & 63, tr = tid >> 6;  // 64 column lanes x 4 row lanes
-    // T of the compact-WY form, column by column (CTA 0), after the panel rows
-    double *tloc = reinterpret_cast<double *>(smem_raw + (((size_t)R * bwp * sizeof(T) + 15) & ~(size_t)15));
-
-    // the panel rows of this CTA, 16 loads of a thread in flight at a time
-    for (int e0 = 0; e0 < R * bw; e0 += 16 * 256) {
-        T v[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            const int e = e0 + u * 256 + tid, i = e % R, c = e / R;
-            v[u] = (e < R * bw && i < nrow) ? P[(size_t)(row0 + i) + (size_t)c * a.lda] : T(0);
-        }
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            const int e = e0 + u * 256 + tid, i = e % R, c = e / R;
-            if (e < R * bw) Ploc[i * bwp + c] = v[u];
-        }
-    }
-    if (g == 0)
-        for (int e = tid; e < 64 * 64; e += blockDim.x) tloc[e] = 0.0;
-    __syncthreads();
-    // sum over the rows gi >= first (gi = row0 + i, i = tr, tr + 4, ...) of x_i Ploc[i][c],
-    // x_i = Ploc[i][col] (1 at gi == col when unit): four independent partial sums
-    auto col_dot = [&](int c, int col, int first, bool unit) -> T {
-        auto xv = [&](int i) -> T {
-            const int gi = row0 + i;
-            return gi < first ? T(0) : ((unit && gi == col) ? T(1) : Ploc[i * bwp + col]);
-        };
-        T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
-        int i = tr;
-        for (; i + 12 < nrow; i += 16) {
-            s0 = fma(xv(i), Ploc[i * bwp + c], s0);
-            s1 = fma(xv(i + 4), Ploc[(i + 4) * bwp + c], s1);
-            s2 = fma(xv(i + 8), Ploc[(i + 8) * bwp + c], s2);
-            s3 = fma(xv(i + 12), Ploc[(i + 12) * bwp + c], s3);
-        }
-        for (; i < nrow; i += 4) s0 = fma(xv(i), Ploc[i * bwp + c], s0);
-        return (s0 + s1) + (s2 + s3);
-    };
-
-    const int nref = min(bw, a.m);
-    // One grid barrier per column. Before it, every CTA publishes (for column j, already
-    // updated by reflectors 0..j-1) the partial sum of squares below the diagonal and the
-    // unscaled partial dot products d_c = sum_{i>j} x_i P[i][c] (c > j); the CTA holding
-    // row j publishes that row. After it, every CTA forms the same reflector
-    // v = [1; x scl] and w_c = v . P_c = P[j][c] + scl d_c, and updates its rows. The
-    // published values alternate between two buffers by column parity: a CTA can be at
-    // most one column ahead of another. The free slots c < j - 1 of the same exchange
-    // carry the partial Gram column G[c][j-1] = v_c . v_(j-1) of the finished reflectors,
-    // from which CTA 0 forms column j - 1 of T (forward recurrence) while the others
-    // update their rows.
-    for (int j = 0; j < nref; ++j) {
-        const int par = j & 1;
-        double *part = a.part + (size_t)par * a.gstride;              // [G]
-        double *dpart = a.wpart + (size_t)par * a.gstride * 64;       // [G][64]
-        double *prow = a.alpha + par * 64;                            // [64]
-        {
-            T ss = T(0), s = T(0);
-            const int c = tc;
-            for (int i = tid; i < nrow; i += blockDim.x)
-                if (row0 + i > j) { T x = Ploc[i * bwp + j]; ss = fma(x, x, ss); }
-            if (c > j && c < bw) s = col_dot(c, j, j + 1, false);
-            // v_c . v_(j-1) over the rows >= j - 1 (v_c is zero above c)
-            if (c < j - 1) s = col_dot(c, j - 1, j - 1, true);
-            colpart[tr][tc] = (double)s;
-            double sst = block_sum((double)ss, red);  // also orders colpart
-            if (tid < bw)
-                dpart[(size_t)g * 64 + tid] = colpart[0][tid] + colpart[1][tid] + colpart[2][tid] + colpart[3][tid];
-            if (tid == 0) part[g] = sst;
-            if (j >= row0 && j < row0 + nrow && tid >= j && tid < bw)
-                prow[tid] = (double)Ploc[(j - row0) * bwp + tid];
-        }
-        if (!grid_barrier(a.count, (unsigned)G * (unsigned)(j + 1), a.status, a.spin_limit)) return;
-        // ---- reflector of column j (every CTA computes the same numbers)
-        {
-            // sigma2 by warp 0; d_c by 64 column lanes x 4 row groups of CTAs
-            if (tid < 32) {
-                double v = 0.0;
-                for (int q = tid; q < G; q += 32) v += __ldcg(part + q);
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (tid == 0) red[0] = v;
-            }
-            // L2-coherent loads (written by other CTAs before the barrier), all issued
-            // before they are summed
-            // (up to 64 CTAs: all 16 loads of a thread in flight at once)
-            // row j entries c >= j, loaded with the partials (one round trip for both)
-            const double pv = (tid >= j && tid < bw) ? __ldcg(prow + tid) : 0.0;
-            double dv = 0.0;
-            if ((tc > j && tc < bw) || tc < j - 1) {
-                double acc[16];
-#pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    const int q = tr + 4 * u;
-                    acc[u] = (q < G) ? __ldcg(dpart + (size_t)q * 64 + tc) : 0.0;
-                }
-                for (int q = tr + 64; q < G; q += 4) acc[0] += __ldcg(dpart + (size_t)q * 64 + tc);
-#pragma unroll
-                for (int h = 8; h > 0; h >>= 1)
-#pragma unroll
-                    for (int u = 0; u < h; ++u) acc[u] += acc[u + h];
-                dv = acc[0];
-            }
-            colpart[tr][tc] = dv;
-            if (tid < bw) prow_s[tid] = pv;
-            __syncthreads();
-            if (tid < bw) wsum[tid] = colpart[0][tid] + colpart[1][tid] + colpart[2][tid] + colpart[3][tid];
-            // the reflector's scalars, once, in the panel's precision (one thread's
-            // binary64 square root and two divisions per column cost microseconds on this
-            // chip, whose binary64 units are few)
-            if (tid == 0) {
-                const T sigma2 = (T)red[0];
-                const T alpha = (T)prow_s[j];
-                if (sigma2 == T(0)) { refl[0] = (double)alpha; refl[1] = 0.0; refl[2] = 0.0; }
-                else {
-                    const T nrm = dsqrt<T>(fma(alpha, alpha, sigma2));
-                    const T bt = (alpha >= T(0)) ? -nrm : nrm;
-                    refl[0] = (double)bt;
-                    refl[1] = (double)((bt - alpha) / bt);
-                    refl[2] = (double)(T(1) / (alpha - bt));
-                }
-            }
-            __syncthreads();
-        }
-        const double beta = refl[0], tau = refl[1], scl = refl[2];
-        // column j - 1 of T: T[c][j-1] = -tau_(j-1) sum_(c <= q < j-1) T[c][q] G[q][j-1]
-        if (g == 0 && j >= 1) {
-            if (tid < j - 1) {
-                double acc = 0.0;
-                for (int q = tid; q < j - 1; ++q) acc += tloc[tid + q * 64] * wsum[q];
-                tloc[tid + (j - 1) * 64] = -tau_s[j - 1] * acc;
-            }
-            if (tid == 0) tloc[(j - 1) + (j - 1) * 64] = tau_s[j - 1];
-            __syncthreads();
-        }
-        // w_c = P[j][c] + scl d_c; stored pre-multiplied by tau
-        if (tid > j && tid < bw) wsum[tid] = tau * (prow_s[tid] + scl * wsum[tid]);
-        __syncthreads();
-        const T sclT = (T)scl;
-        for (int i = tid; i < nrow; i += blockDim.x)
-            if (row0 + i > j) Ploc[i * bwp + j] = Ploc[i * bwp + j] * sclT;
-        __syncthreads();
-        {
-            const int c = tc;
-            if (c > j && c < bw) {
-                const T wt = (T)wsum[c];
-#pragma unroll 4
-                for (int i = tr; i < nrow; i += 4) {
-                    const int gi = row0 + i;
-                    if (gi >= j) {
-                        const T v = (gi == j) ? T(1) : Ploc[i * bwp + j];
-                        Ploc[i * bwp + c] = fma(-v, wt, Ploc[i * bwp + c]);
-                    }
-                }
-            }
-        }
-        if (tid == 0) tau_s[j] = tau;
-        __syncthreads();
-        if (tid == 0 && j >= row0 && j < row0 + nrow) Ploc[(j - row0) * bwp + j] = (T)beta;
-        __syncthreads();
-    }
-    if (tid == 0)
-        for (int j = nref; j < bw; ++j) tau_s[j] = 0.0;
-    __syncthreads();
-
-    // ---- write back the panel (R on/above the diagonal, reflector tails below) and the
-    //      explicit V (unit diagonal, zeros above) for the GEMM updates
-    for (int e = tid; e < nrow * bw; e += blockDim.x) {
-        int i = e % nrow, c = e / nrow;
-        int gi = row0 + i;
-        T pv = Ploc[i * bwp + c];
-        P[(size_t)gi + (size_t)c * a.lda] = pv;
-        T vv = (c >= nref) ? T(0) : ((gi > c) ? pv : ((gi == c) ? T(1) : T(0)));
-        V[(size_t)gi + (size_t)c * a.ldv] = vv;
-    }
-    // ---- the last column of T: partial Gram column G[c][nref-1] (c < nref - 1) through the
-    //      buffer of the next parity, one more barrier, then CTA 0 sums and finishes T
-    const int jl = nref - 1;
-    {
-        double *dpart = a.wpart + (size_t)(nref & 1) * a.gstride * 64;
-        const T s = (tc < jl) ? col_dot(tc, jl, jl, true) : T(0);
-        colpart[tr][tc] = (double)s;
-        __syncthreads();
-        if (tid < bw) dpart[(size_t)g * 64 + tid] = colpart[0][tid] + colpart[1][tid] + colpart[2][tid] + colpart[3][tid];
-    }
-    if (!grid_barrier(a.count, (unsigned)G * (unsigned)(nref + 1), a.status, a.spin_limit)) return;
-    if (g != 0) return;
-    {
-        const double *dpart = a.wpart + (size_t)(nref & 1) * a.gstride * 64;
-        double dv = 0.0;
-        if (tc < jl) {
-            double acc[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) {
-                const int q = tr + 4 * u;
-                acc[u] = (q < G) ? __ldcg(dpart + (size_t)q * 64 + tc) : 0.0;
-            }
-            for (int q = tr + 64; q < G; q += 4) acc[0] += __ldcg(dpart + (size_t)q * 64 + tc);
-#pragma unroll
-            for (int h = 8; h > 0; h >>= 1)
-#pragma unroll
-                for (int u = 0; u < h; ++u) acc[u] += acc[u + h];
-            dv = acc[0];
-        }
-        colpart[tr][tc] = dv;
-        __syncthreads();
-        if (tid < bw) wsum[tid] = colpart[0][tid] + colpart[1][tid] + colpart[2][tid] + colpart[3][tid];
-        __syncthreads();
-        if (tid < jl) {
-            double acc = 0.0;
-            for (int q = tid; q < jl; ++q) acc += tloc[tid + q * 64] * wsum[q];
-            tloc[tid + jl * 64] = -tau_s[jl] * acc;
-        }
-        if (tid == 0) tloc[jl + jl * 64] = tau_s[jl];
-        __syncthreads();
-    }
-    for (int e = tid; e < bw * bw; e += blockDim.x) {
-        int r = e % bw, c = e / bw;
-        Tm[(size_t)r + (size_t)c * ldt] = (T)tloc[r + c * 64];
-    }
-}
 
 // ---- W of the two-sided update, fused (three small launches instead of five GEMMs):
 //   X = (A22 V) T,  Y = V^T X,  Z = T^T Y,  W = X - (1/2) V Z.
@@ -445,16 +189,13 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
 {
     cudaError_t e;
     if (b > 64 || b < 1) return cudaErrorInvalidValue;
-    // sync layout: [0..1] barrier words, then doubles
-    double *dsync = reinterpret_cast<double *>(sync + 64);
-    const int max_g = 512;
-    double *part = dsync;                           // 2 x max_g
-    double *alpha = part + 2 * max_g;               // 2 x 64
-    double *wpart = alpha + 128;                    // 2 x max_g x 64
-    double *gram = wpart + 2 * (size_t)max_g * 64;  // max_g x 64 x 64
-
-    int dev = 0;
-    cudaGetDevice(&dev);
+    // sync layout: partials of the W kernels, then the packets of the panel factorisation
+    T *ypart = reinterpret_cast<T *>(sync + 64);
+    unsigned long long *packets = reinterpret_cast<unsigned long long *>(sync + kSyncWords);
+    const int m_first = n - b;
+    if (m_first >= 2 &&
+        (e = cudaMemsetAsync(packets, 0, sizeof(unsigned long long) * panel_packet_words(m_first, sizeof(T)), st)) != cudaSuccess)
+        return e;
     // V1 explicit and zero outside each panel's reflectors (the back-transformation merges
     // consecutive panels into one block)
     if ((e = cudaMemsetAsync(v1, 0, sizeof(T) * (size_t)n * n, st)) != cudaSuccess) return e;
@@ -466,43 +207,8 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
         T *V = v1 + r0 + (size_t)c0 * n;
         T *Tm = t1 + (size_t)c0 * b;
         int ldt = b;
-        // rows per CTA: 256 (fewer CTAs make the per-column barrier and the reductions of
-        // the partials cheaper; the per-column work of a CTA stays small), more if needed
-        // for co-residency
-        int rows = 256;
-        int G = ceil_div(m, rows);
-        // panel rows, then T (64 x 64 binary64) at the next 16-byte boundary
-        auto panel_smem = [&](int r) {
-            return (((size_t)r * (bw + 1) * sizeof(T) + 15) & ~(size_t)15) + 64 * 64 * sizeof(double);
-        };
-        size_t smem = panel_smem(rows);
-        static PerDeviceOnce attr_set;  // per instantiation
-        e = once_per_device(attr_set, [] {
-            return cudaFuncSetAttribute(panel_qr_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        });
-        if (e != cudaSuccess) return e;
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, panel_qr_kernel<T>, 256, smem);
-        int max_coresident = per_sm * num_sms;
-        while (G > max_coresident || G > max_g) {
-            rows *= 2;
-            G = ceil_div(m, rows);
-            smem = panel_smem(rows);
-            if (smem > 200 * 1024) return cudaErrorInvalidConfiguration;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, panel_qr_kernel<T>, 256, smem);
-            max_coresident = per_sm * num_sms;
-        }
-        if ((e = cudaMemsetAsync(sync, 0, 2 * sizeof(unsigned), st)) != cudaSuccess) return e;
-        PanelArgs pa;
-        pa.m = m; pa.bw = bw; pa.rows_per_cta = rows; pa.lda = lda; pa.ldv = n;
-        pa.count = sync;
-        pa.part = part; pa.alpha = alpha; pa.wpart = wpart; pa.gram = gram; pa.status = status;
-        pa.gstride = max_g;
-        pa.spin_limit = spin_limit();
-        void *args[] = {&P, &V, &Tm, &ldt, &pa};
-        EGB_COUNT_LAUNCH();
-        if ((e = cudaLaunchCooperativeKernel((void *)panel_qr_kernel<T>, dim3(G), dim3(256), args,
-                                             smem, st)) != cudaSuccess) return e;
+        if ((e = panel_qr<T>(st, m, m_first, bw, P, lda, V, n, Tm, ldt, (unsigned)c0, packets, status, num_sms)) != cudaSuccess)
+            return e;
 
         // ---- two-sided update of A22 = a[r0:, r0:] (full symmetric storage)
         T *A22 = a + r0 + (size_t)r0 * lda;
@@ -527,12 +233,10 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
         }
         if (!xdone && (e = gemm<T>(st, 0, 0, m, bw, m, T(1), A22, lda, V, n, T(0), W, m)) != cudaSuccess)
             return e;
-        if (ceil_div(m, kWRows) + 1 <= max_g) {
-            // X = (A22 V) T, W = X - 1/2 V (T^T (V^T X)); the per-block partials of V^T X
-            // and their sum use the (now idle) Gram scratch of the panel factorisation
-            T *yp = reinterpret_cast<T *>(gram);
-            T *ysum = yp + (size_t)ceil_div(m, kWRows) * 64 * 64;
-            if ((e = form_w<T>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, yp)) != cudaSuccess) return e;
+        if (ceil_div(m, kWRows) + 1 <= kSyncBlocks) {
+            // X = (A22 V) T, W = X - 1/2 V (T^T (V^T X))
+            T *ysum = ypart + (size_t)ceil_div(m, kWRows) * 64 * 64;
+            if ((e = form_w<T>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart)) != cudaSuccess) return e;
         } else {
             // X = (A22 V) T
             if ((e = gemm<T>(st, 0, 0, m, bw, bw, T(1), W, m, Tm, ldt, T(0), X, m)) != cudaSuccess) return e;
