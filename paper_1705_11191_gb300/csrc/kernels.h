@@ -94,6 +94,17 @@ template <typename T>
 cudaError_t trsm_left_lower(cudaStream_t st, int trans, int n, int ncol, const T *L, int ldl,
                             const T *inv_diag, T *B, int ldb, T *work);
 
+// Columns that the refinement of the binary32 route works on for k wanted states: at least
+// 16 more (guard) columns, up to the next multiple of 128, the column tile of its products.
+// The correction of a state is divided by its distance to the first column outside the
+// block, so with none to spare a k-th gap of a few 1e-4 Ha stops the convergence; the guard
+// columns put the edge of the block some spacings away at next to no cost.
+inline int refine_block(int n, int k)
+{
+    const long long kg = ((long long)k + 16 + 127) / 128 * 128;
+    return kg < n ? (int)kg : n;
+}
+
 // ---- full -> band (Eq. 11, first line) ----
 // Householder QR of the m x bw panel at P (explicit V, compact-WY T), panel.cu. packets:
 // panel_packet_words(m_first, sizeof(T)) words zeroed before the first panel of a reduction

@@ -73,8 +73,11 @@ __global__ void residual_kernel(int n, int k, const double *g, const double *s, 
 //  rows i < k : from Goo = Xo^T H Xo and Soo = Xo^T S Xo (binary64, k x k); pairs in the
 //               same cluster (cid[i] == cid[j]) only get R_ij / 2
 //  rows i >= k: E_ij = M_ij / (lam_j - w_i), M = Xu^T R_o (binary32, (n-k) x k, ld n-k)
-// Also accumulates max |E| and max |R_oo| into stats[0], stats[1] (as ordered ints).
-__global__ void build_e_kernel(int n, int k, const double *goo, const double *soo,
+// Columns j >= kc are guard columns: they need not converge, only stay close to their start,
+// so a correction above 1/4 (a pair closer than its error, at the edge of the block) is left
+// out. Also accumulates max |E| of the first kc columns and max |R_oo| into stats[0], stats[1]
+// (as ordered ints).
+__global__ void build_e_kernel(int n, int k, int kc, const double *goo, const double *soo,
                                const float *m, const double *lam, const double *w,
                                const int *cid, float *e32, unsigned long long *stats)
 {
@@ -98,7 +101,8 @@ __global__ void build_e_kernel(int n, int k, const double *goo, const double *so
             double mij = (double)m[(size_t)(i - k) + (size_t)j * (n - k)];
             e = (fabs(dl) > 1e-13) ? mij / dl : 0.0;
         }
-        emax = fmax(emax, fabs(e));
+        if (j < kc) emax = fmax(emax, fabs(e));
+        else if (!(fabs(e) <= 0.25)) e = 0.0;
         e32[q] = (float)e;
     }
     // non-negative doubles order like their bit patterns
@@ -302,13 +306,13 @@ __global__ void rotate_gram_kernel(int k, const int *cid, const int *csize, cons
     }
 }
 
-__global__ void orth_defect_kernel(int k, const double *sm, unsigned long long *stats)
+__global__ void orth_defect_kernel(int kc, int ld, const double *sm, unsigned long long *stats)
 {
     double r = 0.0;
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < (size_t)k * k;
+    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < (size_t)kc * kc;
          q += (size_t)gridDim.x * blockDim.x) {
-        int i = (int)(q % k), j = (int)(q / k);
-        r = fmax(r, fabs((i == j ? 1.0 : 0.0) - sm[q]));
+        int i = (int)(q % kc), j = (int)(q / kc);
+        r = fmax(r, fabs((i == j ? 1.0 : 0.0) - sm[(size_t)i + (size_t)j * ld]));
     }
     for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
     if ((threadIdx.x & 31) == 0) atomicMax(stats, (unsigned long long)__double_as_longlong(r));
@@ -316,11 +320,16 @@ __global__ void orth_defect_kernel(int k, const double *sm, unsigned long long *
 
 // out[0] = max_j lam_j - w_k, the largest refined eigenvalue of the wanted block against
 // the binary32-route estimate of the first unwanted one (-inf when k = n); out[1] =
-// max(|w_0|, |w_(n-1)|, max_j |lam_j|), the scale of the spectrum. One CTA.
-__global__ void wanted_order_kernel(int n, int k, const double *lam, const double *w, double *out)
+// max(|w_0|, |w_(n-1)|, max_j |lam_j|), the scale of the spectrum; out[2] = 1 if the kb
+// refined eigenvalues (wanted and guard) do not ascend. One CTA.
+__global__ void wanted_order_kernel(int n, int k, int kb, const double *lam, const double *w, double *out)
 {
     __shared__ double smax[32], sabs[32];
     double m = -INFINITY, a = 0.0;
+    int down = 0;
+    for (int j = threadIdx.x + 1; j < kb; j += blockDim.x) down |= lam[j] < lam[j - 1];
+    down = __syncthreads_or(down);
+    if (threadIdx.x == 0) out[2] = down ? 1.0 : 0.0;
     for (int j = threadIdx.x; j < k; j += blockDim.x) {
         m = fmax(m, lam[j]);
         a = fmax(a, fabs(lam[j]));
@@ -341,6 +350,29 @@ __global__ void wanted_order_kernel(int n, int k, const double *lam, const doubl
         }
         out[0] = k < n ? m - w[k] : -INFINITY;
         out[1] = fmax(a, fmax(fabs(w[0]), fabs(w[n - 1])));
+    }
+}
+
+// Column rank_j of the output is column j of x (n x k), rank_j its place in ascending order
+// of lam (index order between equal values); lamo likewise. *bad = 1 if a column past the kc
+// whose convergence is checked ends among the kw wanted ones. One CTA per column.
+__global__ void sort_columns_kernel(int n, int k, int kw, int kc, const double *lam, const double *x,
+                                    double *lamo, double *xo, double *bad)
+{
+    __shared__ int rank;
+    const int j = blockIdx.x;
+    const double v = lam[j];
+    if (threadIdx.x == 0) rank = 0;
+    __syncthreads();
+    int c = 0;
+    for (int i = threadIdx.x; i < k; i += blockDim.x) c += lam[i] < v || (lam[i] == v && i < j);
+    if (c) atomicAdd(&rank, c);
+    __syncthreads();
+    const int r = rank;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) xo[(size_t)i + (size_t)r * n] = x[(size_t)i + (size_t)j * n];
+    if (threadIdx.x == 0) {
+        lamo[r] = v;
+        if (j >= kc && r < kw) *bad = 1.0;
     }
 }
 
@@ -376,7 +408,9 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
 {
     Workspace &w = h->wk;
     cudaStream_t st = h->stream;
-    const int n = h->n, k = h->n_state, b = h->band_width;
+    const int n = h->n, kw = h->n_state, b = h->band_width;
+    const int k = refine_block(n, kw);  // wanted states and guard columns
+    const int kc = kw + 8 < k ? kw + 8 : k;  // columns whose convergence is checked
     const bool unit = h->overlap_is_unit;
     const bool ev_mode = rq.evec != nullptr;
     int dev = 0, sms = 0;
@@ -477,7 +511,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     if (!unit) CKR(trsm_left_lower<float>(st, 1, n, n, L, n, INVD, X32, n, WORK));
     CKR(cudaEventRecord(w.ev[STAGE_REFINE], st));
 
-    // ---------------- refinement of the k wanted eigenpairs
+    // ---------------- refinement of the kw wanted eigenpairs (and the guard columns)
     const size_t nk = (size_t)n * k;
     double *XO = w.rf;                 // n x k binary64
     double *YH = XO + nk;              // n x k
@@ -488,7 +522,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     double *GD = LAM + k;              // k
     double *SD = GD + k;               // k
     unsigned long long *STATS = reinterpret_cast<unsigned long long *>(SD + k);  // 4
-    int *CID = reinterpret_cast<int *>(STATS + 4);        // k
+    int *CID = reinterpret_cast<int *>(STATS + 8);        // k
     int *CSZ = CID + k;                                   // k
     double *QBUF = reinterpret_cast<double *>(CSZ + k);  // k x 32 x 32 (2k ints: 8-byte aligned)
     float *R32 = reinterpret_cast<float *>(QBUF + (size_t)k * kMaxCluster * kMaxCluster);  // n x k
@@ -559,7 +593,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
             CKR(gemm<float>(st, 1, 0, n - k, k, n, 1.0f, X32 + (size_t)k * n, n, R32, n, 0.0f, M32, n - k));
         CKR(cudaMemsetAsync(STATS, 0, 4 * sizeof(unsigned long long), st));
         EGB_COUNT_LAUNCH();
-        build_e_kernel<<<grid_for(nk), 256, 0, st>>>(n, k, GOO, SOO, M32, LAM, w.w, CID, E32, STATS);
+        build_e_kernel<<<grid_for(nk), 256, 0, st>>>(n, k, kc, GOO, SOO, M32, LAM, w.w, CID, E32, STATS);
         // X_o += [X_o | X_u] E  (binary32 product of small corrections; the X_o block of
         // the binary32 matrix is refreshed from the current binary64 X_o first)
         CKR(copy_matrix<float, double>(st, n, k, XO, n, X32, n));
@@ -579,13 +613,28 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     {
         int rc = products_and_rr(kOzDigits);
         if (rc) return rc;
-        CKR(cudaMemsetAsync(STATS, 0, 4 * sizeof(unsigned long long), st));
+        CKR(cudaMemsetAsync(STATS, 0, 8 * sizeof(unsigned long long), st));
         EGB_COUNT_LAUNCH();
-        orth_defect_kernel<<<grid_for((size_t)k * k), 256, 0, st>>>(k, SOO, STATS);
+        orth_defect_kernel<<<grid_for((size_t)kc * kc), 256, 0, st>>>(kc, k, SOO, STATS);
         EGB_COUNT_LAUNCH();
-        wanted_order_kernel<<<1, 256, 0, st>>>(n, k, LAM, w.w, reinterpret_cast<double *>(STATS + 2));
-        CKR(cudaMemcpyAsync(w.scal_host + 8, STATS, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
+        wanted_order_kernel<<<1, 256, 0, st>>>(n, kw, k, LAM, w.w, reinterpret_cast<double *>(STATS + 2));
+        CKR(cudaMemcpyAsync(w.scal_host + 8, STATS, 5 * sizeof(double), cudaMemcpyDeviceToHost, st));
         CKR(cudaStreamSynchronize(st));
+        if (w.scal_host[12] != 0.0) {
+            // the binary32 route had two close states in the wrong order: the wanted ones are
+            // the lowest of the refined block
+            EGB_COUNT_LAUNCH();
+            sort_columns_kernel<<<k, 256, 0, st>>>(n, k, kw, kc, LAM, XO, GD, YH,
+                                                    reinterpret_cast<double *>(STATS + 5));
+            CKR(cudaMemcpyAsync(XO, YH, sizeof(double) * nk, cudaMemcpyDeviceToDevice, st));
+            CKR(cudaMemcpyAsync(LAM, GD, sizeof(double) * k, cudaMemcpyDeviceToDevice, st));
+            EGB_COUNT_LAUNCH();
+            wanted_order_kernel<<<1, 256, 0, st>>>(n, kw, k, LAM, w.w, reinterpret_cast<double *>(STATS + 2));
+            CKR(cudaMemcpyAsync(w.scal_host + 10, STATS + 2, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
+            CKR(cudaStreamSynchronize(st));
+            if (w.scal_host[13] != 0.0)
+                return set_error(h, ELSI_ERR_NO_CONVERGENCE, "a state past the checked ones is among the lowest %d", kw);
+        }
     }
     h->refine_iters = iters;
     h->orth_err = w.scal_host[8];
@@ -601,23 +650,23 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     if (!(w.scal_host[10] <= 1e-4 * fmax(1.0, w.scal_host[11])))
         return set_error(h, ELSI_ERR_NO_CONVERGENCE,
                          "refined states are not the lowest %d (max refined eigenvalue %.6g above "
-                         "the next binary32 one)", k, w.scal_host[10]);
-    // eigenvalues: refined for the wanted states, binary32-route values for the rest
+                         "the next binary32 one)", kw, w.scal_host[10]);
+    // eigenvalues: refined for the wanted and guard states, binary32-route values for the rest
     EGB_COUNT_LAUNCH();
     copy_eval_kernel<<<grid_for(n), 256, 0, st>>>(n, k, LAM, w.w, w.w);
     CKR(cudaEventRecord(w.ev[STAGE_OCC], st));
     if (ev_mode) {
         CKR(cudaMemcpyAsync(rq.eval, w.w, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
-        CKR(cudaMemcpyAsync(rq.evec, XO, sizeof(double) * nk, cudaMemcpyDeviceToDevice, st));
+        CKR(cudaMemcpyAsync(rq.evec, XO, sizeof(double) * (size_t)n * kw, cudaMemcpyDeviceToDevice, st));
         CKR(cudaEventRecord(w.ev[STAGE_DENSITY], st));
     } else {
-        CKR(occupation(st, k, w.w, h->n_electron, h->scheme, h->kt, h->occ_accuracy,
+        CKR(occupation(st, kw, w.w, h->n_electron, h->scheme, h->kt, h->occ_accuracy,
                        h->mu_max_steps, w.f, w.scal, w.status, h->occ_stride));
         CKR(cudaEventRecord(w.ev[STAGE_DENSITY], st));
-        int kocc = k;
+        int kocc = kw;
         if (h->scheme == ELSI_OCC_INTEGER) {
             kocc = (int)((h->n_electron / h->occ_stride + 1.999999999) / 2.0) * h->occ_stride;
-            if (kocc > k) kocc = k;
+            if (kocc > kw) kocc = kw;
             if (kocc < 1) kocc = 1;
         }
         // P = X_o diag(f) X_o^T and W = X_o diag(f eps) X_o^T, binary64-accurate products

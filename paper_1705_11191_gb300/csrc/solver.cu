@@ -75,7 +75,7 @@ int ensure_workspace(elsi_gb_handle_s *h, int kz)
     ENSURE(sync, unsigned, sync_words(h->n, (int)eb));
     ENSURE(status, int, ST_WORDS);
     if (h->precision == ELSI_PREC_FP32_REFINE) {
-        const size_t k = h->n_state;
+        const size_t k = refine_block(h->n, h->n_state);
         ENSURE(rf, double, 5 * n * k + 2 * k * k + 1040 * k + 64);
         // digits of H, S (n x n), of X_o, Y_H, Y_S (k columns of length n) and of the
         // rows of X_o for P and W (three splits of n rows of length k)

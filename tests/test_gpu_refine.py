@@ -144,3 +144,30 @@ def test_binary64_cholesky_fallback_nearly_dependent_pair():
     assert rel(P.cpu().numpy(), ref["P"]) <= 1e-7
     assert abs(e - ref["energy"]) <= 1e-7 * abs(ref["energy"])
     assert iters == -1 or iters >= 1
+
+
+@pytest.mark.parametrize("gap", [1e-3, 1e-5, 1e-7])
+def test_small_gap_above_the_wanted_states(gap):
+    """The k-th and (k+1)-th eigenvalues 'gap' apart, below the error of the binary32 route for
+    the smallest: the wanted states are the lowest k, without a binary64 repeat (the guard
+    columns keep the edge of the refined block away from the wanted states)."""
+    n, k = 400, 50
+    rng = np.random.default_rng(11)
+    q, _ = np.linalg.qr(rng.standard_normal((n, n)))
+    lam = np.sort(rng.uniform(-4.0, 6.0, n))
+    lam[k] = lam[k - 1] + gap
+    lam = np.sort(lam)
+    h = (q * lam) @ q.T
+    h = 0.5 * (h + h.T)
+    ref = np.linalg.eigvalsh(h)
+    with egb.Handle(n, k, 0.0) as hd:
+        hd.use_current_stream()
+        hd.set_overlap_is_unit(True)
+        hd.set_precision(egb.PREC_FP32_REFINE)
+        ev, C = hd.ev_real(dev(h))
+        iters, orth = hd.refine_info()
+    C = C.cpu().numpy()
+    assert iters > 0 and orth < 1e-10
+    # eigenvalues are accurate to second order in the vectors' error, and to eps ||H||
+    np.testing.assert_allclose(ev.cpu().numpy()[:k], ref[:k], rtol=0, atol=1e-12)
+    assert np.abs(h @ C - C * ref[:k]).max() < 1e-10
