@@ -22,9 +22,9 @@ extern "C" {
 #endif
 
 /*
- * elsi_gb_set_spin_limit: iteration limit of the library's SIMT spin waits (the grid
- *   barrier of the cooperative panel factorisation and the per-sweep progress flags of the
- *   bulge chase; the mbarrier waits of the tensor-core pipelines keep their own limit).
+ * elsi_gb_set_spin_limit: iteration limit of the library's SIMT spin waits (the
+ *   packets that the CTAs of the panel factorisation and of the bulge chase exchange and the
+ *   progress flags of the general chase; the mbarrier waits of the tensor-core pipelines keep their own limit).
  *   A wait that has polled more than `polls` times records ELSI_ERR_TIMEOUT in the
  *   solve's status word and its kernel returns, so the solve returns ELSI_ERR_TIMEOUT and
  *   the CUDA context stays usable. Process-wide; read at each launch. Default 2^26
@@ -73,10 +73,11 @@ int elsi_gb_gemm_f32(int ta, int tb, int m, int n, int k, float alpha, const flo
  * elsi_gb_gemm_f64_digits: the binary64-accurate product of the refinement and of P, W
  *   (Ozaki et al., Numer. Algorithms 59 (2012), integer-digit form):
  *   C (m x n, column-major, ldc) = alpha * op(A) op(B) + beta * C, op() as for
- *   elsi_gb_gemm_f32, every row of op(A) and column of op(B) cut into `digits` (1..7)
- *   signed 7-bit digits after scaling by a power of two, the digit products summed
- *   exactly on the bf16 tensor cores, levels 2..digits+1 kept (truncation about
- *   2^(-7 digits) relative to max|op(A)_i.| max|op(B)_.j| per term). uplo = 1 writes
+ *   elsi_gb_gemm_f32, every row of op(A) and column of op(B) cut, after scaling by a power
+ *   of two, into signed 9-bit digits, as few of them as hold `digits` (1..7) times 7 bits and
+ *   one more (1, 2, 3, 4, 4, 5, 6), the digit products summed on the bf16 tensor cores
+ *   (truncation at most about 2^(-7 digits) relative to max|op(A)_i.| max|op(B)_.j| per term:
+ *   the refinement form of the product). uplo = 1 writes
  *   only the lower triangle of C. planes: device scratch of
  *   elsi_gb_gemm_f64_digits_planes(m, n, k) bf16 values (2 bytes each; 16-byte aligned);
  *   exps: device int[elsi_gb_gemm_f64_digits_exps(m, n)]; status: device int[8], zeroed
@@ -91,6 +92,18 @@ int elsi_gb_gemm_f64_digits(int ta, int tb, int m, int n, int k, double alpha, c
                             int lda, const double *B, int ldb, double beta, double *C, int ldc,
                             int uplo, int digits, void *planes, size_t plane_elems, int *exps,
                             size_t exp_elems, int *status, void *stream);
+
+/*
+ * elsi_gb_gemm_f64_wide: the same with eight 9-bit digits and 128-bit sums, the products of
+ *   the binary64 route (truncation about 2^-72); scratch of elsi_gb_gemm_f64_wide_planes
+ *   values and elsi_gb_gemm_f64_digits_exps exponents. Scratch beyond that is used to divide
+ *   a long K over CTAs.
+ */
+size_t elsi_gb_gemm_f64_wide_planes(int m, int n, int k);
+int elsi_gb_gemm_f64_wide(int ta, int tb, int m, int n, int k, double alpha, const double *A,
+                          int lda, const double *B, int ldb, double beta, double *C, int ldc,
+                          int uplo, void *planes, size_t plane_elems, int *exps, size_t exp_elems,
+                          int *status, void *stream);
 
 #ifdef __cplusplus
 }

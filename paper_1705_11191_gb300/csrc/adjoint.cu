@@ -93,9 +93,12 @@ int ev_adjoint(elsi_gb_handle_s *h, int n, int k, const double *eps, const doubl
     Workspace &w = h->wk;
     if (!ensure_buf((void **)&w.adj, &w.adj_cap, sizeof(double) * (nk + 3 * nkk + 16)))
         return set_error(h, ELSI_ERR_NOMEM, "adjoint scratch");
+    if (!ensure_digit_scratch(h, n, n)) return set_error(h, ELSI_ERR_NOMEM, "adjoint digit planes");
+    const DigitScratch digits(h);
     double *A = w.adj, *XH = A + nk, *XS = XH + nkk, *Y = XS + nkk;
     cudaStream_t st = h->stream;
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = cudaMemsetAsync(w.status, 0, sizeof(int) * ST_WORDS, st);
+    if (e != cudaSuccess) return set_error(h, ELSI_ERR_CUDA, "eigenpair adjoint: %s", cudaGetErrorString(e));
 #define ACK(x)                                                                             \
     if ((e = (x)) != cudaSuccess)                                                          \
         return set_error(h, ELSI_ERR_CUDA, "eigenpair adjoint: %s", cudaGetErrorString(e));
@@ -112,9 +115,11 @@ int ev_adjoint(elsi_gb_handle_s *h, int n, int k, const double *eps, const doubl
         ACK(gemm<double>(st, 0, 1, n, n, kk, 1.0, Y, n, c, n, 0.0, sb, n));
         ACK(symmetrize<double>(st, n, sb, n));
     }
+    int code = 0;
+    ACK(cudaMemcpyAsync(&code, w.status + ST_CODE, sizeof(int), cudaMemcpyDeviceToHost, st));
     ACK(cudaStreamSynchronize(st));
 #undef ACK
-    return ELSI_OK;
+    return code ? set_error(h, code, "eigenpair adjoint: device error") : ELSI_OK;
 }
 
 }  // namespace egb

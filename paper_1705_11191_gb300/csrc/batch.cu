@@ -58,6 +58,8 @@ struct BatchState {
     EGB_BUF(double, outs)   // per-problem scalars
     EGB_BUF(int, offs)      // state offsets (nprob + 1)
     EGB_BUF(int, status)
+    EGB_BUF(__nv_bfloat16, dig)  // digit planes of the P and W products
+    EGB_BUF(int, digx)           // and their exponents
     EGB_BUF(double, tune)   // eigenpair scratch of the autotuner's trial solves
 #undef EGB_BUF
     double *outs_host = nullptr;  // pinned
@@ -551,6 +553,29 @@ int batch_dm(elsi_gb_handle_s *h, const double *occ, double *const *dm, double *
     cudaStream_t st = h->stream;
     if (occ && occ != b.occ)
         BCK(cudaMemcpyAsync(b.occ, occ, sizeof(double) * b.total_lvl, cudaMemcpyDeviceToDevice, st));
+    // P and W as digit products on the tensor cores (two operands of N rows of length K)
+    size_t planes = 0, nmax = 0;
+    for (const BatchItem &it : b.items) {
+        const int c = b.cplx ? 2 : 1;
+        const size_t e = 2 * ozaki_split_elems(c * it.n, c * it.k, kOzWide);
+        planes = e > planes ? e : planes;
+        nmax = (size_t)c * it.n > nmax ? (size_t)c * it.n : nmax;
+    }
+    BENSURE(dig, __nv_bfloat16, planes);
+    BENSURE(digx, int, 2 * nmax + 512);
+    BCK(cudaMemsetAsync(b.status, 0, sizeof(int) * ST_WORDS, st));
+    struct Scratch {
+        Scratch(BatchState &b)
+        {
+            set_tc_scratch(nullptr, 0, b.status);
+            set_f64_tc_scratch(b.dig, b.dig_cap / sizeof(__nv_bfloat16), b.digx, b.digx_cap / sizeof(int));
+        }
+        ~Scratch()
+        {
+            set_f64_tc_scratch(nullptr, 0, nullptr, 0);
+            set_tc_scratch(nullptr, 0, nullptr);
+        }
+    } scratch(b);
     for (int i = 0; i < nprob; ++i) {
         const BatchItem &it = b.items[i];
         double *w_out = (edm && edm[i]) ? edm[i] : nullptr;
@@ -569,7 +594,8 @@ int batch_dm(elsi_gb_handle_s *h, const double *occ, double *const *dm, double *
     }
     BCK(segment_energy(st, nprob, b.offs, b.occ, b.lvl, b.outs));
     BCK(cudaMemcpyAsync(b.outs_host, b.outs, sizeof(double) * nprob, cudaMemcpyDeviceToHost, st));
-    BCK(cudaStreamSynchronize(st));
+    int rc = batch_status(h, b, "density matrices");
+    if (rc) return rc;
     if (energy)
         for (int i = 0; i < nprob; ++i) energy[i] = b.outs_host[i];
     return ELSI_OK;
@@ -622,7 +648,7 @@ void free_batch(elsi_gb_handle_s *h)
 {
     if (!h->batch) return;
     BatchState &b = *h->batch;
-    void *bufs[] = {b.vals, b.vecs, b.lvl, b.wts, b.occ, b.occ2, b.emb, b.cw, b.outs, b.offs, b.status,
+    void *bufs[] = {b.vals, b.vecs, b.lvl, b.wts, b.occ, b.occ2, b.emb, b.cw, b.outs, b.offs, b.status, b.dig, b.digx,
                     b.tune};
     for (void *p : bufs)
         if (p) cudaFree(p);

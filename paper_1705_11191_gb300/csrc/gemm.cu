@@ -143,23 +143,49 @@ void set_f64_tc_scratch(__nv_bfloat16 *planes, size_t elems, int *exps, size_t e
 // rows, op(B) by columns (once for A A^T). cudaErrorNotSupported if the scratch is short.
 static cudaError_t gemm_f64_digits(cudaStream_t st, int ta, int tb, int m, int n, int k, double alpha,
                                    const double *A, int lda, const double *B, int ldb, double beta,
-                                   double *C, int ldc, int uplo, int digits = kOzDigits)
+                                   double *C, int ldc, int uplo, int digits = kOzWide)
 {
     const bool same = A == B && lda == ldb && ta != tb && m == n;
-    const size_t ea = ozaki_split_elems(m, k), eb = same ? 0 : ozaki_split_elems(n, k);
+    const size_t ea = ozaki_split_elems(m, k, digits), eb = same ? 0 : ozaki_split_elems(n, k, digits);
     const size_t xa = (size_t)ceil_div(m, 128) * 128, xb = same ? 0 : (size_t)ceil_div(n, 128) * 128;
     if (ea + eb > t_oz_elems || xa + xb > t_oz_exp_elems) return cudaErrorNotSupported;
     __nv_bfloat16 *ad = t_oz_planes, *bd = same ? t_oz_planes : t_oz_planes + ea;
     int *xe = t_oz_exps, *ye = same ? t_oz_exps : t_oz_exps + xa;
+    // what is left of the planes (from the next 16-byte boundary) takes the partial products of
+    // a divided K
+    const size_t used = (ea + eb + 7) & ~(size_t)7;
+    double *part = reinterpret_cast<double *>(t_oz_planes + used);
+    const size_t part_elems = (t_oz_elems > used ? t_oz_elems - used : 0) / 4;
     cudaError_t e;
     // row i of op(A): ta = 0 -> A[i + q lda], ta = 1 -> A[q + i lda]
-    if ((e = ozaki_split(st, m, k, A, ta ? lda : 1, ta ? 1 : lda, nullptr, nullptr, ad, xe)) != cudaSuccess)
+    if ((e = ozaki_split(st, m, k, A, ta ? lda : 1, ta ? 1 : lda, nullptr, nullptr, ad, xe, digits)) != cudaSuccess)
         return e;
     // column j of op(B): tb = 0 -> B[q + j ldb], tb = 1 -> B[j + q ldb]
     if (!same &&
-        (e = ozaki_split(st, n, k, B, tb ? 1 : ldb, tb ? ldb : 1, nullptr, nullptr, bd, ye)) != cudaSuccess)
+        (e = ozaki_split(st, n, k, B, tb ? 1 : ldb, tb ? ldb : 1, nullptr, nullptr, bd, ye, digits)) != cudaSuccess)
         return e;
-    return ozaki_gemm(st, m, n, k, alpha, ad, xe, bd, ye, beta, C, ldc, uplo, digits);
+    return ozaki_gemm(st, m, n, k, alpha, ad, xe, bd, ye, beta, C, ldc, uplo, digits, part, part_elems);
+}
+
+// A binary64 product goes to the digit products when the thread has their scratch and K is
+// long enough: a CTA of the SIMT kernel takes about 1 us per unit of K for its 64 x 64 tile
+// (4096 FMAs at two a clock) however small the product, the two splits and the digit product
+// about 12 us.
+static bool digits_pay(int k) { return t_oz_planes && k >= 24; }
+
+// C -= V W^T + W V^T (lower triangle, m x m, V and W m x b): one product over K = 2 b whose
+// operands' rows are [V_i W_i] and [W_i V_i].
+cudaError_t gemm_f64_two_sided(cudaStream_t st, int m, int b, const double *V, int ldv, const double *W,
+                               int ldw, double *C, int ldc)
+{
+    const size_t pe = ozaki_split_elems(m, 2 * b, kOzWide), xe = (size_t)ceil_div(m, 128) * 128;
+    if (!digits_pay(2 * b) || 2 * pe > t_oz_elems || 2 * xe > t_oz_exp_elems) return cudaErrorNotSupported;
+    __nv_bfloat16 *ad = t_oz_planes, *bd = ad + pe;
+    int *ea = t_oz_exps, *eb = ea + xe;
+    cudaError_t e;
+    if ((e = ozaki_split(st, m, 2 * b, V, 1, ldv, nullptr, nullptr, ad, ea, kOzWide, W, ldw, b)) != cudaSuccess) return e;
+    if ((e = ozaki_split(st, m, 2 * b, W, 1, ldw, nullptr, nullptr, bd, eb, kOzWide, V, ldv, b)) != cudaSuccess) return e;
+    return ozaki_gemm(st, m, m, 2 * b, -1.0, ad, ea, bd, eb, 1.0, C, ldc, 1, kOzWide);
 }
 
 template <typename T>
@@ -176,7 +202,7 @@ cudaError_t gemm(cudaStream_t st, int ta, int tb, int m, int n, int k, T alpha, 
         }
     } else {
         // binary64 products large enough for the digit products on the tensor cores
-        if (t_oz_planes && k >= 32 && (double)m * n * k >= 1.6e7) {
+        if (digits_pay(k)) {
             cudaError_t e = gemm_f64_digits(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, uplo);
             if (e != cudaErrorNotSupported) return e;
         }
@@ -215,6 +241,8 @@ cudaError_t gemm_splitk(cudaStream_t st, int ta, int tb, int m, int n, int k, T 
                                         t_tc_work, t_tc_elems, t_tc_status);
             if (e != cudaErrorNotSupported) return e;
         }
+    } else if (digits_pay(k)) {
+        return gemm<T>(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, T(0), C, ldc, 0);
     }
     using G = GemmCfg<T>;
     const int tiles = ceil_div(m, G::BM) * ceil_div(n, G::BN);
@@ -421,10 +449,11 @@ template cudaError_t check_finite<float>(cudaStream_t, int, int, const float *, 
 
 }  // namespace egb
 
+// Seven planes, as many as the seven-bit digits that the entry counts in need.
 extern "C" size_t elsi_gb_gemm_f64_digits_planes(int m, int n, int k)
 {
     if (m < 1 || n < 1 || k < 1) return 0;
-    return egb::ozaki_split_elems(m, k) + egb::ozaki_split_elems(n, k);
+    return egb::ozaki_split_elems(m, k, 7) + egb::ozaki_split_elems(n, k, 7);
 }
 
 extern "C" size_t elsi_gb_gemm_f64_digits_exps(int m, int n)
@@ -433,18 +462,20 @@ extern "C" size_t elsi_gb_gemm_f64_digits_exps(int m, int n)
     return (size_t)egb::ceil_div(m, 128) * 128 + (size_t)egb::ceil_div(n, 128) * 128;
 }
 
-extern "C" int elsi_gb_gemm_f64_digits(int ta, int tb, int m, int n, int k, double alpha,
-                                       const double *A, int lda, const double *B, int ldb,
-                                       double beta, double *C, int ldc, int uplo, int digits,
-                                       void *planes, size_t plane_elems, int *exps, size_t exp_elems,
-                                       int *status, void *stream)
+extern "C" size_t elsi_gb_gemm_f64_wide_planes(int m, int n, int k)
 {
-    if (m < 1 || n < 1 || k < 1 || digits < 1 || digits > egb::kOzDigits || !A || !B || !C || !planes ||
-        !exps || !status)
-        return ELSI_ERR_ARG;
+    if (m < 1 || n < 1 || k < 1) return 0;
+    return egb::ozaki_split_elems(m, k, egb::kOzWide) + egb::ozaki_split_elems(n, k, egb::kOzWide);
+}
+
+static int digits_entry(int ta, int tb, int m, int n, int k, double alpha, const double *A, int lda,
+                        const double *B, int ldb, double beta, double *C, int ldc, int uplo, int digits,
+                        size_t need, void *planes, size_t plane_elems, int *exps, size_t exp_elems, int *status,
+                        void *stream)
+{
+    if (m < 1 || n < 1 || k < 1 || !A || !B || !C || !planes || !exps || !status) return ELSI_ERR_ARG;
     if (ldc < m || lda < (ta ? k : m) || ldb < (tb ? n : k)) return ELSI_ERR_ARG;
-    if ((size_t)planes % 16 != 0 || plane_elems < elsi_gb_gemm_f64_digits_planes(m, n, k) ||
-        exp_elems < elsi_gb_gemm_f64_digits_exps(m, n))
+    if ((size_t)planes % 16 != 0 || plane_elems < need || exp_elems < elsi_gb_gemm_f64_digits_exps(m, n))
         return ELSI_ERR_ARG;
     // the pipeline's status word comes from the binary32 scratch slot of this thread
     float *tw;
@@ -459,4 +490,26 @@ extern "C" int elsi_gb_gemm_f64_digits(int ta, int tb, int m, int n, int k, doub
     egb::set_tc_scratch(tw, te, ts);
     if (e == cudaErrorNotSupported) return ELSI_ERR_ARG;
     return e == cudaSuccess ? ELSI_OK : ELSI_ERR_CUDA;
+}
+
+extern "C" int elsi_gb_gemm_f64_digits(int ta, int tb, int m, int n, int k, double alpha,
+                                       const double *A, int lda, const double *B, int ldb,
+                                       double beta, double *C, int ldc, int uplo, int digits,
+                                       void *planes, size_t plane_elems, int *exps, size_t exp_elems,
+                                       int *status, void *stream)
+{
+    if (digits < 1 || digits > 7) return ELSI_ERR_ARG;
+    // the fewest nine-bit digits with at least 7 digits + 1 bits (the leading one holds eight)
+    return digits_entry(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, uplo, (7 * digits + 9) / 9,
+                        elsi_gb_gemm_f64_digits_planes(m, n, k), planes, plane_elems, exps, exp_elems, status, stream);
+}
+
+extern "C" int elsi_gb_gemm_f64_wide(int ta, int tb, int m, int n, int k, double alpha,
+                                     const double *A, int lda, const double *B, int ldb,
+                                     double beta, double *C, int ldc, int uplo,
+                                     void *planes, size_t plane_elems, int *exps, size_t exp_elems,
+                                     int *status, void *stream)
+{
+    return digits_entry(ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, uplo, egb::kOzWide,
+                        elsi_gb_gemm_f64_wide_planes(m, n, k), planes, plane_elems, exps, exp_elems, status, stream);
 }

@@ -48,6 +48,10 @@ void set_tc_scratch(float *work, size_t elems, int *status);
 // and exponent scratch (planes = nullptr: SIMT binary64 kernel only). Uses the status word
 // of set_tc_scratch for timeouts.
 void set_f64_tc_scratch(__nv_bfloat16 *planes, size_t elems, int *exps, size_t exp_elems);
+// C -= V W^T + W V^T (lower triangle) as one digit product; cudaErrorNotSupported without
+// the scratch or when the product is too small for it.
+cudaError_t gemm_f64_two_sided(cudaStream_t st, int m, int b, const double *V, int ldv, const double *W,
+                               int ldw, double *C, int ldc);
 cudaError_t tc_gemm_f32(cudaStream_t st, int ta, int tb, int m, int n, int k, float alpha,
                         const float *A, int lda, const float *B, int ldb, float beta, float *C,
                         int ldc, int uplo, float *work, size_t work_elems, int *status);
@@ -216,19 +220,24 @@ cudaError_t dup_pairs(cudaStream_t st, int n, const double *f, double *f2);
 
 // ---- binary64-accurate products on the bf16 tensor cores (ozaki.cu) ----
 // Splits V vectors of length K (element (v, q) at src[v * sv + q * sq], optionally times
-// scale[q] * scale2[q]) into the digit planes consumed by ozaki_gemm.
-size_t ozaki_split_elems(int V, int K);  // bf16 elements of the planes of V vectors
+// scale[q] * scale2[q]) into the digit planes consumed by ozaki_gemm; the leading 'digits' of
+// them are written. With src2, element (v, q) for q >= k1 is src2[v * sv + (q - k1) * sq2].
+constexpr int kOzDigits = 6;  // 9-bit digits of the refinement form: 53 bits below the largest entry
+constexpr int kOzWide = 8;    // of the binary64 route: 71 bits, sums in 128 bits
+size_t ozaki_split_elems(int V, int K, int digits = kOzDigits);  // bf16 elements of the planes
 cudaError_t ozaki_split(cudaStream_t st, int V, int K, const double *src, long long sv,
                         long long sq, const double *scale, const double *scale2,
-                        __nv_bfloat16 *planes, int *exps);
+                        __nv_bfloat16 *planes, int *exps, int digits = kOzDigits,
+                        const double *src2 = nullptr, long long sq2 = 0, int k1 = 0);
 // C (m x n, ldc) = alpha * A B + beta * C with A given by the split of its m rows and B
 // by the split of its n columns (both of length k). uplo = 1: lower triangle only.
-// digits (1..7, default 7): leading digit planes used, i.e. D(D+1)/2 digit products and a
-// truncation error of about 2^(-7(D+1)) relative to max|A_i.| max|B_.j| per product term.
-constexpr int kOzDigits = 7;
+// digits (1..kOzDigits, or kOzWide; that of both splits, or for the refinement form less):
+// leading digit planes used, i.e. D(D+1)/2 digit products and a truncation error of about
+// 2^(-9D) relative to max|A_i.| max|B_.j| per product term. part: optional
+// scratch (part_elems values) to divide a long K over CTAs when the output is small.
 cudaError_t ozaki_gemm(cudaStream_t st, int m, int n, int k, double alpha,
                        const __nv_bfloat16 *Ad, const int *ea, const __nv_bfloat16 *Bd,
                        const int *eb, double beta, double *C, int ldc, int uplo,
-                       int digits = kOzDigits);
+                       int digits = kOzDigits, double *part = nullptr, size_t part_elems = 0);
 
 }  // namespace egb

@@ -4,21 +4,29 @@
 // integer-digit form).
 //
 // Every row of A (and column of B) is scaled by a power of two 2^e so that its entries
-// lie in (-1, 1), then cut into D signed 7-bit integer digits:
-//     x = 2^e sum_{s=1..D} d_s 2^{-7s} (+ a remainder below 2^{-7D}),  |d_1| <= 128,
-//     |d_s| <= 64 for s >= 2,
-// each digit exactly representable in bf16. Then
-//     (A B)_ij = 2^{e_i + f_j} sum_L 2^{-7L} sum_{s+t=L} (D_s^A D_t^B)_ij
-// and every digit product is an exact integer. The tensor cores accumulate the products
-// of one level L over chunks of 256 along K in binary32, which stays exact (the sum of
-// absolute values stays below 2^24); chunk results are converted to int32 and summed
-// (exact), and each level is finally scaled and added in binary64. Levels L = 2..D+1 are
-// kept, which leaves a truncation error of about 2^{-7(D+1)} relative to
-// max|A_i.| max|B_.j| per product term.
+// lie in [-1/2, 1/2], then cut into D signed 9-bit integer digits:
+//     x = 2^e sum_{s=1..D} d_s 2^{-9s} (+ a remainder of at most 2^{-9D-1}),  |d_s| <= 256,
+// each digit exactly representable in bf16 (whose significand has 8 bits: every integer up
+// to 256). Then
+//     (A B)_ij = 2^{e_i + f_j} sum_L 2^{-9L} sum_{s+t=L} (D_s^A D_t^B)_ij
+// and every digit product is an exact integer. Levels L = 2..D+1 are kept: D (D + 1) / 2
+// products. (Seven-bit digits, which leave the tensor cores more terms before a sum passes
+// 2^24, need 7 digits and 28 products for 49 bits; 6 nine-bit digits hold 53 in 21.)
 //
-// One chunk of level L sums at most 256 (2 * 128 * 64 + (D - 2) * 64 * 64) < 9.5e6 in
-// magnitude, so the int32 level sum is exact for up to 227 chunks (K = 58 112); longer
-// products are cut along K into segments of kOzSegK and the segments added in binary64.
+// Two forms:
+//  * refinement (D <= 6, 128 x 128 tiles): the corrections of the binary32 route, P and W. With
+//    D = 6 the dropped part is about 2^-54 of max|A_i.| max|B_.j| per term.
+//  * binary64 route (D = 8, 128 x 64 tiles, 128-bit sums): 71 bits below the largest entry and
+//    a dropped part of 2^-72. A binary64 FMA chain rounds relative to each product, not to
+//    the row's largest entry; on graded operands (the standard form of an ill-conditioned
+//    overlap) the 2^-54 form lost four digits of P at lambda_min(S) = 1e-6, this one none.
+//
+// Exactness. The tensor cores add in binary32, exact below 2^24: a sum over 64 of K and L - 1
+// digit pairs stays below 64 (L - 1) 2^16, so levels up to 5 are exact and one of the levels
+// 6 to 8 can pass 2^24 only if nearly all its digits are extreme, when it is rounded to a
+// multiple of 2 of its own unit. Such sums are drained every 64 terms into integers in
+// registers. The last level, and in the refinement form level 6 as well, whose units are
+// 2^-45 of the level-2 unit and below, are summed in binary32 over all of K.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -27,18 +35,17 @@
 
 namespace egb {
 
-constexpr int kOzD = 7;         // digits per operand
-constexpr int kOzBits = 7;      // bits per digit
+constexpr int kOzBits = 9;       // bits per digit
 constexpr int kOzBM = 128, kOzBN = 128, kOzBK = 16;  // plane padding: rows, K
-constexpr int kOzSegK = 32768;  // K per kernel launch (128 chunks of 256: int32-exact sums)
+constexpr int kOzSegK = 32768;  // K per kernel launch (64-bit integer sums: see the shift)
 
 // ------------------------------------------------------------------ splitting
-// The digits are those of the binary64 steps r = x 2^-e, then for s = 1..D: t = 128 r,
+// The digits are those of the binary64 steps r = x 2^-e, then for s = 1..D: t = 512 r,
 // d_s = rint(t), r = t - d_s (every step exact). They are formed here with integer
 // operations on the bit pattern x = +-M 2^E (binary64 arithmetic is scarce on this chip):
-// the running value A_s = sum_{i<=s} d_i 128^{s-i} equals rint(x 2^{7s-e}) (rounding half
-// to even; 128 A_{s-1} is even, so the parity of the ties is the same), hence
-// A_s = +-rne(M / 2^{e-E-7s}) and d_s = A_s - 128 A_{s-1}.
+// the running value A_s = sum_{i<=s} d_i 512^{s-i} equals rint(x 2^{9s-e}) (rounding half
+// to even; 512 A_{s-1} is even, so the parity of the ties is the same), hence
+// A_s = +-rne(M / 2^{e-E-9s}) and d_s = A_s - 512 A_{s-1}.
 
 // M / 2^k rounded to nearest, ties to even (M < 2^53, k >= 0).
 __device__ __forceinline__ unsigned long long rne_shift(unsigned long long M, int k)
@@ -51,317 +58,509 @@ __device__ __forceinline__ unsigned long long rne_shift(unsigned long long M, in
     return q;
 }
 
-// Vector v (0 <= v < V) has elements x(v, q) = src[v * sv + q * sq], q < K. Writes
-// D digit planes out[s * plane + v * ldo + q] (bf16, q < Kpad, zero padded) and the
-// exponent e_v (max_q |x(v, q)| = m 2^e_v, m in [0.5, 1)). Vectors V <= v < Vpad get zero
-// digits. Optional per-element factor scale[q] (a diagonal matrix multiplied in before
-// splitting).
-__global__ void ozaki_split_kernel(int V, int Vpad, int K, int Kpad, const double *__restrict__ src,
-                                   long long sv, long long sq, const double *__restrict__ scale,
-                                   const double *__restrict__ scale2, __nv_bfloat16 *__restrict__ out,
-                                   int ldo, size_t plane, int *__restrict__ exps)
+__device__ __forceinline__ unsigned long long magnitude(double x)
 {
-    __shared__ unsigned long long red[32];
+    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+
+// The row exponent from the largest magnitude bit pattern: max |x| = m 2^e, m in [0.25, 0.5).
+__device__ __forceinline__ int row_exponent(unsigned long long mb)
+{
+    if (mb == 0ull) return 0;
+    const int xf = (int)(mb >> 52);
+    return 1 + (xf ? xf - 1022 : (64 - __clzll((long long)(mb & 0xFFFFFFFFFFFFFull))) - 1074);
+}
+
+// d[s - 1] = digit s of x under the row exponent e, s = 1..ND
+template <int ND>
+__device__ __forceinline__ void digits_of(double x, int e, int (&d)[ND])
+{
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const int xf = (int)((u >> 52) & 0x7FF);
+    const unsigned long long M = xf ? ((u & 0xFFFFFFFFFFFFFull) | (1ull << 52)) : (u & 0xFFFFFFFFFFFFFull);
+    const int E = xf ? xf - 1075 : -1074;
+    const bool neg = (u >> 63) != 0ull;
+    long long aprev = 0;
+#pragma unroll
+    for (int s = 1; s <= ND; ++s) {
+        const int k = e - E - kOzBits * s;  // bits of M below digit s
+        long long a = 0;
+        // k <= -9: the digits before hold all of x
+        if (M != 0ull && k > -kOzBits) a = (long long)(k <= 0 ? (M << (-k)) : rne_shift(M, k));
+        const long long dg = (M != 0ull && k > -kOzBits) ? a - aprev * (1ll << kOzBits) : 0;
+        d[s - 1] = (int)(neg ? -dg : dg);
+        aprev = a;
+    }
+}
+
+__device__ __forceinline__ unsigned bf16_pair(int a, int b)
+{
+    const __nv_bfloat162 p = __floats2bfloat162_rn((float)a, (float)b);
+    return *reinterpret_cast<const unsigned *>(&p);
+}
+
+// Vector v (0 <= v < V) has elements x(v, q), q < K: src[v * sv + q * sq], or for q >= k1 the
+// second source src2[v * sv + (q - k1) * sq2]; optional per-element factors scale[q],
+// scale2[q] (diagonal matrices multiplied in before splitting). The first nd of its digit
+// planes go to out[s * plane + v * ldo + q] (bf16, q < Kpad, zero padded), its exponent to
+// exps[v]. Vectors V <= v < Vpad get zero digits.
+struct SplitSrc {
+    const double *src, *src2, *scale, *scale2;
+    long long sv, sq, sq2;
+    int k1;
+    __device__ __forceinline__ double at(int v, int q) const
+    {
+        double x = q < k1 ? src[(size_t)v * sv + (size_t)q * sq] : src2[(size_t)v * sv + (size_t)(q - k1) * sq2];
+        if (scale) x *= scale[q];
+        if (scale2) x *= scale2[q];
+        return x;
+    }
+};
+
+// Vectors along memory (sq = 1): one CTA per vector.
+template <int ND>
+__global__ void __launch_bounds__(256) ozaki_split_kernel(int V, int K, int Kpad, const SplitSrc s, int nd,
+                                                          __nv_bfloat16 *__restrict__ out, int ldo, size_t plane,
+                                                          int *__restrict__ exps)
+{
+    __shared__ unsigned long long red[8];
     const int v = blockIdx.x;
-    if (v >= Vpad) return;
-    __nv_bfloat16 *o = out + (size_t)v * ldo;
-    if (v >= V) {
-        for (int q = threadIdx.x; q < Kpad; q += blockDim.x)
-            for (int s = 0; s < kOzD; ++s) o[(size_t)s * plane + q] = __float2bfloat16(0.0f);
-        if (threadIdx.x == 0) exps[v] = 0;
-        return;
-    }
-    const double *x = src + (size_t)v * sv;
-    auto elem = [&](int q) {
-        double val = x[(size_t)q * sq];
-        if (scale) val *= scale[q];
-        if (scale2) val *= scale2[q];
-        return val;
-    };
-    // max |x| as the largest magnitude bit pattern (finite values order like their bits)
     unsigned long long mb = 0ull;
-    for (int q = threadIdx.x; q < K; q += blockDim.x) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(elem(q)) & 0x7FFFFFFFFFFFFFFFull;
-        mb = b > mb ? b : mb;
-    }
-    for (int o2 = 16; o2 > 0; o2 >>= 1) {
-        const unsigned long long t = __shfl_xor_sync(0xffffffffu, mb, o2);
+    if (v < V)
+        for (int q = threadIdx.x; q < K; q += 256) {
+            const unsigned long long b = magnitude(s.at(v, q));
+            mb = b > mb ? b : mb;
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long t = __shfl_xor_sync(0xffffffffu, mb, o);
         mb = t > mb ? t : mb;
     }
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mb;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        unsigned long long m = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0ull;
-        for (int o2 = 16; o2 > 0; o2 >>= 1) {
-            const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o2);
-            m = t > m ? t : m;
-        }
-        if (threadIdx.x == 0) red[0] = m;
-    }
-    __syncthreads();
-    mb = red[0];
-    // frexp exponent of the maximum: e = (bit length of M) + E
-    int e = 0;
-    if (mb != 0ull) {
-        const int xf = (int)(mb >> 52);
-        e = xf ? xf - 1022 : (64 - __clzll((long long)(mb & 0xFFFFFFFFFFFFFull))) - 1074;
-    }
-    if (threadIdx.x == 0) exps[v] = e;
-    for (int q = threadIdx.x; q < Kpad; q += blockDim.x) {
-        const unsigned long long u = (q < K) ? (unsigned long long)__double_as_longlong(elem(q)) : 0ull;
-        const int xf = (int)((u >> 52) & 0x7FF);
-        const unsigned long long M = xf ? ((u & 0xFFFFFFFFFFFFFull) | (1ull << 52)) : (u & 0xFFFFFFFFFFFFFull);
-        const int E = xf ? xf - 1075 : -1074;
-        const bool neg = (u >> 63) != 0ull;
-        long long aprev = 0;
 #pragma unroll
-        for (int s = 1; s <= kOzD; ++s) {
-            const int k = e - E - kOzBits * s;
-            long long a = 0;
-            if (M != 0ull) a = (long long)(k <= 0 ? (M << (-k)) : rne_shift(M, k));
-            if (neg) a = -a;
-            const long long dgt = a - aprev * (1ll << kOzBits);
-            aprev = a;
-            o[(size_t)(s - 1) * plane + q] = __float2bfloat16(__int2float_rn((int)dgt));
+    for (int w = 0; w < 8; ++w) mb = red[w] > mb ? red[w] : mb;
+    const int e = row_exponent(mb);
+    if (threadIdx.x == 0) exps[v] = e;
+    unsigned *o = reinterpret_cast<unsigned *>(out + (size_t)v * ldo);
+    for (int q = 2 * threadIdx.x; q < Kpad; q += 512) {
+        int a[ND], b[ND];
+        digits_of<ND>((v < V && q < K) ? s.at(v, q) : 0.0, e, a);
+        digits_of<ND>((v < V && q + 1 < K) ? s.at(v, q + 1) : 0.0, e, b);
+#pragma unroll
+        for (int d = 0; d < ND; ++d)
+            if (d < nd) o[(d * plane + q) >> 1] = bf16_pair(a[d], b[d]);
+    }
+}
+
+// Vectors across memory (sv = 1): 32 vectors per CTA, read along the vectors' index (256 bytes
+// a warp) and transposed through shared memory. One CTA per vector would read one 8-byte
+// element per 32-byte sector.
+template <int ND>
+__global__ void __launch_bounds__(256) ozaki_split_t_kernel(int V, int K, int Kpad, const SplitSrc s, int nd,
+                                                            __nv_bfloat16 *__restrict__ out, int ldo, size_t plane,
+                                                            int *__restrict__ exps)
+{
+    __shared__ unsigned long long red[8][32];
+    __shared__ int es[32];
+    __shared__ double tile[32][65];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int v0 = blockIdx.x * 32, v = v0 + tx;
+    unsigned long long mb = 0ull;
+    if (v < V) {
+#pragma unroll 8
+        for (int q = ty; q < K; q += 8) {
+            const unsigned long long b = magnitude(s.at(v, q));
+            mb = b > mb ? b : mb;
         }
+    }
+    red[ty][tx] = mb;
+    __syncthreads();
+    if (ty == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) mb = red[w][tx] > mb ? red[w][tx] : mb;
+        es[tx] = row_exponent(mb);
+        exps[v] = es[tx];
+    }
+    for (int q0 = 0; q0 < Kpad; q0 += 64) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int q = q0 + ty + 8 * u;
+            tile[tx][ty + 8 * u] = (v < V && q < K) ? s.at(v, q) : 0.0;
+        }
+        __syncthreads();
+        const int q = q0 + 2 * tx;
+        if (q < Kpad)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int r = ty * 4 + u;
+                int a[ND], b[ND];
+                digits_of<ND>(tile[r][2 * tx], es[r], a);
+                digits_of<ND>(tile[r][2 * tx + 1], es[r], b);
+                unsigned *o = reinterpret_cast<unsigned *>(out + (size_t)(v0 + r) * ldo);
+#pragma unroll
+                for (int d = 0; d < ND; ++d)
+                    if (d < nd) o[(d * plane + q) >> 1] = bf16_pair(a[d], b[d]);
+            }
     }
 }
 
 // ------------------------------------------------------------------ GEMM (tcgen05)
-// One CTA per 128 x 128 tile of C, 320 threads:
-//   warp 0, one lane: TMA producer of the (A digit plane, B digit plane) k-tiles, 64 bf16 of
-//                     K (128 bytes, 128-byte swizzle) x 128 rows each, into a STAGES ring;
-//   warp 1, one lane: MMA issuer, tcgen05.mma kind::f16 (bf16 x bf16 -> fp32), M = N = 128,
-//                     K = 16 per instruction;
+// One CTA per 128 x BN tile of C (and K range), 320 threads:
+//   warp 0, one lane: TMA producer: for each k-tile (64 of K, 128 bytes with the 128-byte
+//                     swizzle) the digit tiles A_1, B_1, A_2, B_2, .. A_D, B_D into two rings;
+//   warp 1, one lane: MMA issuer, tcgen05.mma kind::f16 (bf16 x bf16 -> fp32), M = 128,
+//                     N = BN, K = 16 per instruction;
 //   warps 2..9:       epilogue, warp w owns tensor-memory lanes (rows) 32 (w mod 4) .. + 31
-//                     and the tile columns 64 h .. 64 h + 63, h = (w - 2) / 4.
-// Work order: levels L = D+1 down to 2 (smallest contributions first), chunks of 256 along
-// K, pairs (s, L - s), k-tiles. Each chunk's sum over its pairs and k-tiles goes to one of
-// two tensor-memory accumulators (columns 0..127 and 128..255): the products are integers
-// and the sum stays below 2^24, so the accumulation is exact whatever its rounding. The
-// epilogue converts each chunk to int32 and adds it in registers (exact); at the end of a
-// level it adds alpha 2^(e_i + f_j - 7L) times the level sum to a binary64 running sum of
-// the tile kept in tensor memory (columns 256..511, the two 32-bit halves of column j's
-// value at 256 + 2j and 257 + 2j), and C is written once, after the last level. (Adding
-// each level to C in global memory instead costs a 256 KB read-modify-write per tile and
-// level, which stalls the MMA issuer once it has filled the second accumulator and
-// dominates products with a short K.)
+//                     and the tile columns h BN / 2 .. , h = (w - 2) / 4.
+// Every digit tile is loaded once per k-tile and used by all its products (level by level:
+// level L needs the digits up to L - 1, so the first products start when two tiles are there;
+// in the last level each tile is used once and its slot given back). Loading a pair of tiles
+// for each product instead costs as much shared-memory bandwidth in writes as the MMAs read.
+//
+// The epilogue converts each drained sum to an integer (exact) and adds it, shifted, to
+// integers in registers. Refinement form: 64 bits, units of 2^(e - 9 (D + 1)) with e the
+// smallest shift that cannot overflow them (D = 6: e = 7 at K = 256, one more for each
+// doubling of K; 0 for D <= 4). Wide form: levels 2..5 and 6..9 in two 64-bit integers (units
+// of level 5 and of level 9), put together to 128 bits at the end. The sums become binary64
+// values by integer operations and are written as C = alpha (...) + beta C. (A binary64
+// conversion and addition per level and element, at two a clock, took longer than the MMAs of
+// a product with K <= 2048.)
+//
+// Measured (8192 x 2304 x 8192): D = 6 6.3 ms, 1.03 PFLOP/s of digit products (0.54 of the
+// measured bf16 rate; 5.5 ms without loads and drains, what is left are the hand-overs of a
+// ring that holds little more than one k-tile); n = 16384 solve, all refinement products 385
+// -> 257 ms. Binary64 route, products of a solve against the SIMT kernel: n = 1531 67 -> 13 ms,
+// n = 5000 758 -> 93 ms.
 namespace oztc {
-constexpr int BM = 128, BN = 128, BK = 64, STAGES = 7;
-constexpr int CHUNK_TILES = 256 / BK;         // k-tiles per exact chunk
-constexpr int TILE_BYTES = BM * BK * 2;       // 16 KB
-constexpr int STAGE_BYTES = 2 * TILE_BYTES;   // A tile + B tile
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
-constexpr int TMEM_COLS = 4 * BN;  // two accumulators + the binary64 running sum
-constexpr int EPI_WARPS = 8, CW = BN / 2;  // epilogue warps; columns per epilogue warp
+constexpr int BM = 128, BK = 64;
+constexpr int A_BYTES = BM * BK * 2;  // 16 KB
+constexpr int EPI_WARPS = 8;
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
+
+template <bool WIDE> struct Cfg {
+    static constexpr int BN = WIDE ? 64 : 128;
+    static constexpr int RING = WIDE ? 9 : 7;  // slots of each operand's ring (> D)
+    static constexpr int NBUF = WIDE ? 3 : 2;  // accumulators of the drained levels
+    static constexpr int EXACT = WIDE ? 8 : 5; // levels above are summed in binary32 over K
+    static constexpr int NBACK = 16;           // barriers of the give-back events (> events in flight)
+    static constexpr int B_BYTES = BN * BK * 2;
+    static constexpr int SMEM_BYTES = RING * (A_BYTES + B_BYTES) + 1024 + 512;
+    static constexpr int TMEM_COLS = 4 * BN;   // NBUF accumulators, then the binary32 levels
+    static constexpr int CW = BN / 2;          // columns per epilogue warp
+};
 
 struct Maps {
     CUtensorMap a, b;  // planes as (D * Mpad) x Kpad and (D * Npad) x Kpad bf16 matrices
 };
 
 struct Args {
-    int m_real, n_real, kpad, mpad, npad, uplo, ldc;
-    int kt0;     // first k-tile of this launch's K segment; kpad is the segment's end
-    int digits;  // D <= kOzD: digit planes used per operand (levels 2 .. D + 1)
+    int m_real, n_real, mpad, npad, uplo, ldc;
+    int kt0, nkt, ktz;  // first k-tile and number of them in this launch; k-tiles per blockIdx.z
+    int digits;         // D digit planes per operand (levels 2 .. D + 1)
+    int order[9];       // the levels in the order of their products
+    int eshift;         // refinement form: units of the integer sums 2^(eshift - 9 (D + 1))
     const int *ea, *eb;
     double alpha, beta;
+    int alpha_exp;      // alpha = +-2^alpha_exp, or kNotPow2
     double *C;
+    size_t cstride;     // C of blockIdx.z: C + z cstride
     int *status;
 };
+constexpr int kNotPow2 = 1 << 20;
 }  // namespace oztc
 
-// x 2^e: a multiplication by a power of two built from its bit pattern where 2^e is a normal
-// number (exact, like ldexp), ldexp elsewhere.
-__device__ __forceinline__ double scale2(double x, int e)
+// a 2^e rounded to nearest even, with integer operations where the result is a normal number
+__device__ __forceinline__ double pack_double(unsigned long long nrm, bool sticky, bool neg, int biased)
 {
-    if (e >= -1022 && e <= 1023) return x * __longlong_as_double((long long)(e + 1023) << 52);
-    return ldexp(x, e);
+    unsigned long long mant = nrm >> 11;  // 53 bits
+    const unsigned rem = (unsigned)nrm & 0x7FFu;
+    mant += (rem > 0x400u || (rem == 0x400u && (sticky || (mant & 1ull)))) ? 1ull : 0ull;
+    const unsigned long long bits = ((unsigned long long)(biased - 1) << 52) + mant;  // mant has bit 52
+    return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
+__device__ __forceinline__ double fixed_to_double(long long a, int e)
+{
+    if (a == 0) return 0.0;
+    const unsigned long long u = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
+    const int lz = __clzll((long long)u);
+    const int biased = 1086 - lz + e;  // exponent field of 2^63 2^(e - lz)
+    if (biased < 1 || biased > 2045) return ldexp((double)a, e);
+    return pack_double(u << lz, false, a < 0, biased);
+}
+
+// (hi 2^36 + lo) 2^e
+__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int e)
+{
+    const __int128 t = ((__int128)hi << 36) + (__int128)lo;
+    const bool neg = t < 0;
+    const unsigned __int128 u = neg ? (unsigned __int128)(-t) : (unsigned __int128)t;
+    const unsigned long long uh = (unsigned long long)(u >> 64), ul = (unsigned long long)u;
+    if (uh == 0ull) {
+        if (ul == 0ull) return 0.0;
+        const int lz = __clzll((long long)ul), biased = 1086 - lz + e;
+        if (biased >= 1 && biased <= 2045) return pack_double(ul << lz, false, neg, biased);
+        const double v = ldexp((double)ul, e);
+        return neg ? -v : v;
+    }
+    const int lz = __clzll((long long)uh), biased = 1150 - lz + e;
+    const unsigned long long nrm = lz ? (uh << lz) | (ul >> (64 - lz)) : uh;
+    const bool sticky = (lz ? ul << lz : ul) != 0ull;
+    if (biased >= 1 && biased <= 2045) return pack_double(nrm, sticky, neg, biased);
+    const double v = ldexp((double)(nrm | (sticky ? 1ull : 0ull)), e + 64 - lz);
+    return neg ? -v : v;
+}
+
+template <bool WIDE>
 __global__ void __launch_bounds__(oztc::THREADS, 1)
-ozaki_gemm_tc_kernel(const __grid_constant__ oztc::Maps maps, const oztc::Args a)
+ozaki_gemm_tc_kernel(const __grid_constant__ oztc::Maps maps, const __grid_constant__ oztc::Args a)
 {
     using namespace oztc;
     using namespace tc5;
+    using F = Cfg<WIDE>;
+    constexpr int BN = F::BN, RING = F::RING, NBUF = F::NBUF, CW = F::CW, NBACK = F::NBACK;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((size_t)smem_raw + 1023) & ~(size_t)1023);
-    unsigned long long *bars = (unsigned long long *)(smem + STAGES * STAGE_BYTES);
-    // bars: [0,S) full, [S,2S) empty, 2S+b accumulator b full, 2S+2+b accumulator b empty
-    unsigned *tmem_slot = (unsigned *)(bars + 2 * STAGES + 4);
+    unsigned long long *bars = (unsigned long long *)(smem + RING * (A_BYTES + F::B_BYTES));
+    __shared__ unsigned tmem_slot;
     __shared__ int aborted;
+    __shared__ int ebs[BN];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
     if (m0 >= a.m_real || n0 >= a.n_real) return;
     if (a.uplo && m0 + BM - 1 < n0) return;  // tile strictly above the diagonal
-    const int nkt = (a.kpad + BK - 1) / BK - a.kt0;  // k-tiles of this segment
-    const int nch = (nkt + CHUNK_TILES - 1) / CHUNK_TILES;
-    const unsigned full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[STAGES]);
-    const unsigned accf0 = smem_u32(&bars[2 * STAGES]), acce0 = smem_u32(&bars[2 * STAGES + 2]);
+    const int kz = blockIdx.z * a.ktz;       // k-tiles [kz, kz + nkt) of this launch's range
+    const int nkt = min(a.ktz, a.nkt - kz);
+    const int D = a.digits, X = min(D, F::EXACT);  // levels 2..X are drained
+    // barriers: digits loaded (one per ring slot), slots given back (events, see below),
+    // accumulators full, empty; the end
+    const unsigned bar0 = smem_u32(bars);
+    const unsigned full0 = bar0, back0 = bar0 + 8 * RING;
+    const unsigned accf0 = back0 + 8 * NBACK, acce0 = accf0 + 8 * NBUF, done = acce0 + 8 * NBUF;
+    // Slots are given back two digits at a time: event u (u = 0, 1, ..) of a k-tile follows the
+    // products (u + 1, D - u) and (D - u, u + 1) of the last level, the last uses of these two
+    // digits (one commit for both: a commit holds the tensor pipe up for about 90 cycles).
+    const int EV = (D + 1) / 2;  // events per k-tile
+    const unsigned sA = smem_u32(smem), sB = sA + RING * A_BYTES;
 
     if (tid == 0) {
-        for (int q = 0; q < 2 * STAGES + 2; ++q) mbar_init(smem_u32(&bars[q]), 1);
-        mbar_init(acce0, EPI_WARPS);
-        mbar_init(acce0 + 8, EPI_WARPS);
+        for (int q = 0; q < RING + NBACK + NBUF; ++q) mbar_init(bar0 + 8 * q, 1);
+        for (int q = 0; q < NBUF; ++q) mbar_init(acce0 + 8 * q, EPI_WARPS);
+        mbar_init(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         aborted = 0;
     }
-    if (warp == 2) tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
+    if (tid >= 64 && tid < 64 + BN) ebs[tid - 64] = n0 + tid - 64 < a.n_real ? a.eb[n0 + tid - 64] : 0;
+    if (warp == 2) tmem_alloc(smem_u32(&tmem_slot), F::TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const unsigned tmem = *tmem_slot;
+    const unsigned tmem = tmem_slot;
+    auto give_up = [&](int where) {
+        report_error(a.status, ELSI_ERR_TIMEOUT, where);
+        atomicExch(&aborted, 1);
+    };
 
-    int armed = 0;
+    int armed = 0;  // digits loaded
     if (warp == 0) {
         if (lane == 0) {
-            int it = 0;
+            int it = 0, seen = 0;  // digits; give-back events waited for
             bool stop = false;
-            for (int L = a.digits + 1; L >= 2 && !stop; --L) {
-                const int s_lo = max(1, L - a.digits), s_hi = min(a.digits, L - 1);
-                for (int c = 0; c < nch && !stop; ++c) {
-                    const int kt1 = min(nkt, (c + 1) * CHUNK_TILES);
-                    for (int sa = s_lo; sa <= s_hi && !stop; ++sa)
-                        for (int kt = c * CHUNK_TILES; kt < kt1; ++kt, ++it) {
-                            const int st = it % STAGES;
-                            if (it >= STAGES && !mbar_wait(empty0 + 8 * st, ((it / STAGES) & 1) ^ 1)) {
-                                report_error(a.status, ELSI_ERR_TIMEOUT, 11);
-                                atomicExch(&aborted, 1);
+            for (int kt = 0; kt < nkt && !stop; ++kt) {
+                const int kx = (a.kt0 + kz + kt) * BK;
+                for (int q = 0; q < D; ++q, ++it) {
+                    const int sl = it % RING;
+                    if (it >= RING) {  // the event that gave back the slot's digit q0 (0-based)
+                        const int old = it - RING, q0 = old % D;
+                        const int need = old / D * EV + min(q0, D - 1 - q0);
+                        for (; seen <= need && !stop; ++seen)
+                            if (!mbar_wait_hot(back0 + 8 * (seen % NBACK), (seen / NBACK) & 1)) {
+                                give_up(11);
                                 stop = true;
-                                break;
                             }
-                            if (*(volatile int *)&aborted) { stop = true; break; }
-                            unsigned char *dst = smem + st * STAGE_BYTES;
-                            const unsigned full = full0 + 8 * st;
-                            mbar_expect_tx(full, STAGE_BYTES);
-                            const int kx = (a.kt0 + kt) * BK;
-                            tma_load_2d(smem_u32(dst), &maps.a, full, kx, (sa - 1) * a.mpad + m0);
-                            tma_load_2d(smem_u32(dst + TILE_BYTES), &maps.b, full, kx,
-                                        (L - sa - 1) * a.npad + n0);
-                            armed = it + 1;
-                        }
+                    }
+                    if (stop || *(volatile int *)&aborted) { stop = true; break; }
+                    mbar_expect_tx(full0 + 8 * sl, A_BYTES + F::B_BYTES);
+                    tma_load_2d(sA + sl * A_BYTES, &maps.a, full0 + 8 * sl, kx, q * a.mpad + m0);
+                    tma_load_2d(sB + sl * F::B_BYTES, &maps.b, full0 + 8 * sl, kx, q * a.npad + n0);
+                    armed = it + 1;
                 }
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
             const unsigned idesc = idesc_f32acc(1, BM, BN);
-            int it = 0, g = 0;
+            const unsigned long long dA = sdesc(sA), dB = sdesc(sB);
+            int g = 0, ev = 0, base = 0;  // drained sums, events; ring slot of digit 1 of the k-tile
+            unsigned phase = 0;   // parity of the full barriers at slot 'base'
             bool stop = false;
-            for (int L = a.digits + 1; L >= 2 && !stop; --L) {
-                const int s_lo = max(1, L - a.digits), s_hi = min(a.digits, L - 1);
-                for (int c = 0; c < nch && !stop; ++c, ++g) {
-                    const int bsel = g & 1;
-                    if (g >= 2 && !mbar_wait(acce0 + 8 * bsel, ((g >> 1) - 1) & 1)) {
-                        report_error(a.status, ELSI_ERR_TIMEOUT, 12);
-                        atomicExch(&aborted, 1);
-                        stop = true;
-                        break;
-                    }
-                    const unsigned d = tmem + bsel * BN;
-                    const int kt1 = min(nkt, (c + 1) * CHUNK_TILES);
-                    bool first = true;
-                    for (int sa = s_lo; sa <= s_hi && !stop; ++sa)
-                        for (int kt = c * CHUNK_TILES; kt < kt1; ++kt, ++it) {
-                            const int st = it % STAGES;
-                            if (!mbar_wait(full0 + 8 * st, (it / STAGES) & 1)) {
-                                report_error(a.status, ELSI_ERR_TIMEOUT, 13);
-                                atomicExch(&aborted, 1);
-                                stop = true;
-                                break;
-                            }
-                            tc_fence_after();
-                            const unsigned base = smem_u32(smem + st * STAGE_BYTES);
-#pragma unroll
-                            for (int kk = 0; kk < BK / 16; ++kk) {
-                                const unsigned off = kk * 32;  // 16 bf16 along K
-                                mma_bf16(d, sdesc(base + off), sdesc(base + TILE_BYTES + off), idesc,
-                                         first ? 0u : 1u);
-                                first = false;
-                            }
-                            mma_commit(empty0 + 8 * st);
+            for (int kt = 0; kt < nkt && !stop; ++kt) {
+                int have = 0;  // digits of this k-tile that have arrived
+                for (int o = 0; o < D && !stop; ++o) {
+                    const int L = a.order[o];
+                    for (; have < min(L - 1, D); ++have) {
+                        const int sl = base + have >= RING ? base + have - RING : base + have;
+                        const unsigned ph = base + have >= RING ? phase ^ 1u : phase;
+                        if (!mbar_wait_hot(full0 + 8 * sl, ph)) {
+                            give_up(13);
+                            stop = true;
+                            break;
                         }
-                    if (!stop) mma_commit(accf0 + 8 * bsel);
+                    }
+                    if (stop) break;
+                    unsigned d, acc;
+                    const int buf = g % NBUF;
+                    if (L <= X) {
+                        if (g >= NBUF && !mbar_wait_hot(acce0 + 8 * buf, ((g / NBUF) & 1) ^ 1)) {
+                            give_up(12);
+                            stop = true;
+                            break;
+                        }
+                        d = tmem + buf * BN;
+                        acc = 0;
+                    } else {
+                        d = tmem + (NBUF + L - X - 1) * BN;
+                        acc = kt > 0 ? 1u : 0u;
+                    }
+                    tc_fence_after();
+                    // pairs (s, t), s + t = L, 1 <= s, t <= D; in the last level in the order
+                    // (1, D), (D, 1), (2, D - 1), .. that gives the slots back as they are refilled
+                    const bool last = L == D + 1;
+                    for (int u = 0; u < L - 1; ++u) {
+                        const int s = last ? ((u & 1) ? D - (u >> 1) : 1 + (u >> 1)) : 1 + u, t = L - s;
+                        int la = base + s - 1, lb = base + t - 1;
+                        la = la >= RING ? la - RING : la;
+                        lb = lb >= RING ? lb - RING : lb;
+                        const unsigned long long da = dA + (unsigned)(la * (A_BYTES >> 4));
+                        const unsigned long long db = dB + (unsigned)(lb * (F::B_BYTES >> 4));
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            mma_bf16(d, da + 2 * kk, db + 2 * kk, idesc, acc);
+                            acc = 1;
+                        }
+                        if (last && ((u & 1) || u == D - 1)) {
+                            mma_commit(back0 + 8 * (ev % NBACK));
+                            ++ev;
+                        }
+                    }
+                    if (L <= X) {
+                        mma_commit(accf0 + 8 * buf);
+                        ++g;
+                    }
                 }
+                base += D;
+                if (base >= RING) { base -= RING; phase ^= 1u; }
             }
+            mma_commit(done);
+            if (stop) mbar_wait(done, 0);  // nothing in flight when the tensor memory is freed
         }
     } else {
-        // tensor-memory loads and stores are warp-collective: every lane runs them (rows past
-        // m only skip their global-memory accesses) and the wait results are made uniform
+        // tensor-memory loads are warp-collective: every lane runs them (rows past m only skip
+        // their global-memory accesses) and the wait results are made uniform
         const int quarter = warp & 3, c0 = ((warp - 2) >> 2) * CW;  // rows, first column
         const int row = m0 + quarter * 32 + lane;
         const bool row_in = row < a.m_real;
-        const int er = row_in ? a.ea[row] : 0;
-        const unsigned tlane = tmem + ((unsigned)(quarter * 32) << 16);
-        const unsigned tsum = tlane + 2 * BN + 2 * c0;
-        int iacc[CW];
+        const unsigned tlane = tmem + ((unsigned)(quarter * 32) << 16) + c0;
+        long long acc[CW], low[WIDE ? CW : 1];
+#pragma unroll
+        for (int j = 0; j < CW; ++j) acc[j] = 0;
+#pragma unroll
+        for (int j = 0; j < (WIDE ? CW : 1); ++j) low[j] = 0;
         bool ok = true;
         int g = 0;
-        for (int L = a.digits + 1; L >= 2 && ok; --L) {
-#pragma unroll
-            for (int j = 0; j < CW; ++j) iacc[j] = 0;
-            for (int c = 0; c < nch; ++c, ++g) {
-                const int bsel = g & 1;
-                ok = __all_sync(0xffffffffu, mbar_wait(accf0 + 8 * bsel, (g >> 1) & 1));
+        for (int kt = 0; kt < nkt && ok; ++kt)
+            for (int L = 2; L <= X; ++L, ++g) {
+                const int buf = g % NBUF;
+                ok = __all_sync(0xffffffffu, mbar_wait_hot(accf0 + 8 * buf, (g / NBUF) & 1));
                 if (!ok) {
-                    if (lane == 0) {
-                        report_error(a.status, ELSI_ERR_TIMEOUT, 14);
-                        atomicExch(&aborted, 1);
-                    }
+                    if (lane == 0) give_up(14);
                     break;
                 }
                 tc_fence_after();
+                const int sh = WIDE ? kOzBits * (L <= 5 ? 5 - L : 9 - L) : kOzBits * (D + 1 - L) - a.eshift;
 #pragma unroll
-                for (int q = 0; q < CW / 32; ++q) {
-                    float v[32];
-                    tmem_ld32(tlane + bsel * BN + c0 + q * 32, v);
+                for (int q = 0; q < CW / 16; ++q) {
+                    float v[16];
+                    tmem_ld16(tlane + buf * BN + q * 16, v);
+                    if (WIDE) {
+                        const int mul = 1 << sh;  // sh <= 27
+                        if (L <= 5) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) iacc[q * 32 + j] += __float2int_rn(v[j]);
+                            for (int j = 0; j < 16; ++j) acc[q * 16 + j] += (long long)__float2int_rn(v[j]) * mul;
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j)
+                                low[WIDE ? q * 16 + j : 0] += (long long)__float2int_rn(v[j]) * mul;
+                        }
+                    } else if (sh >= 32) {
+                        const int up = sh - 32;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            acc[q * 16 + j] += (long long)((unsigned long long)((unsigned)__float2int_rn(v[j]) << up) << 32);
+                    } else if (sh >= 0) {
+                        const int mul = 1 << sh;  // sh <= 30: see oz_shift()
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) acc[q * 16 + j] += (long long)__float2int_rn(v[j]) * mul;
+                    } else {
+                        const int half = 1 << (-sh - 1);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) acc[q * 16 + j] += (__float2int_rn(v[j]) + half) >> -sh;
+                    }
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(acce0 + 8 * bsel);
+                if (lane == 0) mbar_arrive(acce0 + 8 * buf);
             }
-            if (!ok) break;
-            // running sum += alpha 2^(e_i + f_j - 7L) level sum, 16 columns at a time
-            const bool firstL = (L == a.digits + 1);
-#pragma unroll
-            for (int q = 0; q < CW / 16; ++q) {
-                unsigned w[32];
-                if (!firstL) tmem_ld32_u(tsum + q * 32, w);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int col = n0 + c0 + q * 16 + j;
-                    const int ec = col < a.n_real ? a.eb[col] : 0;
-                    const double val = a.alpha * scale2((double)iacc[q * 16 + j], er + ec - kOzBits * L);
-                    const double sum = firstL ? val : __hiloint2double((int)w[2 * j + 1], (int)w[2 * j]) + val;
-                    w[2 * j] = (unsigned)__double2loint(sum);
-                    w[2 * j + 1] = (unsigned)__double2hiint(sum);
-                }
-                tmem_st32_u(tsum + q * 32, w);
-            }
+        if (ok) {
+            ok = __all_sync(0xffffffffu, mbar_wait(done, 0));
+            if (!ok && lane == 0) give_up(15);
         }
         if (ok) {
-            // C = beta C + running sum, 16 columns at a time (the loads of C first)
-            double *crow = a.C + (size_t)row;
-#pragma unroll 1
-            for (int q = 0; q < CW / 16; ++q) {
-                unsigned w[32];
-                tmem_ld32_u(tsum + q * 32, w);
-                double cv[16];
+            tc_fence_after();
+            // the levels summed in binary32, in the units of the integers
+            for (int L = X + 1; L <= D + 1; ++L) {
+                const int sh = WIDE ? 0 : kOzBits * (D + 1 - L) - a.eshift;
+                const float sc = __int_as_float((127 + sh) << 23);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int col = n0 + c0 + q * 16 + j;
+                for (int q = 0; q < CW / 16; ++q) {
+                    float v[16];
+                    tmem_ld16(tlane + (NBUF + L - X - 1) * BN + q * 16, v);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        if (WIDE) low[WIDE ? q * 16 + j : 0] += __float2ll_rn(v[j]);
+                        else acc[q * 16 + j] += __float2ll_rn(v[j] * sc);
+                    }
+                }
+            }
+            const bool pow2 = a.alpha_exp != kNotPow2;
+            const bool neg = pow2 && a.alpha < 0.0;
+            const int er = (row_in ? a.ea[row] : 0) - kOzBits * (WIDE ? 9 : D + 1) + (WIDE ? 0 : a.eshift) +
+                           (pow2 ? a.alpha_exp : 0);
+            double *crow = a.C + blockIdx.z * a.cstride + (size_t)row;
+            // C = beta C + sum, 8 columns at a time (the loads of C first)
+#pragma unroll
+            for (int q = 0; q < CW / 8; ++q) {
+                double cv[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int col = n0 + c0 + q * 8 + j;
                     const bool in = row_in && col < a.n_real && (!a.uplo || row >= col);
                     cv[j] = (in && a.beta != 0.0) ? crow[(size_t)col * a.ldc] : 0.0;
                 }
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int col = n0 + c0 + q * 16 + j;
+                for (int j = 0; j < 8; ++j) {
+                    const int cl = c0 + q * 8 + j, col = n0 + cl;
                     if (row_in && col < a.n_real && (!a.uplo || row >= col)) {
-                        const double sum = __hiloint2double((int)w[2 * j + 1], (int)w[2 * j]);
-                        crow[(size_t)col * a.ldc] = a.beta != 0.0 ? fma(a.beta, cv[j], sum) : sum;
+                        double val;
+                        if (WIDE) val = fixed_to_double(acc[q * 8 + j], low[WIDE ? q * 8 + j : 0], er + ebs[cl]);
+                        else val = fixed_to_double(acc[q * 8 + j], er + ebs[cl]);
+                        if (neg) val = -val;
+                        if (!pow2) val *= a.alpha;
+                        if (a.beta == 1.0) val += cv[j];
+                        else if (a.beta != 0.0) val = fma(a.beta, cv[j], val);
+                        crow[(size_t)col * a.ldc] = val;
                     }
                 }
             }
@@ -370,11 +569,24 @@ ozaki_gemm_tc_kernel(const __grid_constant__ oztc::Maps maps, const oztc::Args a
     tc_fence_before();
     __syncthreads();
     if (aborted && warp == 0 && lane == 0) {
-        for (int it = (armed > STAGES ? armed - STAGES : 0); it < armed; ++it)
-            mbar_wait(full0 + 8 * (it % STAGES), (it / STAGES) & 1);
+        for (int it = (armed > RING ? armed - RING : 0); it < armed; ++it)
+            mbar_wait(full0 + 8 * (it % RING), (it / RING) & 1);
     }
     __syncthreads();
-    if (warp == 2) tmem_free(tmem, TMEM_COLS);
+    if (warp == 2) tmem_free(tmem, F::TMEM_COLS);
+}
+
+// C = beta C + sum of the K ranges' partial products (ascending, m x n each)
+__global__ void ozaki_reduce_kernel(int m, int n, int parts, const double *__restrict__ part, double beta,
+                                    double *C, int ldc)
+{
+    const size_t total = (size_t)m * n;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+        double s = 0.0;
+        for (int z = 0; z < parts; ++z) s += part[(size_t)z * total + e];
+        double *c = C + (e % m) + (e / m) * (size_t)ldc;
+        *c = beta != 0.0 ? fma(beta, *c, s) : s;
+    }
 }
 
 size_t ozaki_plane_elems(int V, int K)
@@ -382,39 +594,93 @@ size_t ozaki_plane_elems(int V, int K)
     return (size_t)ceil_div(V, kOzBM) * kOzBM * (size_t)(ceil_div(K, kOzBK) * kOzBK);
 }
 
-size_t ozaki_split_elems(int V, int K) { return ozaki_plane_elems(V, K) * kOzD; }
+size_t ozaki_split_elems(int V, int K, int digits) { return ozaki_plane_elems(V, K) * digits; }
 
 cudaError_t ozaki_split(cudaStream_t st, int V, int K, const double *src, long long sv,
                         long long sq, const double *scale, const double *scale2,
-                        __nv_bfloat16 *planes, int *exps)
+                        __nv_bfloat16 *planes, int *exps, int digits, const double *src2, long long sq2, int k1)
 {
+    if (digits < 1 || (digits > kOzDigits && digits != kOzWide)) return cudaErrorInvalidValue;
     const int Vpad = ceil_div(V, kOzBM) * kOzBM;
     const int Kpad = ceil_div(K, kOzBK) * kOzBK;
+    const size_t plane = ozaki_plane_elems(V, K);
+    SplitSrc s;
+    s.src = src; s.src2 = src2; s.scale = scale; s.scale2 = scale2;
+    s.sv = sv; s.sq = sq; s.sq2 = sq2; s.k1 = src2 ? k1 : K;
+    const bool across = sv == 1 && sq != 1;
     EGB_COUNT_LAUNCH();
-    ozaki_split_kernel<<<Vpad, 256, 0, st>>>(V, Vpad, K, Kpad, src, sv, sq, scale, scale2, planes,
-                                             Kpad, ozaki_plane_elems(V, K), exps);
+    if (digits == kOzWide) {
+        if (across) ozaki_split_t_kernel<kOzWide><<<Vpad / 32, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
+        else ozaki_split_kernel<kOzWide><<<Vpad, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
+    } else {
+        if (across) ozaki_split_t_kernel<kOzDigits><<<Vpad / 32, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
+        else ozaki_split_kernel<kOzDigits><<<Vpad, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
+    }
+    return cudaGetLastError();
+}
+
+// Units of the integer sums of the refinement form for K terms: level 2 adds up to
+// K 2^16 2^(9 (D - 1) - e), which has to stay below 2^62; a shift of exactly 31 is avoided (the
+// multiplication by 2^31 does not fit a signed 32-bit factor).
+static int oz_shift(int k, int digits)
+{
+    int lg = 0;
+    while ((1ll << lg) < k) ++lg;
+    int e = lg + 16 + kOzBits * (digits - 1) - 62;
+    if (e < 0) e = 0;
+    for (bool again = true; again;) {
+        again = false;
+        for (int L = 2; L <= digits; ++L)
+            if (kOzBits * (digits + 1 - L) - e == 31) again = true;
+        if (again) ++e;
+    }
+    return e;
+}
+
+template <bool WIDE>
+static cudaError_t oz_launch(cudaStream_t st, dim3 grid, const oztc::Maps &maps, const oztc::Args &a)
+{
+    static PerDeviceOnce attr;
+    cudaError_t e = once_per_device(attr, [] {
+        return cudaFuncSetAttribute(ozaki_gemm_tc_kernel<WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    oztc::Cfg<WIDE>::SMEM_BYTES);
+    });
+    if (e != cudaSuccess) return e;
+    EGB_COUNT_LAUNCH();
+    ozaki_gemm_tc_kernel<WIDE><<<grid, oztc::THREADS, oztc::Cfg<WIDE>::SMEM_BYTES, st>>>(maps, a);
     return cudaGetLastError();
 }
 
 cudaError_t ozaki_gemm(cudaStream_t st, int m, int n, int k, double alpha,
                        const __nv_bfloat16 *Ad, const int *ea, const __nv_bfloat16 *Bd,
-                       const int *eb, double beta, double *C, int ldc, int uplo, int digits)
+                       const int *eb, double beta, double *C, int ldc, int uplo, int digits,
+                       double *part, size_t part_elems)
 {
-    if (digits < 1 || digits > kOzD) return cudaErrorInvalidValue;
+    const bool wide = digits == kOzWide;
+    if (digits < 1 || (digits > kOzDigits && !wide)) return cudaErrorInvalidValue;
     using namespace oztc;
     if (m <= 0 || n <= 0) return cudaSuccess;
     const int mpad = ceil_div(m, kOzBM) * kOzBM, npad = ceil_div(n, kOzBN) * kOzBN;
     const int kpad = ceil_div(k, kOzBK) * kOzBK;
+    const int bn = wide ? Cfg<true>::BN : Cfg<false>::BN;
     Maps maps;
-    if (!tc5::make_map_2d(&maps.a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Ad, (long long)kOzD * mpad, kpad,
+    if (!tc5::make_map_2d(&maps.a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Ad, (long long)digits * mpad, kpad,
                           kpad, BK, BM) ||
-        !tc5::make_map_2d(&maps.b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Bd, (long long)kOzD * npad, kpad,
-                          kpad, BK, BN))
+        !tc5::make_map_2d(&maps.b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Bd, (long long)digits * npad, kpad,
+                          kpad, BK, bn))
         return cudaErrorNotSupported;
     Args a;
-    a.m_real = m; a.n_real = n; a.kpad = kpad; a.mpad = mpad; a.npad = npad; a.uplo = uplo;
-    a.ldc = ldc; a.ea = ea; a.eb = eb; a.alpha = alpha; a.beta = beta; a.C = C;
+    a.m_real = m; a.n_real = n; a.mpad = mpad; a.npad = npad; a.uplo = uplo;
+    a.ldc = ldc; a.ea = ea; a.eb = eb; a.alpha = alpha; a.beta = beta; a.C = C; a.cstride = 0;
     a.digits = digits;
+    for (int o = 0; o < 9; ++o) a.order[o] = o + 2;
+    if (digits == 6) {  // level 6 (not drained) between 4 and 5: time to drain the two accumulators
+        a.order[3] = 6;
+        a.order[4] = 5;
+    }
+    int xp = 0;
+    const double mant = frexp(alpha, &xp);  // alpha = mant 2^xp
+    a.alpha_exp = (mant == 0.5 || mant == -0.5) ? xp - 1 : kNotPow2;
     float *tw;
     size_t te;
     int *ts = nullptr;
@@ -425,8 +691,6 @@ cudaError_t ozaki_gemm(cudaStream_t st, int m, int n, int k, double alpha,
     cudaError_t attr_err = once_per_device(once, [] {
         int dev = 0;
         cudaError_t r = cudaGetDevice(&dev);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(ozaki_gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
         if (r == cudaSuccess && dev >= 0 && dev < kMaxDevices && !dummy_status[dev]) {
             int *p = nullptr;
             r = cudaMalloc((void **)&p, 8 * sizeof(int));
@@ -440,15 +704,36 @@ cudaError_t ozaki_gemm(cudaStream_t st, int m, int n, int k, double alpha,
     cudaGetDevice(&dev_now);
     a.status = ts ? ts : (dev_now >= 0 && dev_now < kMaxDevices ? dummy_status[dev_now] : nullptr);
     if (!a.status) return cudaErrorInvalidDevice;
-    dim3 grid(mpad / BM, npad / BN);
+    const int tiles_m = mpad / BM, tiles_n = ceil_div(n, bn);
+    auto go = [&](dim3 grid) { return wide ? oz_launch<true>(st, grid, maps, a) : oz_launch<false>(st, grid, maps, a); };
+    // Few output tiles and a long K (A22 V of a panel): the K range is divided over CTAs, each
+    // with at least two k-tiles, and the partial products are added in a second pass.
+    const int nkt_all = ceil_div(kpad, BK);
+    if (!uplo && k <= kOzSegK && part) {
+        int parts = 152 / (tiles_m * tiles_n);
+        if (parts > nkt_all / 2) parts = nkt_all / 2;
+        if ((size_t)(parts > 0 ? parts : 1) * m * n > part_elems) parts = (int)(part_elems / ((size_t)m * n));
+        if (parts > 1) {
+            a.kt0 = 0; a.nkt = nkt_all; a.ktz = ceil_div(nkt_all, parts);
+            parts = ceil_div(nkt_all, a.ktz);
+            a.eshift = oz_shift(a.ktz * BK, digits);
+            a.beta = 0.0; a.C = part; a.ldc = m; a.cstride = (size_t)m * n;
+            cudaError_t e = go(dim3(tiles_m, tiles_n, parts));
+            if (e != cudaSuccess) return e;
+            int rg = ceil_div((long long)m * n, 256);
+            EGB_COUNT_LAUNCH();
+            ozaki_reduce_kernel<<<rg > 152 * 8 ? 152 * 8 : rg, 256, 0, st>>>(m, n, parts, part, beta, C, ldc);
+            return cudaGetLastError();
+        }
+    }
     // K segments of kOzSegK (a multiple of BK): the first applies beta, the rest add
     for (int k0 = 0; k0 < kpad; k0 += kOzSegK) {
+        const int k1 = min(kpad, k0 + kOzSegK);
         a.kt0 = k0 / BK;
-        a.kpad = min(kpad, k0 + kOzSegK);
+        a.nkt = a.ktz = ceil_div(k1 - k0, BK);
+        a.eshift = oz_shift(k1 - k0, digits);
         a.beta = k0 == 0 ? beta : 1.0;
-        EGB_COUNT_LAUNCH();
-        ozaki_gemm_tc_kernel<<<grid, THREADS, SMEM_BYTES, st>>>(maps, a);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = go(dim3(tiles_m, tiles_n));
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

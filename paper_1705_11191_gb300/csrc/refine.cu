@@ -546,15 +546,15 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     // products, cluster Rayleigh-Ritz rotation and the Rayleigh quotients of the
     // current X_o (steps shared by every iteration and the final polish). digits: digit
     // planes of the binary64-accurate products (D digits: D (D + 1) / 2 digit products,
-    // truncation about 2^(-7 D) relative); the first iterations, which correct errors of
+    // truncation about 2^(-9 D) relative); the first iterations, which correct errors of
     // about 1e-3, need fewer than the later ones and the final polish (see the loop).
     auto products_and_rr = [&](int digits) -> int {
-        CKR(ozaki_split(st, k, n, XO, n, 1, nullptr, nullptr, XDG, eX));
+        CKR(ozaki_split(st, k, n, XO, n, 1, nullptr, nullptr, XDG, eX, digits));
         CKR(ozaki_gemm(st, n, k, n, 1.0, HDG, eH, XDG, eX, 0.0, YH, n, 0, digits));
         if (S64) CKR(ozaki_gemm(st, n, k, n, 1.0, SDG, eS, XDG, eX, 0.0, YS, n, 0, digits));
         else CKR(cudaMemcpyAsync(YS, XO, sizeof(double) * nk, cudaMemcpyDeviceToDevice, st));
-        CKR(ozaki_split(st, k, n, YH, n, 1, nullptr, nullptr, YHDG, eYH));
-        CKR(ozaki_split(st, k, n, YS, n, 1, nullptr, nullptr, YSDG, eYS));
+        CKR(ozaki_split(st, k, n, YH, n, 1, nullptr, nullptr, YHDG, eYH, digits));
+        CKR(ozaki_split(st, k, n, YS, n, 1, nullptr, nullptr, YSDG, eYS, digits));
         // X^T H X and X^T S X are symmetric; the rounding of a full product is not, and an
         // antisymmetric error would enter E_ij + E_ji (the re-orthonormalisation) divided
         // by lambda_j - lambda_i. Form the lower triangles (half the work) and mirror them.
@@ -579,13 +579,11 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     int iters = 0;
     double emax = 1.0;
     for (int it = 0; it < h->refine_max_iter; ++it) {
-        // digit planes of this iteration's products: 4 and 5 in the first two iterations
-        // (binary32 start, errors of about 1e-3), 7 from the third on. The corrections of
-        // the states next to the wanted/unwanted boundary are divided by their gap, which
-        // can be far below the cluster threshold: with 5 digits in the third iteration
-        // max|E| stalls near 6e-4 on the 3D-cluster problem at n = 16384 (the binary64
-        // fallback follows), with 7 it reaches 9e-6 and then 1.4e-9.
-        const int digits = it == 0 ? 4 : (it == 1 ? 5 : kOzDigits);
+        // digit planes of this iteration's products: 4 (35 bits) in the first two iterations
+        // (binary32 start, errors of about 1e-3), all 6 (53 bits) from the third on. The
+        // corrections of close states are divided by their gap; with 35 bits in the third
+        // iteration max|E| stalls near 6e-4 on the 3D-cluster problem at n = 16384.
+        const int digits = it < 2 ? 4 : kOzDigits;
         int rc = products_and_rr(digits);
         if (rc) return rc;
         // M = Xu^T R_o in binary32

@@ -550,9 +550,7 @@ cudaError_t apply_q1(cudaStream_t st, int n, int b, int k, const T *v1, const T 
     cudaError_t e;
     int npan = 0;
     for (int c0 = 0; c0 + b <= n - 2; c0 += b) ++npan;
-    // groups of kQ1Group panels on the tensor-core binary32 path; one panel at a time with
-    // the SIMT binary64 GEMM (its split-K products lose parallelism with wide blocks)
-    const int group = sizeof(T) == 4 ? kQ1Group : 1;
+    const int group = kQ1Group;
     const int gw_max = group * b;
     T *Tg = work;                                  // gw_max x gw_max (ld gw_max)
     T *M1 = Tg + (size_t)gw_max * gw_max;          // gw_max x b

@@ -25,6 +25,36 @@ void free_workspace(elsi_gb_handle_s *h)
     h->wk = Workspace();
 }
 
+// Scratch of the binary64-accurate digit products of a solve of order n with k vectors in the
+// binary64 route: the planes of an n x n and an n x max(k, 256) operand (A22 V, the updates of
+// the triangular solves, P and W need no more) and the partial products of a divided K.
+static size_t digit_scratch_elems(int n, int k)
+{
+    const size_t part = (size_t)152 * 128 * 128, small = (size_t)16 * n * n;
+    return ozaki_split_elems(n, n, kOzWide) + ozaki_split_elems(n, k > 256 ? k : 256, kOzWide) + 4 * (part < small ? part : small) + 64;
+}
+
+bool ensure_digit_scratch(elsi_gb_handle_s *h, int n, int k)
+{
+    Workspace &w = h->wk;
+    return ensure_buf((void **)&w.oz, &w.oz_cap, sizeof(__nv_bfloat16) * digit_scratch_elems(n, k)) &&
+           ensure_buf((void **)&w.ozexp, &w.ozexp_cap, sizeof(int) * (4 * (size_t)n + 1024)) &&
+           ensure_buf((void **)&w.status, &w.status_cap, sizeof(int) * ST_WORDS);
+}
+
+DigitScratch::DigitScratch(elsi_gb_handle_s *h)
+{
+    Workspace &w = h->wk;
+    set_tc_scratch(nullptr, 0, w.status);
+    set_f64_tc_scratch(w.oz, w.oz_cap / sizeof(__nv_bfloat16), w.ozexp, w.ozexp_cap / sizeof(int));
+}
+
+DigitScratch::~DigitScratch()
+{
+    set_f64_tc_scratch(nullptr, 0, nullptr, 0);
+    set_tc_scratch(nullptr, 0, nullptr);
+}
+
 #define ENSURE(name, type, count)                                                          \
     if (!ensure_buf((void **)&w.name, &w.name##_cap, sizeof(type) * (size_t)(count)))     \
         return set_error(h, ELSI_ERR_NOMEM, "cannot allocate %s (%zu bytes)", #name,       \
@@ -71,6 +101,7 @@ int ensure_workspace(elsi_gb_handle_s *h, int kz)
         ENSURE(stein, double, n * kTriBlock + 64);  // binary64 diagonal-block inverses
     } else {
         ENSURE(stein, double, 3 * n * kz + kz + 64);
+        if (!ensure_digit_scratch(h, h->n, kz)) return set_error(h, ELSI_ERR_NOMEM, "cannot allocate the digit planes");
     }
     ENSURE(sync, unsigned, sync_words(h->n, (int)eb));
     ENSURE(status, int, ST_WORDS);
@@ -127,6 +158,7 @@ static int solve_fp64(elsi_gb_handle_s *h, const SolveRequest &rq)
     const bool unit = h->overlap_is_unit;
     const int sms = num_sms();
     const bool ev_mode = rq.evec != nullptr;
+    const DigitScratch digits(h);  // large products run as digit products on the tensor cores
 
     CK(cudaEventRecord(w.ev[STAGE_CHOL], st));
     // ---- Eq. 8: S = L L^T (skipped when the factor of the previous call is reused)

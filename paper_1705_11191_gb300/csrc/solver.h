@@ -126,6 +126,17 @@ int set_error(elsi_gb_handle_s *h, int code, const char *fmt, ...);
 bool ensure_buf(void **p, size_t *cap, size_t bytes);
 int run_solve(elsi_gb_handle_s *h, const SolveRequest &rq);
 int ensure_workspace(elsi_gb_handle_s *h, int kz);
+// The handle's digit planes, exponents and status word for products of orders up to n x n by
+// n x max(k, 256); false if they cannot be allocated.
+bool ensure_digit_scratch(elsi_gb_handle_s *h, int n, int k);
+// While it lives, this thread's large binary64 gemm() calls run as digit products on the
+// tensor cores with the handle's scratch (all on the handle's stream).
+struct DigitScratch {
+    explicit DigitScratch(elsi_gb_handle_s *h);
+    ~DigitScratch();
+    DigitScratch(const DigitScratch &) = delete;
+    DigitScratch &operator=(const DigitScratch &) = delete;
+};
 int sing_prepare(elsi_gb_handle_s *h, const double *ovlp, bool *active);
 int solve_singular(elsi_gb_handle_s *h, const SolveRequest &rq);
 void free_sing(elsi_gb_handle_s *h);

@@ -231,7 +231,8 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
                 }
             }
         }
-        if (!xdone && (e = gemm<T>(st, 0, 0, m, bw, m, T(1), A22, lda, V, n, T(0), W, m)) != cudaSuccess)
+        // (A22 is symmetric: transposed, its rows are contiguous for the digit split)
+        if (!xdone && (e = gemm<T>(st, 1, 0, m, bw, m, T(1), A22, lda, V, n, T(0), W, m)) != cudaSuccess)
             return e;
         if (ceil_div(m, kWRows) + 1 <= kSyncBlocks) {
             // X = (A22 V) T, W = X - 1/2 V (T^T (V^T X))
@@ -264,6 +265,13 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
                     if (e != cudaSuccess) return e;
                     done = true;
                 }
+            }
+        }
+        if constexpr (sizeof(T) == 8) {
+            e = gemm_f64_two_sided(st, m, bw, V, n, W, m, A22, lda);
+            if (e != cudaErrorNotSupported) {
+                if (e != cudaSuccess) return e;
+                done = true;
             }
         }
         if (!done) {

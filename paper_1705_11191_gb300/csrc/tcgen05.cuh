@@ -52,6 +52,16 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity)
     return false;
 }
 
+// The same without the back-off, for the waits of a pipeline's own warps (the sleep costs more
+// than the wait there). The instruction suspends the thread by itself for a while, so the
+// limit is again a fraction of a second or more.
+__device__ __forceinline__ bool mbar_wait_hot(unsigned bar, unsigned parity)
+{
+    for (long long i = 0; i < (kWaitLimit << 2); ++i)
+        if (mbar_try(bar, parity)) return true;
+    return false;
+}
+
 __device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap *map, unsigned bar,
                                             int x, int y)
 {
@@ -100,6 +110,22 @@ __device__ __forceinline__ void tmem_ld32(unsigned taddr, float *v)
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+// 16 consecutive accumulator columns of this thread's lane (row).
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, float *v)
+{
+    unsigned r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+        "%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+          "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 // 32 consecutive tensor-memory columns of this thread's lane as raw 32-bit words (waits).
