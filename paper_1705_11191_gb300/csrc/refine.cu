@@ -119,24 +119,42 @@ __global__ void build_e_kernel(int n, int k, int kc, const double *goo, const do
 constexpr int kMaxCluster = 32;
 
 // Clusters: maximal runs of consecutive indices whose Rayleigh quotients
-// lam = G_jj / S_jj differ by less than delta, cut after kMaxCluster entries. One thread
-// scans the k values: cid[i] = first index of i's cluster, csize[first] = its size.
-__global__ void cluster_scan_kernel(int k, const double *goo, const double *soo, double delta,
-                                    int *cid, int *csize)
+// lam = G_jj / S_jj differ by less than delta, cut after every kMaxCluster entries:
+// cid[i] = first index of i's cluster, csize[first] = its size. One CTA of 1024 threads, each
+// with a contiguous segment: the run starts inside the segments, then carried from left to
+// right (one thread walking all k quotients, a division and two dependent loads each, took
+// 0.72 us an index: 0.77 ms at k = 1024, five times a solve).
+__global__ void __launch_bounds__(1024) cluster_scan_kernel(int k, const double *goo, const double *soo,
+                                                            double delta, int *cid, int *csize)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int start = 0;
-    double prev = goo[0] / soo[0];
-    for (int i = 1; i <= k; ++i) {
-        double cur = (i < k) ? goo[(size_t)i * k + i] / soo[(size_t)i * k + i] : 0.0;
-        bool cut = (i == k) || !(fabs(cur - prev) < delta) || (i - start >= kMaxCluster);
-        if (cut) {
-            for (int q = start; q < i; ++q) cid[q] = start;
-            csize[start] = i - start;
-            start = i;
-        }
+    __shared__ int last[1024];
+    const int t = threadIdx.x, nt = blockDim.x;
+    const int seg = (k + nt - 1) / nt, a = min(k, t * seg), b = min(k, a + seg);
+    auto quot = [&](int i) { return goo[(size_t)i * k + i] / soo[(size_t)i * k + i]; };
+    int run = -1;  // start of the current run (-1: it began left of the segment)
+    double prev = (a > 0 && a < b) ? quot(a - 1) : 0.0;
+    for (int i = a; i < b; ++i) {
+        const double cur = quot(i);
+        if (i == 0 || !(fabs(cur - prev) < delta)) run = i;
+        cid[i] = run;
         prev = cur;
     }
+    last[t] = run;
+    __syncthreads();
+    for (int o = 1; o < nt; o <<= 1) {  // largest run start of the segments up to t
+        const int v = t >= o ? last[t - o] : -1;
+        __syncthreads();
+        last[t] = max(last[t], v);
+        __syncthreads();
+    }
+    const int left = t > 0 ? last[t - 1] : 0;
+    for (int i = a; i < b; ++i) {
+        const int r = cid[i] < 0 ? left : cid[i];
+        cid[i] = r + (i - r) / kMaxCluster * kMaxCluster;
+    }
+    __syncthreads();
+    for (int i = a; i < b; ++i)  // the last index of each cluster
+        if (i == k - 1 || cid[i + 1] != cid[i]) csize[cid[i]] = i - cid[i] + 1;
 }
 
 // The small Rayleigh-Ritz problem of every cluster C of size c >= 2 (one CTA per index,
@@ -562,7 +580,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
         CKR(ozaki_gemm(st, k, k, n, 1.0, XDG, eX, YSDG, eYS, 0.0, SOO, k, 1, digits));
         CKR(mirror_lower<double>(st, k, GOO, k));
         CKR(mirror_lower<double>(st, k, SOO, k));
-        cluster_scan_kernel<<<1, 1, 0, st>>>(k, GOO, SOO, delta, CID, CSZ);
+        cluster_scan_kernel<<<1, 1024, 0, st>>>(k, GOO, SOO, delta, CID, CSZ);
         cluster_rr_kernel<<<k, 32, 0, st>>>(k, GOO, SOO, CID, CSZ, QBUF);
         rotate_cols_kernel<<<dim3(k, ceil_div(n, 256)), 256, 0, st>>>(n, k, CID, CSZ, QBUF, XO, YH, YS);
         rotate_gram_kernel<<<dim3(k, 1), 256, 0, st>>>(k, CID, CSZ, QBUF, GOO, SOO, 0);
