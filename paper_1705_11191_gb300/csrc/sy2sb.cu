@@ -13,58 +13,64 @@
 namespace egb {
 
 // ---- W of the two-sided update, fused (three small launches instead of five GEMMs):
-//   X = (A22 V) T,  Y = V^T X,  Z = T^T Y,  W = X - (1/2) V Z.
-// Row blocks of kWRows rows; tiles of 64 x 64 (bw <= 64, zero padded) in shared memory,
-// each of the 256 threads computing a 4 x 4 block of a tile product.
-constexpr int kWRows = 64;
+//   X = (A22 V) T,  Y = V^T X,  W = X - (1/2) V (T^T Y).
+// Row blocks of WRows<T> rows; tiles of 64 columns (bw <= 64, zero padded) in shared memory,
+// each of the 256 threads computing R x 4 or 4 x 4 elements of a tile product. Binary64 has
+// two FMAs a clock and SM, so its blocks are 16 rows: four times the CTAs of 64-row blocks
+// (two launches of 135 us at any order), and V (T^T Y) is formed as (V T^T) Y, whose work
+// shrinks with the rows, where T^T Y costs every block 64^3 FMAs: 27 and 20 us at n = 1531,
+// b = 32.
+template <typename T> constexpr int WRows = sizeof(T) == 4 ? 64 : 16;
 constexpr int kWLd = 65;
 
-// c[4][4] = sum_k A[r0 + i][k] B[k][c0 + j] for tiles A (64 x kWLd), B (64 x kWLd)
-template <typename T>
-__device__ __forceinline__ void tile_mm(const T *A, const T *B, int kmax, T (&c)[4][4])
+// c[R][4] = sum_{k < kmax} A[R ty + i][k] B[k][4 tx + j] for tiles A, B with leading dimension
+// kWLd, ty = tid / 16, tx = tid % 16
+template <typename T, int R>
+__device__ __forceinline__ void tile_mm(const T *A, const T *B, int kmax, T (&c)[R][4])
 {
-    const int tr = (threadIdx.x >> 4) * 4, tc = (threadIdx.x & 15) * 4;
+    const int tr = (threadIdx.x >> 4) * R, tc = (threadIdx.x & 15) * 4;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) c[i][j] = T(0);
     for (int k = 0; k < kmax; ++k) {
-        T a[4], b[4];
+        T a[R], b[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = A[(tr + i) * kWLd + k];
+        for (int i = 0; i < R; ++i) a[i] = A[(tr + i) * kWLd + k];
 #pragma unroll
         for (int j = 0; j < 4; ++j) b[j] = B[k * kWLd + tc + j];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < R; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) c[i][j] = fma(a[i], b[j], c[i][j]);
     }
 }
 
-// A 64 x 64 tile from global memory, element (i, c) = ld(i, c) stored by st(i, c, value):
-// 16 elements per thread (256 threads), all loads in flight before the first store.
-template <typename T, typename Ld, typename St>
+// A ROWS x 64 tile from global memory, element (i, c) = ld(i, c) stored by st(i, c, value); all
+// loads of a thread (256 threads) in flight before the first store.
+template <typename T, int ROWS, typename Ld, typename St>
 __device__ __forceinline__ void tile_in(Ld ld, St st)
 {
-    T v[16];
+    constexpr int U = ROWS * 64 / 256;
+    T v[U];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
+    for (int u = 0; u < U; ++u) {
         const int e = threadIdx.x + 256 * u;
-        v[u] = ld(e & 63, e >> 6);
+        v[u] = ld(e % ROWS, e / ROWS);
     }
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
+    for (int u = 0; u < U; ++u) {
         const int e = threadIdx.x + 256 * u;
-        st(e & 63, e >> 6, v[u]);
+        st(e % ROWS, e / ROWS, v[u]);
     }
 }
 
 // tile[i][c] = src[(r0 + i) + c * ld] for i < rows, c < bw; zero elsewhere
-template <typename T>
+template <typename T, int ROWS>
 __device__ __forceinline__ void load_rows(T *tile, const T *src, int ld, int r0, int rows, int bw)
 {
-    tile_in<T>([&](int i, int c) { return (i < rows && c < bw) ? src[(size_t)(r0 + i) + (size_t)c * ld] : T(0); },
-               [&](int i, int c, T x) { tile[i * kWLd + c] = x; });
+    tile_in<T, ROWS>([&](int i, int c) { return (i < rows && c < bw) ? src[(size_t)(r0 + i) + (size_t)c * ld] : T(0); },
+                     [&](int i, int c, T x) { tile[i * kWLd + c] = x; });
 }
 
 // X rows = Xa rows T; partial Y (64 x 64 per block, column-major) = V rows^T X rows
@@ -72,17 +78,18 @@ template <typename T>
 __global__ void __launch_bounds__(256) w_stage1_kernel(int m, int bw, const T *xa, const T *V, int ldv,
                                                        const T *Tm, int ldt, T *X, T *ypart)
 {
+    constexpr int ROWS = WRows<T>, R = ROWS / 16;
     extern __shared__ unsigned char wsm_raw[];
     T *sT = reinterpret_cast<T *>(wsm_raw), *sA = sT + 64 * kWLd, *sX = sA + 64 * kWLd;
-    const int r0 = blockIdx.x * kWRows, rows = min(kWRows, m - r0);
-    load_rows(sT, Tm, ldt, 0, bw, bw);
-    load_rows(sA, xa, m, r0, rows, bw);
+    const int r0 = blockIdx.x * ROWS, rows = min(ROWS, m - r0);
+    load_rows<T, 64>(sT, Tm, ldt, 0, bw, bw);
+    load_rows<T, ROWS>(sA, xa, m, r0, rows, bw);
     __syncthreads();
-    T c[4][4];
-    tile_mm(sA, sT, bw, c);
-    const int tr = (threadIdx.x >> 4) * 4, tc = (threadIdx.x & 15) * 4;
+    T c[R][4];
+    tile_mm<T, R>(sA, sT, bw, c);
+    const int tr = (threadIdx.x >> 4) * R, tc = (threadIdx.x & 15) * 4;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             sX[(tr + i) * kWLd + tc + j] = c[i][j];
@@ -90,62 +97,68 @@ __global__ void __launch_bounds__(256) w_stage1_kernel(int m, int bw, const T *x
         }
     __syncthreads();
     // V rows transposed into sA: sA[a][i] = V[r0 + i][a]
-    tile_in<T>([&](int i, int a) { return (i < rows && a < bw) ? V[(size_t)(r0 + i) + (size_t)a * ldv] : T(0); },
-               [&](int i, int a, T x) { sA[a * kWLd + i] = x; });
+    tile_in<T, ROWS>([&](int i, int a) { return (i < rows && a < bw) ? V[(size_t)(r0 + i) + (size_t)a * ldv] : T(0); },
+                     [&](int i, int a, T x) { sA[a * kWLd + i] = x; });
     __syncthreads();
-    tile_mm(sA, sX, kWRows, c);
+    T y[4][4];
+    tile_mm<T, 4>(sA, sX, ROWS, y);
+    const int ta = (threadIdx.x >> 4) * 4;
     T *yp = ypart + (size_t)blockIdx.x * 64 * 64;
+    if (ta < bw && tc < bw)
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) yp[(tr + i) + (tc + j) * 64] = c[i][j];
+            for (int j = 0; j < 4; ++j) yp[(ta + i) + (tc + j) * 64] = y[i][j];
 }
 
 // Y[e] = sum over blocks g of ypart[g][e] (e < 64 * 64, ascending g)
 template <typename T>
-__global__ void w_stage2_kernel(int nblk, const T *ypart, T *Y)
+__global__ void w_stage2_kernel(int nblk, int bw, const T *ypart, T *Y)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= 64 * 64) return;
     T s = T(0);
-    int g = 0;
-    for (; g + 8 <= nblk; g += 8) {
-        T v[8];
+    if ((e & 63) < bw && (e >> 6) < bw) {
+        int g = 0;
+        for (; g + 8 <= nblk; g += 8) {
+            T v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = ypart[(size_t)(g + u) * 64 * 64 + e];
+            for (int u = 0; u < 8; ++u) v[u] = ypart[(size_t)(g + u) * 64 * 64 + e];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) s += v[u];
+            for (int u = 0; u < 8; ++u) s += v[u];
+        }
+        for (; g < nblk; ++g) s += ypart[(size_t)g * 64 * 64 + e];
     }
-    for (; g < nblk; ++g) s += ypart[(size_t)g * 64 * 64 + e];
     Y[e] = s;
 }
 
-// Z = T^T Y (every block, in shared memory); W rows = X rows - (1/2) V rows Z
+// W rows = X rows - (1/2) (V rows T^T) Y
 template <typename T>
 __global__ void __launch_bounds__(256) w_stage3_kernel(int m, int bw, const T *X, const T *V, int ldv,
                                                        const T *Tm, int ldt, const T *Y, T *W)
 {
+    constexpr int ROWS = WRows<T>, R = ROWS / 16;
     extern __shared__ unsigned char wsm_raw[];
     T *sA = reinterpret_cast<T *>(wsm_raw), *sB = sA + 64 * kWLd, *sZ = sB + 64 * kWLd;
-    const int r0 = blockIdx.x * kWRows, rows = min(kWRows, m - r0);
-    // sA = T^T (sA[a][k] = T[k][a]), sB = Y
-    tile_in<T>([&](int i, int c) { return (i < bw && c < bw) ? Tm[(size_t)i + (size_t)c * ldt] : T(0); },
-               [&](int i, int c, T x) { sA[c * kWLd + i] = x; });
-    tile_in<T>([&](int i, int c) { return Y[i + c * 64]; }, [&](int i, int c, T x) { sB[i * kWLd + c] = x; });
+    const int r0 = blockIdx.x * ROWS, rows = min(ROWS, m - r0);
+    // sA = T^T (sA[a][k] = T[k][a]), sB = Y, sZ = V rows
+    tile_in<T, 64>([&](int i, int c) { return (i < bw && c < bw) ? Tm[(size_t)i + (size_t)c * ldt] : T(0); },
+                   [&](int i, int c, T x) { sA[c * kWLd + i] = x; });
+    tile_in<T, 64>([&](int i, int c) { return Y[i + c * 64]; }, [&](int i, int c, T x) { sB[i * kWLd + c] = x; });
+    load_rows<T, ROWS>(sZ, V, ldv, r0, rows, bw);
     __syncthreads();
-    T c[4][4];
-    tile_mm(sA, sB, bw, c);
-    const int tr = (threadIdx.x >> 4) * 4, tc = (threadIdx.x & 15) * 4;
+    T c[R][4];
+    tile_mm<T, R>(sZ, sA, bw, c);
+    const int tr = (threadIdx.x >> 4) * R, tc = (threadIdx.x & 15) * 4;
+    __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) sZ[(tr + i) * kWLd + tc + j] = c[i][j];
     __syncthreads();
-    load_rows(sA, V, ldv, r0, rows, bw);
-    __syncthreads();
-    tile_mm(sA, sZ, bw, c);
+    tile_mm<T, R>(sZ, sB, bw, c);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             if (tr + i < rows && tc + j < bw) {
@@ -158,7 +171,7 @@ template <typename T>
 static cudaError_t form_w(cudaStream_t st, int m, int bw, const T *xa, const T *V, int ldv,
                           const T *Tm, int ldt, T *X, T *Y, T *W, T *ypart)
 {
-    const int nblk = ceil_div(m, kWRows);
+    const int nblk = ceil_div(m, WRows<T>);
     const size_t smem = (size_t)3 * 64 * kWLd * sizeof(T);
     static PerDeviceOnce attr;  // per instantiation
     cudaError_t e = once_per_device(attr, [&] {
@@ -171,7 +184,7 @@ static cudaError_t form_w(cudaStream_t st, int m, int bw, const T *xa, const T *
     EGB_COUNT_LAUNCH();
     w_stage1_kernel<T><<<nblk, 256, smem, st>>>(m, bw, xa, V, ldv, Tm, ldt, X, ypart);
     EGB_COUNT_LAUNCH();
-    w_stage2_kernel<T><<<16, 256, 0, st>>>(nblk, ypart, Y);
+    w_stage2_kernel<T><<<64, 64, 0, st>>>(nblk, bw, ypart, Y);
     EGB_COUNT_LAUNCH();
     w_stage3_kernel<T><<<nblk, 256, smem, st>>>(m, bw, X, V, ldv, Tm, ldt, Y, W);
     return cudaGetLastError();
@@ -234,9 +247,9 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
         // (A22 is symmetric: transposed, its rows are contiguous for the digit split)
         if (!xdone && (e = gemm<T>(st, 1, 0, m, bw, m, T(1), A22, lda, V, n, T(0), W, m)) != cudaSuccess)
             return e;
-        if (ceil_div(m, kWRows) + 1 <= kSyncBlocks) {
+        if (ceil_div(m, WRows<T>) + 1 <= kSyncBlocks) {
             // X = (A22 V) T, W = X - 1/2 V (T^T (V^T X))
-            T *ysum = ypart + (size_t)ceil_div(m, kWRows) * 64 * 64;
+            T *ysum = ypart + (size_t)ceil_div(m, WRows<T>) * 64 * 64;
             if ((e = form_w<T>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart)) != cudaSuccess) return e;
         } else {
             // X = (A22 V) T
