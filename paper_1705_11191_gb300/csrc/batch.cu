@@ -129,7 +129,7 @@ static int default_workers(size_t N) { return N <= 4096 ? 4 : (N <= 8192 ? 2 : 1
 static double instance_bytes(size_t N, int prec)
 {
     const double n2 = (double)N * (double)N;
-    return (prec == ELSI_PREC_FP32_REFINE ? 150.0 : 80.0) * n2 + 64.0 * 1048576.0;
+    return (prec == ELSI_PREC_FP32_REFINE ? 150.0 : 120.0) * n2 + 64.0 * 1048576.0;
 }
 
 static BatchState *batch_state(elsi_gb_handle_s *h)
@@ -254,6 +254,7 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
         s->mu_max_steps = h->mu_max_steps;
         s->precision = h->precision;
         s->band_width = tv.band;
+        s->band_set = true;
         s->elpa_solver = tv.solver;
         s->refine_max_iter = h->refine_max_iter;
         s->stream = wst;
@@ -422,7 +423,7 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
         TuneVal v;
         const bool known = tune_get(dev, prec, cplx, size_bucket(N), &v);
         if (!known) {
-            v.band = h->band_width;
+            v.band = band_of(h, prec);
             v.solver = h->elpa_solver;
             v.workers = h->batch_workers > 0 ? h->batch_workers : default_workers(N);
             if (h->batch_autotune) {

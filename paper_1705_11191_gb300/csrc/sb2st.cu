@@ -1,7 +1,7 @@
 // Band -> tridiagonal reduction T = Q2^T B Q2 by bulge chasing (arXiv:1705.11191 Eq. 11,
 // second line; step (2) of the two-stage tridiagonalisation, sec. 3.1, after Bischof,
 // Lang & Sun's successive band reduction), and the back-transformation of eigenvectors
-// through Q2 (step (4)).
+// through Q1 (step (5)).
 //
 // Sweep j (0 <= j <= n-3) annihilates column j below the subdiagonal and chases the
 // resulting bulge down the band in steps t = 0, 1, ...; step t owns the index window
@@ -12,8 +12,8 @@
 // until that sweep has finished step t+1. No grid-wide barrier is involved.
 //
 // Each step stores its Householder reflector (b entries, v[0] = 1) and tau in slot
-// j * S + t (S = steps of sweep 0); the back-transformation applies them in the
-// reverse of a valid application order.
+// j * S + t (S = steps of sweep 0); the back-transformation (q2tc.cu, q2f64.cu) applies them
+// in the reverse of a valid application order.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -364,177 +364,6 @@ template cudaError_t sb2st<double>(cudaStream_t, int, int, double *, int, double
                                    double *, double *, int *, unsigned *, int);
 template cudaError_t sb2st<float>(cudaStream_t, int, int, float *, int, double *, double *,
                                   float *, float *, int *, unsigned *, int);
-
-// ------------------------------------------------------------------ Q2 back-transform
-// Z <- Q2 Z. Q2 = prod over sweep blocks J (ascending) of prod over steps t (descending)
-// of W(J,t) = H(J,t) H(J+1,t) ... H(J+m-1,t); so Z is updated for J descending, t
-// ascending and, inside W(J,t), sweeps descending. Every lane owns one column of Z and
-// keeps the rows of the current window in a shared-memory ring (row-major across the
-// CTA's columns, so a warp's accesses are conflict-free); the dot product v^T z of each
-// reflector is lane-local. The reflectors of one (J, t) are staged once per CTA.
-constexpr int kQ2Sweeps = 64;   // m: sweeps per block
-constexpr int kQ2Ring = 256;    // ring rows (>= m + 2b - 1 for b <= 64), power of two
-constexpr int kQ2Lanes = 8;     // lanes per column
-constexpr int kQ2RingLd = kQ2Ring + 8;  // column stride of the ring: the 4 columns of a warp
-                                        // start 8 banks apart
-// columns per CTA: binary32 32 (256 threads); binary64 8 (64 threads), so that the
-// n_state columns of the binary64 route still spread over all SMs
-template <typename T> struct Q2Cols;
-template <> struct Q2Cols<float> { static constexpr int v = 32; };
-template <> struct Q2Cols<double> { static constexpr int v = 8; };
-
-__device__ __forceinline__ void cp_async_bytes(void *dst, const void *src, int bytes)
-{
-    unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    if (bytes == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src));
-    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src));
-}
-__device__ __forceinline__ void q2_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-__device__ __forceinline__ void q2_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::); }
-
-template <typename T>
-__global__ void __launch_bounds__(256)
-apply_q2_kernel(int n, int b, int S, const T *__restrict__ v2, const T *__restrict__ tau2, int k,
-                T *z, int ldz)
-{
-    constexpr int kQ2Cols = Q2Cols<T>::v;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *ring = reinterpret_cast<T *>(smem_raw);          // kQ2Cols x kQ2RingLd, [col][slot]
-    T *vsb = ring + kQ2Cols * kQ2RingLd;                // 2 x (m x b) staged reflectors
-    T *tsb = vsb + 2 * kQ2Sweeps * b;                   // 2 x m taus
-    const int tid = threadIdx.x;
-    const int lc = tid / kQ2Lanes;                      // local column
-    const int sub = tid % kQ2Lanes;                     // row lane
-    const int c0 = blockIdx.x * kQ2Cols;
-    const int ncol = min(kQ2Cols, k - c0);
-    const bool col_ok = lc < ncol;
-    const int nsweep = n - 2;
-    const int nblk = (nsweep + kQ2Sweeps - 1) / kQ2Sweeps;
-    const unsigned gmask = 0xffu << ((tid & 31) & ~7);
-    T *myring = ring + lc * kQ2RingLd;
-
-    // asynchronous copy of rows [r0, r1) of the CTA's columns into the ring
-    auto fetch_rows = [&](int r0, int r1) {
-        const int nr = r1 - r0;
-        for (int e = tid; e < nr * ncol; e += blockDim.x) {
-            int r = r0 + e % nr, c = e / nr;
-            cp_async_bytes(ring + c * kQ2RingLd + (r & (kQ2Ring - 1)), z + (size_t)r + (size_t)(c0 + c) * ldz,
-                           (int)sizeof(T));
-        }
-    };
-    auto store_rows = [&](int r0, int r1) {
-        const int nr = r1 - r0;
-        for (int e = tid; e < nr * ncol; e += blockDim.x) {
-            int r = r0 + e % nr, c = e / nr;
-            z[(size_t)r + (size_t)(c0 + c) * ldz] = ring[c * kQ2RingLd + (r & (kQ2Ring - 1))];
-        }
-    };
-    // asynchronous staging of the reflectors of step t of sweeps [J, Jend) (zeros / tau 0
-    // for sweeps that have no step t)
-    auto fetch_refl = [&](int J, int Jend, int t, int buf) {
-        T *vs = vsb + buf * kQ2Sweeps * b;
-        T *ts = tsb + buf * kQ2Sweeps;
-        for (int e = tid; e < (Jend - J) * b; e += blockDim.x) {
-            int jj = e / b, i = e % b;
-            int j = J + jj;
-            int Sj = (n - 2 - j) / b + 1;
-            if (t < Sj) cp_async_bytes(vs + jj * b + i, v2 + ((size_t)j * S + t) * b + i, (int)sizeof(T));
-            else vs[jj * b + i] = T(0);
-        }
-        for (int jj = tid; jj < Jend - J; jj += blockDim.x) {
-            int j = J + jj;
-            int Sj = (n - 2 - j) / b + 1;
-            if (t < Sj) cp_async_bytes(ts + jj, tau2 + (size_t)j * S + t, (int)sizeof(T));
-            else ts[jj] = T(0);
-        }
-    };
-
-    for (int jb = nblk - 1; jb >= 0; --jb) {
-        const int J = jb * kQ2Sweeps;
-        const int Jend = min(nsweep, J + kQ2Sweeps);  // sweeps J .. Jend-1
-        const int SJ = (n - 2 - J) / b + 1;
-        int lo = J + 1;                                // window [lo, hi)
-        int hi = min(n, Jend + b);
-        __syncthreads();
-        fetch_rows(lo, hi);
-        fetch_refl(J, Jend, 0, 0);
-        q2_commit();
-        for (int t = 0; t < SJ; ++t) {
-            const int buf = t & 1;
-            q2_wait_all();
-            __syncthreads();
-            // prefetch what step t+1 needs: its reflectors and the b rows entering the window
-            const int nlo = min(lo + b, n), nhi = min(hi + b, n);
-            if (t + 1 < SJ) {
-                fetch_refl(J, Jend, t + 1, buf ^ 1);
-                fetch_rows(hi, nhi);
-            }
-            q2_commit();
-            const T *vs = vsb + buf * kQ2Sweeps * b;
-            const T *ts = tsb + buf * kQ2Sweeps;
-            for (int j = Jend - 1; j >= J; --j) {
-                const int jj = j - J;
-                const T tau = ts[jj];
-                if (tau == T(0)) continue;
-                const int r0 = j + 1 + t * b;
-                const int L = min(b, n - r0);
-                if (L <= 0) continue;
-                const T *v = vs + jj * b;
-                T sdot = T(0);
-#pragma unroll 8
-                for (int i = sub; i < L; i += kQ2Lanes)
-                    sdot = fma(v[i], myring[(r0 + i) & (kQ2Ring - 1)], sdot);
-                sdot += __shfl_xor_sync(gmask, sdot, 4);
-                sdot += __shfl_xor_sync(gmask, sdot, 2);
-                sdot += __shfl_xor_sync(gmask, sdot, 1);
-                const T sc = tau * sdot;
-#pragma unroll 8
-                for (int i = sub; i < L; i += kQ2Lanes) {
-                    T &zr = myring[(r0 + i) & (kQ2Ring - 1)];
-                    zr = fma(-sc, v[i], zr);
-                }
-                __syncwarp(gmask);
-            }
-            __syncthreads();
-            // rows [lo, nlo) are final for this block of sweeps
-            if (t + 1 < SJ) {
-                store_rows(lo, nlo);
-                lo = nlo;
-                hi = nhi;
-            } else {
-                store_rows(lo, hi);
-            }
-            (void)col_ok;
-        }
-    }
-    q2_wait_all();
-}
-
-template <typename T>
-cudaError_t apply_q2(cudaStream_t st, int n, int b, const T *v2, const T *tau2, int k, T *z,
-                     int ldz, int *status)
-{
-    (void)status;
-    if (n < 3 || k <= 0) return cudaSuccess;
-    if (b > 64 || kQ2Sweeps + 2 * b - 1 > kQ2Ring) return cudaErrorInvalidValue;
-    const int S = sb2st_steps(n, b);
-    constexpr int kQ2Cols = Q2Cols<T>::v;
-    size_t smem = ((size_t)kQ2Cols * kQ2RingLd + 2 * (size_t)kQ2Sweeps * b + 2 * kQ2Sweeps) * sizeof(T);
-    static PerDeviceOnce attr_set;  // per instantiation
-    cudaError_t e = once_per_device(attr_set, [] {
-        const size_t smax =
-            ((size_t)kQ2Cols * kQ2RingLd + 2 * (size_t)kQ2Sweeps * 64 + 2 * kQ2Sweeps) * sizeof(T);
-        return cudaFuncSetAttribute(apply_q2_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax);
-    });
-    if (e != cudaSuccess) return e;
-    EGB_COUNT_LAUNCH();
-    apply_q2_kernel<T><<<ceil_div(k, kQ2Cols), kQ2Cols * kQ2Lanes, smem, st>>>(n, b, S, v2, tau2, k, z, ldz);
-    return cudaGetLastError();
-}
-template cudaError_t apply_q2<double>(cudaStream_t, int, int, const double *, const double *, int,
-                                      double *, int, int *);
-template cudaError_t apply_q2<float>(cudaStream_t, int, int, const float *, const float *, int,
-                                     float *, int, int *);
 
 // ------------------------------------------------------------------ Q1 back-transform
 // Z <- Q1 Z, Q1 = Q_0 Q_1 ... Q_{P-1}, Q_p = I - V_p T_p V_p^T: panels descending.

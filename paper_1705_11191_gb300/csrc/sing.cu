@@ -127,6 +127,7 @@ int sing_prepare(elsi_gb_handle_s *h, const double *ovlp, bool *active)
     s->overlap_is_unit = true;
     s->precision = ELSI_PREC_FP64;
     s->band_width = h->band_width;
+    s->band_set = h->band_set;
     s->stream = st;
     SolveRequest q;
     q.ham = g.negs;
@@ -194,6 +195,7 @@ int solve_singular(elsi_gb_handle_s *h, const SolveRequest &rq)
     r->overlap_is_unit = true;
     r->precision = h->precision;
     r->band_width = h->band_width;
+    r->band_set = h->band_set;
     r->elpa_solver = h->elpa_solver;
     r->refine_max_iter = h->refine_max_iter;
     r->stream = st;

@@ -69,7 +69,7 @@ int ensure_workspace(elsi_gb_handle_s *h, int kz)
 {
     Workspace &w = h->wk;
     const size_t n = h->n;
-    const int b = h->band_width;
+    const int b = band_of(h, h->precision);
     const int S = sb2st_steps(h->n, b);
     const size_t nsweep = n >= 3 ? n - 2 : 1;
     const bool fp32 = h->precision == ELSI_PREC_FP32_REFINE;
@@ -154,7 +154,7 @@ static int solve_fp64(elsi_gb_handle_s *h, const SolveRequest &rq)
 {
     Workspace &w = h->wk;
     cudaStream_t st = h->stream;
-    const int n = h->n, k = h->n_state, b = h->band_width;
+    const int n = h->n, k = h->n_state, b = band_of(h, ELSI_PREC_FP64);
     const bool unit = h->overlap_is_unit;
     const int sms = num_sms();
     const bool ev_mode = rq.evec != nullptr;
@@ -205,7 +205,7 @@ static int solve_fp64(elsi_gb_handle_s *h, const SolveRequest &rq)
     CK(stein<double>(st, n, w.d, w.e, k, w.w, w.z, n, w.stein, w.status));
     CK(cudaEventRecord(w.ev[STAGE_Q2], st));
     // ---- step (4): Z <- Q2 Z
-    if (!one_stage) CK(apply_q2<double>(st, n, b, w.v2, w.tau2, k, w.z, n, w.status));
+    if (!one_stage) CK(apply_q2_f64(st, n, b, w.v2, w.tau2, k, w.z, n, w.status));
     CK(cudaEventRecord(w.ev[STAGE_Q1], st));
     // ---- step (5): Z <- Q1 Z (one-stage: Z <- Q Z)
     if (one_stage) CK(apply_q_onestage<double>(st, n, k, w.v1, w.t1, w.z, n, w.work));
