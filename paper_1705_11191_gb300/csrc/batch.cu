@@ -121,6 +121,12 @@ bool batch_tuning_lookup(elsi_gb_handle_s *h, int n, bool cplx, int *band, int *
     return true;
 }
 
+// What the calling thread's solves share the GPU with, for as long as this lives.
+struct ConcurrentSolves {
+    void set(int n) { set_concurrent_solves(n); }
+    ~ConcurrentSolves() { set_concurrent_solves(1); }
+};
+
 // Concurrency without tuning: 4 instances for real-form sizes up to 4096, 2 up to 8192.
 static int default_workers(size_t N) { return N <= 4096 ? 4 : (N <= 8192 ? 2 : 1); }
 
@@ -364,6 +370,8 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
                     instance(t, &s, &wst);
                     double *vals, *vecs;
                     scratch(t, &vals, &vecs);
+                    ConcurrentSolves share;
+                    share.set(W);
                     if (solve_one(s, wst, i, v, vals, vecs, rr[t])) {
                         const cudaError_t ce = cudaStreamSynchronize(wst);
                         if (ce != cudaSuccess && rr[t].rc == ELSI_OK) {
@@ -469,11 +477,13 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
         cudaStream_t wst;
         instance(t, &s, &wst);
         Result &r = res[t];
+        ConcurrentSolves share;
         for (;;) {
             const int q = next.fetch_add(1);
             if (q >= nprob) break;
             const int i = order[q];
             const BatchItem &it = b.items[i];
+            share.set(W < nprob - q ? W : nprob - q);
             if (!solve_one(s, wst, i, tv[i], b.vals + it.off_val, b.vecs + it.off_vec, r)) {
                 next.store(nprob);  // the other instances stop after their current problem
                 return;

@@ -148,11 +148,14 @@ cudaError_t extract_band(cudaStream_t st, int n, int b, const T *a, int lda, T *
 // Eigenvalues 0..count-1 (ascending) of the symmetric tridiagonal (d, e) by Sturm
 // bisection (w needs count + 8 entries: the Gershgorin bounds follow the values), then
 // eigenvectors of the first kvec of them into z (n x kvec, ldz) as type T.
-// scratch: 3*n*kvec + kvec + 16 doubles.
+// scratch of stein: 3*n*kvec + kvec + 16 doubles.
 // tol_rel: stop when the bracket is narrower than tol_rel * ||T|| (0: full binary64).
 // Off-diagonals of e below 2 eps ||T|| are set to zero first (T splits into blocks).
+// scratch of stebz: 2 n values. set_concurrent_solves: how many solves the calling thread's
+// solve shares the GPU with (itself included; 1 unless set), for the choice of its threads.
+void set_concurrent_solves(int solves);
 cudaError_t stebz(cudaStream_t st, int n, const double *d, double *e, int count,
-                  double *w, int *status, double tol_rel = 0.0);
+                  double *w, int *status, double *scratch, double tol_rel = 0.0);
 template <typename T>
 cudaError_t stein(cudaStream_t st, int n, const double *d, const double *e, int kvec,
                   const double *w, T *z, int ldz, double *scratch, int *status);

@@ -517,7 +517,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     // neither the eigenvalues nor, through the twisted factorisations, the eigenvectors
     // beyond that level. (At 1e-7 ||T|| the refinement of the 3D-cluster problem at
     // n = 16384 no longer converges and the solve falls back to the binary64 route.)
-    CKR(stebz(st, n, w.d, w.e, n, w.w, w.status, 1e-8));
+    CKR(stebz(st, n, w.d, w.e, n, w.w, w.status, reinterpret_cast<double *>(w.oz), 1e-8));
     // eigenvector scratch (3 n^2 + n binary64 values) in the digit-plane buffer, free here
     CKR(stein<float>(st, n, w.d, w.e, n, w.w, X32, n, reinterpret_cast<double *>(w.oz), w.status));
     CKR(cudaEventRecord(w.ev[STAGE_Q2], st));

@@ -201,7 +201,7 @@ static int solve_fp64(elsi_gb_handle_s *h, const SolveRequest &rq)
     CK(cudaEventRecord(w.ev[STAGE_TRIDIAG], st));
     // ---- step (3): eigenvalues (all n for ev, the n_state lowest for dm), k vectors
     const int nval = ev_mode ? n : k;
-    CK(stebz(st, n, w.d, w.e, nval, w.w, w.status));
+    CK(stebz(st, n, w.d, w.e, nval, w.w, w.status, w.stein));
     CK(stein<double>(st, n, w.d, w.e, k, w.w, w.z, n, w.stein, w.status));
     CK(cudaEventRecord(w.ev[STAGE_Q2], st));
     // ---- step (4): Z <- Q2 Z

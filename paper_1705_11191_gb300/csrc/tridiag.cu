@@ -30,35 +30,42 @@ __device__ __forceinline__ double guard_pivot(double q, double pivmin)
 
 // number of eigenvalues < sigma: the sign changes of the leading principal minors
 // p_i = det(T[0:i, 0:i] - sigma I), p_0 = 1, p_{i+1} = (d_i - sigma) p_i - e_{i-1}^2 p_{i-1}
-// (Sturm; Givens 1954). The ratio q_i = p_{i+1} / p_i is the pivot of the LDL^T
+// (Sturm; Givens 1954), e2 = e^2. The ratio q_i = p_{i+1} / p_i is the pivot of the LDL^T
 // factorisation of T - sigma I, and a pivot smaller than pivmin in magnitude is replaced
-// by -pivmin as in the pivot form. This form needs no division (binary64 division is a long
-// sequence of the few binary64 FMA units of this chip); the pair (p_i, p_{i-1}) is rescaled
-// by an exact power of two whenever |p_i| leaves [2^-600, 2^600] (checked every 8 steps;
-// one step changes |p| by at most a factor of about 2 ||T|| / pivmin, far below 2^50).
-__device__ int sturm_count(int n, const double *__restrict__ d, const double *__restrict__ e,
+// by -pivmin as in the pivot form. This form needs no division, and everything but the three
+// operations of the recurrence is done on the bit patterns: on this chip a warp holds its
+// scheduler's binary64 unit for 64 cycles with every addition, product or comparison. Signs
+// come from the sign bits; the test for a tiny pivot is made when the exponent of p_{i+1} is
+// below that of pivmin 2^460 >= pivmin |p_i| (it always is for a zero). The pair (p_i, p_{i-1})
+// is rescaled by an exact power of two when |p_i| leaves [2^-200, 2^200], every 8 steps, which
+// keeps |p| below 2^460 for ||T|| up to 2^31.
+// Measured against a form with a binary64 product and comparison for the pivot test, sign
+// comparisons and e^2 formed on the way (8 such operations a step, eigenvalues by 8 or 2 lanes
+// at every count), the bisection: n = 1531, 382 values 8.7 -> 4.1 ms; n = 4096, all 15.2 -> 7.1
+// ms; n = 16384, all 111 -> 65 ms; 8 solves of n = 2000 at a time 25 -> 10 ms each.
+__device__ int sturm_count(int n, const double *__restrict__ d, const double *__restrict__ e2,
                            double sigma, double pivmin)
 {
+    const int tiny = (__double2hiint(pivmin) & 0x7FF00000) + (461 << 20);
     double pm = 1.0;                                // p_{i-1}
     double p = guard_pivot(d[0] - sigma, pivmin);   // p_1 = q_0
-    int cnt = p < 0.0;
+    unsigned cnt = (unsigned)__double2hiint(p) >> 31;
     int i = 1;
     while (i < n) {
         const int iend = min(n, i + 8);
         for (; i < iend; ++i) {
-            const double ei = e[i - 1];
-            double pn = fma(d[i] - sigma, p, -(ei * ei) * pm);
+            double pn = fma(d[i] - sigma, p, -e2[i - 1] * pm);
             // pivot q = pn / p below pivmin in magnitude: q = -pivmin
-            if (fabs(pn) < pivmin * fabs(p)) pn = -pivmin * p;
-            cnt += (pn < 0.0) != (p < 0.0);
+            if ((__double2hiint(pn) & 0x7FF00000) <= tiny && fabs(pn) < pivmin * fabs(p)) pn = -pivmin * p;
+            cnt += (unsigned)(__double2hiint(pn) ^ __double2hiint(p)) >> 31;
             pm = p;
             p = pn;
         }
-        const double ap = fabs(p);
-        if (ap > 0x1p600) { p *= 0x1p-600; pm *= 0x1p-600; }
-        else if (ap < 0x1p-600) { p *= 0x1p600; pm *= 0x1p600; }
+        const int ex = __double2hiint(p) & 0x7FF00000;
+        if (ex > ((1023 + 200) << 20)) { p *= 0x1p-200; pm *= 0x1p-200; }
+        else if (ex < ((1023 - 200) << 20)) { p *= 0x1p200; pm *= 0x1p200; }
     }
-    return cnt;
+    return (int)cnt;
 }
 
 // [0]=gl, [1]=gu, [2]=pivmin, [3]=||T|| bound, [4]=1 if T splits into blocks, else 0
@@ -103,16 +110,16 @@ __global__ void gershgorin_kernel(int n, const double *d, const double *e, doubl
     if (threadIdx.x == 0) out[4] = split ? 1.0 : 0.0;
 }
 
-// number of eigenvalues < sigma, binary32 (used only to bracket)
-__device__ int sturm_count32(int n, const double *__restrict__ d, const double *__restrict__ e,
+// number of eigenvalues < sigma, binary32 (used only to bracket); d and e^2 rounded once for
+// all counts (a conversion is a binary64 operation too)
+__device__ int sturm_count32(int n, const float *__restrict__ d, const float *__restrict__ e2,
                              float sigma, float pivmin)
 {
-    float q = (float)d[0] - sigma;
+    float q = d[0] - sigma;
     if (fabsf(q) < pivmin) q = -pivmin;
     int cnt = q < 0.0f;
     for (int i = 1; i < n; ++i) {
-        float ei = (float)e[i - 1];
-        q = (float)d[i] - sigma - __fdividef(ei * ei, q);
+        q = d[i] - sigma - __fdividef(e2[i - 1], q);
         if (fabsf(q) < pivmin) q = -pivmin;
         cnt += q < 0.0f;
     }
@@ -128,7 +135,8 @@ __device__ int sturm_count32(int n, const double *__restrict__ d, const double *
 // with binary64 counts (falling back to the Gershgorin interval if the check fails). Phase 2: binary64 counts down to
 // max(tol_rel * ||T||, 2 eps max|lo|,|hi|).
 template <int LANES>
-__global__ void bisect_kernel(int n, const double *d, const double *e, int count,
+__global__ void bisect_kernel(int n, const double *__restrict__ d, const double *__restrict__ e2,
+                              const float *__restrict__ d32, const float *__restrict__ e232, int count,
                               const double *bounds, double *w, double tol_rel, int bracket32)
 {
     const int group = threadIdx.x / LANES, lane = threadIdx.x % LANES;
@@ -143,7 +151,7 @@ __global__ void bisect_kernel(int n, const double *d, const double *e, int count
         const float fpiv = fmaxf(1e-30f, (float)pivmin);
         for (int it = 0; it < 64 && (double)(fhi - flo) > 1e-6 * tn; ++it) {
             float sig = flo + (fhi - flo) * (float)(lane + 1) / (float)(LANES + 1);
-            int c = sturm_count32(n, d, e, sig, fpiv);
+            int c = sturm_count32(n, d32, e232, sig, fpiv);
             unsigned ok = __ballot_sync(gmask, c <= idx) & gmask;
             int pcount = __popc(ok);
             float nlo = __shfl_sync(gmask, sig, (threadIdx.x & 31) / LANES * LANES + max(pcount - 1, 0));
@@ -156,10 +164,10 @@ __global__ void bisect_kernel(int n, const double *d, const double *e, int count
         if (lo < gl) lo = gl;
         if (hi > gu) hi = gu;
         // verify the bracket in binary64: count(lo) <= idx < count(hi)
-        int c = sturm_count(n, d, e, lane == 0 ? lo : hi, pivmin);
+        int c = sturm_count(n, d, e2, lane == 0 ? lo : hi, pivmin);
         int clo = __shfl_sync(gmask, c, (threadIdx.x & 31) / LANES * LANES);
         int chi = (LANES > 1) ? __shfl_sync(gmask, c, (threadIdx.x & 31) / LANES * LANES + 1)
-                              : sturm_count(n, d, e, hi, pivmin);
+                              : sturm_count(n, d, e2, hi, pivmin);
         if (!(clo <= idx && idx < chi)) { lo = gl; hi = gu; }
     }
     if (active) {
@@ -170,7 +178,7 @@ __global__ void bisect_kernel(int n, const double *d, const double *e, int count
             double tol = fmax(tol_rel * scale, 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi))) + 4.0 * pivmin;
             if (hi - lo <= tol) break;
             double sig = lo + (hi - lo) * (double)(lane + 1) / (double)(LANES + 1);
-            int c = sturm_count(n, d, e, sig, pivmin);
+            int c = sturm_count(n, d, e2, sig, pivmin);
             unsigned ok = __ballot_sync(gmask, c <= idx) & gmask;
             int pcount = __popc(ok);
             double nlo = __shfl_sync(gmask, sig, (threadIdx.x & 31) / LANES * LANES + max(pcount - 1, 0));
@@ -186,33 +194,70 @@ __global__ void bisect_kernel(int n, const double *d, const double *e, int count
 // changes no eigenvalue by more than 2 eps ||T|| and lets exactly degenerate eigenvalues
 // (e.g. those of a complex Hermitian matrix written as a real one) be found in
 // different blocks.
-__global__ void split_kernel(int n, double *e, const double *bounds)
+// Also the forms of T that the counts read: e^2, and d and e^2 in binary32.
+__global__ void split_kernel(int n, const double *d, double *e, const double *bounds, double *e2, float *d32,
+                             float *e232)
 {
     const double tn = bounds[3];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n - 1; i += gridDim.x * blockDim.x)
-        if (fabs(e[i]) <= 2.0 * DBL_EPSILON * tn) e[i] = 0.0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        d32[i] = (float)d[i];
+        if (i < n - 1) {
+            double x = e[i];
+            if (fabs(x) <= 2.0 * DBL_EPSILON * tn) e[i] = x = 0.0;
+            e2[i] = x * x;
+            e232[i] = (float)x * (float)x;
+        }
+    }
 }
 
+static thread_local int t_concurrent_solves = 1;
+void set_concurrent_solves(int solves) { t_concurrent_solves = solves; }
+
 cudaError_t stebz(cudaStream_t st, int n, const double *d, double *e, int count,
-                  double *w, int *status, double tol_rel)
+                  double *w, int *status, double *scratch, double tol_rel)
 {
     (void)status;
     if (n <= 0 || count <= 0) return cudaSuccess;
     // the Gershgorin bounds live right after the count eigenvalues (w has count + 8)
     double *bounds = w + count;
+    double *e2 = scratch;
+    float *d32 = reinterpret_cast<float *>(scratch + n), *e232 = d32 + n;
     EGB_COUNT_LAUNCH();
     gershgorin_kernel<<<1, 1024, 0, st>>>(n, d, e, bounds);
     EGB_COUNT_LAUNCH();
-    split_kernel<<<ceil_div(n, 256), 256, 0, st>>>(n, e, bounds);
-    // enough threads to cover the latency: multisection when there are few eigenvalues
-    if (count <= 4096) {
-        EGB_COUNT_LAUNCH();
-        bisect_kernel<8><<<ceil_div(count, 16), 128, 0, st>>>(n, d, e, count, bounds, w, tol_rel, n > 512);
-    } else {
-        EGB_COUNT_LAUNCH();
-        bisect_kernel<2><<<ceil_div(count, 64), 128, 0, st>>>(n, d, e, count, bounds, w, tol_rel, 1);
+    split_kernel<<<ceil_div(n, 256), 256, 0, st>>>(n, d, e, bounds, e2, d32, e232);
+    // Lanes per eigenvalue. A count of L points gains log2(L + 1) bits, so one lane is the best
+    // use of a busy binary64 unit and many lanes the shortest chain on idle ones: the most lanes
+    // that keep a warp per scheduler (608, divided among the solves that run at the same time).
+    // n = 120: 32 lanes; n = 4096 with all eigenvalues: 4; n = 16384: 1.
+    const int budget = 608 * 32 / (t_concurrent_solves > 0 ? t_concurrent_solves : 1);
+    int lanes = 1;
+    while (lanes < 32 && (long long)count * lanes * 2 <= budget) lanes *= 2;
+    const int b32 = n > 512;
+    const int grid = ceil_div(count, 128 / lanes);
+    EGB_COUNT_LAUNCH();
+    switch (lanes) {
+    case 1: bisect_kernel<1><<<grid, 128, 0, st>>>(n, d, e2, d32, e232, count, bounds, w, tol_rel, b32); break;
+    case 2: bisect_kernel<2><<<grid, 128, 0, st>>>(n, d, e2, d32, e232, count, bounds, w, tol_rel, b32); break;
+    case 4: bisect_kernel<4><<<grid, 128, 0, st>>>(n, d, e2, d32, e232, count, bounds, w, tol_rel, b32); break;
+    case 8: bisect_kernel<8><<<grid, 128, 0, st>>>(n, d, e2, d32, e232, count, bounds, w, tol_rel, b32); break;
+    case 16: bisect_kernel<16><<<grid, 128, 0, st>>>(n, d, e2, d32, e232, count, bounds, w, tol_rel, b32); break;
+    default: bisect_kernel<32><<<grid, 128, 0, st>>>(n, d, e2, d32, e232, count, bounds, w, tol_rel, b32); break;
     }
     return cudaGetLastError();
+}
+
+// The count in the pivot form, from e (rare: only where T splits).
+__device__ int sturm_count_e(int n, const double *__restrict__ d, const double *__restrict__ e, double sigma,
+                             double pivmin)
+{
+    double q = guard_pivot(d[0] - sigma, pivmin);
+    int cnt = q < 0.0;
+    for (int i = 1; i < n; ++i) {
+        q = guard_pivot(d[i] - sigma - e[i - 1] * e[i - 1] / q, pivmin);
+        cnt += q < 0.0;
+    }
+    return cnt;
 }
 
 // Block of each eigenvalue: with [lo, hi] a small interval around w[l], the eigenvalues of
@@ -231,7 +276,7 @@ __global__ void block_assign_kernel(int n, const double *d, const double *e, int
     const double tn = bounds[3], pivmin = bounds[2];
     const double delta = 8.0 * DBL_EPSILON * fmax(fabs(w[l]), tn) + 4.0 * pivmin;
     const double lo = w[l] - delta, hi = w[l] + delta;
-    const int clo = sturm_count(n, d, e, lo, pivmin);
+    const int clo = sturm_count_e(n, d, e, lo, pivmin);
     int r = l - clo;  // rank among the eigenvalues in [lo, hi]
     if (r < 0) r = 0;
     double qlo = 1.0, qhi = 1.0;
@@ -265,6 +310,25 @@ __global__ void block_assign_kernel(int n, const double *d, const double *e, int
 // the backward one, the twist index r = argmin |gamma_i| with gamma_r (signed), and
 // ||z||^2 of the vector z with z_r = 1 that solves (T_b - lam I) z = gamma_r e_r.
 // Arrays are indexed [i * kvec + l].
+// 1 / x to about an ulp: the hardware's 20-bit approximation and two Newton steps (four FMAs);
+// a binary64 division is about three times as many operations of the scarce binary64 unit. The
+// approximation flushes subnormals, but pivots are at least pivmin >= DBL_MIN; a huge x, whose
+// reciprocal would be subnormal, takes the division.
+__device__ __forceinline__ double recip(double x)
+{
+    if ((__double2hiint(x) & 0x7FF00000) >= (2044 << 20)) return 1.0 / x;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(fma(-x, r, 1.0), r, r);
+    return fma(fma(-x, r, 1.0), r, r);
+}
+
+// |a| < |b| on the bit patterns
+__device__ __forceinline__ bool mag_less(double a, double b)
+{
+    return (__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFll) < (__double_as_longlong(b) & 0x7FFFFFFFFFFFFFFFll);
+}
+
 struct Twist {
     int r;
     double gamma, nrm2;
@@ -277,9 +341,10 @@ __device__ Twist twisted_factor(const double *__restrict__ d, const double *__re
     double dp = guard_pivot(d[bs] - lam, pivmin);
     dplus[(size_t)bs * kvec + l] = dp;
     for (int i = bs; i < be - 1; ++i) {
-        const double lp = e[i] / dp;
+        const double lp = e[i] * recip(dp);
         lplus[(size_t)i * kvec + l] = lp;
-        dp = guard_pivot(d[i + 1] - lam - lp * e[i], pivmin);
+        dp = d[i + 1] - lam - lp * e[i];
+        if (mag_less(dp, pivmin)) dp = -pivmin;
         dplus[(size_t)(i + 1) * kvec + l] = dp;
     }
     double dm = guard_pivot(d[be - 1] - lam, pivmin);
@@ -288,11 +353,12 @@ __device__ Twist twisted_factor(const double *__restrict__ d, const double *__re
     t.r = be - 1;
     double best = fabs(t.gamma);
     for (int i = be - 2; i >= bs; --i) {
-        const double um = e[i] / dm;
+        const double um = e[i] * recip(dm), dl = d[i] - lam;
         uminus[(size_t)i * kvec + l] = um;
-        dm = guard_pivot(d[i] - lam - um * e[i], pivmin);
-        const double g = dplus[(size_t)i * kvec + l] + dm - (d[i] - lam);
-        if (fabs(g) < best) { best = fabs(g); t.gamma = g; t.r = i; }
+        dm = dl - um * e[i];
+        if (mag_less(dm, pivmin)) dm = -pivmin;
+        const double g = dplus[(size_t)i * kvec + l] + dm - dl;
+        if (mag_less(g, best)) { best = fabs(g); t.gamma = g; t.r = i; }
     }
     double nrm2 = 1.0, zi = 1.0;
     for (int i = t.r - 1; i >= bs; --i) {
