@@ -152,56 +152,70 @@ __global__ void __launch_bounds__(256) ozaki_split_kernel(int V, int K, int Kpad
     }
 }
 
-// Vectors across memory (sv = 1): 32 vectors per CTA, read along the vectors' index (256 bytes
-// a warp) and transposed through shared memory. One CTA per vector would read one 8-byte
-// element per 32-byte sector.
+// Vectors across memory (sv = 1): 8 vectors per CTA, read along the vectors' index (64 bytes of
+// each line) and transposed through shared memory; one CTA per vector would read one 8-byte
+// element per 32-byte sector. Up to 256 elements of a vector are read once and kept in
+// registers; longer ones are read twice. (32 vectors per CTA read whole lines but left two
+// thirds of the SMs idle at n = 1531: 34 us at K = 256.)
 template <int ND>
 __global__ void __launch_bounds__(256) ozaki_split_t_kernel(int V, int K, int Kpad, const SplitSrc s, int nd,
                                                             __nv_bfloat16 *__restrict__ out, int ldo, size_t plane,
                                                             int *__restrict__ exps)
 {
-    __shared__ unsigned long long red[8][32];
-    __shared__ int es[32];
-    __shared__ double tile[32][65];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int v0 = blockIdx.x * 32, v = v0 + tx;
+    constexpr int R = 8, C = 256;  // vectors, elements of a tile
+    __shared__ unsigned long long red[8][R];
+    __shared__ double tile[R][C + 2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tx = tid & (R - 1), ty = tid / R;  // vector; elements ty, ty + 32, ..
+    const int v0 = blockIdx.x * R, v = v0 + tx;
     unsigned long long mb = 0ull;
-    if (v < V) {
-#pragma unroll 8
-        for (int q = ty; q < K; q += 8) {
-            const unsigned long long b = magnitude(s.at(v, q));
+    double x[C / 32];
+    for (int q0 = 0; q0 < K; q0 += C) {
+#pragma unroll
+        for (int u = 0; u < C / 32; ++u) {
+            const int q = q0 + ty + 32 * u;
+            x[u] = (v < V && q < K) ? s.at(v, q) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < C / 32; ++u) {
+            const unsigned long long b = magnitude(x[u]);
             mb = b > mb ? b : mb;
         }
     }
-    red[ty][tx] = mb;
-    __syncthreads();
-    if (ty == 0) {
 #pragma unroll
-        for (int w = 1; w < 8; ++w) mb = red[w][tx] > mb ? red[w][tx] : mb;
-        es[tx] = row_exponent(mb);
-        exps[v] = es[tx];
+    for (int o = 16; o >= R; o >>= 1) {
+        const unsigned long long t = __shfl_xor_sync(0xffffffffu, mb, o);
+        mb = t > mb ? t : mb;
     }
-    for (int q0 = 0; q0 < Kpad; q0 += 64) {
-        __syncthreads();
+    if (lane < R) red[warp][lane] = mb;
+    __syncthreads();
+    // warp w cuts vector v0 + w
+    mb = 0ull;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int q = q0 + ty + 8 * u;
-            tile[tx][ty + 8 * u] = (v < V && q < K) ? s.at(v, q) : 0.0;
-        }
-        __syncthreads();
-        const int q = q0 + 2 * tx;
-        if (q < Kpad)
+    for (int w = 0; w < 8; ++w) mb = red[w][warp] > mb ? red[w][warp] : mb;
+    const int e = row_exponent(mb);
+    if (lane == 0) exps[v0 + warp] = e;
+    unsigned *o = reinterpret_cast<unsigned *>(out + (size_t)(v0 + warp) * ldo);
+    for (int q0 = 0; q0 < Kpad; q0 += C) {
+        if (K > C) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int r = ty * 4 + u;
-                int a[ND], b[ND];
-                digits_of<ND>(tile[r][2 * tx], es[r], a);
-                digits_of<ND>(tile[r][2 * tx + 1], es[r], b);
-                unsigned *o = reinterpret_cast<unsigned *>(out + (size_t)(v0 + r) * ldo);
-#pragma unroll
-                for (int d = 0; d < ND; ++d)
-                    if (d < nd) o[(d * plane + q) >> 1] = bf16_pair(a[d], b[d]);
+            for (int u = 0; u < C / 32; ++u) {
+                const int q = q0 + ty + 32 * u;
+                x[u] = (v < V && q < K) ? s.at(v, q) : 0.0;
             }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int u = 0; u < C / 32; ++u) tile[tx][ty + 32 * u] = x[u];
+        __syncthreads();
+        for (int c = 2 * lane; c < C && q0 + c < Kpad; c += 64) {
+            int a[ND], b[ND];
+            digits_of<ND>(tile[warp][c], e, a);
+            digits_of<ND>(tile[warp][c + 1], e, b);
+#pragma unroll
+            for (int d = 0; d < ND; ++d)
+                if (d < nd) o[(d * plane + q0 + c) >> 1] = bf16_pair(a[d], b[d]);
+        }
     }
 }
 
@@ -270,6 +284,9 @@ struct Args {
 constexpr int kNotPow2 = 1 << 20;
 }  // namespace oztc
 
+// x 2^e where the result may not be a normal number (out of line: it is hardly ever taken)
+__device__ __noinline__ double scale_slow(double x, int e) { return ldexp(x, e); }
+
 // a 2^e rounded to nearest even, with integer operations where the result is a normal number
 __device__ __forceinline__ double pack_double(unsigned long long nrm, bool sticky, bool neg, int biased)
 {
@@ -286,7 +303,7 @@ __device__ __forceinline__ double fixed_to_double(long long a, int e)
     const unsigned long long u = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
     const int lz = __clzll((long long)u);
     const int biased = 1086 - lz + e;  // exponent field of 2^63 2^(e - lz)
-    if (biased < 1 || biased > 2045) return ldexp((double)a, e);
+    if (biased < 1 || biased > 2045) return scale_slow((double)a, e);
     return pack_double(u << lz, false, a < 0, biased);
 }
 
@@ -301,14 +318,14 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, in
         if (ul == 0ull) return 0.0;
         const int lz = __clzll((long long)ul), biased = 1086 - lz + e;
         if (biased >= 1 && biased <= 2045) return pack_double(ul << lz, false, neg, biased);
-        const double v = ldexp((double)ul, e);
+        const double v = scale_slow((double)ul, e);
         return neg ? -v : v;
     }
     const int lz = __clzll((long long)uh), biased = 1150 - lz + e;
     const unsigned long long nrm = lz ? (uh << lz) | (ul >> (64 - lz)) : uh;
     const bool sticky = (lz ? ul << lz : ul) != 0ull;
     if (biased >= 1 && biased <= 2045) return pack_double(nrm, sticky, neg, biased);
-    const double v = ldexp((double)(nrm | (sticky ? 1ull : 0ull)), e + 64 - lz);
+    const double v = scale_slow((double)(nrm | (sticky ? 1ull : 0ull)), e + 64 - lz);
     return neg ? -v : v;
 }
 
@@ -539,29 +556,38 @@ ozaki_gemm_tc_kernel(const __grid_constant__ oztc::Maps maps, const __grid_const
             const int er = (row_in ? a.ea[row] : 0) - kOzBits * (WIDE ? 9 : D + 1) + (WIDE ? 0 : a.eshift) +
                            (pow2 ? a.alpha_exp : 0);
             double *crow = a.C + blockIdx.z * a.cstride + (size_t)row;
-            // C = beta C + sum, 8 columns at a time (the loads of C first)
+            // C = beta C + sum, 4 columns at a time (the loads of C first). The sums go through
+            // shared memory (the rings are done), each thread reading back its own: a loop over
+            // registers would have to be unrolled, and that much straight-line code, run once,
+            // waits for instructions (12 us of a tile's 34).
+            long long *stage = reinterpret_cast<long long *>(smem) + (tid - 64);
+            constexpr int ET = 32 * EPI_WARPS;
 #pragma unroll
-            for (int q = 0; q < CW / 8; ++q) {
-                double cv[8];
+            for (int j = 0; j < CW; ++j) {
+                stage[j * ET] = acc[j];
+                if (WIDE) stage[(CW + j) * ET] = low[WIDE ? j : 0];
+            }
+#pragma unroll 1
+            for (int q = 0; q < CW; q += 4) {
+                double cv[4];
+                bool in[4];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int col = n0 + c0 + q * 8 + j;
-                    const bool in = row_in && col < a.n_real && (!a.uplo || row >= col);
-                    cv[j] = (in && a.beta != 0.0) ? crow[(size_t)col * a.ldc] : 0.0;
+                for (int j = 0; j < 4; ++j) {
+                    const int col = n0 + c0 + q + j;
+                    in[j] = row_in && col < a.n_real && (!a.uplo || row >= col);
+                    cv[j] = (in[j] && a.beta != 0.0) ? crow[(size_t)col * a.ldc] : 0.0;
                 }
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int cl = c0 + q * 8 + j, col = n0 + cl;
-                    if (row_in && col < a.n_real && (!a.uplo || row >= col)) {
-                        double val;
-                        if (WIDE) val = fixed_to_double(acc[q * 8 + j], low[WIDE ? q * 8 + j : 0], er + ebs[cl]);
-                        else val = fixed_to_double(acc[q * 8 + j], er + ebs[cl]);
-                        if (neg) val = -val;
-                        if (!pow2) val *= a.alpha;
-                        if (a.beta == 1.0) val += cv[j];
-                        else if (a.beta != 0.0) val = fma(a.beta, cv[j], val);
-                        crow[(size_t)col * a.ldc] = val;
-                    }
+                for (int j = 0; j < 4; ++j) {
+                    const int cl = c0 + q + j, col = n0 + cl;
+                    double val;
+                    if (WIDE) val = fixed_to_double(stage[(q + j) * ET], stage[(CW + q + j) * ET], er + ebs[cl]);
+                    else val = fixed_to_double(stage[(q + j) * ET], er + ebs[cl]);
+                    if (neg) val = -val;
+                    if (!pow2) val *= a.alpha;
+                    if (a.beta == 1.0) val += cv[j];
+                    else if (a.beta != 0.0) val = fma(a.beta, cv[j], val);
+                    if (in[j]) crow[(size_t)col * a.ldc] = val;
                 }
             }
         }
@@ -610,10 +636,10 @@ cudaError_t ozaki_split(cudaStream_t st, int V, int K, const double *src, long l
     const bool across = sv == 1 && sq != 1;
     EGB_COUNT_LAUNCH();
     if (digits == kOzWide) {
-        if (across) ozaki_split_t_kernel<kOzWide><<<Vpad / 32, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
+        if (across) ozaki_split_t_kernel<kOzWide><<<Vpad / 8, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
         else ozaki_split_kernel<kOzWide><<<Vpad, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
     } else {
-        if (across) ozaki_split_t_kernel<kOzDigits><<<Vpad / 32, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
+        if (across) ozaki_split_t_kernel<kOzDigits><<<Vpad / 8, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
         else ozaki_split_kernel<kOzDigits><<<Vpad, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
     }
     return cudaGetLastError();
