@@ -141,9 +141,7 @@ cudaError_t potrf(cudaStream_t st, int n, T *a, int lda, T *inv_diag, T *work, i
             if (m2 > 0) {
                 T *a21 = a + (j0 + jb) + (size_t)j0 * lda;
                 T *a22 = a + (j0 + jb) + (size_t)(j0 + jb) * lda;
-                if ((e = gemm<T>(st, 0, 1, m2, jb, jb, T(1), a21, lda, inv11, n, T(0), work, m2)) != cudaSuccess) return e;
-                if ((e = cudaMemcpy2DAsync(a21, sizeof(T) * lda, work, sizeof(T) * m2, sizeof(T) * m2, jb,
-                                           cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+                if ((e = tri_apply<T>(st, 1, 0, jb, m2, inv11, n, a21, lda)) != cudaSuccess) return e;
                 if ((e = gemm<T>(st, 0, 1, m2, m2, jb, T(-1), a21, lda, a21, lda, T(1), a22, lda, 1)) != cudaSuccess) return e;
             }
         }
@@ -159,9 +157,7 @@ cudaError_t potrf(cudaStream_t st, int n, T *a, int lda, T *inv_diag, T *work, i
                 if ((e = gemm<T>(st, 0, 1, m2, jb, j0 - p0, T(-1), a21, lda, a + j0 + (size_t)p0 * lda, lda,
                                  T(1), xj, lda)) != cudaSuccess) return e;
             }
-            if ((e = gemm<T>(st, 0, 1, m2, jb, jb, T(1), xj, lda, inv_diag + j0, n, T(0), work, m2)) != cudaSuccess) return e;
-            if ((e = cudaMemcpy2DAsync(xj, sizeof(T) * lda, work, sizeof(T) * m2, sizeof(T) * m2, jb,
-                                       cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+            if ((e = tri_apply<T>(st, 1, 0, jb, m2, inv_diag + j0, n, xj, lda)) != cudaSuccess) return e;
         }
         // (3) A22 -= L21 L21^T (lower triangle), K = panel width
         T *a22 = a + p1 + (size_t)p1 * lda;
@@ -191,9 +187,7 @@ static cudaError_t trsm_range(cudaStream_t st, int trans, int r0, int r1, int nc
         const T *inv11 = inv_diag + j0;
         T *bj = B + j0;
         // B_j := inv(L_jj) B_j   or   inv(L_jj)^T B_j
-        if ((e = gemm<T>(st, trans, 0, jb, ncol, jb, T(1), inv11, ldi, bj, ldb, T(0), work, jb)) != cudaSuccess) return e;
-        if ((e = cudaMemcpy2DAsync(bj, sizeof(T) * ldb, work, sizeof(T) * jb, sizeof(T) * jb, ncol,
-                                   cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+        if ((e = tri_apply<T>(st, 0, trans, jb, ncol, inv11, ldi, bj, ldb)) != cudaSuccess) return e;
         if (!trans) {
             const int m2 = r1 - j0 - jb;
             if (m2 > 0) {

@@ -1,9 +1,8 @@
-// Register-tiled SIMT GEMM and small matrix utilities.
+// SIMT GEMM and small matrix utilities.
 //
-// The binary64 path of this solver is bound by the FP64 FMA rate of the chip, which
-// any register-tiled kernel saturates, so the GEMM here is a plain shared-memory tiled
-// kernel: each CTA computes a BM x BN tile of C, staging BK-deep slices of op(A) and
-// op(B) in shared memory, each thread accumulating a TM x TN block in registers.
+// Large products run on the tensor cores (tc_gemm.cu in binary32, ozaki.cu in binary64); the
+// kernels here serve the small ones, where three launches and two operand passes cost more
+// than the product, and calls without the scratch of those paths.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -98,9 +97,138 @@ gemm_kernel(int m, int n, int k, T alpha, const T *__restrict__ A, int lda, int 
     }
 }
 
-template <typename T> struct GemmCfg;
-template <> struct GemmCfg<double> { static constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4; };
-template <> struct GemmCfg<float> { static constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8; };
+// Small tiles: BT x BT per CTA, TM x TN per thread, the next 16-deep slices in registers while
+// the current ones are used. A 64^3 product is 16 CTAs of 16 x 16 in binary64, where a tile
+// costs BT^2 / 2 clocks per unit of K on its SM: 6 us against 64 us for one CTA of 64 x 64.
+// Binary64 uses it for every shape (at that rate the extra operand traffic does not show).
+template <typename T, int BT, int TM, int TN>
+__global__ void __launch_bounds__((BT / TM) * (BT / TN))
+gemm_small_kernel(int m, int n, int k, T alpha, const T *__restrict__ A, int lda, int ta,
+                  const T *__restrict__ B, int ldb, int tb, T beta, T *__restrict__ C, int ldc, int uplo)
+{
+    constexpr int NT = (BT / TM) * (BT / TN), BK = 16, PER = BT * BK / NT;
+    __shared__ T As[2][BK][BT + 1], Bs[2][BK][BT + 1];
+    const int m0 = blockIdx.x * BT, n0 = blockIdx.y * BT;
+    if (uplo == 1 && m0 + BT - 1 < n0) return;  // tile entirely above the diagonal
+    const int tid = threadIdx.x, tx = tid % (BT / TN), ty = tid / (BT / TN);
+    T av[PER], bv[PER];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const int e = tid + r * NT;
+            int i = ta ? e / BK : e % BT, kk = ta ? e % BK : e / BT;
+            av[r] = (m0 + i < m && k0 + kk < k)
+                        ? (ta ? A[(size_t)(k0 + kk) + (size_t)(m0 + i) * lda] : A[(size_t)(m0 + i) + (size_t)(k0 + kk) * lda])
+                        : T(0);
+            i = tb ? e % BT : e / BK;
+            kk = tb ? e / BT : e % BK;
+            bv[r] = (n0 + i < n && k0 + kk < k)
+                        ? (tb ? B[(size_t)(n0 + i) + (size_t)(k0 + kk) * ldb] : B[(size_t)(k0 + kk) + (size_t)(n0 + i) * ldb])
+                        : T(0);
+        }
+    };
+    auto store = [&](int buf) {
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const int e = tid + r * NT;
+            if (ta) As[buf][e % BK][e / BK] = av[r]; else As[buf][e / BT][e % BT] = av[r];
+            if (tb) Bs[buf][e / BT][e % BT] = bv[r]; else Bs[buf][e % BK][e / BK] = bv[r];
+        }
+    };
+    T acc[TM][TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
+    load(0);
+    store(0);
+    __syncthreads();
+    for (int k0 = 0, buf = 0; k0 < k; k0 += BK, buf ^= 1) {
+        if (k0 + BK < k) load(k0 + BK);
+#pragma unroll
+        for (int kk = 0; kk < BK; ++kk)
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j)
+                    acc[i][j] = fma(As[buf][kk][ty + i * (BT / TM)], Bs[buf][kk][tx + j * (BT / TN)], acc[i][j]);
+        if (k0 + BK < k) store(buf ^ 1);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int j = 0; j < TN; ++j)
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            const int gi = m0 + ty + i * (BT / TM), gj = n0 + tx + j * (BT / TN);
+            if (gi >= m || gj >= n || (uplo == 1 && gi < gj)) continue;
+            T *c = C + (size_t)gi + (size_t)gj * ldc;
+            T v = alpha * acc[i][j];
+            if (beta != T(0)) v = fma(beta, *c, v);
+            *c = v;
+        }
+}
+
+// B (w x ncol, w <= 64, ldb) := op(inv) B (left) or X (m x w, ldb) := X inv^T (right), in place,
+// inv the lower-triangular inverse of a diagonal block: a CTA holds whole columns (rows) of
+// the block, so no copy of the product is needed. One 64-column (row) slice of COLS per CTA.
+template <typename T, int COLS>
+__global__ void __launch_bounds__(256) tri_apply_kernel(int right, int trans, int w, int ncol, const T *__restrict__ inv,
+                                                        int ldi, T *B, int ldb)
+{
+    __shared__ T Ls[64][65];        // Ls[k][i] = op(inv)[i][k]
+    __shared__ T Bs[64][COLS + 1];  // Bs[k][c]
+    constexpr int CPT = COLS / 4;   // columns of a thread
+    const int c0 = blockIdx.x * COLS, tid = threadIdx.x;
+    // right: X_row = X_row inv^T, i.e. out_i = sum_k inv[i][k] x_k for each row
+    for (int e = tid; e < 64 * 64; e += 256) {
+        const int r = e & 63, c = e >> 6;  // inv[r][c], c <= r
+        const T v = (r < w && c <= r) ? inv[(size_t)r + (size_t)c * ldi] : T(0);
+        if (trans) Ls[r][c] = v; else Ls[c][r] = v;
+    }
+    for (int e = tid; e < 64 * COLS; e += 256) {
+        const int k = right ? e / COLS : e & 63, c = right ? e % COLS : e >> 6;
+        Bs[k][c] = (k < w && c0 + c < ncol) ? (right ? B[(size_t)(c0 + c) + (size_t)k * ldb] : B[(size_t)k + (size_t)(c0 + c) * ldb])
+                                            : T(0);
+    }
+    __syncthreads();
+    const int i = tid & 63, cg = (tid >> 6) * CPT;
+    T acc[CPT];
+#pragma unroll
+    for (int j = 0; j < CPT; ++j) acc[j] = T(0);
+    // op(inv)[i][k] is zero for k > i (k < i when transposed); a warp holds 32 consecutive i
+    const int kb = trans ? (i & 32) : 0, ke = trans ? 64 : (i & 32) + 32;
+#pragma unroll 4
+    for (int k = kb; k < ke; ++k)
+#pragma unroll
+        for (int j = 0; j < CPT; ++j) acc[j] = fma(Ls[k][i], Bs[k][cg + j], acc[j]);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < CPT; ++j) Bs[i][cg + j] = acc[j];
+    __syncthreads();
+    for (int e = tid; e < 64 * COLS; e += 256) {
+        const int k = right ? e / COLS : e & 63, c = right ? e % COLS : e >> 6;
+        if (k < w && c0 + c < ncol) {
+            if (right) B[(size_t)(c0 + c) + (size_t)k * ldb] = Bs[k][c];
+            else B[(size_t)k + (size_t)(c0 + c) * ldb] = Bs[k][c];
+        }
+    }
+}
+
+template <typename T>
+cudaError_t tri_apply(cudaStream_t st, int right, int trans, int w, int ncol, const T *inv, int ldi, T *B, int ldb)
+{
+    constexpr int COLS = sizeof(T) == 8 ? 4 : 16;
+    if (w <= 0 || ncol <= 0) return cudaSuccess;
+    if (w > 64) return cudaErrorInvalidValue;
+    EGB_COUNT_LAUNCH();
+    tri_apply_kernel<T, COLS><<<ceil_div(ncol, COLS), 256, 0, st>>>(right, trans, w, ncol, inv, ldi, B, ldb);
+    return cudaGetLastError();
+}
+template cudaError_t tri_apply<double>(cudaStream_t, int, int, int, int, const double *, int, double *, int);
+template cudaError_t tri_apply<float>(cudaStream_t, int, int, int, int, const float *, int, float *, int);
+
+// Binary32 tiles of the large SIMT kernel.
+struct GemmCfg { static constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8; };
 
 // Scratch for the tensor-core binary32 GEMM of the calling thread's current solve (set by
 // the solver around a binary32-route solve; absent elsewhere).
@@ -167,11 +295,15 @@ static cudaError_t gemm_f64_digits(cudaStream_t st, int ta, int tb, int m, int n
     return ozaki_gemm(st, m, n, k, alpha, ad, xe, bd, ye, beta, C, ldc, uplo, digits, part, part_elems);
 }
 
-// A binary64 product goes to the digit products when the thread has their scratch and K is
-// long enough: a CTA of the SIMT kernel takes about 1 us per unit of K for its 64 x 64 tile
-// (4096 FMAs at two a clock) however small the product, the two splits and the digit product
-// about 12 us.
-static bool digits_pay(int k) { return t_oz_planes && k >= 24; }
+// A binary64 product goes to the digit products when the thread has their scratch and the
+// small-tile kernel would take longer: that one needs 128 clocks of an SM per unit of K and
+// 16 x 16 tile, the two splits and the digit product 35 to 45 us (and as much host time).
+static bool digits_pay(int m, int n, int k)
+{
+    const double tiles = (double)ceil_div(m, 16) * ceil_div(n, 16);
+    const double waves = tiles <= 152.0 ? 1.0 : tiles / 152.0;
+    return t_oz_planes && k >= 24 && waves * k >= 450.0;
+}
 
 // C -= V W^T + W V^T (lower triangle, m x m, V and W m x b): one product over K = 2 b whose
 // operands' rows are [V_i W_i] and [W_i V_i].
@@ -179,7 +311,7 @@ cudaError_t gemm_f64_two_sided(cudaStream_t st, int m, int b, const double *V, i
                                int ldw, double *C, int ldc)
 {
     const size_t pe = ozaki_split_elems(m, 2 * b, kOzWide), xe = (size_t)ceil_div(m, 128) * 128;
-    if (!digits_pay(2 * b) || 2 * pe > t_oz_elems || 2 * xe > t_oz_exp_elems) return cudaErrorNotSupported;
+    if (!digits_pay(m, m, 2 * b) || 2 * pe > t_oz_elems || 2 * xe > t_oz_exp_elems) return cudaErrorNotSupported;
     __nv_bfloat16 *ad = t_oz_planes, *bd = ad + pe;
     int *ea = t_oz_exps, *eb = ea + xe;
     cudaError_t e;
@@ -194,25 +326,35 @@ cudaError_t gemm(cudaStream_t st, int ta, int tb, int m, int n, int k, T alpha, 
 {
     if (m <= 0 || n <= 0) return cudaSuccess;
     if constexpr (sizeof(T) == 4) {
-        // binary32 products large enough for the tensor-core path
-        if (t_tc_work && k >= 16 && (double)m * n * k >= 4.0e6) {
+        // Large binary32 products go to the tensor cores: two operand passes and the product take
+        // 17 us at least, the small-tile kernel 10 us per 1e8 multiplications.
+        if (t_tc_work && k >= 16 && (double)m * n * k >= 8.0e7) {
             cudaError_t e = tc_gemm_f32(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc,
                                         uplo, t_tc_work, t_tc_elems, t_tc_status);
             if (e != cudaErrorNotSupported) return e;
         }
     } else {
         // binary64 products large enough for the digit products on the tensor cores
-        if (digits_pay(k)) {
+        if (digits_pay(m, n, k)) {
             cudaError_t e = gemm_f64_digits(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, uplo);
             if (e != cudaErrorNotSupported) return e;
         }
     }
-    using G = GemmCfg<T>;
-    dim3 grid(ceil_div(m, G::BM), ceil_div(n, G::BN));
-    dim3 block((G::BM / G::TM) * (G::BN / G::TN));
     EGB_COUNT_LAUNCH();
-    gemm_kernel<T, G::BM, G::BN, G::BK, G::TM, G::TN><<<grid, block, 0, st>>>(
-        m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, uplo, k > 0 ? k : 1, 0);
+    if constexpr (sizeof(T) == 8) {
+        gemm_small_kernel<T, 16, 2, 1><<<dim3(ceil_div(m, 16), ceil_div(n, 16)), 128, 0, st>>>(
+            m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, uplo);
+    } else {
+        // binary32: 32 x 32 tiles for the products below the tensor-core path
+        using G = GemmCfg;
+        if ((double)m * n * k < 8.0e7)
+            gemm_small_kernel<T, 32, 2, 2><<<dim3(ceil_div(m, 32), ceil_div(n, 32)), 256, 0, st>>>(
+                m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, uplo);
+        else
+            gemm_kernel<T, G::BM, G::BN, G::BK, G::TM, G::TN>
+                <<<dim3(ceil_div(m, G::BM), ceil_div(n, G::BN)), (G::BM / G::TM) * (G::BN / G::TN), 0, st>>>(
+                    m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, uplo, k > 0 ? k : 1, 0);
+    }
     return cudaGetLastError();
 }
 
@@ -241,30 +383,32 @@ cudaError_t gemm_splitk(cudaStream_t st, int ta, int tb, int m, int n, int k, T 
                                         t_tc_work, t_tc_elems, t_tc_status);
             if (e != cudaErrorNotSupported) return e;
         }
-    } else if (digits_pay(k)) {
-        return gemm<T>(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, T(0), C, ldc, 0);
     }
-    using G = GemmCfg<T>;
-    const int tiles = ceil_div(m, G::BM) * ceil_div(n, G::BN);
-    int splits = ceil_div(2 * 152, tiles);
-    int maxs = k / 256;
-    if (splits > maxs) splits = maxs;
-    if ((size_t)splits * m * n > part_elems) splits = (int)(part_elems / ((size_t)m * n));
-    if (splits <= 1) return gemm<T>(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, T(0), C, ldc, 0);
-    int kchunk = ceil_div(k, splits);
-    kchunk = ceil_div(kchunk, G::BK) * G::BK;
-    splits = ceil_div(k, kchunk);
-    dim3 grid(ceil_div(m, G::BM), ceil_div(n, G::BN), splits);
-    dim3 block((G::BM / G::TM) * (G::BN / G::TN));
-    EGB_COUNT_LAUNCH();
-    gemm_kernel<T, G::BM, G::BN, G::BK, G::TM, G::TN><<<grid, block, 0, st>>>(
-        m, n, k, T(1), A, lda, ta, B, ldb, tb, T(0), part, m, 0, kchunk, (size_t)m * n);
-    size_t total = (size_t)m * n;
-    int rg = (int)((total + 255) / 256);
-    if (rg > 152 * 8) rg = 152 * 8;
-    EGB_COUNT_LAUNCH();
-    splitk_reduce_kernel<T><<<rg, 256, 0, st>>>(m, n, splits, part, alpha, C, ldc);
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        return gemm<T>(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, T(0), C, ldc, 0);
+    } else {
+        using G = GemmCfg;
+        const int tiles = ceil_div(m, G::BM) * ceil_div(n, G::BN);
+        int splits = ceil_div(2 * 152, tiles);
+        int maxs = k / 256;
+        if (splits > maxs) splits = maxs;
+        if ((size_t)splits * m * n > part_elems) splits = (int)(part_elems / ((size_t)m * n));
+        if (splits <= 1) return gemm<T>(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, T(0), C, ldc, 0);
+        int kchunk = ceil_div(k, splits);
+        kchunk = ceil_div(kchunk, G::BK) * G::BK;
+        splits = ceil_div(k, kchunk);
+        dim3 grid(ceil_div(m, G::BM), ceil_div(n, G::BN), splits);
+        dim3 block((G::BM / G::TM) * (G::BN / G::TN));
+        EGB_COUNT_LAUNCH();
+        gemm_kernel<T, G::BM, G::BN, G::BK, G::TM, G::TN><<<grid, block, 0, st>>>(
+            m, n, k, T(1), A, lda, ta, B, ldb, tb, T(0), part, m, 0, kchunk, (size_t)m * n);
+        size_t total = (size_t)m * n;
+        int rg = (int)((total + 255) / 256);
+        if (rg > 152 * 8) rg = 152 * 8;
+        EGB_COUNT_LAUNCH();
+        splitk_reduce_kernel<T><<<rg, 256, 0, st>>>(m, n, splits, part, alpha, C, ldc);
+        return cudaGetLastError();
+    }
 }
 template cudaError_t gemm_splitk<double>(cudaStream_t, int, int, int, int, int, double, const double *,
                                          int, const double *, int, double *, int, double *, size_t);

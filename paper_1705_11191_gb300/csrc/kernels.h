@@ -56,6 +56,11 @@ cudaError_t tc_gemm_f32(cudaStream_t st, int ta, int tb, int m, int n, int k, fl
                         const float *A, int lda, const float *B, int ldb, float beta, float *C,
                         int ldc, int uplo, float *work, size_t work_elems, int *status);
 
+// In place, with the inverse of a lower-triangular diagonal block (w <= 64): B (w x ncol) :=
+// op(inv) B, or right: B (ncol x w) := B inv^T.
+template <typename T>
+cudaError_t tri_apply(cudaStream_t st, int right, int trans, int w, int ncol, const T *inv, int ldi, T *B, int ldb);
+
 // C = alpha * op(A) * op(B) with K split over several CTAs (for small outputs with a long
 // K); part: scratch of part_elems elements for the partial products.
 template <typename T>
