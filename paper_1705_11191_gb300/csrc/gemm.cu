@@ -327,8 +327,8 @@ cudaError_t gemm(cudaStream_t st, int ta, int tb, int m, int n, int k, T alpha, 
     if (m <= 0 || n <= 0) return cudaSuccess;
     if constexpr (sizeof(T) == 4) {
         // Large binary32 products go to the tensor cores: two operand passes and the product take
-        // 17 us at least, the small-tile kernel 10 us per 1e8 multiplications.
-        if (t_tc_work && k >= 16 && (double)m * n * k >= 8.0e7) {
+        // 17 us at least, the small-tile kernel about 16 us at this limit (50 us at 64 x 64 x 16384).
+        if (t_tc_work && k >= 16 && (double)m * n * k >= 3.0e7) {
             cudaError_t e = tc_gemm_f32(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc,
                                         uplo, t_tc_work, t_tc_elems, t_tc_status);
             if (e != cudaErrorNotSupported) return e;
@@ -347,7 +347,7 @@ cudaError_t gemm(cudaStream_t st, int ta, int tb, int m, int n, int k, T alpha, 
     } else {
         // binary32: 32 x 32 tiles for the products below the tensor-core path
         using G = GemmCfg;
-        if ((double)m * n * k < 8.0e7)
+        if ((double)m * n * k < 3.0e7)
             gemm_small_kernel<T, 32, 2, 2><<<dim3(ceil_div(m, 32), ceil_div(n, 32)), 256, 0, st>>>(
                 m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, uplo);
         else
