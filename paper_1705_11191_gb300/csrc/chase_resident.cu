@@ -25,10 +25,10 @@
 // The column sums x^T X0 and D x are taken with the unscaled x (x_first apart), so that
 // three block barriers serve a whole step.
 //
-// Measured, b = 64, against the kernel of sb2st.cu: binary32 n = 777 10.6 -> 3.0 ms,
-// n = 4096 60.3 -> 17.3 ms, n = 16384 245 -> 76 ms (14.7 -> 4.2 - 4.7 us a sweep, two block
-// barriers' worth of arithmetic and two L2 hand-overs); binary64 n = 512 15.2 -> 11.0 ms,
-// n = 1531 51.3 -> 35.7 ms (a step's 28 000 FMAs at two a clock bound it).
+// Measured against the kernel of sb2st.cu: binary32, b = 64, n = 777 10.6 -> 2.7 ms, n = 4096
+// 60.3 -> 16.0 ms, n = 16384 245 -> 70 ms (14.7 -> 3.5 - 4.3 us a sweep, two L2 hand-overs and
+// two steps' arithmetic); binary64, b = 64, n = 512 15.2 -> 11.0 ms, n = 1531 51.3 -> 35.7 ms (a
+// step's 28 000 FMAs at two a clock bound it), and with b = 32 4.5 and 14.0 ms.
 #include "common.cuh"
 #include "kernels.h"
 #include "packets.cuh"
@@ -99,6 +99,13 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         const int pr = rs == 0 ? B - 1 : rs - 1;           // slot that leaves / enters
         const bool have_row = j > 0 && r - 1 + B <= n - 1;  // position t + 1 had a step in sweep j - 1
         const bool have_next = r + B <= n - 1;              // position t + 1 has one in this sweep
+        // ---- the window moves, the part that needs no message: the column that leaves D enters X
+        if (j > 0) {
+            if (t == 0) x0 = __shfl_sync(0xffffffffu, pick(D, pr % CPT), quad | (pr / CPT));
+            if (i != pr && part == pr / CPT)
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) move_if(X[q], D[q], pr % CPT, q);
+        }
         // ---- what this step waits for
         {
             bool ok = true;
@@ -124,9 +131,8 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         }
         __syncthreads();
         if (failed) return;
-        // ---- the window moves: slot pr takes the new row and column
+        // ---- slot pr takes the new row and column
         if (j > 0) {
-            const T dold = __shfl_sync(0xffffffffu, pick(D, pr % CPT), quad | (pr / CPT));
             if (i == pr) {
 #pragma unroll
                 for (int q = 0; q < CPT; ++q) {
@@ -135,22 +141,23 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
                     D[q] = (c == pr) ? msc[par][1] : rows_[par][c];
                 }
                 x0 = rows_[par][pr];
-            } else {
-                if (part == pr / CPT) {
-                    const T ri = rows_[par][i];
+            } else if (part == pr / CPT) {
+                const T ri = rows_[par][i];
 #pragma unroll
-                    for (int q = 0; q < CPT; ++q)
-                        if (q == pr % CPT) { X[q] = D[q]; D[q] = ri; }
-                }
-                x0 = dold;
+                for (int q = 0; q < CPT; ++q) move_if(D[q], ri, pr % CPT, q);
             }
         }
         // ---- y, x and the partial sums over rows
         const bool first = i == rs;
         T y = T(0), x = x0;
         if (t > 0) {
+            T y1 = T(0);
 #pragma unroll
-            for (int q = 0; q < CPT; ++q) y = fma(X[q], vps[par][c0 + q], y);
+            for (int q = 0; q < CPT; q += 2) {
+                y = fma(X[q], vps[par][c0 + q], y);
+                y1 = fma(X[q + 1], vps[par][c0 + q + 1], y1);
+            }
+            y += y1;
             y += __shfl_xor_sync(0xffffffffu, y, 1);
             y += __shfl_xor_sync(0xffffffffu, y, 2);
             y *= msc[par][0];
@@ -188,12 +195,12 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
 #pragma unroll
                 for (int q = 0; q < PH; ++q) upart[warp][c0 + base + q] = u[q];
             }
-#pragma unroll
-            for (int o = 16; o >= 4; o >>= 1) {
-                ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                if (t > 0) xy += __shfl_xor_sync(0xffffffffu, xy, o);
-            }
-            if (lane == 0) { red[0][warp] = ss; red[1][warp] = xy; }
+            // |xz|^2 in the lanes of the lower half, xz . y in the upper half
+            const T keep = (lane & 16) ? xy : ss, give = (lane & 16) ? ss : xy;
+            T r2 = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+            r2 += __shfl_xor_sync(0xffffffffu, r2, 8);
+            r2 += __shfl_xor_sync(0xffffffffu, r2, 4);
+            if ((lane & 15) == 0) red[lane >> 4][warp] = r2;
         }
         __syncthreads();
         // ---- the reflector (every thread computes the same scalars) and q = tau D v
@@ -215,9 +222,13 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         }
         T qd;
         {
-            T g = T(0);
+            T g = T(0), g1 = T(0);
 #pragma unroll
-            for (int q = 0; q < CPT; ++q) g = fma(D[q], xs[c0 + q], g);
+            for (int q = 0; q < CPT; q += 2) {
+                g = fma(D[q], xs[c0 + q], g);
+                g1 = fma(D[q + 1], xs[c0 + q + 1], g1);
+            }
+            g += g1;
             g += __shfl_xor_sync(0xffffffffu, g, 1);
             g += __shfl_xor_sync(0xffffffffu, g, 2);
             const T dc = __shfl_sync(0xffffffffu, pick(D, rs % CPT), quad | (rs / CPT));
@@ -241,13 +252,12 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         T K = T(0);
 #pragma unroll
         for (int w = 0; w < NW; ++w) K += red[2][w];
-        K *= T(0.5) * tau;
-        const T wi = fma(-K, v, qd);
+        // D - v w^T - w v^T with w = q - K v / 2, as D - v q^T - (q - K v) v^T
+        const T w2 = fma(-K * tau, v, qd);
 #pragma unroll
         for (int q = 0; q < CPT; ++q) {
             const int c = c0 + q;
-            const T vc = vs[c], wc = fma(-K, vc, qs[c]);
-            D[q] = fma(-v, wc, fma(-wi, vc, D[q]));
+            D[q] = fma(-v, qs[c], fma(-w2, vs[c], D[q]));
         }
         if (t > 0) {
 #pragma unroll

@@ -58,7 +58,7 @@ potrf_diag_kernel(int jb, T *a, int lda, T *inv, int ldi, int *status, int pivot
                     d = T(1);  // keep going with a harmless pivot; the status reports the failure
                 }
                 piv[k] = d;
-                prec[k & 1] = T(1) / d;
+                prec[k & 1] = recip(d);
             }
         }
     };

@@ -69,11 +69,46 @@ __device__ __forceinline__ bool get(const u64 *p, unsigned seq, T &v, long long 
 
 }  // namespace pkt
 
-// 1 / sqrt(x): in binary64 the division and the square root are long sequences on the chip's
-// few binary64 units, the reciprocal square root a shorter one.
-template <typename T> __device__ __forceinline__ T rsq(T x);
-template <> __device__ __forceinline__ float rsq(float x) { return 1.0f / sqrtf(x); }
-template <> __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+// 1 / x and 1 / sqrt(x) to about an ulp: the hardware's approximation and Newton steps. A
+// library division or square root is two to three times as long a chain, and in binary64 two
+// to three times as many operations of the chip's few binary64 units. Arguments whose result
+// or whose approximation would be subnormal or overflow take the library's path.
+__device__ __forceinline__ double recip(double x)
+{
+    const int ex = __double2hiint(x) & 0x7FF00000;
+    if (ex >= (2044 << 20) || ex == 0) return 1.0 / x;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(fma(-x, r, 1.0), r, r);
+    return fma(fma(-x, r, 1.0), r, r);
+}
+__device__ __forceinline__ float recip(float x)
+{
+    const float a = fabsf(x);
+    if (!(a > 1e-36f && a < 1e36f)) return 1.0f / x;
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaf(fmaf(-x, r, 1.0f), r, r);
+}
+__device__ __forceinline__ double rsq(double x)
+{
+    const int ex = __double2hiint(x) & 0x7FF00000;
+    if (ex >= (2000 << 20) || ex <= (40 << 20)) return rsqrt(x);
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    // r += r (1 - x r^2) / 2, twice
+    double h = fma(-x * r, r, 1.0);
+    r = fma(0.5 * r, h, r);
+    h = fma(-x * r, r, 1.0);
+    return fma(0.5 * r, h, r);
+}
+__device__ __forceinline__ float rsq(float x)
+{
+    if (!(x > 1e-36f && x < 1e36f)) return 1.0f / sqrtf(x);
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
+}
 
 // Householder scalars of x = (alpha, tail) with |tail|^2 = ss: v = (1, scl tail), H = I - tau
 // v v^T, H x = beta e_1.
@@ -83,10 +118,10 @@ __device__ __forceinline__ void reflector(T alpha, T ss, T &beta, T &tau, T &scl
     beta = alpha;
     tau = scl = T(0);
     if (ss != T(0)) {
-        const T s2 = fma(alpha, alpha, ss), rn = rsq<T>(s2), nrm = s2 * rn;
+        const T s2 = fma(alpha, alpha, ss), rn = rsq(s2), nrm = s2 * rn;
         beta = (alpha >= T(0)) ? -nrm : nrm;
         tau = fma(fabs(alpha), rn, T(1));  // (beta - alpha) / beta
-        scl = T(1) / (alpha - beta);
+        scl = recip(alpha - beta);
     }
 }
 

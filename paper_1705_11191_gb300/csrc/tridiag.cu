@@ -20,6 +20,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "packets.cuh"
 
 namespace egb {
 
@@ -310,19 +311,6 @@ __global__ void block_assign_kernel(int n, const double *d, const double *e, int
 // the backward one, the twist index r = argmin |gamma_i| with gamma_r (signed), and
 // ||z||^2 of the vector z with z_r = 1 that solves (T_b - lam I) z = gamma_r e_r.
 // Arrays are indexed [i * kvec + l].
-// 1 / x to about an ulp: the hardware's 20-bit approximation and two Newton steps (four FMAs);
-// a binary64 division is about three times as many operations of the scarce binary64 unit. The
-// approximation flushes subnormals, but pivots are at least pivmin >= DBL_MIN; a huge x, whose
-// reciprocal would be subnormal, takes the division.
-__device__ __forceinline__ double recip(double x)
-{
-    if ((__double2hiint(x) & 0x7FF00000) >= (2044 << 20)) return 1.0 / x;
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(fma(-x, r, 1.0), r, r);
-    return fma(fma(-x, r, 1.0), r, r);
-}
-
 // |a| < |b| on the bit patterns
 __device__ __forceinline__ bool mag_less(double a, double b)
 {
