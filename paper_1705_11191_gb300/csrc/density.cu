@@ -16,6 +16,7 @@ __device__ __forceinline__ double occ_phi(int scheme, double x)
 {
     if (scheme == ELSI_OCC_GAUSSIAN || scheme == ELSI_OCC_MP0) return 0.5 * erfc(x);
     if (scheme == ELSI_OCC_MP1) return 0.5 * erfc(x) - x * exp(-x * x) * 0.28209479177387814347;
+    if (x < -37.0) return 1.0;  // 1 + exp(x) rounds to 1
     if (x > 0.0) { double e = exp(-x); return e / (1.0 + e); }
     return 1.0 / (1.0 + exp(x));
 }
@@ -67,9 +68,16 @@ __global__ void occupation_kernel(int k, const double *eps_all, double n_el_all,
             out[2] = 0.0;
         }
     } else {
+        const double rkt = 1.0 / kt;
+        // Far from mu an exponential adds nothing to the count (above x = 80 less than 2e-35 a
+        // state, below -37 exactly 1): a warp of such states skips the 50 or so operations of the
+        // binary64 unit that are most of the cost of a bisection step.
         auto count = [&](double mu) {
             double s2 = 0.0;
-            for (int l = tid; l < kk; l += nt) s2 += g * occ_phi(scheme, (eps(l) - mu) / kt);
+            for (int l = tid; l < kk; l += nt) {
+                const double x = (eps(l) - mu) * rkt;
+                if (scheme != ELSI_OCC_FERMI || x < 80.0) s2 += g * occ_phi(scheme, x);
+            }
             return block_sum(s2, red);
         };
         double lo = eps(0), hi = eps(kk - 1);

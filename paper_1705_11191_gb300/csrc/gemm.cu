@@ -97,20 +97,33 @@ gemm_kernel(int m, int n, int k, T alpha, const T *__restrict__ A, int lda, int 
     }
 }
 
-// Small tiles: BT x BT per CTA, TM x TN per thread, the next 16-deep slices in registers while
-// the current ones are used. A 64^3 product is 16 CTAs of 16 x 16 in binary64, where a tile
-// costs BT^2 / 2 clocks per unit of K on its SM: 6 us against 64 us for one CTA of 64 x 64.
-// Binary64 uses it for every shape (at that rate the extra operand traffic does not show).
+// Small tiles: BT x BT per CTA, TM x TN consecutive elements per thread, read from shared memory
+// 16 bytes at a time, the next 16-deep slices in registers while the current ones are used. A
+// 64^3 product is 16 CTAs of 16 x 16 in binary64, where a tile costs BT^2 / 2 clocks per unit of
+// K on its SM: 6 us against 64 us for one CTA of 64 x 64. Binary64 uses it for every shape (at
+// that rate the extra operand traffic does not show).
+template <typename T, int N>
+__device__ __forceinline__ void lds_vec(const T *p, T (&v)[N])
+{
+    if constexpr (sizeof(T) * N == 16) {
+        const uint4 u = *reinterpret_cast<const uint4 *>(p);
+        memcpy(v, &u, 16);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = p[i];
+    }
+}
+
 template <typename T, int BT, int TM, int TN>
 __global__ void __launch_bounds__((BT / TM) * (BT / TN))
 gemm_small_kernel(int m, int n, int k, T alpha, const T *__restrict__ A, int lda, int ta,
                   const T *__restrict__ B, int ldb, int tb, T beta, T *__restrict__ C, int ldc, int uplo)
 {
-    constexpr int NT = (BT / TM) * (BT / TN), BK = 16, PER = BT * BK / NT;
-    __shared__ T As[2][BK][BT + 1], Bs[2][BK][BT + 1];
+    constexpr int NT = (BT / TM) * (BT / TN), BK = 16, PER = BT * BK / NT, LD = BT + 16 / (int)sizeof(T);
+    __shared__ __align__(16) T As[2][BK][LD], Bs[2][BK][LD];
     const int m0 = blockIdx.x * BT, n0 = blockIdx.y * BT;
     if (uplo == 1 && m0 + BT - 1 < n0) return;  // tile entirely above the diagonal
-    const int tid = threadIdx.x, tx = tid % (BT / TN), ty = tid / (BT / TN);
+    const int tid = threadIdx.x, r0 = tid % (BT / TM) * TM, q0 = tid / (BT / TM) * TN;
     T av[PER], bv[PER];
     auto load = [&](int k0) {
 #pragma unroll
@@ -146,12 +159,15 @@ gemm_small_kernel(int m, int n, int k, T alpha, const T *__restrict__ A, int lda
     for (int k0 = 0, buf = 0; k0 < k; k0 += BK, buf ^= 1) {
         if (k0 + BK < k) load(k0 + BK);
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk)
+        for (int kk = 0; kk < BK; ++kk) {
+            T x[TM], y[TN];
+            lds_vec<T, TM>(&As[buf][kk][r0], x);
+            lds_vec<T, TN>(&Bs[buf][kk][q0], y);
 #pragma unroll
             for (int i = 0; i < TM; ++i)
 #pragma unroll
-                for (int j = 0; j < TN; ++j)
-                    acc[i][j] = fma(As[buf][kk][ty + i * (BT / TM)], Bs[buf][kk][tx + j * (BT / TN)], acc[i][j]);
+                for (int j = 0; j < TN; ++j) acc[i][j] = fma(x[i], y[j], acc[i][j]);
+        }
         if (k0 + BK < k) store(buf ^ 1);
         __syncthreads();
     }
@@ -159,7 +175,7 @@ gemm_small_kernel(int m, int n, int k, T alpha, const T *__restrict__ A, int lda
     for (int j = 0; j < TN; ++j)
 #pragma unroll
         for (int i = 0; i < TM; ++i) {
-            const int gi = m0 + ty + i * (BT / TM), gj = n0 + tx + j * (BT / TN);
+            const int gi = m0 + r0 + i, gj = n0 + q0 + j;
             if (gi >= m || gj >= n || (uplo == 1 && gi < gj)) continue;
             T *c = C + (size_t)gi + (size_t)gj * ldc;
             T v = alpha * acc[i][j];
@@ -348,7 +364,7 @@ cudaError_t gemm(cudaStream_t st, int ta, int tb, int m, int n, int k, T alpha, 
         // binary32: 32 x 32 tiles for the products below the tensor-core path
         using G = GemmCfg;
         if ((double)m * n * k < 3.0e7)
-            gemm_small_kernel<T, 32, 2, 2><<<dim3(ceil_div(m, 32), ceil_div(n, 32)), 256, 0, st>>>(
+            gemm_small_kernel<T, 32, 4, 4><<<dim3(ceil_div(m, 32), ceil_div(n, 32)), 64, 0, st>>>(
                 m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, uplo);
         else
             gemm_kernel<T, G::BM, G::BN, G::BK, G::TM, G::TN>
