@@ -38,6 +38,14 @@
 // issues the copies and the MMAs. Every wait is bounded; on expiry the CTA records
 // ELSI_ERR_TIMEOUT, waits (bounded) for its own operations in flight, frees its tensor
 // memory and returns.
+//
+// Pipeline over the blocks. A group is a chain of two products, so what bounds a CTA is the
+// latency of a group (6.3 us), and there is one CTA per 128 columns: at n = 4096 32 of 152 SMs.
+// The unit of work is therefore (block, 128 columns): rows of block J are final for it when block
+// J + 64 has passed them, so block J runs ceil(64 / b) + 1 steps behind block J + 64, on another SM.
+// The rows go through L2; a progress word per unit says how many steps are stored. Units are
+// handed out by a counter in the order of the blocks, so a unit waits only for one that was
+// handed out before it, whatever the number of CTAs that run at a time.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -241,16 +249,16 @@ __device__ __forceinline__ void tmem_ld8(unsigned taddr, float *v)
 
 // Eight consecutive rows r0 .. r0+7 of a column (rows >= n read as 0 / not stored); two
 // 16-byte accesses when the column start allows it (vec: ld a multiple of 4) and the eight
-// rows exist, since r0 is a multiple of 8.
+// rows exist, since r0 is a multiple of 8. Loads go to L2: another SM may have stored the rows.
 __device__ __forceinline__ void load8(const float *zc, int r0, int n, bool ok, bool vec, float *v)
 {
     if (ok && vec && r0 + 8 <= n) {
-        const float4 a = *reinterpret_cast<const float4 *>(zc + r0);
-        const float4 c = *reinterpret_cast<const float4 *>(zc + r0 + 4);
+        const float4 a = __ldcg(reinterpret_cast<const float4 *>(zc + r0));
+        const float4 c = __ldcg(reinterpret_cast<const float4 *>(zc + r0 + 4));
         v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = c.x; v[5] = c.y; v[6] = c.z; v[7] = c.w;
     } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = (ok && r0 + i < n) ? zc[r0 + i] : 0.f;
+        for (int i = 0; i < 8; ++i) v[i] = (ok && r0 + i < n) ? __ldcg(zc + r0 + i) : 0.f;
     }
 }
 
@@ -272,11 +280,13 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 
 struct ApplyArgs {
     int n, b, jb_lo, jb_hi, k;  // blocks jb_lo <= jb < jb_hi, their groups packed in fac
-    long long ldz;
+    long long ldz, spin_limit;
     const float *fac;
     float *z;
     int *status;
+    unsigned *sync;  // kSyncNext: units handed out, kSyncStop: a CTA gave up, kSyncHead + unit: steps stored
 };
+constexpr int kSyncNext = 0, kSyncStop = 1, kSyncHead = 2;
 
 __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyArgs a)
 {
@@ -284,22 +294,23 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
     unsigned char *smem = (unsigned char *)(((size_t)smem_raw + 1023) & ~(size_t)1023);
     unsigned long long *bars = (unsigned long long *)(smem + kGroupBytes);
     unsigned *tmem_slot = (unsigned *)(bars + 4);
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, unit_next;
     const unsigned bar_v = smem_u32(&bars[0]), bar_w = smem_u32(&bars[1]);
     const unsigned bar_m1 = smem_u32(&bars[2]), bar_m2 = smem_u32(&bars[3]);
     const unsigned sV = smem_u32(smem), sW = sV + 2 * kVPlane;
     const int n = a.n, b = a.b;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int quarter = warp & 3, part = warp >> 2;
-    const int gc = blockIdx.x * kCols + quarter * 32 + lane;  // column of Z
-    const bool colok = gc < a.k;
-    float *zc = a.z + (size_t)(colok ? gc : 0) * (size_t)a.ldz;
+    const int ncg = (a.k + kCols - 1) / kCols;       // column groups
+    const int units = (a.jb_hi - a.jb_lo) * ncg;     // unit u: block jb_hi - 1 - u / ncg, columns u % ncg
+    constexpr int kWaiter = kThreads - 32;           // thread that publishes and polls progress
     const bool vec = (a.ldz & 3) == 0 && (((size_t)a.z) & 15) == 0;
 
     if (tid == 0) {
         for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&bars[i]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         abort_flag = 0;
+        unit_next = (int)atomicAdd(a.sync + kSyncNext, 1u);
     }
     if (warp == 0) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
     tc_fence_before();
@@ -312,8 +323,6 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
     bool v_out = false, w_out = false, m1_out = false, m2_out = false;
     unsigned gidx = 0;  // groups processed by this CTA (parity of every barrier)
 
-    // packed index of group (jb, 0), kept up to date as jb decreases
-    long long gbase = a.jb_hi > a.jb_lo ? group_base(n, b, a.jb_hi - 1) - group_base(n, b, a.jb_lo) : 0;
     auto fac_of = [&](long long g) -> const unsigned char * {
         return reinterpret_cast<const unsigned char *>(a.fac) + (size_t)g * kGroupBytes;
     };
@@ -328,7 +337,10 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
         for (int p = 0; p < 4; ++p)
             bulk_g2s(sW + p * (kWPlane / 2), g + 2 * kVPlane + p * (kWPlane / 2), kWPlane / 2, bar_w);
     };
-    if (tid == 0 && a.jb_hi > a.jb_lo) {
+    int unit = unit_next;
+    long long gbase = 0;  // (thread 0) packed index of the first group of the unit's block
+    if (tid == 0 && unit < units) {
+        for (int i = a.jb_lo; i < a.jb_hi - 1 - unit / ncg; ++i) gbase += block_steps(n, b, i * kM);
         const unsigned char *g0 = fac_of(gbase);
         load_v(g0);
         load_w(g0);
@@ -341,11 +353,37 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
     const unsigned idesc2 = idesc_f32acc(2, 128, 128);
     bool ok = true;
 
-    for (int jb = a.jb_hi - 1; jb >= a.jb_lo && ok; --jb) {
+    while (unit < units && ok) {
+        const int jb = a.jb_hi - 1 - unit / ncg;
         const int J = jb * kM;
         const int SJ = block_steps(n, b, J);
-        // packed index of the group after (jb, t): (jb, t + 1), or (jb - 1, 0) after the last
-        const long long gnext_block = jb > a.jb_lo ? gbase - block_steps(n, b, J - kM) : -1;
+        const int gc = unit % ncg * kCols + quarter * 32 + lane;  // column of Z
+        const bool colok = gc < a.k;
+        float *zc = a.z + (size_t)(colok ? gc : 0) * (size_t)a.ldz;
+        unsigned *mine = a.sync + kSyncHead + unit;
+        // the block above (handed out ncg units before) must have stored the rows up to the end of
+        // the window of step t: its steps up to t + ceil(64 / b) - 1, or all of them
+        const int Sabove = unit >= ncg ? block_steps(n, b, J + kM) : 0;
+        int seen = unit >= ncg ? 0 : 1 << 30;  // (kWaiter) its steps known to be stored
+        auto wait_above = [&](int t) {
+            const int need = min(t + (kM + b - 1) / b, Sabove);
+            for (long long it = 0; seen < need; ++it) {
+                unsigned v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(mine - ncg) : "memory");
+                seen = (int)v;
+                if (seen >= need) break;
+                unsigned stop = 0;
+                if ((it & 63) == 63)
+                    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(stop) : "l"(a.sync + kSyncStop));
+                if (stop || it > a.spin_limit) {
+                    report_error(a.status, ELSI_ERR_TIMEOUT, 15);
+                    seen = -1;
+                    break;
+                }
+            }
+        };
+        if (tid == kWaiter) wait_above(1);  // rows of the windows of steps 0 and 1
+        if (__syncthreads_or(seen < 0)) { ok = false; break; }
         // initial window of the block: rows J .. J+127
 #pragma unroll
         for (int c = 0; c < kChunks; ++c) {
@@ -379,6 +417,9 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
             tmem_wait_st();
             tc_fence_before();
             __syncthreads();
+            // the rows that the last step stored are visible to the block below (while MMA 1 runs)
+            if (tid == kWaiter && t > 0)
+                asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(mine), "r"((unsigned)t) : "memory");
             // ---- MMA 1: Y^T = Z_w^T V
             if (tid == 0) {
                 if (!mbar_wait(bar_v, gidx & 1)) {
@@ -411,9 +452,16 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
             }
             tc_fence_after();
             // next group's V (MMA 1 has read the buffer)
-            const long long gnext = last ? gnext_block : gbase + t + 1;
+            long long gnext = gbase + t + 1;  // (thread 0) the group after this one
             if (tid == 0 && !abort_flag) {
                 m1_out = false;
+                if (last) {
+                    const int u = (int)atomicAdd(a.sync + kSyncNext, 1u);
+                    unit_next = u;
+                    if (u < units)
+                        for (int i = jb - 1; i >= a.jb_hi - 1 - u / ncg; --i) gbase -= block_steps(n, b, i * kM);
+                    gnext = u < units ? gbase : -1;
+                }
                 if (gnext >= 0) { load_v(fac_of(gnext)); v_out = true; }
             }
             // ---- A of MMA 2: Y^T (hi, lo); warp part q takes a = 16 q .. 16 q + 15
@@ -468,12 +516,14 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
             }
             __syncthreads();
             if (abort_flag) { ok = false; break; }
-            if (!mbar_wait(bar_m2, gidx & 1)) {
+            if (tid == kWaiter && !last) wait_above(t + 2);  // rows that the next step prefetches, while MMA 2 runs
+            const bool done2 = mbar_wait(bar_m2, gidx & 1);
+            if (!done2) {
                 report_error(a.status, ELSI_ERR_TIMEOUT, 14);
                 abort_flag = 1;
             }
             tc_fence_after();
-            if (tid == 0 && !abort_flag) {
+            if (tid == 0 && done2) {
                 m2_out = false;
                 if (gnext >= 0) { load_w(fac_of(gnext)); w_out = true; }
             }
@@ -504,11 +554,13 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
                     }
                 }
             }
-            __syncthreads();
-            if (abort_flag) { ok = false; break; }
+            if (__syncthreads_or(seen < 0 || abort_flag)) { ok = false; break; }
         }
-        gbase = gnext_block;
+        if (ok && tid == kWaiter)
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(mine), "r"((unsigned)SJ) : "memory");
+        unit = unit_next;
     }
+    if (!ok && tid == 0) atomicExch(a.sync + kSyncStop, 1u);
     // exit: nothing of this CTA may still be in flight when its shared and tensor memory go
     __syncthreads();
     if (tid == 0) {
@@ -544,15 +596,22 @@ static int q2_blocks_per_range(int n, int b)
     return (int)(r < (size_t)nblk ? r : (size_t)nblk);
 }
 
+// floats of operand blocks; the largest range is the one that starts at block 0
+static size_t q2_group_floats(int n, int b)
+{
+    return (size_t)q2tc::group_base(n, b, q2_blocks_per_range(n, b)) * q2tc::kGroupFloats;
+}
+
+// the counter and progress words of a range, for up to n columns at a time
+static size_t q2_sync_words(int n, int b)
+{
+    return q2tc::kSyncHead + (size_t)q2_blocks_per_range(n, b) * ceil_div(n, q2tc::kCols);
+}
+
 size_t q2_factor_elems(int n, int b)
 {
-    using namespace q2tc;
     if (n < 3) return 1;
-    const int nblk = (n - 2 + kM - 1) / kM;
-    const int r = q2_blocks_per_range(n, b);
-    // the largest range is the one that starts at block 0
-    const int hi = r < nblk ? r : nblk;
-    return (size_t)group_base(n, b, hi) * kGroupFloats;
+    return q2_group_floats(n, b) + q2_sync_words(n, b);
 }
 
 cudaError_t apply_q2_tc(cudaStream_t st, int n, int b, const float *v2, const float *tau2, int k,
@@ -563,6 +622,9 @@ cudaError_t apply_q2_tc(cudaStream_t st, int n, int b, const float *v2, const fl
     if (b < 8 || b > kM || (b & 7) || ((size_t)fac & 15)) return cudaErrorInvalidValue;
     const int S = sb2st_steps(n, b);
     const int nblk = (n - 2 + kM - 1) / kM;
+    int dev = 0, num_sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t fsmem = (size_t)(4 * kM * (kM + 1) + 2 * kM) * sizeof(float);
     static PerDeviceOnce fattr, aattr;
     cudaError_t e = once_per_device(fattr, [&] {
@@ -574,19 +636,32 @@ cudaError_t apply_q2_tc(cudaStream_t st, int n, int b, const float *v2, const fl
                                     kSmemBytes);
     });
     if (e != cudaSuccess) return e;
+    unsigned *sync = reinterpret_cast<unsigned *>(fac + q2_group_floats(n, b));
+    const int kmax = ceil_div(n, kCols) * kCols;  // columns that the progress words are there for
     // ranges of blocks from the last (applied first) to the first
     const int per = q2_blocks_per_range(n, b);
     for (int hi = nblk; hi > 0; hi -= per) {
         const int lo = hi - per > 0 ? hi - per : 0;
         EGB_COUNT_LAUNCH();
         q2_factor_kernel<<<dim3(S, hi - lo), 256, fsmem, st>>>(n, b, S, lo, v2, tau2, fac);
-        ApplyArgs a;
-        a.n = n; a.b = b; a.jb_lo = lo; a.jb_hi = hi; a.k = k; a.ldz = ldz; a.fac = fac; a.z = z;
-        a.status = status;
-        EGB_COUNT_LAUNCH();
-        q2_apply_tc5_kernel<<<ceil_div(k, kCols), kThreads, kSmemBytes, st>>>(a);
-        cudaError_t le = cudaGetLastError();
-        if (le != cudaSuccess) return le;
+        for (int c = 0; c < k; c += kmax) {
+            const int kc = k - c < kmax ? k - c : kmax, ncg = ceil_div(kc, kCols), units = (hi - lo) * ncg;
+            ApplyArgs a;
+            a.n = n; a.b = b; a.jb_lo = lo; a.jb_hi = hi; a.k = kc; a.ldz = ldz; a.fac = fac;
+            a.z = z + (size_t)c * ldz;
+            a.status = status; a.sync = sync; a.spin_limit = spin_limit();
+            e = cudaMemsetAsync(sync, 0, (size_t)(kSyncHead + units) * sizeof(unsigned), st);
+            if (e != cudaSuccess) return e;
+            // a block runs 1 + ceil(64 / b) steps behind the one above it: more CTAs than blocks that
+            // can be under way at a time would only wait
+            const int deep = ceil_div(block_steps(n, b, lo * kM), 1 + ceil_div(kM, b));
+            int grid = units < num_sms ? units : num_sms;
+            if ((long long)deep * ncg < grid) grid = deep * ncg;
+            EGB_COUNT_LAUNCH();
+            q2_apply_tc5_kernel<<<grid, kThreads, kSmemBytes, st>>>(a);
+            cudaError_t le = cudaGetLastError();
+            if (le != cudaSuccess) return le;
+        }
     }
     return cudaSuccess;
 }
