@@ -166,8 +166,10 @@ cudaError_t stein(cudaStream_t st, int n, const double *d, const double *e, int 
                   const double *w, T *z, int ldz, double *scratch, int *status);
 
 // ---- back-transformations (steps 4 and 5) ----
+// sync: scratch of q2_f64_sync_words(n) words (k <= n), or more
+size_t q2_f64_sync_words(int n);
 cudaError_t apply_q2_f64(cudaStream_t st, int n, int b, const double *v2, const double *tau2, int k, double *z,
-                         int ldz, int *status);
+                         int ldz, int *status, unsigned *sync, size_t sync_words);
 // binary32 Z <- Q2 Z with compact-WY groups of 64 reflectors on the tcgen05 tensor cores
 // (q2tc.cu); fac: scratch of q2_factor_elems(n, b) floats (16-byte aligned) for the
 // per-group operand blocks; b a multiple of 8 in 8..64. Timeouts of its bounded waits go

@@ -1,5 +1,6 @@
 // Stage sequence of one solve (arXiv:1705.11191 sec. 3.1, Eqs. 8-11 and steps (1)-(5);
 // sec. 4.4 for the occupation and density matrix).
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -103,7 +104,7 @@ int ensure_workspace(elsi_gb_handle_s *h, int kz)
         ENSURE(stein, double, 3 * n * kz + kz + 64);
         if (!ensure_digit_scratch(h, h->n, kz)) return set_error(h, ELSI_ERR_NOMEM, "cannot allocate the digit planes");
     }
-    ENSURE(sync, unsigned, sync_words(h->n, (int)eb));
+    ENSURE(sync, unsigned, fp32 ? sync_words(h->n, (int)eb) : std::max(sync_words(h->n, (int)eb), q2_f64_sync_words(h->n)));
     ENSURE(status, int, ST_WORDS);
     if (h->precision == ELSI_PREC_FP32_REFINE) {
         const size_t k = refine_block(h->n, h->n_state);
@@ -205,7 +206,7 @@ static int solve_fp64(elsi_gb_handle_s *h, const SolveRequest &rq)
     CK(stein<double>(st, n, w.d, w.e, k, w.w, w.z, n, w.stein, w.status));
     CK(cudaEventRecord(w.ev[STAGE_Q2], st));
     // ---- step (4): Z <- Q2 Z
-    if (!one_stage) CK(apply_q2_f64(st, n, b, w.v2, w.tau2, k, w.z, n, w.status));
+    if (!one_stage) CK(apply_q2_f64(st, n, b, w.v2, w.tau2, k, w.z, n, w.status, w.sync, w.sync_cap / sizeof(unsigned)));
     CK(cudaEventRecord(w.ev[STAGE_Q1], st));
     // ---- step (5): Z <- Q1 Z (one-stage: Z <- Q Z)
     if (one_stage) CK(apply_q_onestage<double>(st, n, k, w.v1, w.t1, w.z, n, w.work));
