@@ -1,6 +1,6 @@
 // Back-transformation through Q2 (step (4) of the two-stage method, arXiv:1705.11191 sec. 3.1)
-// in binary64: Z <- Q2 Z, Q2 = prod over sweep blocks J (32 sweeps, ascending) of prod over
-// steps t (descending) of H(J,t) H(J+1,t) ... H(J+31,t); so the blocks are applied from the
+// in binary64: Z <- Q2 Z, Q2 = prod over sweep blocks J (16 sweeps, ascending) of prod over
+// steps t (descending) of H(J,t) H(J+1,t) ... H(J+15,t); so the blocks are applied from the
 // last to the first, t ascending, and inside a group the later sweep first.
 //
 // What bounds it: binary64 operations, a warp's instruction every 64 clocks on each of the 608
@@ -12,14 +12,19 @@
 //
 // Pipeline over the blocks. There are too few columns to fill the chip, so the unit of work of a
 // warp is (block, 32 / LPC columns): step t of block J ends above the rows of step t + 1 of block
-// J + 32, so block J runs one step behind block J + 32, in whatever warp that is. The rows go
-// through L2 (a step takes 14 us or more, a hand-over about one); a progress word per unit says
+// J + 16, so block J runs one step behind block J + 16, in whatever warp that is. The rows go
+// through L2 (a step takes 7 us or more, a hand-over about one); a progress word per unit says
 // how many steps are stored. Units are handed out by a counter in the order of the blocks, so a
 // unit waits only for one that was handed out before it, whatever the number of warps that run.
 //
 // The b rows under a reflector stay in registers: row g is in slot g mod b, and from one reflector
 // to the next one row leaves and one enters in its slot, both loaded and stored in L2 directly.
 // The reflector is in shared memory in the order of the slots, loaded one ahead by the lanes together.
+//
+// Measured against eight lanes per column and a pipeline of eight blocks of 64 sweeps inside a CTA, its
+// rows in a ring in shared memory (b = 32): n = 5000, k = 668 97 -> 36 ms (two lanes; the 390 000
+// reflectors are 30 ms of the binary64 units); n = 1531, k = 381 5.7 -> 3.4 ms (four); n = 1000 2.7 ->
+// 1.6 ms and n = k = 512 0.91 -> 0.80 ms (eight). Blocks of 32 sweeps: 39, 4.1, 2.0 and 0.99 ms.
 #include "common.cuh"
 #include "kernels.h"
 #include "packets.cuh"
@@ -27,7 +32,7 @@
 namespace egb {
 namespace q2d {
 
-constexpr int kM = 32;      // sweeps per block
+constexpr int kM = 16;      // sweeps per block
 constexpr int kWarps = 4;   // warps per CTA, each with its own units
 
 // sync words: units handed out, a warp gave up, steps stored by each unit
@@ -191,7 +196,7 @@ cudaError_t launch(cudaStream_t st, const Args &a, int num_sms)
 }
 
 // Lanes per column, by the longer of two times in units of a warp instruction on one scheduler: all
-// reflectors of all columns over the 608 schedulers, and the chain through the blocks (n / 32
+// reflectors of all columns over the 608 schedulers, and the chain through the blocks (n / 16
 // blocks, a step apart, and the n / b steps of the last one).
 inline double cost(int n, int b, int k, int lpc)
 {
