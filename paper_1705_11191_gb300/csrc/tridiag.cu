@@ -5,7 +5,7 @@
 //    1967), a few threads per wanted eigenvalue index (multisection);
 //  * eigenvectors: one twisted factorisation T - lambda I = N_r D_r N_r^T per
 //    eigenvalue (Parlett & Dhillon 1997/2000), which gives the vector with residual
-//    O(eps ||T||) in O(n) work; one thread per vector;
+//    O(eps ||T||) in O(n) work;
 //  * vectors of eigenvalues closer than 1e-5 ||T|| are re-orthogonalised (two passes of
 //    Gram-Schmidt within the cluster, as in inverse-iteration codes), which bounds the
 //    loss of orthogonality between close vectors by about eps*1e5. A cluster is worked
@@ -40,32 +40,69 @@ __device__ __forceinline__ double guard_pivot(double q, double pivmin)
 // below that of pivmin 2^460 >= pivmin |p_i| (it always is for a zero). The pair (p_i, p_{i-1})
 // is rescaled by an exact power of two when |p_i| leaves [2^-200, 2^200], every 8 steps, which
 // keeps |p| below 2^460 for ||T|| up to 2^31.
+// A warp issues in order, so eight steps are one straight piece without a branch: the next d and
+// e^2 are on their way, the eight d_i - sigma do not wait for the chain, and a piece with a tiny
+// pivot (seen afterwards, from the smallest exponent) is done again step by step.
 // Measured against a form with a binary64 product and comparison for the pivot test, sign
 // comparisons and e^2 formed on the way (8 such operations a step, eigenvalues by 8 or 2 lanes
 // at every count), the bisection: n = 1531, 382 values 8.7 -> 4.1 ms; n = 4096, all 15.2 -> 7.1
-// ms; n = 16384, all 111 -> 65 ms; 8 solves of n = 2000 at a time 25 -> 10 ms each.
+// ms; n = 16384, all 111 -> 65 ms; 8 solves of n = 2000 at a time 25 -> 10 ms each; and then
+// with the straight pieces 2.2, 4.3, 38 and 7.4 ms.
+// e2[i] = e_{i-1}^2, e2[0] = 0.
 __device__ int sturm_count(int n, const double *__restrict__ d, const double *__restrict__ e2,
                            double sigma, double pivmin)
 {
+    constexpr int P = 8;
     const int tiny = (__double2hiint(pivmin) & 0x7FF00000) + (461 << 20);
-    double pm = 1.0;                                // p_{i-1}
-    double p = guard_pivot(d[0] - sigma, pivmin);   // p_1 = q_0
-    unsigned cnt = (unsigned)__double2hiint(p) >> 31;
-    int i = 1;
-    while (i < n) {
-        const int iend = min(n, i + 8);
-        for (; i < iend; ++i) {
-            double pn = fma(d[i] - sigma, p, -e2[i - 1] * pm);
+    double pm = 0.0, p = 1.0;  // p_{i-1}, p_i
+    unsigned cnt = 0;
+    auto steps = [&](int i0, int i1) {
+        for (int i = i0; i < i1; ++i) {
+            double pn = fma(d[i] - sigma, p, -e2[i] * pm);
             // pivot q = pn / p below pivmin in magnitude: q = -pivmin
             if ((__double2hiint(pn) & 0x7FF00000) <= tiny && fabs(pn) < pivmin * fabs(p)) pn = -pivmin * p;
             cnt += (unsigned)(__double2hiint(pn) ^ __double2hiint(p)) >> 31;
             pm = p;
             p = pn;
         }
+    };
+    const int whole = n / P * P;
+    double dn[P], en[P];
+    if (whole > 0) {
+#pragma unroll
+        for (int q = 0; q < P; ++q) { dn[q] = d[q]; en[q] = e2[q]; }
+    }
+    for (int i = 0; i < whole; i += P) {
+        double x[P], y[P];
+#pragma unroll
+        for (int q = 0; q < P; ++q) { x[q] = dn[q] - sigma; y[q] = en[q]; }
+        if (i + P < whole) {
+#pragma unroll
+            for (int q = 0; q < P; ++q) { dn[q] = d[i + P + q]; en[q] = e2[i + P + q]; }
+        }
+        const double p0 = p, pm0 = pm;
+        unsigned c = 0;
+        int least = 0x7FF00000;
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            const double pn = fma(x[q], p, -y[q] * pm);
+            least = min(least, __double2hiint(pn) & 0x7FF00000);
+            c += (unsigned)(__double2hiint(pn) ^ __double2hiint(p)) >> 31;
+            pm = p;
+            p = pn;
+        }
+        if (least <= tiny) {
+            p = p0;
+            pm = pm0;
+            steps(i, i + P);
+        } else {
+            cnt += c;
+        }
         const int ex = __double2hiint(p) & 0x7FF00000;
         if (ex > ((1023 + 200) << 20)) { p *= 0x1p-200; pm *= 0x1p-200; }
         else if (ex < ((1023 - 200) << 20)) { p *= 0x1p200; pm *= 0x1p200; }
     }
+    steps(whole, n);
     return (int)cnt;
 }
 
@@ -195,7 +232,7 @@ __global__ void bisect_kernel(int n, const double *__restrict__ d, const double 
 // changes no eigenvalue by more than 2 eps ||T|| and lets exactly degenerate eigenvalues
 // (e.g. those of a complex Hermitian matrix written as a real one) be found in
 // different blocks.
-// Also the forms of T that the counts read: e^2, and d and e^2 in binary32.
+// Also the forms of T that the counts read: e^2 (from index 1), and d and e^2 in binary32.
 __global__ void split_kernel(int n, const double *d, double *e, const double *bounds, double *e2, float *d32,
                              float *e232)
 {
@@ -205,9 +242,10 @@ __global__ void split_kernel(int n, const double *d, double *e, const double *bo
         if (i < n - 1) {
             double x = e[i];
             if (fabs(x) <= 2.0 * DBL_EPSILON * tn) e[i] = x = 0.0;
-            e2[i] = x * x;
+            e2[i + 1] = x * x;
             e232[i] = (float)x * (float)x;
         }
+        if (i == 0) e2[0] = 0.0;
     }
 }
 
@@ -306,93 +344,173 @@ __global__ void block_assign_kernel(int n, const double *d, const double *e, int
     blk[2 * l + 1] = be;
 }
 
-// One twisted factorisation of T_b - lam I on the block [bs, be): the pivots D+ (dplus)
-// and ratios L+ = e / D+ (lplus) of the forward factorisation, the ratios U- (uminus) of
-// the backward one, the twist index r = argmin |gamma_i| with gamma_r (signed), and
-// ||z||^2 of the vector z with z_r = 1 that solves (T_b - lam I) z = gamma_r e_r.
-// Arrays are indexed [i * kvec + l].
 // |a| < |b| on the bit patterns
 __device__ __forceinline__ bool mag_less(double a, double b)
 {
     return (__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFll) < (__double_as_longlong(b) & 0x7FFFFFFFFFFFFFFFll);
 }
 
-struct Twist {
-    int r;
-    double gamma, nrm2;
-};
-
-__device__ Twist twisted_factor(const double *__restrict__ d, const double *__restrict__ e,
-                                int bs, int be, double lam, double pivmin, int kvec, int l,
-                                double *dplus, double *lplus, double *uminus)
+// Twisted factorisation of T_b - lam I on the block [bs, be) of each eigenvalue lam = w[l], in two
+// kernels. The first one runs the two recurrences, a thread each: the pivots D+ (dplus) and ratios
+// L+ = e / D+ (lplus) of the forward factorisation, the ratios U- = e / D- (uminus) of the
+// backward one. Arrays are indexed [i * kvec + l].
+//
+// What bounds it: the recurrence, seven dependent binary64 operations a row (a reciprocal from the
+// hardware's approximation, L+, the pivot), each 64 clocks of a warp's unit; so the two directions go
+// to different warps, and everything that is not in the recurrence goes to the second kernel. There
+// 32 vectors belong to a CTA of eight warps: the search for the twist index r = argmin |gamma_i|,
+// gamma_i = D+_i + D-_i - (d_i - lam), is divided by rows (D- is formed again from U-, the same
+// operations); the products z_i = -L+_i z_{i+1} above r and z_{i+1} = -U-_i z_i below it (z_r = 1)
+// are two chains for two warps, whose lanes step through the rows together; then all warps scale by
+// 1 / ||z|| and transpose through shared memory into whole lines of z.
+// Measured against one thread per vector from the forward recurrence to the store of z, with the
+// loads of each row waited for: n = 1531, 381 vectors 2.2 -> 0.9 ms; n = 4096, all 9.3 -> 2.8 ms;
+// n = 16384, all 47 -> 19 ms.
+__global__ void __launch_bounds__(32)
+twist_factor_kernel(const double *__restrict__ d, const double *__restrict__ e, int kvec,
+                    const double *__restrict__ w, const double *bounds, const int *__restrict__ blk,
+                    double *dplus, double *lplus, double *uminus)
 {
-    double dp = guard_pivot(d[bs] - lam, pivmin);
-    dplus[(size_t)bs * kvec + l] = dp;
-    for (int i = bs; i < be - 1; ++i) {
-        const double lp = e[i] * recip(dp);
-        lplus[(size_t)i * kvec + l] = lp;
-        dp = d[i + 1] - lam - lp * e[i];
-        if (mag_less(dp, pivmin)) dp = -pivmin;
-        dplus[(size_t)(i + 1) * kvec + l] = dp;
+    const int l = blockIdx.x * 32 + threadIdx.x;
+    if (l >= kvec) return;
+    const double pivmin = bounds[2], lam = w[l];
+    const int bs = blk[2 * l], be = blk[2 * l + 1];  // the eigenvalue's block [bs, be)
+    if (blockIdx.y == 0) {
+        double dp = guard_pivot(d[bs] - lam, pivmin);
+        dplus[(size_t)bs * kvec + l] = dp;
+        double en = 0.0, dn = 0.0;  // read one row ahead
+        if (bs + 1 < be) { en = e[bs]; dn = d[bs + 1]; }
+        for (int i = bs; i < be - 1; ++i) {
+            const double ei = en, dl = dn - lam;
+            if (i + 2 < be) { en = e[i + 1]; dn = d[i + 2]; }
+            const double lp = ei * recip(dp);
+            lplus[(size_t)i * kvec + l] = lp;
+            dp = fma(-lp, ei, dl);
+            if (mag_less(dp, pivmin)) dp = -pivmin;
+            dplus[(size_t)(i + 1) * kvec + l] = dp;
+        }
+    } else {
+        double dm = guard_pivot(d[be - 1] - lam, pivmin);
+        double en = 0.0, dn = 0.0;
+        if (bs + 1 < be) { en = e[be - 2]; dn = d[be - 2]; }
+        for (int i = be - 2; i >= bs; --i) {
+            const double ei = en, dl = dn - lam;
+            if (i > bs) { en = e[i - 1]; dn = d[i - 1]; }
+            const double um = ei * recip(dm);
+            uminus[(size_t)i * kvec + l] = um;
+            dm = fma(-um, ei, dl);
+            if (mag_less(dm, pivmin)) dm = -pivmin;
+        }
     }
-    double dm = guard_pivot(d[be - 1] - lam, pivmin);
-    Twist t;
-    t.gamma = dplus[(size_t)(be - 1) * kvec + l] + dm - (d[be - 1] - lam);
-    t.r = be - 1;
-    double best = fabs(t.gamma);
-    for (int i = be - 2; i >= bs; --i) {
-        const double um = e[i] * recip(dm), dl = d[i] - lam;
-        uminus[(size_t)i * kvec + l] = um;
-        dm = dl - um * e[i];
-        if (mag_less(dm, pivmin)) dm = -pivmin;
-        const double g = dplus[(size_t)i * kvec + l] + dm - dl;
-        if (mag_less(g, best)) { best = fabs(g); t.gamma = g; t.r = i; }
-    }
-    double nrm2 = 1.0, zi = 1.0;
-    for (int i = t.r - 1; i >= bs; --i) {
-        zi = -lplus[(size_t)i * kvec + l] * zi;
-        nrm2 += zi * zi;
-    }
-    zi = 1.0;
-    for (int i = t.r; i < be - 1; ++i) {
-        zi = -uminus[(size_t)i * kvec + l] * zi;
-        nrm2 += zi * zi;
-    }
-    t.nrm2 = nrm2;
-    return t;
 }
 
-// Twisted factorisation eigenvector for each of the first kvec eigenvalues (w[l] is the
-// eigenvalue of index l, zero outside its block).
+constexpr int kTwistWarps = 8, kTwistRows = 16;
+
+// z / ||z|| for each of the first kvec eigenvalues (zero outside its block), from the factors;
+// lplus and uminus are overwritten by z.
 template <typename T>
-__global__ void twisted_kernel(int n, const double *__restrict__ d, const double *__restrict__ e,
-                               int kvec, const double *__restrict__ w, const double *bounds,
-                               const int *__restrict__ blk, T *z, int ldz, double *dplus,
-                               double *uminus, double *lplus, int *status)
+__global__ void __launch_bounds__(32 * kTwistWarps)
+twist_vector_kernel(int n, const double *__restrict__ d, const double *__restrict__ e, int kvec,
+                    const double *__restrict__ w, const double *bounds, const int *__restrict__ blk,
+                    const double *__restrict__ dplus, double *lplus, double *uminus, T *z, int ldz, int *status)
 {
-    int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= kvec) return;
-    const double pivmin = bounds[2];
-    const int bs = blk[2 * l], be = blk[2 * l + 1];  // the eigenvalue's block [bs, be)
-    const Twist t = twisted_factor(d, e, bs, be, w[l], pivmin, kvec, l, dplus, lplus, uminus);
-    const double nrm2 = t.nrm2;
-    const int r = t.r;
-    if (!(nrm2 < DBL_MAX)) { report_error(status, ELSI_ERR_NO_CONVERGENCE, l); }
-    const double s = (nrm2 < DBL_MAX) ? 1.0 / sqrt(nrm2) : 1.0;
-    // write z / ||z|| (zero outside the block)
-    T *zc = z + (size_t)l * ldz;
-    for (int i = 0; i < bs; ++i) zc[i] = T(0);
-    for (int i = be; i < n; ++i) zc[i] = T(0);
-    zc[r] = (T)s;
-    double zi = 1.0;
-    for (int i = r - 1; i >= bs; --i) {
-        zi = -lplus[(size_t)i * kvec + l] * zi;
-        zc[i] = (T)(zi * s);
+    __shared__ T tile[kTwistWarps][32][kTwistRows + 1];
+    __shared__ double best_w[kTwistWarps][32], nrm_w[2][32];
+    __shared__ int r_w[kTwistWarps][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int l = blockIdx.x * 32 + lane;
+    const bool have = l < kvec;
+    const double pivmin = bounds[2], lam = have ? w[l] : 0.0;
+    const int bs = have ? blk[2 * l] : 0, be = have ? blk[2 * l + 1] : 0;
+    // ---- twist index: the last row of the smallest |gamma|
+    double best = __longlong_as_double(0x7FFFFFFFFFFFFFFFll);
+    int r = be - 1;
+    const int per = (n + kTwistWarps - 1) / kTwistWarps;
+    const int lo = min(n, warp * per), hi = min(n, lo + per);
+#pragma unroll 4
+    for (int i = hi - 1; i >= lo; --i) {
+        if (i < bs || i >= be) continue;
+        const double dl = d[i] - lam;
+        double dm = dl;
+        if (i < be - 1) dm = fma(-uminus[(size_t)i * kvec + l], e[i], dl);
+        if (mag_less(dm, pivmin)) dm = -pivmin;
+        const double g = dplus[(size_t)i * kvec + l] + dm - dl;
+        if (mag_less(g, best)) { best = g; r = i; }
     }
-    zi = 1.0;
-    for (int i = r; i < be - 1; ++i) {
-        zi = -uminus[(size_t)i * kvec + l] * zi;
-        zc[i + 1] = (T)(zi * s);
+    best_w[warp][lane] = best;
+    r_w[warp][lane] = r;
+    __syncthreads();
+    best = best_w[kTwistWarps - 1][lane];
+    r = r_w[kTwistWarps - 1][lane];
+#pragma unroll
+    for (int q = kTwistWarps - 2; q >= 0; --q)
+        if (mag_less(best_w[q][lane], best)) { best = best_w[q][lane]; r = r_w[q][lane]; }
+    // ---- the two chains of products
+    constexpr int P = 8;
+    if (warp == 0) {
+        const int top = __reduce_max_sync(0xffffffffu, r), bot = __reduce_min_sync(0xffffffffu, have ? bs : n);
+        double zi = 1.0, s = 0.0;
+        for (int i0 = top - 1; i0 >= bot; i0 -= P) {
+            double f[P];
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const int i = i0 - q;
+                f[q] = i >= bs && i < r ? lplus[(size_t)i * kvec + l] : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const int i = i0 - q;
+                if (i >= bs && i < r) {
+                    zi = -f[q] * zi;
+                    s = fma(zi, zi, s);
+                    lplus[(size_t)i * kvec + l] = zi;
+                }
+            }
+        }
+        nrm_w[0][lane] = s;
+    } else if (warp == 1) {
+        const int first = __reduce_min_sync(0xffffffffu, have ? r : n), last = __reduce_max_sync(0xffffffffu, be);
+        double zi = 1.0, s = 0.0;
+        for (int i0 = first; i0 < last - 1; i0 += P) {
+            double f[P];
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const int i = i0 + q;
+                f[q] = i >= r && i < be - 1 ? uminus[(size_t)i * kvec + l] : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const int i = i0 + q;
+                if (i >= r && i < be - 1) {
+                    zi = -f[q] * zi;
+                    s = fma(zi, zi, s);
+                    uminus[(size_t)i * kvec + l] = zi;
+                }
+            }
+        }
+        nrm_w[1][lane] = s;
+    }
+    __syncthreads();
+    const double nrm2 = 1.0 + nrm_w[0][lane] + nrm_w[1][lane];
+    if (warp == 0 && have && !(nrm2 < DBL_MAX)) report_error(status, ELSI_ERR_NO_CONVERGENCE, l);
+    const double s = (nrm2 < DBL_MAX) ? 1.0 / sqrt(nrm2) : 1.0;
+    // ---- scaled into the columns of z
+    for (int i0 = warp * kTwistRows; i0 < n; i0 += kTwistWarps * kTwistRows) {
+#pragma unroll
+        for (int q = 0; q < kTwistRows; ++q) {
+            const int i = i0 + q;
+            double x = 0.0;
+            if (i >= bs && i < be)
+                x = i < r ? lplus[(size_t)i * kvec + l] : i > r ? uminus[(size_t)(i - 1) * kvec + l] : 1.0;
+            tile[warp][lane][q] = (T)(x * s);
+        }
+        __syncwarp();
+        const int q = lane % kTwistRows;
+#pragma unroll
+        for (int c = lane / kTwistRows; c < 32; c += 32 / kTwistRows)
+            if (blockIdx.x * 32 + c < kvec && i0 + q < n)
+                z[(size_t)(blockIdx.x * 32 + c) * ldz + i0 + q] = tile[warp][c][q];
+        __syncwarp();
     }
 }
 
@@ -562,8 +680,10 @@ cudaError_t stein(cudaStream_t st, int n, const double *d, const double *e, int 
     EGB_COUNT_LAUNCH();
     block_assign_kernel<<<ceil_div(kvec, 64), 64, 0, st>>>(n, d, e, kvec, w, bounds, blk);
     EGB_COUNT_LAUNCH();
-    twisted_kernel<T><<<ceil_div(kvec, 64), 64, 0, st>>>(n, d, e, kvec, w, bounds, blk, z, ldz, dplus,
-                                                        uminus, lplus, status);
+    twist_factor_kernel<<<dim3(ceil_div(kvec, 32), 2), 32, 0, st>>>(d, e, kvec, w, bounds, blk, dplus, lplus, uminus);
+    EGB_COUNT_LAUNCH();
+    twist_vector_kernel<T><<<ceil_div(kvec, 32), 32 * kTwistWarps, 0, st>>>(n, d, e, kvec, w, bounds, blk, dplus, lplus,
+                                                                           uminus, z, ldz, status);
     // cluster starts (in the L+ scratch, no longer needed), then pieces and seams
     int *cstart = reinterpret_cast<int *>(lplus);
     EGB_COUNT_LAUNCH();
