@@ -5,19 +5,24 @@
 // term is below binary32 rounding). This is the binary32 GEMM of the reduction and the
 // back-transformations of the binary32 route.
 //
-// Structure of one CTA (320 threads; persistent over 128 x 128 tiles of C):
+// Structure of one CTA (576 threads; persistent over 128 x 128 tiles of C):
 //   warp 0, one lane : TMA producer. Loads the K-major hi and lo tiles of A and B (32 fp32 of
 //                      K = 128 bytes per row, 128-byte swizzle) into a 3-stage ring, one
 //                      mbarrier per stage with the transaction byte count;
 //   warp 1, one lane : MMA issuer. tcgen05.mma kind::tf32, M = 128, N = 128, K = 8 per
 //                      instruction, accumulator in tensor memory (128 lanes x 128 columns);
 //                      tcgen05.commit frees a stage when its MMAs have read it;
-//   warps 2-9        : epilogue: warp w owns rows 32 (w mod 4) .. + 31 and columns
-//                      64 h .. 64 h + 63 (h = (w - 2) / 4) of the tile. It sums the K
-//                      chunks of the two tensor-memory accumulators (tcgen05.ld) in
-//                      registers, then loads its part of C (beta != 0; 32 columns in flight
-//                      at once) and writes C = alpha acc + beta C with coalesced
-//                      column-major stores; warp 2 allocates and frees the tensor memory.
+//   warps 2-17       : epilogue: warp w owns rows 32 (w mod 4) .. + 31 and columns
+//                      32 h .. 32 h + 31 (h = (w - 2) / 4) of the tile. It loads its part of C
+//                      (beta != 0), sums the K chunks of the two tensor-memory accumulators
+//                      (tcgen05.ld) in registers and writes C = alpha acc + beta C with
+//                      coalesced column-major stores; warp 2 allocates and frees the tensor
+//                      memory.
+// What bounds it: the planes, 64 KB per 128 x 128 x 32 products from L2 (0.7 us an SM, 14 TB/s in
+// all, against 0.5 us of products; 220 TFLOP/s useful at K = 8192), and at K = 64 .. 256 (full to
+// band, Q1, the triangular solves) C, read and written once per tile. With 8 epilogue warps that
+// asked for C after the products: 4096 x 4096 with K = 64 36 -> 29 us, K = 256 71 -> 64 us;
+// 16384 x 16384, K = 256 907 -> 929 us.
 // Every wait is bounded; on expiry the kernel records ELSI_ERR_TIMEOUT and finishes without
 // further waits on the pipeline (after a bounded wait for its own TMA copies in flight).
 #include <cuda.h>
@@ -39,7 +44,7 @@ constexpr int TILE_BYTES = BM * BK * 4;  // 16 KB (BN == BM)
 constexpr int STAGE_BYTES = 4 * TILE_BYTES;  // A_hi, A_lo, B_hi, B_lo
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
 constexpr int TMEM_COLS = 4 * BN;  // two buffers x (hi*hi sum, cross-term sum)
-constexpr int EPI_WARPS = 8, CW = BN / 2;  // epilogue warps; columns per epilogue warp
+constexpr int EPI_WARPS = 16, CW = BN / 4;  // epilogue warps; columns per epilogue warp
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
 
 __device__ __forceinline__ void mma_tf32(unsigned tmem_d, unsigned long long a, unsigned long long b,
@@ -57,7 +62,7 @@ struct Maps {
 };
 
 
-// Warps: 0 = TMA producer (one lane), 1 = MMA issuer (one lane), 2..9 = epilogue (warp w
+// Warps: 0 = TMA producer (one lane), 1 = MMA issuer (one lane), 2..17 = epilogue (warp w
 // reads tensor-memory lanes 32 (w mod 4) .. + 31, i.e. those rows of the tile). K is
 // accumulated in chunks of CH k-tiles in one of two tensor-memory buffers, each holding the
 // hi*hi sum and the (2^-11 times smaller) cross-term sum separately; the epilogue warps add
@@ -157,13 +162,13 @@ gemm_tf32x3_kernel(const __grid_constant__ Maps maps, int m, int n, int kp, floa
                     const int s = ktg % STAGES, g = gbase + kt / CH, bsel = g & 1;
                     const unsigned ph = (ktg / STAGES) & 1;
                     const bool first = (kt % CH) == 0;
-                    if (first && g >= 2 && !mbar_wait(acce0 + 8 * bsel, ((g >> 1) - 1) & 1)) {
+                    if (first && g >= 2 && !mbar_wait_hot(acce0 + 8 * bsel, ((g >> 1) - 1) & 1)) {
                         report_error(status, ELSI_ERR_TIMEOUT, 4);
                         atomicExch(&aborted, 1);
                         stop = true;
                         break;
                     }
-                    if (!mbar_wait(full0 + 8 * s, ph)) {
+                    if (!mbar_wait_hot(full0 + 8 * s, ph)) {
                         report_error(status, ELSI_ERR_TIMEOUT, 2);
                         atomicExch(&aborted, 1);
                         stop = true;
@@ -200,10 +205,15 @@ gemm_tf32x3_kernel(const __grid_constant__ Maps maps, int m, int n, int kp, floa
             if (!tile_of(t, tiles_m, uplo, &m0, &n0)) continue;
             const int row = m0 + quarter * 32 + lane;
             const bool row_in = row < m;
-            float *crow = C + (size_t)row;
-            float acc[CW];
+            float *cp = C + (size_t)row + (size_t)(n0 + c0) * ldc;
+            auto in = [&](int j) { return row_in && n0 + c0 + j < n && (!uplo || row >= n0 + c0 + j); };
+            // C is on its way while the products run (one 128-byte line per column and warp)
+            float acc[CW], cv[CW];
 #pragma unroll
-            for (int j = 0; j < CW; ++j) acc[j] = 0.0f;
+            for (int j = 0; j < CW; ++j) {
+                acc[j] = 0.0f;
+                cv[j] = (beta != 0.0f && in(j)) ? cp[(size_t)j * ldc] : 0.0f;
+            }
             for (int c = 0; c < nchunk && ok; ++c) {
                 const int g = gbase + c, bsel = g & 1;
                 ok = __all_sync(0xffffffffu, mbar_wait(accf0 + 8 * bsel, (g >> 1) & 1));
@@ -216,42 +226,26 @@ gemm_tf32x3_kernel(const __grid_constant__ Maps maps, int m, int n, int kp, floa
                 }
                 tc_fence_after();
 #pragma unroll
-                for (int q = 0; q < CW / 32; ++q) {
-                    float v[32];
+                for (int q = 0; q < CW / 16; ++q) {
+                    float v[16];
                     const unsigned ta =
-                        tmem + ((unsigned)(quarter * 32) << 16) + bsel * 2 * BN + c0 + q * 32;
-                    tmem_ld32(ta + BN, v);  // cross terms
+                        tmem + ((unsigned)(quarter * 32) << 16) + bsel * 2 * BN + c0 + q * 16;
+                    tmem_ld16(ta + BN, v);  // cross terms
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) acc[q * 32 + j] += v[j];
-                    tmem_ld32(ta, v);  // hi * hi
+                    for (int j = 0; j < 16; ++j) acc[q * 16 + j] += v[j];
+                    tmem_ld16(ta, v);  // hi * hi
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) acc[q * 32 + j] += v[j];
+                    for (int j = 0; j < 16; ++j) acc[q * 16 + j] += v[j];
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(acce0 + 8 * bsel);
             }
             gbase += nchunk;
-            if (ok && row_in) {
-                // 32 loads of C at a time (one 128-byte line per column and warp, 32 KB in
-                // flight per CTA), then their stores
+            if (ok) {
 #pragma unroll
-                for (int h = 0; h < CW / 32; ++h) {
-                    float cv[32];
-                    float *cp = crow + (size_t)(n0 + c0 + h * 32) * ldc;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int col = n0 + c0 + h * 32 + j;
-                        const bool in = col < n && (!uplo || row >= col);
-                        cv[j] = (beta != 0.0f && in) ? cp[(size_t)j * ldc] : 0.0f;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int col = n0 + c0 + h * 32 + j;
-                        if (col < n && (!uplo || row >= col))
-                            cp[(size_t)j * ldc] = alpha * acc[h * 32 + j] + beta * cv[j];
-                    }
-                }
+                for (int j = 0; j < CW; ++j)
+                    if (in(j)) cp[(size_t)j * ldc] = alpha * acc[j] + beta * cv[j];
             }
         }
     }
@@ -268,41 +262,81 @@ gemm_tf32x3_kernel(const __grid_constant__ Maps maps, int m, int n, int kp, floa
                      : "memory");
 }
 
+__device__ __forceinline__ void split_tf32(float x, float &hi, float &lo)
+{
+    unsigned h, l;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(h) : "f"(x));
+    hi = __uint_as_float(h & 0xFFFFE000u);
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(l) : "f"(x - hi));
+    lo = __uint_as_float(l & 0xFFFFE000u);
+}
+
 // Columns [q_off, q_off + kw) of the rows x kp plane (K-major) of hi / lo TF32 parts of the
 // operand piece element (r, q) = src[r * sr + q * sq] (one of sr, sq is 1), q < k, zero for
-// k <= q < kw. 32 x 32 tiles through shared memory so that reads and writes coalesce.
-__global__ void split_planes_kernel(int rows, int k, int kw, int kp, int q_off,
-                                    const float *__restrict__ src, long long sr, long long sq,
-                                    float *__restrict__ hi, float *__restrict__ lo)
+// k <= q < kw. Bound by memory (4 bytes read, 8 written): four 16-byte loads a thread in flight.
+// sq = 1: 32 rows x 128 q straight from registers; sr = 1: 128 rows x 32 q transposed in shared
+// memory. vec: src and the other stride are multiples of 16 bytes.
+// Against 32 x 32 tiles with one 4-byte load at a time: 16384 x 16384 along K 860 -> 460 us (3.2 GB),
+// 16384 x 256 across 15 -> 8 us.
+constexpr int kSplitLong = 128, kSplitShort = 32;
+__global__ void __launch_bounds__(256)
+split_planes_kernel(int rows, int k, int kw, int kp, int q_off, const float *__restrict__ src, long long sr,
+                    long long sq, int vec, float *__restrict__ hi, float *__restrict__ lo)
 {
-    __shared__ float t[32][33];
-    const int r0 = blockIdx.y * 32, q0 = blockIdx.x * 32;
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+    auto put = [&](int r, int q, const float (&x)[4]) {  // q < kw, a multiple of 4
+        float4 h, l;
+        split_tf32(x[0], h.x, l.x);
+        split_tf32(x[1], h.y, l.y);
+        split_tf32(x[2], h.z, l.z);
+        split_tf32(x[3], h.w, l.w);
+        const size_t o = (size_t)r * kp + q_off + q;
+        *reinterpret_cast<float4 *>(hi + o) = h;
+        *reinterpret_cast<float4 *>(lo + o) = l;
+    };
+    // four consecutive elements from p, those before cnt
+    auto get = [&](const float *p, int cnt, float (&x)[4]) {
+        if (vec && cnt >= 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(p);
+            x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) x[c] = c < cnt ? p[c] : 0.0f;
+        }
+    };
     if (sq == 1) {
-        for (int i = ty; i < 32; i += 8) {
-            const int r = r0 + i, q = q0 + tx;
-            t[i][tx] = (r < rows && q < k) ? src[r * sr + q] : 0.0f;
+        const int q = blockIdx.x * kSplitLong + 4 * tx;
+        float x[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = blockIdx.y * kSplitShort + ty + 8 * i;
+            get(src + (long long)r * sr + q, r < rows ? k - q : 0, x[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = blockIdx.y * kSplitShort + ty + 8 * i;
+            if (r < rows && q < kw) put(r, q, x[i]);
         }
     } else {
-        for (int i = ty; i < 32; i += 8) {
-            const int q = q0 + i, r = r0 + tx;
-            t[tx][i] = (r < rows && q < k) ? src[r + q * sq] : 0.0f;
+        __shared__ float t[kSplitShort][kSplitLong + 1];  // [q][r]
+        const int r = blockIdx.y * kSplitLong + 4 * tx;
+        float x[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int q = blockIdx.x * kSplitShort + ty + 8 * i;
+            get(src + (long long)q * sq + r, q < k ? rows - r : 0, x[i]);
         }
-    }
-    __syncthreads();
-    for (int i = ty; i < 32; i += 8) {
-        const int r = r0 + i, q = q0 + tx;
-        if (r < rows && q < kw) {
-            const float x = t[i][tx];
-            unsigned h;
-            asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(h) : "f"(x));
-            h &= 0xFFFFE000u;
-            const float xh = __uint_as_float(h);
-            unsigned l;
-            asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(l) : "f"(x - xh));
-            l &= 0xFFFFE000u;
-            hi[(size_t)r * kp + q_off + q] = xh;
-            lo[(size_t)r * kp + q_off + q] = __uint_as_float(l);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) t[ty + 8 * i][4 * tx + c] = x[i][c];
+        __syncthreads();
+        const int ql = 4 * (tx & 7);  // eight lanes a row
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int rl = (tx >> 3) + 4 * (ty + 8 * i), rr = blockIdx.y * kSplitLong + rl;
+            const float y[4] = {t[ql][rl], t[ql + 1][rl], t[ql + 2][rl], t[ql + 3][rl]};
+            if (rr < rows) put(rr, blockIdx.x * kSplitShort + ql, y);
         }
     }
 }
@@ -336,21 +370,21 @@ cudaError_t tc_gemm_f32_parts(cudaStream_t st, int m, int n, int nparts, const T
     if (kp <= 0 || work_elems < 2 * ((size_t)m + n) * kp + 64 || ((size_t)work & 15))
         return cudaErrorNotSupported;
     float *ahi = work, *alo = ahi + (size_t)m * kp, *bhi = alo + (size_t)m * kp, *blo = bhi + (size_t)n * kp;
-    dim3 tb32(32, 8);
+    // rows x kw of a plane from src[r * sr + q * sq]
+    auto split = [&](int rows, int k, int off, const float *src, long long sr, long long sq, float *hi, float *lo) {
+        const int kw = kround(k), vec = ((size_t)src & 15) == 0 && (sr == 1 ? sq : sr) % 4 == 0;
+        const dim3 grid = sq == 1 ? dim3(ceil_div(kw, kSplitLong), ceil_div(rows, kSplitShort))
+                                  : dim3(ceil_div(kw, kSplitShort), ceil_div(rows, kSplitLong));
+        EGB_COUNT_LAUNCH();
+        split_planes_kernel<<<grid, dim3(32, 8), 0, st>>>(rows, k, kw, kp, off, src, sr, sq, vec, hi, lo);
+    };
     int off = 0;
     for (int i = 0; i < nparts; ++i) {
-        const int kw = kround(a[i].k);
         // op(A) element (i, q): trans = 0 -> A[i + q ld]; trans = 1 -> A[q + i ld]
-        EGB_COUNT_LAUNCH();
-        split_planes_kernel<<<dim3(kw / 32, (m + 31) / 32), tb32, 0, st>>>(
-            m, a[i].k, kw, kp, off, a[i].p, a[i].trans ? (long long)a[i].ld : 1,
-            a[i].trans ? 1 : (long long)a[i].ld, ahi, alo);
+        split(m, a[i].k, off, a[i].p, a[i].trans ? (long long)a[i].ld : 1, a[i].trans ? 1 : (long long)a[i].ld, ahi, alo);
         // op(B) element (q, j) is plane row j: trans = 0 -> B[q + j ld]; trans = 1 -> B[j + q ld]
-        EGB_COUNT_LAUNCH();
-        split_planes_kernel<<<dim3(kw / 32, (n + 31) / 32), tb32, 0, st>>>(
-            n, b[i].k, kw, kp, off, b[i].p, b[i].trans ? 1 : (long long)b[i].ld,
-            b[i].trans ? (long long)b[i].ld : 1, bhi, blo);
-        off += kw;
+        split(n, b[i].k, off, b[i].p, b[i].trans ? 1 : (long long)b[i].ld, b[i].trans ? (long long)b[i].ld : 1, bhi, blo);
+        off += kround(a[i].k);
     }
     Maps maps;
     if (!make_map(&maps.a_hi, ahi, m, kp) || !make_map(&maps.a_lo, alo, m, kp) ||
