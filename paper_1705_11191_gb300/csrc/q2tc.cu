@@ -28,6 +28,11 @@
 // each group's products start from fresh accumulators, so tensor-memory accumulation never
 // sums more than 3 x K/8 partial products into one value.
 //
+// Rows enter and leave the window through shared memory (two buffers of 64 rows x 128 columns, 16-byte
+// pieces permuted within 128 bytes): a thread owns a column there, and lanes along a column make
+// whole lines in memory. A thread that read its own column from L2 and stored it back took 32
+// lines an instruction (and 32 loads where a column starts unaligned).
+//
 // CTA (512 threads, 16 warps, one CTA per SM): 128 columns of Z; warp w owns the columns
 // 32 (w mod 4) .. +31 (one per lane, the tensor-memory lane quarter of the warp) and the
 // window slots 32 (w / 4) .. +31 of them, in registers. The A operands (Z_w^T, then Y^T,
@@ -42,10 +47,14 @@
 // Pipeline over the blocks. A group is a chain of two products, so what bounds a CTA is the
 // latency of a group (6.3 us), and there is one CTA per 128 columns: at n = 4096 32 of 152 SMs.
 // The unit of work is therefore (block, 128 columns): rows of block J are final for it when block
-// J + 64 has passed them, so block J runs ceil(64 / b) + 1 steps behind block J + 64, on another SM.
+// J + 64 has passed them, so block J runs ceil(64 / b) + 2 steps behind block J + 64, on another SM.
 // The rows go through L2; a progress word per unit says how many steps are stored. Units are
 // handed out by a counter in the order of the blocks, so a unit waits only for one that was
 // handed out before it, whatever the number of CTAs that run at a time.
+// Measured (all n columns, b = 64), one CTA per 128 columns -> units -> rows through shared memory:
+// n = 777 0.80 -> 0.54 -> 0.44 ms, n = 2000 3.2 -> 0.76 -> 0.81, n = 4096 12.4 -> 3.1 -> 3.0,
+// n = 16384 211 -> 187 -> 182. There all SMs are busy and a group is 6.6 us: 1.9 us of products, the rest
+// the hand-overs between tensor memory, registers and the five barriers of a group.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -68,7 +77,8 @@ constexpr int kVPlane = kWin * kM * 4;  // bytes of one plane of V: 4 K-chunks o
 constexpr int kWPlane = kWin * kM * 4;  // bytes of one plane of W: 2 K-chunks of [128 rows][32 a]
 constexpr int kGroupBytes = 2 * kVPlane + 2 * kWPlane;  // VH | VL | WH | WL = 128 KB
 constexpr int kGroupFloats = kGroupBytes / 4;
-constexpr int kSmemBytes = kGroupBytes + 1024 + 128;
+constexpr int kZBytes = kCols * kM * 4;  // rows that enter or leave the window in a step
+constexpr int kSmemBytes = kGroupBytes + 2 * kZBytes + 1024 + 128;
 constexpr unsigned kTmemCols = 512;
 // tensor-memory columns
 constexpr unsigned kZH = 0, kZL = 128;      // Z_w^T (A of MMA 1), later Y^T (A of MMA 2)
@@ -292,7 +302,7 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((size_t)smem_raw + 1023) & ~(size_t)1023);
-    unsigned long long *bars = (unsigned long long *)(smem + kGroupBytes);
+    unsigned long long *bars = (unsigned long long *)(smem + kGroupBytes + 2 * kZBytes);
     unsigned *tmem_slot = (unsigned *)(bars + 4);
     __shared__ int abort_flag, unit_next;
     const unsigned bar_v = smem_u32(&bars[0]), bar_w = smem_u32(&bars[1]);
@@ -348,7 +358,16 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
     }
 
     float zr[kSlots];   // slots kSlots * part + i of this thread's column
-    float pre[kSlots];  // rows entering the window after the current group
+    constexpr int kIn = kCols * kM / kThreads;
+    float in[kIn];      // part of the rows entering the window after the current group
+    // byte offset of row r of column c in a buffer of entering / leaving rows
+    auto zoff = [](int c, int r) { return c * (kM * 4) + ((((r >> 2) ^ (c & 7))) << 4) + ((r & 3) << 2); };
+    // piece i of a thread in whole lines: vec 4 rows of a column, else one
+    auto piece = [&](int i, int &c, int &r) {
+        const int e = tid + i * kThreads;
+        if (vec) { c = e >> 4; r = (e & 15) * 4; }
+        else { c = e >> 6; r = e & 63; }
+    };
     const unsigned idesc1 = idesc_f32acc(2, 128, 64);
     const unsigned idesc2 = idesc_f32acc(2, 128, 128);
     bool ok = true;
@@ -357,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
         const int jb = a.jb_hi - 1 - unit / ncg;
         const int J = jb * kM;
         const int SJ = block_steps(n, b, J);
-        const int gc = unit % ncg * kCols + quarter * 32 + lane;  // column of Z
+        const int c0 = unit % ncg * kCols, gc = c0 + quarter * 32 + lane;  // first column, this thread's
         const bool colok = gc < a.k;
         float *zc = a.z + (size_t)(colok ? gc : 0) * (size_t)a.ldz;
         unsigned *mine = a.sync + kSyncHead + unit;
@@ -393,12 +412,33 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
         for (int t = 0; t < SJ; ++t) {
             const int w0 = J + t * b;
             const bool last = t + 1 == SJ;
+            unsigned char *zbuf = smem + kGroupBytes + (t & 1) * kZBytes;
             // prefetch the rows that replace the ones leaving after this group
             if (!last) {
+                if (vec) {
 #pragma unroll
-                for (int c = 0; c < kChunks; ++c) {
-                    const int p = (part * kSlots + c * 8 - w0) & (kWin - 1);
-                    if (p < b) load8(zc, w0 + p + kWin, n, colok, vec, pre + c * 8);
+                    for (int i = 0; i < kIn / 4; ++i) {
+                        int c, r;
+                        piece(i, c, r);
+                        const bool ok4 = c0 + c < a.k && r < b;
+                        const float *src = a.z + (size_t)(ok4 ? c0 + c : 0) * (size_t)a.ldz;
+                        const int row = w0 + kWin + r;
+                        if (ok4 && row + 4 <= n) {
+                            const float4 x = __ldcg(reinterpret_cast<const float4 *>(src + row));
+                            in[4 * i] = x.x; in[4 * i + 1] = x.y; in[4 * i + 2] = x.z; in[4 * i + 3] = x.w;
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) in[4 * i + q] = ok4 && row + q < n ? __ldcg(src + row + q) : 0.f;
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kIn; ++i) {
+                        int c, r;
+                        piece(i, c, r);
+                        const int row = w0 + kWin + r;
+                        in[i] = c0 + c < a.k && r < b && row < n ? __ldcg(a.z + (size_t)(c0 + c) * (size_t)a.ldz + row) : 0.f;
+                    }
                 }
             }
             // ---- A of MMA 1: Z_w^T (hi, lo) at logical window positions
@@ -417,9 +457,6 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
             tmem_wait_st();
             tc_fence_before();
             __syncthreads();
-            // the rows that the last step stored are visible to the block below (while MMA 1 runs)
-            if (tid == kWaiter && t > 0)
-                asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(mine), "r"((unsigned)t) : "memory");
             // ---- MMA 1: Y^T = Z_w^T V
             if (tid == 0) {
                 if (!mbar_wait(bar_v, gidx & 1)) {
@@ -446,6 +483,24 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
             }
             __syncthreads();
             if (abort_flag) { ok = false; break; }
+            // the rows that left after the last group, in whole lines (while MMA 1 runs)
+            if (t > 0) {
+                const unsigned char *zold = smem + kGroupBytes + ((t - 1) & 1) * kZBytes;
+#pragma unroll
+                for (int i = 0; i < (vec ? kIn / 4 : kIn); ++i) {
+                    int c, r;
+                    piece(i, c, r);
+                    const int row = w0 - b + r;
+                    if (c0 + c >= a.k || r >= b) continue;
+                    float *dst = a.z + (size_t)(c0 + c) * (size_t)a.ldz + row;
+                    if (vec && row + 4 <= n) {
+                        *reinterpret_cast<float4 *>(dst) = *reinterpret_cast<const float4 *>(zold + zoff(c, r));
+                    } else {
+                        for (int q = 0; q < (vec ? 4 : 1); ++q)
+                            if (row + q < n) dst[q] = *reinterpret_cast<const float *>(zold + zoff(c, r + q));
+                    }
+                }
+            }
             if (!mbar_wait(bar_m1, gidx & 1)) {
                 report_error(a.status, ELSI_ERR_TIMEOUT, 12);
                 abort_flag = 1;
@@ -487,6 +542,24 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
                     tmem_st8(tq + kZL + kA * part + 8 * g, lo);
                 }
             }
+            if (!last) {
+                if (vec) {
+#pragma unroll
+                    for (int i = 0; i < kIn / 4; ++i) {
+                        int c, r;
+                        piece(i, c, r);
+                        *reinterpret_cast<float4 *>(zbuf + zoff(c, r)) =
+                            make_float4(in[4 * i], in[4 * i + 1], in[4 * i + 2], in[4 * i + 3]);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kIn; ++i) {
+                        int c, r;
+                        piece(i, c, r);
+                        *reinterpret_cast<float *>(zbuf + zoff(c, r)) = in[i];
+                    }
+                }
+            }
             tmem_wait_st();
             tc_fence_before();
             __syncthreads();
@@ -516,6 +589,8 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
             }
             __syncthreads();
             if (abort_flag) { ok = false; break; }
+            if (tid == kWaiter && t > 0)  // the rows stored above are visible to the block below
+                asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(mine), "r"((unsigned)t) : "memory");
             if (tid == kWaiter && !last) wait_above(t + 2);  // rows that the next step prefetches, while MMA 2 runs
             const bool done2 = mbar_wait(bar_m2, gidx & 1);
             if (!done2) {
@@ -542,15 +617,20 @@ __global__ void __launch_bounds__(kThreads, 1) q2_apply_tc5_kernel(const ApplyAr
             }
             tc_fence_before();
             ++gidx;
-            // ---- rows leaving the window: store, and take the prefetched rows in their slots
+            // ---- rows leaving the window change places with the ones that enter in their slots
 #pragma unroll
             for (int c = 0; c < kChunks; ++c) {
                 const int p = (part * kSlots + c * 8 - w0) & (kWin - 1);
-                if (last || p < b) {
+                if (last) {
                     store8(zc, w0 + p, n, colok, vec, zr + c * 8);
-                    if (!last) {
+                } else if (p < b) {
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) zr[c * 8 + i] = pre[c * 8 + i];
+                    for (int h = 0; h < 2; ++h) {
+                        float4 *x = reinterpret_cast<float4 *>(zbuf + zoff(quarter * 32 + lane, p + 4 * h));
+                        float *zq = zr + c * 8 + 4 * h;
+                        const float4 y = *x;
+                        *x = make_float4(zq[0], zq[1], zq[2], zq[3]);
+                        zq[0] = y.x; zq[1] = y.y; zq[2] = y.z; zq[3] = y.w;
                     }
                 }
             }
@@ -652,9 +732,9 @@ cudaError_t apply_q2_tc(cudaStream_t st, int n, int b, const float *v2, const fl
             a.status = status; a.sync = sync; a.spin_limit = spin_limit();
             e = cudaMemsetAsync(sync, 0, (size_t)(kSyncHead + units) * sizeof(unsigned), st);
             if (e != cudaSuccess) return e;
-            // a block runs 1 + ceil(64 / b) steps behind the one above it: more CTAs than blocks that
+            // a block runs 2 + ceil(64 / b) steps behind the one above it: more CTAs than blocks that
             // can be under way at a time would only wait
-            const int deep = ceil_div(block_steps(n, b, lo * kM), 1 + ceil_div(kM, b));
+            const int deep = ceil_div(block_steps(n, b, lo * kM), 2 + ceil_div(kM, b));
             int grid = units < num_sms ? units : num_sms;
             if ((long long)deep * ncg < grid) grid = deep * ncg;
             EGB_COUNT_LAUNCH();
