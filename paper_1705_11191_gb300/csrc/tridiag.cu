@@ -514,25 +514,93 @@ twist_vector_kernel(int n, const double *__restrict__ d, const double *__restric
     }
 }
 
-// Gram-Schmidt of vector zv against the cluster vectors i0 .. v-1 (two passes); returns
-// the squared norm left.
+// Sums and updates of the Gram-Schmidt step with at least the precision of binary64 arithmetic
+// rounded to T. A binary32 product and a sum are kept as two binary32 numbers (products split by
+// an FMA, Knuth's two-sum: Ogita, Rump & Oishi 2005), a dozen operations of a unit that has 64
+// times the rate of the binary64 one; a conversion and an FMA there hold it for 128 clocks.
+template <typename T> struct Wide;
+template <> struct Wide<double> {
+    double v;
+    __device__ __forceinline__ explicit Wide(double x = 0.0) : v(x) {}
+    __device__ __forceinline__ void fma_(double a, double b) { v = fma(a, b, v); }
+    __device__ __forceinline__ void fms(double2 c, double b) { v = fma(-c.x, b, v); }
+    __device__ __forceinline__ double rounded() const { return v; }
+    __device__ __forceinline__ double value() const { return v; }
+    __device__ __forceinline__ static double2 coef(double s) { return make_double2(s, 0.0); }
+    using Coef = double2;
+};
+template <> struct Wide<float> {
+    float h, l;
+    __device__ __forceinline__ explicit Wide(float x = 0.f) : h(x), l(0.f) {}
+    __device__ __forceinline__ void add(float p, float e)
+    {
+        const float s = h + p, b = s - h;
+        l += ((h - (s - b)) + (p - b)) + e;
+        h = s;
+    }
+    __device__ __forceinline__ void fma_(float a, float b)
+    {
+        const float p = __fmul_rn(a, b);  // not contracted with the sum
+        add(p, fmaf(a, b, -p));
+    }
+    __device__ __forceinline__ void fms(float2 c, float b)  // minus (c.x + c.y) b
+    {
+        const float p = __fmul_rn(-c.x, b);
+        add(p, fmaf(-c.y, b, fmaf(-c.x, b, -p)));
+    }
+    __device__ __forceinline__ float rounded() const { return h + l; }
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+    __device__ __forceinline__ static float2 coef(double s)
+    {
+        const float h = (float)s;
+        return make_float2(h, (float)(s - (double)h));
+    }
+    using Coef = float2;
+};
+
+// Gram-Schmidt of vector zv against the cluster vectors i0 .. v-1 (two passes, each with all
+// products first: Giraud et al. 2005); returns the squared norm left. What bounds it: the rows of
+// the cluster, read from L2 twice a pass; a warp per product, so a pass has two barriers, where one
+// product and one update at a time by the whole CTA had three per vector.
+// Measured together with inverse_iteration below, both phases: n = 16384 39 -> 3.6 ms, eight solves of
+// n = 2000 at a time 49 -> 5.3 ms in all (of which this form 2 and 1).
+constexpr int kOrthPiece = 64;  // vectors orthogonalised together (pieces and seams)
+
 template <typename T>
 __device__ double cluster_project(int n, int i0, int v, T *z, int ldz, double *red)
 {
+    using W = Wide<T>;
+    __shared__ typename W::Coef coef[kOrthPiece];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     T *zv = z + (size_t)v * ldz;
     for (int pass = 0; pass < 2; ++pass) {
-        for (int u = i0; u < v; ++u) {
+        for (int u = i0 + warp; u < v; u += nw) {
             const T *zu = z + (size_t)u * ldz;
-            double s = 0.0;
-            for (int i = threadIdx.x; i < n; i += blockDim.x) s += (double)zu[i] * (double)zv[i];
-            s = block_sum(s, red);
-            for (int i = threadIdx.x; i < n; i += blockDim.x) zv[i] = (T)((double)zv[i] - s * (double)zu[i]);
-            __syncthreads();
+            W a, b;
+            int i = lane;
+            for (; i + 32 < n; i += 64) {
+                a.fma_(zu[i], zv[i]);
+                b.fma_(zu[i + 32], zv[i + 32]);
+            }
+            if (i < n) a.fma_(zu[i], zv[i]);
+            double s = a.value() + b.value();
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) coef[u - i0] = W::coef(s);
         }
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            W x(zv[i]);
+            const T *zu = z + (size_t)i0 * ldz + i;
+#pragma unroll 4
+            for (int u = 0; u < v - i0; ++u) x.fms(coef[u], zu[(size_t)u * ldz]);
+            zv[i] = x.rounded();
+        }
+        __syncthreads();
     }
-    double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += (double)zv[i] * (double)zv[i];
-    return block_sum(s, red);
+    W s;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) s.fma_(zv[i], zv[i]);
+    return block_sum(s.value(), red);
 }
 
 __device__ __forceinline__ double hash_unit(unsigned a, unsigned b)
@@ -541,8 +609,6 @@ __device__ __forceinline__ double hash_unit(unsigned a, unsigned b)
     h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
     return (double)h * (2.0 / 4294967296.0) - 1.0;
 }
-
-constexpr int kOrthPiece = 64;  // vectors orthogonalised together (pieces and seams)
 
 // cstart[i] = first index of the cluster of i (chains of eigenvalues closer than
 // tol_rel * ||T||). One CTA: each thread scans a contiguous segment, then the segment
@@ -570,6 +636,101 @@ __global__ void cluster_start_kernel(int kvec, const double *w, const double *bo
         const int carry = last[t - 1];
         for (int i = a; i < b && cstart[i] < 0; ++i) cstart[i] = carry;
     }
+}
+
+// zv <- x / max |x|, x = (T_b - lambda I)^{-1} zv on the block [bs, be) from the factors L+ D+ L+^T of
+// vector v (dplus; L+ = e / D+): forward L+ y = b, backward L+^T x = D+^{-1} y. Entries are rescaled
+// (all at once) whenever one exceeds 2^500. work: x[i * kvec], the vector's spent U- column. By the
+// whole CTA (kOrthThreads threads): a chunk of rows is loaded and divided in parallel, one thread runs the
+// recurrence over it in shared memory, an FMA a row.
+// Measured against one thread that loaded and divided row by row (1.1 us a row): n = 16384 18.5 -> 1.8 ms
+// a phase.
+constexpr int kOrthThreads = 256;
+template <typename T>
+__device__ void inverse_iteration(int n, int bs, int be, int kvec, int v, const double *__restrict__ e,
+                                  const double *__restrict__ dplus, double *work, T *zv, double *red)
+{
+    __shared__ double sr[kOrthThreads], sb[kOrthThreads], sy[kOrthThreads];
+    __shared__ int scales;  // rescalings in this chunk
+    constexpr int C = kOrthThreads, kBig = (1023 + 500) << 20;
+    const double shrink = 0x1p-500;
+    const int tid = threadIdx.x;
+    double *x = work + v;
+    // the recurrence over rows first, first + dir, .. of the chunk: val = sb - sr val
+    auto chain = [&](int first, int dir, int cnt, double val) {
+        int times = 0;
+        for (int j0 = 0; j0 < cnt; j0 += 4) {
+            double r[4], c[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = first + dir * min(j0 + q, cnt - 1);
+                r[q] = sr[j];
+                c[q] = sb[j];
+            }
+            const int at = times;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (j0 + q >= cnt) break;
+                const int j = first + dir * (j0 + q);
+                for (int s = at; s < times; ++s)
+                    if (dir < 0) c[q] *= shrink;  // right-hand sides loaded before a rescaling
+                val = fma(-r[q], val, c[q]);
+                if ((__double2hiint(val) & 0x7FFFFFFF) >= kBig) {
+                    for (int i = 0; i < j0 + q; ++i) sy[first + dir * i] *= shrink;
+                    if (dir < 0)  // the rows that are still to come are y of the forward pass
+                        for (int i = j0 + 4; i < cnt; ++i) sb[first + dir * i] *= shrink;
+                    val *= shrink;
+                    ++times;
+                }
+                sy[j] = val;
+            }
+        }
+        scales = times;
+        return val;
+    };
+    double val = 0.0;  // (thread 0) last value of the recurrence
+    for (int r0 = bs; r0 < be; r0 += C) {
+        const int i = r0 + tid, cnt = min(C, be - r0);
+        if (i < be) {
+            sb[tid] = (double)zv[i];
+            sr[tid] = i > bs ? e[i - 1] / dplus[(size_t)(i - 1) * kvec + v] : 0.0;
+        }
+        __syncthreads();
+        if (tid == 0) val = chain(0, 1, cnt, val);
+        __syncthreads();
+        for (int s = 0; s < scales; ++s)
+            for (int j = bs + tid; j < r0; j += C) x[(size_t)j * kvec] *= shrink;
+        if (i < be) x[(size_t)i * kvec] = sy[tid];
+        __syncthreads();
+    }
+    val = 0.0;
+    int times = 0;  // rescalings so far, which rows not yet loaded still need
+    for (int r0 = bs + (be - bs - 1) / C * C; r0 >= bs; r0 -= C) {
+        const int i = r0 + tid, cnt = min(C, be - r0);
+        if (i < be) {
+            double y = x[(size_t)i * kvec];
+            for (int s = 0; s < times; ++s) y *= shrink;
+            const double d = dplus[(size_t)i * kvec + v];
+            sb[tid] = y / d;
+            sr[tid] = i < be - 1 ? e[i] / d : 0.0;
+        }
+        __syncthreads();
+        if (tid == 0) val = chain(cnt - 1, -1, cnt, val);
+        __syncthreads();
+        times += scales;
+        for (int s = 0; s < scales; ++s)
+            for (int j = r0 + C + tid; j < be; j += C) x[(size_t)j * kvec] *= shrink;
+        if (i < be) x[(size_t)i * kvec] = sy[tid];
+        __syncthreads();
+    }
+    double mx = 0.0;
+    for (int i = bs + tid; i < be; i += C) mx = fmax(mx, fabs(x[(size_t)i * kvec]));
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((tid & 31) == 0) red[tid >> 5] = mx;
+    __syncthreads();
+    for (int q = 0; q < C / 32; ++q) mx = fmax(mx, red[q]);
+    const double sc = (mx > 0.0 && mx <= DBL_MAX) ? 1.0 / mx : 0.0;
+    for (int i = tid; i < n; i += C) zv[i] = (i >= bs && i < be) ? (T)(x[(size_t)i * kvec] * sc) : T(0);
 }
 
 // Gram-Schmidt (two passes) within clusters of eigenvalues closer than tol_rel * ||T||,
@@ -614,38 +775,7 @@ __global__ void cluster_orth_kernel(int n, int kvec, const int *cstart, int phas
                 zv[i] = (i >= bs && i < be) ? (T)hash_unit((unsigned)(v * 7919 + attempt), (unsigned)i) : T(0);
             __syncthreads();
             cluster_project(n, i0, v, z, ldz, red);
-            if (threadIdx.x == 0) {
-                double *x = work + v;  // x[i * kvec]
-                // forward: L+ y = b; backward: L+^T x = D+^{-1} y. Entries are rescaled
-                // (all at once) whenever one exceeds 2^500.
-                const double big = 0x1p500, shrink = 0x1p-500;
-                double y = 0.0;
-                for (int i = bs; i < be; ++i) {
-                    const double bi = (double)zv[i];
-                    y = (i == bs) ? bi : bi - (e[i - 1] / dplus[(size_t)(i - 1) * kvec + v]) * y;
-                    if (fabs(y) > big) {
-                        for (int j = bs; j < i; ++j) x[(size_t)j * kvec] *= shrink;
-                        y *= shrink;
-                    }
-                    x[(size_t)i * kvec] = y;
-                }
-                double xi = 0.0;
-                for (int i = be - 1; i >= bs; --i) {
-                    const double yi = x[(size_t)i * kvec] / dplus[(size_t)i * kvec + v];
-                    xi = (i == be - 1) ? yi : yi - (e[i] / dplus[(size_t)i * kvec + v]) * xi;
-                    if (fabs(xi) > big) {
-                        for (int j = i + 1; j < be; ++j) x[(size_t)j * kvec] *= shrink;
-                        for (int j = bs; j < i; ++j) x[(size_t)j * kvec] *= shrink;
-                        xi *= shrink;
-                    }
-                    x[(size_t)i * kvec] = xi;
-                }
-                double mx = 0.0;
-                for (int i = bs; i < be; ++i) mx = fmax(mx, fabs(x[(size_t)i * kvec]));
-                const double sc = (mx > 0.0 && mx <= DBL_MAX) ? 1.0 / mx : 0.0;
-                for (int i = 0; i < n; ++i)
-                    zv[i] = (i >= bs && i < be) ? (T)(x[(size_t)i * kvec] * sc) : T(0);
-            }
+            inverse_iteration(n, bs, be, kvec, v, e, dplus, work, zv, red);
             __syncthreads();
             double nr = 0.0;
             for (int i = threadIdx.x; i < n; i += blockDim.x) nr += (double)zv[i] * (double)zv[i];
@@ -690,7 +820,7 @@ cudaError_t stein(cudaStream_t st, int n, const double *d, const double *e, int 
     cluster_start_kernel<<<1, 1024, 0, st>>>(kvec, w, bounds, 1e-5, cstart);
     for (int phase = 0; phase < 2; ++phase) {
         EGB_COUNT_LAUNCH();
-        cluster_orth_kernel<T><<<kvec, 256, 0, st>>>(n, kvec, cstart, phase, e, blk, dplus, uminus, z,
+        cluster_orth_kernel<T><<<kvec, kOrthThreads, 0, st>>>(n, kvec, cstart, phase, e, blk, dplus, uminus, z,
                                                      ldz, status);
     }
     return cudaGetLastError();
