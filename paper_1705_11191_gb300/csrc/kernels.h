@@ -177,12 +177,15 @@ cudaError_t apply_q2_f64(cudaStream_t st, int n, int b, const double *v2, const 
 size_t q2_factor_elems(int n, int b);
 cudaError_t apply_q2_tc(cudaStream_t st, int n, int b, const float *v2, const float *tau2, int k,
                         float *z, int ldz, float *fac, int *status);
-// Z <- Q1 Z in groups of kQ1Group panels; work: q1_work_elems(b, k) elements.
-constexpr int kQ1Group = 4;
-inline size_t q1_work_elems(int b, int k)
+// Z <- Q1 Z in groups of q1_group(n) panels (q1.cu); work: q1_work_elems(n, b, k) elements. Eight panels
+// a group halve the passes over Z, and merging their T takes longer: n = 777 0.77 ms against 0.30 with
+// four, n = 1531 the same, n = 4096 2.35 against 2.54, n = 5000 9.7 against 10.9, n = 16384 62 against 74.
+constexpr int kQ1MaxGroup = 8;
+inline int q1_group(int n) { return n >= 4096 ? kQ1MaxGroup : 4; }
+inline size_t q1_work_elems(int n, int b, int k)
 {
-    const size_t g = (size_t)kQ1Group * b;
-    return g * g + 2 * g * b + 4 * g * (size_t)k + 64;
+    const size_t g = (size_t)q1_group(n) * b, groups = (size_t)n / g + 1;
+    return groups * g * g + 4 * g * (size_t)k + 64;
 }
 template <typename T>
 cudaError_t apply_q1(cudaStream_t st, int n, int b, int k, const T *v1, const T *t1, T *z,
