@@ -15,34 +15,35 @@ namespace egb {
 // ---- W of the two-sided update, fused (three small launches instead of five GEMMs):
 //   X = (A22 V) T,  Y = V^T X,  W = X - (1/2) V (T^T Y).
 // Row blocks of WRows<T> rows; tiles of 64 columns (bw <= 64, zero padded) in shared memory,
-// each of the 256 threads computing R x 4 or 4 x 4 elements of a tile product. Binary64 has
+// each of the 256 threads computing R x CJ or CJ x CJ elements of a tile product (CJ = 4, or 2 for
+// bw <= 32, where half of every tile is padding). Binary64 has
 // two FMAs a clock and SM, so its blocks are 16 rows: four times the CTAs of 64-row blocks
 // (two launches of 135 us at any order), and V (T^T Y) is formed as (V T^T) Y, whose work
 // shrinks with the rows, where T^T Y costs every block 64^3 FMAs: 27 and 20 us at n = 1531,
-// b = 32.
+// b = 32, and 11 and 13 us with CJ = 2.
 template <typename T> constexpr int WRows = sizeof(T) == 4 ? 64 : 16;
 constexpr int kWLd = 65;
 
-// c[R][4] = sum_{k < kmax} A[R ty + i][k] B[k][4 tx + j] for tiles A, B with leading dimension
+// c[R][CJ] = sum_{k < kmax} A[R ty + i][k] B[k][CJ tx + j] for tiles A, B with leading dimension
 // kWLd, ty = tid / 16, tx = tid % 16
-template <typename T, int R>
-__device__ __forceinline__ void tile_mm(const T *A, const T *B, int kmax, T (&c)[R][4])
+template <typename T, int R, int CJ>
+__device__ __forceinline__ void tile_mm(const T *A, const T *B, int kmax, T (&c)[R][CJ])
 {
-    const int tr = (threadIdx.x >> 4) * R, tc = (threadIdx.x & 15) * 4;
+    const int tr = (threadIdx.x >> 4) * R, tc = (threadIdx.x & 15) * CJ;
 #pragma unroll
     for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) c[i][j] = T(0);
+        for (int j = 0; j < CJ; ++j) c[i][j] = T(0);
     for (int k = 0; k < kmax; ++k) {
-        T a[R], b[4];
+        T a[R], b[CJ];
 #pragma unroll
         for (int i = 0; i < R; ++i) a[i] = A[(tr + i) * kWLd + k];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = B[k * kWLd + tc + j];
+        for (int j = 0; j < CJ; ++j) b[j] = B[k * kWLd + tc + j];
 #pragma unroll
         for (int i = 0; i < R; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) c[i][j] = fma(a[i], b[j], c[i][j]);
+            for (int j = 0; j < CJ; ++j) c[i][j] = fma(a[i], b[j], c[i][j]);
     }
 }
 
@@ -74,7 +75,7 @@ __device__ __forceinline__ void load_rows(T *tile, const T *src, int ld, int r0,
 }
 
 // X rows = Xa rows T; partial Y (64 x 64 per block, column-major) = V rows^T X rows
-template <typename T>
+template <typename T, int CJ>
 __global__ void __launch_bounds__(256) w_stage1_kernel(int m, int bw, const T *xa, const T *V, int ldv,
                                                        const T *Tm, int ldt, T *X, T *ypart)
 {
@@ -85,13 +86,13 @@ __global__ void __launch_bounds__(256) w_stage1_kernel(int m, int bw, const T *x
     load_rows<T, 64>(sT, Tm, ldt, 0, bw, bw);
     load_rows<T, ROWS>(sA, xa, m, r0, rows, bw);
     __syncthreads();
-    T c[R][4];
-    tile_mm<T, R>(sA, sT, bw, c);
-    const int tr = (threadIdx.x >> 4) * R, tc = (threadIdx.x & 15) * 4;
+    T c[R][CJ];
+    tile_mm<T, R, CJ>(sA, sT, bw, c);
+    const int tr = (threadIdx.x >> 4) * R, tc = (threadIdx.x & 15) * CJ;
 #pragma unroll
     for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < CJ; ++j) {
             sX[(tr + i) * kWLd + tc + j] = c[i][j];
             if (tr + i < rows && tc + j < bw) X[(size_t)(r0 + tr + i) + (size_t)(tc + j) * m] = c[i][j];
         }
@@ -100,40 +101,44 @@ __global__ void __launch_bounds__(256) w_stage1_kernel(int m, int bw, const T *x
     tile_in<T, ROWS>([&](int i, int a) { return (i < rows && a < bw) ? V[(size_t)(r0 + i) + (size_t)a * ldv] : T(0); },
                      [&](int i, int a, T x) { sA[a * kWLd + i] = x; });
     __syncthreads();
-    T y[4][4];
-    tile_mm<T, 4>(sA, sX, ROWS, y);
-    const int ta = (threadIdx.x >> 4) * 4;
+    T y[CJ][CJ];
+    tile_mm<T, CJ, CJ>(sA, sX, ROWS, y);
+    const int ta = (threadIdx.x >> 4) * CJ;
     T *yp = ypart + (size_t)blockIdx.x * 64 * 64;
     if (ta < bw && tc < bw)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < CJ; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) yp[(ta + i) + (tc + j) * 64] = y[i][j];
+            for (int j = 0; j < CJ; ++j) yp[(ta + i) + (tc + j) * 64] = y[i][j];
 }
 
-// Y[e] = sum over blocks g of ypart[g][e] (e < 64 * 64, ascending g)
+// Y[e] = sum over blocks g of ypart[g][e] (e < 64 * 64): four threads an element, each over a
+// quarter of the blocks in ascending order
 template <typename T>
-__global__ void w_stage2_kernel(int nblk, int bw, const T *ypart, T *Y)
+__global__ void __launch_bounds__(256) w_stage2_kernel(int nblk, int bw, const T *ypart, T *Y)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= 64 * 64) return;
+    __shared__ T part[4][64];
+    const int el = threadIdx.x & 63, q = threadIdx.x >> 6, e = blockIdx.x * 64 + el;
     T s = T(0);
-    if ((e & 63) < bw && (e >> 6) < bw) {
-        int g = 0;
-        for (; g + 8 <= nblk; g += 8) {
+    if (el < bw && (int)blockIdx.x < bw) {
+        const int per = (nblk + 3) / 4, g1 = min(nblk, (q + 1) * per);
+        int g = q * per;
+        for (; g + 8 <= g1; g += 8) {
             T v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) v[u] = ypart[(size_t)(g + u) * 64 * 64 + e];
 #pragma unroll
             for (int u = 0; u < 8; ++u) s += v[u];
         }
-        for (; g < nblk; ++g) s += ypart[(size_t)g * 64 * 64 + e];
+        for (; g < g1; ++g) s += ypart[(size_t)g * 64 * 64 + e];
     }
-    Y[e] = s;
+    part[q][el] = s;
+    __syncthreads();
+    if (q == 0) Y[e] = (part[0][el] + part[1][el]) + (part[2][el] + part[3][el]);
 }
 
 // W rows = X rows - (1/2) (V rows T^T) Y
-template <typename T>
+template <typename T, int CJ>
 __global__ void __launch_bounds__(256) w_stage3_kernel(int m, int bw, const T *X, const T *V, int ldv,
                                                        const T *Tm, int ldt, const T *Y, T *W)
 {
@@ -147,27 +152,27 @@ __global__ void __launch_bounds__(256) w_stage3_kernel(int m, int bw, const T *X
     tile_in<T, 64>([&](int i, int c) { return Y[i + c * 64]; }, [&](int i, int c, T x) { sB[i * kWLd + c] = x; });
     load_rows<T, ROWS>(sZ, V, ldv, r0, rows, bw);
     __syncthreads();
-    T c[R][4];
-    tile_mm<T, R>(sZ, sA, bw, c);
-    const int tr = (threadIdx.x >> 4) * R, tc = (threadIdx.x & 15) * 4;
+    T c[R][CJ];
+    tile_mm<T, R, CJ>(sZ, sA, bw, c);
+    const int tr = (threadIdx.x >> 4) * R, tc = (threadIdx.x & 15) * CJ;
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) sZ[(tr + i) * kWLd + tc + j] = c[i][j];
+        for (int j = 0; j < CJ; ++j) sZ[(tr + i) * kWLd + tc + j] = c[i][j];
     __syncthreads();
-    tile_mm<T, R>(sZ, sB, bw, c);
+    tile_mm<T, R, CJ>(sZ, sB, bw, c);
 #pragma unroll
     for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < CJ; ++j)
             if (tr + i < rows && tc + j < bw) {
                 const size_t q = (size_t)(r0 + tr + i) + (size_t)(tc + j) * m;
                 W[q] = X[q] - T(0.5) * c[i][j];
             }
 }
 
-template <typename T>
+template <typename T, int CJ>
 static cudaError_t form_w(cudaStream_t st, int m, int bw, const T *xa, const T *V, int ldv,
                           const T *Tm, int ldt, T *X, T *Y, T *W, T *ypart)
 {
@@ -175,18 +180,18 @@ static cudaError_t form_w(cudaStream_t st, int m, int bw, const T *xa, const T *
     const size_t smem = (size_t)3 * 64 * kWLd * sizeof(T);
     static PerDeviceOnce attr;  // per instantiation
     cudaError_t e = once_per_device(attr, [&] {
-        cudaError_t r = cudaFuncSetAttribute(w_stage1_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t r = cudaFuncSetAttribute(w_stage1_kernel<T, CJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(w_stage3_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            r = cudaFuncSetAttribute(w_stage3_kernel<T, CJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         return r;
     });
     if (e != cudaSuccess) return e;
     EGB_COUNT_LAUNCH();
-    w_stage1_kernel<T><<<nblk, 256, smem, st>>>(m, bw, xa, V, ldv, Tm, ldt, X, ypart);
+    w_stage1_kernel<T, CJ><<<nblk, 256, smem, st>>>(m, bw, xa, V, ldv, Tm, ldt, X, ypart);
     EGB_COUNT_LAUNCH();
-    w_stage2_kernel<T><<<64, 64, 0, st>>>(nblk, bw, ypart, Y);
+    w_stage2_kernel<T><<<64, 256, 0, st>>>(nblk, bw, ypart, Y);
     EGB_COUNT_LAUNCH();
-    w_stage3_kernel<T><<<nblk, 256, smem, st>>>(m, bw, X, V, ldv, Tm, ldt, Y, W);
+    w_stage3_kernel<T, CJ><<<nblk, 256, smem, st>>>(m, bw, X, V, ldv, Tm, ldt, Y, W);
     return cudaGetLastError();
 }
 
@@ -250,7 +255,9 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
         if (ceil_div(m, WRows<T>) + 1 <= kSyncBlocks) {
             // X = (A22 V) T, W = X - 1/2 V (T^T (V^T X))
             T *ysum = ypart + (size_t)ceil_div(m, WRows<T>) * 64 * 64;
-            if ((e = form_w<T>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart)) != cudaSuccess) return e;
+            e = bw <= 32 ? form_w<T, 2>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart)
+                         : form_w<T, 4>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart);
+            if (e != cudaSuccess) return e;
         } else {
             // X = (A22 V) T
             if ((e = gemm<T>(st, 0, 0, m, bw, bw, T(1), W, m, Tm, ldt, T(0), X, m)) != cudaSuccess) return e;
