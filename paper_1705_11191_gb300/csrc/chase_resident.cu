@@ -22,8 +22,11 @@
 //   y = tau_p X0 v_p, x = X0[:, first] - y, v = house(x), p = tau v^T (X0 - y v_p^T),
 //   q = tau D v, w = q - (1/2) tau (v.q) v,
 //   X = X0 - y v_p^T - v p^T,  D = D - v w^T - w v^T.
-// The column sums x^T X0 and D x are taken with the unscaled x (x_first apart), so that
-// three block barriers serve a whole step.
+// The column sums x^T X0 and D x are taken with the unscaled x (x_first apart). A sweep's share of
+// the chain is one step from its reflector's arrival to the row it sends back and one from a row's
+// arrival to the reflector it sends on, so each step sends as early as it can: the reflector
+// before the sums x^T X0 and D x, the row before the update of D (in binary64, where an
+// operation holds a warp's unit 64 clocks, 57 -> 40 and 121 -> 101 operations).
 //
 // Measured against the kernel of sb2st.cu: binary32, b = 64, n = 777 10.6 -> 2.7 ms, n = 4096
 // 60.3 -> 16.0 ms, n = 16384 245 -> 70 ms (14.7 -> 3.5 - 4.3 us a sweep, two L2 hand-overs and
@@ -44,6 +47,10 @@ struct Args {
     int *status;
     long long spin_limit;
 };
+
+// A value that what follows cannot be computed before this point
+__device__ __forceinline__ void pin(double &x) { asm volatile("" : "+d"(x)); }
+__device__ __forceinline__ void pin(float &x) { asm volatile("" : "+f"(x)); }
 
 template <typename T, int B>
 __global__ void __launch_bounds__(4 * B, 512 / (4 * B))
@@ -169,32 +176,7 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
             if (first) { ysl[0] = x; ysl[1] = y; }
         }
         {
-            T ss = xz * xz, xy = xz * y;
-            if (t > 0) {
-                // column sums of xz X0 over the warp's eight rows: exchange halves so that each
-                // lane ends with PH columns
-                T u[CPT];
-#pragma unroll
-                for (int q = 0; q < CPT; ++q) u[q] = xz * X[q];
-                if (first)
-#pragma unroll
-                    for (int q = 0; q < CPT; ++q) xrow[c0 + q] = X[q];
-                int base = 0;
-#pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    const int o = 16 >> s;
-                    const int half = CPT >> (s + 1);
-                    const bool up = (lane & o) != 0;
-#pragma unroll
-                    for (int q = 0; q < half; ++q) {
-                        const T keep = up ? u[q + half] : u[q], give = up ? u[q] : u[q + half];
-                        u[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-                    }
-                    base += up ? half : 0;
-                }
-#pragma unroll
-                for (int q = 0; q < PH; ++q) upart[warp][c0 + base + q] = u[q];
-            }
+            const T ss = xz * xz, xy = xz * y;
             // |xz|^2 in the lanes of the lower half, xz . y in the upper half
             const T keep = (lane & 16) ? xy : ss, give = (lane & 16) ? ss : xy;
             T r2 = keep + __shfl_xor_sync(0xffffffffu, give, 16);
@@ -205,9 +187,9 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         __syncthreads();
         // ---- the reflector (every thread computes the same scalars) and q = tau D v
         const T alpha = ysl[0];
-        T ss = T(0), xy = T(0);
+        T ss = red[0][0], xy = red[1][0];
 #pragma unroll
-        for (int w = 0; w < NW; ++w) { ss += red[0][w]; xy += red[1][w]; }
+        for (int w = 1; w < NW; ++w) { ss += red[0][w]; xy += red[1][w]; }
         T beta, tau, scl;
         reflector<T>(alpha, ss, beta, tau, scl);
         const T v = first ? T(1) : xz * scl;
@@ -219,6 +201,33 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
             const size_t slot = (size_t)j * a.S + t;
             v2[slot * B + (i >= rs ? i - rs : i - rs + B)] = v;
             if (i == 0) tau2[slot] = tau;
+        }
+        if (t > 0) {
+            T xp = xz;
+            pin(xp);  // after the reflector is on its way
+            // column sums of xz X0 over the warp's eight rows: exchange halves so that each
+            // lane ends with PH columns
+            T u[CPT];
+#pragma unroll
+            for (int q = 0; q < CPT; ++q) u[q] = xp * X[q];
+            if (first)
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) xrow[c0 + q] = X[q];
+            int base = 0;
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                const int o = 16 >> s;
+                const int half = CPT >> (s + 1);
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int q = 0; q < half; ++q) {
+                    const T keep = up ? u[q + half] : u[q], give = up ? u[q] : u[q + half];
+                    u[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+                base += up ? half : 0;
+            }
+#pragma unroll
+            for (int q = 0; q < PH; ++q) upart[warp][c0 + base + q] = u[q];
         }
         T qd;
         {
@@ -234,12 +243,6 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
             const T dc = __shfl_sync(0xffffffffu, pick(D, rs % CPT), quad | (rs / CPT));
             qd = tau * fma(scl, g, dc);
         }
-        if (t > 0 && tid < B) {
-            T s = T(0);
-#pragma unroll
-            for (int w = 0; w < NW; ++w) s += upart[w][tid];
-            ps[tid] = tau * (fma(scl, s, xrow[tid]) - fma(scl, xy, ysl[1]) * vps[par][tid]);
-        }
         if (part == 0) qs[i] = qd;
         {
             T kp = v * qd;
@@ -248,32 +251,43 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
             if (lane == 0) red[2][warp] = kp;
         }
         __syncthreads();
-        // ---- updates
-        T K = T(0);
+        T K = red[2][0];
 #pragma unroll
-        for (int w = 0; w < NW; ++w) K += red[2][w];
+        for (int w = 1; w < NW; ++w) K += red[2][w];
         // D - v w^T - w v^T with w = q - K v / 2, as D - v q^T - (q - K v) v^T
-        const T w2 = fma(-K * tau, v, qd);
-#pragma unroll
-        for (int q = 0; q < CPT; ++q) {
-            const int c = c0 + q;
-            D[q] = fma(-v, qs[c], fma(-w2, vs[c], D[q]));
-        }
+        T vd = v, w2 = fma(-K * tau, v, qd);
         if (t > 0) {
+            if (tid < B) {
+                T s = upart[0][tid];
+#pragma unroll
+                for (int w = 1; w < NW; ++w) s += upart[w][tid];
+                ps[tid] = tau * (fma(scl, s, xrow[tid]) - fma(scl, xy, ysl[1]) * vps[par][tid]);
+            }
+            __syncthreads();
+            // ---- updates: X first, and the row that position t - 1 takes in at its next sweep
 #pragma unroll
             for (int q = 0; q < CPT; ++q) {
                 const int c = c0 + q;
                 X[q] = fma(-v, ps[c], fma(-y, vps[par][c], X[q]));
             }
-            if (first) {  // the row that position t - 1 takes in at its next sweep
+            if (first) {
 #pragma unroll
                 for (int q = 0; q < CPT; ++q) {
                     const int c = c0 + q;
                     put(rout + c * kWords<T>, c == rs ? beta : X[q], (unsigned)j + 1);
                 }
-                if (part == rs / CPT) put(rout + B * kWords<T>, pick(D, rs % CPT), (unsigned)j + 1);
+                if (part == rs / CPT)
+                    put(rout + B * kWords<T>, fma(-v, qs[rs], fma(-w2, vs[rs], pick(D, rs % CPT))), (unsigned)j + 1);
             }
-        } else {
+            pin(vd);
+            pin(w2);  // D after the row is on its way
+        }
+#pragma unroll
+        for (int q = 0; q < CPT; ++q) {
+            const int c = c0 + q;
+            D[q] = fma(-vd, qs[c], fma(-w2, vs[c], D[q]));
+        }
+        if (t == 0) {
             if (first && part == rs / CPT) {
                 dout[j + 1] = (double)pick(D, rs % CPT);
                 eout[j] = (double)beta;

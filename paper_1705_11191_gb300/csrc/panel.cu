@@ -179,11 +179,18 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
         T row = T(0);
         if (G > 1 || g == G) {
             tot = Sum<T>();
+            // row j comes with the first of them (the loads are in flight together)
+            bool have_row = g == 0 || xg != 0;
             for (int q0 = xg; q0 < G && ok; q0 += LPC * FLY) {
-                u64 w0[FLY], w1[FLY];
+                u64 w0[FLY], w1[FLY], wr[2];
                 long long it = 0;
                 for (;;) {
                     bool ready = true;
+                    const u64 *rp = a.rpk + (size_t)(j * 64 + xc) * 2;
+                    if (!have_row) {
+                        wr[0] = ld_relaxed(rp);
+                        if (sizeof(T) == 8) wr[1] = ld_relaxed(rp + 1);
+                    }
 #pragma unroll
                     for (int u = 0; u < FLY; ++u) {
                         const int q = q0 + LPC * u;
@@ -192,7 +199,12 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
 #pragma unroll
                     for (int u = 0; u < FLY; ++u)
                         if (q0 + LPC * u < G) ready = ready && seq_of(w0[u]) == seq && seq_of(w1[u]) == seq;
-                    if (ready) break;
+                    if (!have_row) {
+                        have_row = seq_of(wr[0]) == seq && (sizeof(T) == 4 || seq_of(wr[1]) == seq);
+                        if (sizeof(T) == 4) row = (T)__uint_as_float((unsigned)wr[0]);
+                        else row = (T)__hiloint2double((int)(unsigned)wr[1], (int)(unsigned)wr[0]);
+                    }
+                    if (ready && have_row) break;
                     if (!poll_again(it, a.spin_limit, a.status, j)) { ok = false; break; }
                 }
 #pragma unroll
@@ -205,7 +217,6 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
         }
         if (xg == 0) {
             if (g == 0) row = rowown[xc];
-            else ok = get(a.rpk + (size_t)(j * 64 + xc) * 2, seq, row, a.spin_limit, a.status) && ok;
             const T d = tot.value();
             dsum[xc] = d;
             rowj[xc] = row;
