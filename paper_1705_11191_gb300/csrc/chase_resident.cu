@@ -31,7 +31,8 @@
 // Measured against the kernel of sb2st.cu: binary32, b = 64, n = 777 10.6 -> 2.7 ms, n = 4096
 // 60.3 -> 16.0 ms, n = 16384 245 -> 70 ms (14.7 -> 3.5 - 4.3 us a sweep, two L2 hand-overs and
 // two steps' arithmetic); binary64, b = 64, n = 512 15.2 -> 11.0 ms, n = 1531 51.3 -> 35.7 ms (a
-// step's 28 000 FMAs at two a clock bound it), and with b = 32 4.5 and 14.0 ms.
+// step's 28 000 FMAs at two a clock bound it), and with b = 32 4.5 and 14.0 ms, 3.8 and 11.9 with
+// the early messages (3.9, 12.3) and the shorter reciprocals of packets.cuh.
 #include "common.cuh"
 #include "kernels.h"
 #include "packets.cuh"

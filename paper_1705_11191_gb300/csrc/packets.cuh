@@ -69,7 +69,8 @@ __device__ __forceinline__ bool get(const u64 *p, unsigned seq, T &v, long long 
 
 }  // namespace pkt
 
-// 1 / x and 1 / sqrt(x) to about an ulp: the hardware's approximation and Newton steps. A
+// 1 / x and 1 / sqrt(x) to about an ulp: the hardware's approximation (about 2^-20 in binary64) and
+// a step of third order (two of Newton's are a longer chain), one of Newton's in binary32. A
 // library division or square root is two to three times as long a chain, and in binary64 two
 // to three times as many operations of the chip's few binary64 units. Arguments whose result
 // or whose approximation would be subnormal or overflow take the library's path.
@@ -79,8 +80,8 @@ __device__ __forceinline__ double recip(double x)
     if (ex >= (2044 << 20) || ex == 0) return 1.0 / x;
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(fma(-x, r, 1.0), r, r);
-    return fma(fma(-x, r, 1.0), r, r);
+    const double h = fma(-x, r, 1.0);  // r (1 + h + h^2): a relative error of h^3
+    return fma(r, fma(h, h, h), r);
 }
 __device__ __forceinline__ float recip(float x)
 {
@@ -96,11 +97,8 @@ __device__ __forceinline__ double rsq(double x)
     if (ex >= (2000 << 20) || ex <= (40 << 20)) return rsqrt(x);
     double r;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    // r += r (1 - x r^2) / 2, twice
-    double h = fma(-x * r, r, 1.0);
-    r = fma(0.5 * r, h, r);
-    h = fma(-x * r, r, 1.0);
-    return fma(0.5 * r, h, r);
+    const double h = fma(-x * r, r, 1.0);  // r (1 + h / 2 + 3 h^2 / 8): a relative error of 5 h^3 / 16
+    return fma(h * r, fma(0.375, h, 0.5), r);
 }
 __device__ __forceinline__ float rsq(float x)
 {

@@ -22,7 +22,8 @@
 //
 // Measured per 64-column panel, before -> now: binary32 n = 777 0.73 -> 0.21 ms, n = 4096 0.82
 // -> 0.24 ms, n = 16384 0.85 -> 0.29 ms; binary64 n = 512 1.09 -> 0.40 ms, n = 5000 1.24 ->
-// 0.51 ms. What is left is one L2 exchange a column (about 1.5 us) and, in binary64, the
+// 0.51 ms; per 32-column panel, binary64 n = 512 0.152 -> 0.133 ms, n = 5000 0.192 -> 0.169 ms with
+// the late scale, the row fetched with the sums and the shorter reciprocals of packets.cuh. What is left is one L2 exchange a column (about 1.5 us) and, in binary64, the
 // 2 x 64 x 64 FMAs of a CTA's rows at two a clock.
 #include "common.cuh"
 #include "kernels.h"
@@ -99,11 +100,14 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
     constexpr int LPC = 32 * NW / NC;  // threads per column in the exchange
     constexpr int RPL = 32 / RW;       // columns of a warp's rows moved by one access
     constexpr int FLY = 8;             // packets of a thread in flight
+    // binary64: the storage holds x, scaled to the reflector at the end (binary32 would lose sums of
+    // two columns of 1e-16 and less)
+    constexpr bool LATE = sizeof(T) == 8;
     static_assert(LPC >= 4 && LPC <= 16 && NW % LPC == 0 && RW <= 32, "layout");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(16) T xbuf[NW][RW];
     __shared__ T partw[NW][NC];
-    __shared__ T rowown[NC], dsum[NC], rowj[NC], scal[3];
+    __shared__ T rowown[NC], dsum[NC], rowj[NC], scal[3], scls[NC];  // scls: 1 / x scale of column c's reflector
     __shared__ int failed;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.x, G = a.G, bw = a.bw;
@@ -223,7 +227,7 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
             if (xc == j) {
                 T beta, tau, scl;
                 reflector<T>(row, d, beta, tau, scl);
-                scal[0] = beta; scal[1] = tau; scal[2] = scl;
+                scal[0] = beta; scal[1] = tau; scal[2] = scls[j] = scl;
             }
         }
         if (!ok) failed = 1;
@@ -231,20 +235,24 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
         if (failed) return;
         const T beta = scal[0], tau = scal[1], scl = scal[2];
         if (g < G) {
-            // ---- P_c -= v (tau v . P_c), c > j; column j becomes the reflector
+            // ---- P_c -= v (tau v . P_c), c > j, v = scl x; column j becomes the reflector (binary64: at
+            //      the end, LATE; the scale would be as many operations as the products)
             T wv[CPL];
 #pragma unroll
             for (int c = 0; c < CPL; ++c) {
                 const int col = c * 32 + lane;
                 wv[c] = col > j ? tau * fma(scl, dsum[col], rowj[col]) : T(0);
             }
+            T wx[CPL];
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) wx[c] = LATE ? scl * wv[c] : wv[c];
 #pragma unroll
             for (int i = 0; i < RW; ++i) {
-                const T v = xbuf[warp][i] * scl;
+                const T v = LATE ? xbuf[warp][i] : xbuf[warp][i] * scl;
 #pragma unroll
                 for (int c = 0; c < CPL; ++c) {
-                    p[c][i] = fma(-v, wv[c], p[c][i]);
-                    if (c * 32 + lane == j && row0 + i > j) p[c][i] = v;
+                    p[c][i] = fma(-v, wx[c], p[c][i]);
+                    if (!LATE && c * 32 + lane == j && row0 + i > j) p[c][i] = v;
                 }
             }
             if (g == 0 && warp == j / RW) {
@@ -258,7 +266,7 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
             // ---- T[0:j, j] = -tau T[0:j, 0:j] (v_c . v_j), forward recurrence
             double acc = 0.0;
             if (xc < j)
-                for (int q = xc + xg; q < j; q += LPC) acc += Ts[xc][q] * ((double)scl * (double)dsum[q] + (double)rowj[q]);
+                for (int q = xc + xg; q < j; q += LPC) acc += Ts[xc][q] * ((double)scl * (double)dsum[q] + (double)rowj[q]) * (LATE ? (double)scls[q] : 1.0);
             __syncwarp();
 #pragma unroll
             for (int o = 1; o < LPC; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -285,7 +293,8 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
     if (gi < a.m)
 #pragma unroll 4
         for (int c = cl; c < bw; c += RPL) {
-            const T pv = tile[c * (RW + 1) + rl];
+            T pv = tile[c * (RW + 1) + rl];
+            if (LATE && gi > c && c < nref) pv *= scls[c];
             P[(size_t)gi + (size_t)c * a.lda] = pv;
             V[(size_t)gi + (size_t)c * a.ldv] = (c >= nref || gi < c) ? T(0) : (gi == c ? T(1) : pv);
         }
