@@ -103,7 +103,7 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
     // binary64: the storage holds x, scaled to the reflector at the end (binary32 would lose sums of
     // two columns of 1e-16 and less)
     constexpr bool LATE = sizeof(T) == 8;
-    static_assert(LPC >= 4 && LPC <= 16 && NW % LPC == 0 && RW <= 32, "layout");
+    static_assert(LPC >= 4 && LPC <= 16 && NW % LPC == 0 && RW <= 32 && RW * NW >= NC, "layout");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(16) T xbuf[NW][RW];
     __shared__ T partw[NW][NC];
@@ -323,16 +323,21 @@ cudaError_t launch(cudaStream_t st, T *P, T *V, T *Tm, int ldt, Args a, int num_
 template <typename T, int CPL>
 cudaError_t choose(cudaStream_t st, T *P, T *V, T *Tm, int ldt, const Args &a, int num_sms)
 {
-    // Rows per CTA. Binary32: the exchange costs more than the arithmetic, so 256, and 512 once
-    // that gives more than 32 CTAs (one round of packets in flight). Binary64: two FMAs a clock
-    // make the arithmetic of a CTA's rows the larger part, so 64 where the CTAs fit.
+    // Rows per CTA: few while the packets of a column still come in one round (64 / CPL CTAs: the
+    // threads of a column with 8 in flight each), since a column is the latency of a warp's
+    // instructions over its rows and of one exchange, which more CTAs hardly lengthen up to there.
+    // Binary32 128 rows against 256: n = 777 210 -> 190 us a panel, n = 4096 234 -> 224 us; above,
+    // 256, and 512 once that gives more than 32 CTAs (n = 16384: 321 us, 335 with 128). Binary64 32
+    // rows against 64: n = 1531 141 -> 131 us; n = 5000 188 us against 169 with 64.
+    constexpr int kFew = sizeof(T) == 4 ? 128 : 32 * CPL;  // the rows j < bw are all in the first CTA
     bool fits = false;
     cudaError_t e = cudaSuccess;
+    if (ceil_div(a.m, kFew) <= 64 / CPL) e = launch<T, kFew / 8, CPL, 8>(st, P, V, Tm, ldt, a, num_sms, &fits);
     if constexpr (sizeof(T) == 4) {
-        if (a.m <= 32 * 256) e = launch<T, 32, CPL, 8>(st, P, V, Tm, ldt, a, num_sms, &fits);
+        if (e == cudaSuccess && !fits && a.m <= 32 * 256) e = launch<T, 32, CPL, 8>(st, P, V, Tm, ldt, a, num_sms, &fits);
         if (e == cudaSuccess && !fits) e = launch<T, 32, CPL, 16>(st, P, V, Tm, ldt, a, num_sms, &fits);
     } else {
-        e = launch<T, 8, CPL, 8>(st, P, V, Tm, ldt, a, num_sms, &fits);
+        if (e == cudaSuccess && !fits) e = launch<T, 8, CPL, 8>(st, P, V, Tm, ldt, a, num_sms, &fits);
         if (e == cudaSuccess && !fits) e = launch<T, 16, CPL, 16>(st, P, V, Tm, ldt, a, num_sms, &fits);
     }
     if (e != cudaSuccess) return e;
@@ -341,11 +346,14 @@ cudaError_t choose(cudaStream_t st, T *P, T *V, T *Tm, int ldt, const Args &a, i
 
 }  // namespace pan
 
-size_t panel_packet_words(int m, int elem)
+// CTAs of a panel with at most m rows, at most: see choose()
+static int max_ctas(int m, int elem)
 {
-    const int gs = ceil_div(m, elem == 4 ? 256 : 64);
-    return (size_t)64 * 64 * 2 * (gs + 1);
+    const int most = ceil_div(m, elem == 4 ? 256 : 64), few = ceil_div(m, elem == 4 ? 128 : 32);
+    return few < 64 ? few : (most > 64 ? most : 64);
 }
+
+size_t panel_packet_words(int m, int elem) { return (size_t)64 * 64 * 2 * (max_ctas(m, elem) + 1); }
 
 template <typename T>
 cudaError_t panel_qr(cudaStream_t st, int m, int m_first, int bw, T *P, int lda, T *V, int ldv, T *Tm, int ldt,
@@ -354,7 +362,7 @@ cudaError_t panel_qr(cudaStream_t st, int m, int m_first, int bw, T *P, int lda,
     if (bw < 1 || bw > 64) return cudaErrorInvalidValue;
     pan::Args a;
     a.m = m; a.bw = bw; a.lda = lda; a.ldv = ldv; a.G = 0;
-    a.gs = ceil_div(m_first, sizeof(T) == 4 ? 256 : 64);
+    a.gs = max_ctas(m_first, sizeof(T));
     a.seq0 = seq0; a.rpk = packets; a.dpk = packets + 64 * 64 * 2;
     a.status = status; a.spin_limit = spin_limit();
     return bw <= 32 ? pan::choose<T, 1>(st, P, V, Tm, ldt, a, num_sms)
