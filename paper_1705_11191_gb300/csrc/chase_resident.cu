@@ -60,6 +60,8 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
     constexpr int CPT = B / 4;       // columns of a row per thread (four threads per row)
     constexpr int NW = 4 * B / 32;   // warps
     constexpr int PH = CPT / 8;      // columns per lane after the in-warp column sums
+    // binary32: the column sums cost less than the barrier that taking them later needs
+    constexpr bool EARLY = sizeof(T) == 4;
     __shared__ __align__(16) T vps[2][B];      // v_p by slot (double buffered: see the end)
     __shared__ __align__(16) T rows_[2][B];    // row message by slot
     __shared__ T msc[2][2];                    // tau_p, d of the row message
@@ -176,6 +178,34 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
             xs[i] = xz;
             if (first) { ysl[0] = x; ysl[1] = y; }
         }
+        auto column_sums = [&]() {
+            T xp = xz;
+            if (!EARLY) pin(xp);  // after the reflector is on its way
+            // column sums of xz X0 over the warp's eight rows: exchange halves so that each
+            // lane ends with PH columns
+            T u[CPT];
+#pragma unroll
+            for (int q = 0; q < CPT; ++q) u[q] = xp * X[q];
+            if (first)
+#pragma unroll
+                for (int q = 0; q < CPT; ++q) xrow[c0 + q] = X[q];
+            int base = 0;
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                const int o = 16 >> s;
+                const int half = CPT >> (s + 1);
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int q = 0; q < half; ++q) {
+                    const T keep = up ? u[q + half] : u[q], give = up ? u[q] : u[q + half];
+                    u[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+                base += up ? half : 0;
+            }
+#pragma unroll
+            for (int q = 0; q < PH; ++q) upart[warp][c0 + base + q] = u[q];
+        };
+        if (t > 0 && EARLY) column_sums();
         {
             const T ss = xz * xz, xy = xz * y;
             // |xz|^2 in the lanes of the lower half, xz . y in the upper half
@@ -203,33 +233,15 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
             v2[slot * B + (i >= rs ? i - rs : i - rs + B)] = v;
             if (i == 0) tau2[slot] = tau;
         }
-        if (t > 0) {
-            T xp = xz;
-            pin(xp);  // after the reflector is on its way
-            // column sums of xz X0 over the warp's eight rows: exchange halves so that each
-            // lane ends with PH columns
-            T u[CPT];
+        auto form_p = [&]() {
+            if (tid < B) {
+                T s = upart[0][tid];
 #pragma unroll
-            for (int q = 0; q < CPT; ++q) u[q] = xp * X[q];
-            if (first)
-#pragma unroll
-                for (int q = 0; q < CPT; ++q) xrow[c0 + q] = X[q];
-            int base = 0;
-#pragma unroll
-            for (int s = 0; s < 3; ++s) {
-                const int o = 16 >> s;
-                const int half = CPT >> (s + 1);
-                const bool up = (lane & o) != 0;
-#pragma unroll
-                for (int q = 0; q < half; ++q) {
-                    const T keep = up ? u[q + half] : u[q], give = up ? u[q] : u[q + half];
-                    u[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-                }
-                base += up ? half : 0;
+                for (int w = 1; w < NW; ++w) s += upart[w][tid];
+                ps[tid] = tau * (fma(scl, s, xrow[tid]) - fma(scl, xy, ysl[1]) * vps[par][tid]);
             }
-#pragma unroll
-            for (int q = 0; q < PH; ++q) upart[warp][c0 + base + q] = u[q];
-        }
+        };
+        if (t > 0 && !EARLY) column_sums();
         T qd;
         {
             T g = T(0), g1 = T(0);
@@ -244,6 +256,7 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
             const T dc = __shfl_sync(0xffffffffu, pick(D, rs % CPT), quad | (rs / CPT));
             qd = tau * fma(scl, g, dc);
         }
+        if (t > 0 && EARLY) form_p();
         if (part == 0) qs[i] = qd;
         {
             T kp = v * qd;
@@ -258,13 +271,10 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         // D - v w^T - w v^T with w = q - K v / 2, as D - v q^T - (q - K v) v^T
         T vd = v, w2 = fma(-K * tau, v, qd);
         if (t > 0) {
-            if (tid < B) {
-                T s = upart[0][tid];
-#pragma unroll
-                for (int w = 1; w < NW; ++w) s += upart[w][tid];
-                ps[tid] = tau * (fma(scl, s, xrow[tid]) - fma(scl, xy, ysl[1]) * vps[par][tid]);
+            if (!EARLY) {
+                form_p();
+                __syncthreads();
             }
-            __syncthreads();
             // ---- updates: X first, and the row that position t - 1 takes in at its next sweep
 #pragma unroll
             for (int q = 0; q < CPT; ++q) {
