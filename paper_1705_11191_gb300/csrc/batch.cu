@@ -42,6 +42,7 @@ struct BatchWorker {
 
 struct BatchState {
     elsi_gb_handle_s *sub = nullptr;  // solver instance the problems run in (worker 0)
+    cudaStream_t stream0 = nullptr;   // its stream next to other workers (created here)
     std::vector<BatchWorker> workers; // workers 1 .. W-1 (own handle, stream, host thread)
     std::vector<BatchItem> items;
     bool cplx = false;
@@ -316,11 +317,18 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
         }
         return true;
     };
-    auto instance = [&](int t, elsi_gb_handle_s **s, cudaStream_t *wst) {
+    // Instance t of W. Next to others the first one has a stream of its own too: streams are dealt out
+    // to the GPU's hardware queues (8 unless the process asks for more) in the order of their
+    // creation, so that 8 created one after the other have a queue each, and the caller's stream would
+    // share one with a worker's, whose two solves then run one after the other (8 solves of
+    // n = 2000: 92 ms against 69).
+    auto instance = [&](int t, int W, elsi_gb_handle_s **s, cudaStream_t *wst) {
         *s = (t == 0) ? b.sub : b.workers[t - 1].sub;
-        *wst = (t == 0) ? st : b.workers[t - 1].stream;
+        *wst = (t == 0) ? (W > 1 ? b.stream0 : st) : b.workers[t - 1].stream;
     };
     auto add_workers = [&](int W) -> int {
+        if (W > 1 && !b.stream0 && cudaStreamCreateWithFlags(&b.stream0, cudaStreamNonBlocking) != cudaSuccess)
+            return set_error(h, ELSI_ERR_CUDA, "batch worker stream");
         while ((int)b.workers.size() < W - 1) {
             BatchWorker wk;
             wk.sub = new (std::nothrow) elsi_gb_handle_s();
@@ -367,7 +375,7 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
                     cudaSetDevice(dev);
                     elsi_gb_handle_s *s;
                     cudaStream_t wst;
-                    instance(t, &s, &wst);
+                    instance(t, W, &s, &wst);
                     double *vals, *vecs;
                     scratch(t, &vals, &vecs);
                     ConcurrentSolves share;
@@ -378,6 +386,8 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
                             rr[t].rc = ELSI_ERR_CUDA;
                             rr[t].msg = cudaGetErrorString(ce);
                         }
+                    } else {
+                        cudaStreamSynchronize(wst);
                     }
                 };
                 for (int t = 1; t < W; ++t) th.emplace_back(one, t);
@@ -469,13 +479,35 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
     }
     rc = add_workers(W);
     if (rc) return rc;
+    // Every instance has room for the largest problem from the start (W is bounded for that): which
+    // instance takes which problem changes from call to call, and one that has to grow frees and
+    // allocates while the others compute (90 to 130 ms for a batch of 55).
+    if (W > 1) {
+        size_t nmax = 0, kmax = 0;
+        int imax = 0;
+        for (int i = 0; i < nprob; ++i) {
+            const size_t N = (size_t)mult * b.items[i].n, K = (size_t)mult * b.items[i].k;
+            if (N > nmax) { nmax = N; imax = i; }
+            if (K > kmax) kmax = K;
+        }
+        for (int t = 0; t < W; ++t) {
+            elsi_gb_handle_s *s;
+            cudaStream_t wst;
+            instance(t, W, &s, &wst);
+            configure(s, wst, tv[imax]);
+            s->n = (int)nmax;
+            s->n_state = (int)(kmax < nmax ? kmax : nmax);
+            const int kz = s->precision == ELSI_PREC_FP32_REFINE ? s->n : s->n_state;
+            if (ensure_workspace(s, kz) != ELSI_OK) free_workspace(s);  // the solve asks for what it needs
+        }
+    }
     std::vector<Result> res(W);
     std::atomic<int> next{0};
     auto work = [&](int t) {
         cudaSetDevice(dev);
         elsi_gb_handle_s *s;
         cudaStream_t wst;
-        instance(t, &s, &wst);
+        instance(t, W, &s, &wst);
         Result &r = res[t];
         ConcurrentSolves share;
         for (;;) {
@@ -486,6 +518,7 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
             share.set(W < nprob - q ? W : nprob - q);
             if (!solve_one(s, wst, i, tv[i], b.vals + it.off_val, b.vecs + it.off_vec, r)) {
                 next.store(nprob);  // the other instances stop after their current problem
+                cudaStreamSynchronize(wst);  // nothing reads the inputs any more
                 return;
             }
             const cudaError_t ce = cplx ? pair_evals(wst, it.k, b.vals + it.off_val, b.lvl + it.off_lvl)
@@ -678,6 +711,7 @@ void free_batch(elsi_gb_handle_s *h)
         }
         if (wk.stream) cudaStreamDestroy(wk.stream);
     }
+    if (b.stream0) cudaStreamDestroy(b.stream0);
     delete h->batch;
     h->batch = nullptr;
 }
