@@ -32,7 +32,8 @@
 // 60.3 -> 16.0 ms, n = 16384 245 -> 70 ms (14.7 -> 3.5 - 4.3 us a sweep, two L2 hand-overs and
 // two steps' arithmetic); binary64, b = 64, n = 512 15.2 -> 11.0 ms, n = 1531 51.3 -> 35.7 ms (a
 // step's 28 000 FMAs at two a clock bound it), and with b = 32 4.5 and 14.0 ms, 3.8 and 11.9 with
-// the early messages (3.9, 12.3) and the shorter reciprocals of packets.cuh.
+// the early messages (3.9, 12.3) and the shorter reciprocals of packets.cuh. As one cluster, up to 16
+// positions: n = 512 3.8 -> 3.5 ms, binary32 n = 777 2.65 -> 2.27 ms.
 #include "common.cuh"
 #include "kernels.h"
 #include "packets.cuh"
@@ -53,7 +54,7 @@ struct Args {
 __device__ __forceinline__ void pin(double &x) { asm volatile("" : "+d"(x)); }
 __device__ __forceinline__ void pin(float &x) { asm volatile("" : "+f"(x)); }
 
-template <typename T, int B>
+template <typename T, int B, bool CL>
 __global__ void __launch_bounds__(4 * B, 512 / (4 * B))
 chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, double *eout, const Args a)
 {
@@ -76,6 +77,28 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
     constexpr int REC = kWords<T> * (B + 2);
     u64 *vin = a.vmsg + (size_t)(t > 0 ? t - 1 : 0) * REC, *vout = a.vmsg + (size_t)t * REC;
     u64 *rin = a.rmsg + (size_t)t * REC, *rout = a.rmsg + (size_t)(t > 0 ? t - 1 : 0) * REC;
+    // CL: the positions are one cluster (and some idle CTAs), messages go to the reader's shared memory
+    __shared__ u64 vbox[CL ? REC : 1], rbox[CL ? REC : 1];
+    unsigned vto = 0, rto = 0;
+    if (CL) {
+        for (int q = tid; q < REC; q += 4 * B) vbox[CL ? q : 0] = rbox[CL ? q : 0] = 0;
+        vto = cluster_addr(vbox, min(t + 1, (int)gridDim.x - 1));
+        rto = cluster_addr(rbox, max(t - 1, 0));
+        __syncwarp();
+        cluster_sync();
+    }
+    auto put_v = [&](int q, T x, unsigned seq) {
+        if (CL) put_cluster(vto + 8 * kWords<T> * q, x, seq); else put(vout + q * kWords<T>, x, seq);
+    };
+    auto put_r = [&](int q, T x, unsigned seq) {
+        if (CL) put_cluster(rto + 8 * kWords<T> * q, x, seq); else put(rout + q * kWords<T>, x, seq);
+    };
+    auto get_v = [&](int q, unsigned seq, T &x) {
+        return CL ? get_own(vbox + q * kWords<T>, seq, x, a.spin_limit, a.status) : get(vin + q * kWords<T>, seq, x, a.spin_limit, a.status);
+    };
+    auto get_r = [&](int q, unsigned seq, T &x) {
+        return CL ? get_own(rbox + q * kWords<T>, seq, x, a.spin_limit, a.status) : get(rin + q * kWords<T>, seq, x, a.spin_limit, a.status);
+    };
 
     if (t == 0)  // defined values should a wait run out below
         for (int q = tid; q < n; q += 4 * B) {
@@ -99,10 +122,10 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         if (t == 0 && gi < n) x0 = band[gi];  // column 0, rows 1 .. B
     }
     __syncthreads();
-    if (failed) return;
+    const bool off = failed || t >= a.S;
 
     int rs = 1 % B;      // slot of the first row (and, for t > 0, of the first column of X)
-    for (int j = 0; j < nsweep; ++j) {
+    for (int j = 0; j < nsweep && !off; ++j) {
         const int r = j + 1 + t * B;
         if (r > n - 1) break;
         const int par = j & 1;
@@ -121,26 +144,26 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
             bool ok = true;
             if (tid < B) {
                 T v = T(0);
-                if (t > 0) ok = get(vin + tid * kWords<T>, (unsigned)j + 1, v, a.spin_limit, a.status);
+                if (t > 0) ok = get_v(tid, (unsigned)j + 1, v);
                 vps[par][tid] = v;
             } else if (tid < 2 * B) {
                 const int c = tid - B;
                 T v = T(0);
-                if (have_row) ok = get(rin + c * kWords<T>, (unsigned)j, v, a.spin_limit, a.status);
+                if (have_row) ok = get_r(c, (unsigned)j, v);
                 rows_[par][c] = v;
             } else if (tid == 2 * B) {
                 T v = T(0);
-                if (t > 0) ok = get(vin + B * kWords<T>, (unsigned)j + 1, v, a.spin_limit, a.status);
+                if (t > 0) ok = get_v(B, (unsigned)j + 1, v);
                 msc[par][0] = v;
             } else if (tid == 2 * B + 32) {
                 T v = T(0);
-                if (have_row) ok = get(rin + B * kWords<T>, (unsigned)j, v, a.spin_limit, a.status);
+                if (have_row) ok = get_r(B, (unsigned)j, v);
                 msc[par][1] = v;
             }
             if (!ok) failed = 1;
         }
         __syncthreads();
-        if (failed) return;
+        if (failed) break;
         // ---- slot pr takes the new row and column
         if (j > 0) {
             if (i == pr) {
@@ -225,8 +248,8 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         reflector<T>(alpha, ss, beta, tau, scl);
         const T v = first ? T(1) : xz * scl;
         if (part == 0) {
-            if (have_next) put(vout + i * kWords<T>, v, (unsigned)j + 1);
-            if (i == 0 && have_next) put(vout + B * kWords<T>, tau, (unsigned)j + 1);
+            if (have_next) put_v(i, v, (unsigned)j + 1);
+            if (i == 0 && have_next) put_v(B, tau, (unsigned)j + 1);
             vs[i] = v;
         } else if (part == 1) {
             const size_t slot = (size_t)j * a.S + t;
@@ -285,10 +308,10 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
 #pragma unroll
                 for (int q = 0; q < CPT; ++q) {
                     const int c = c0 + q;
-                    put(rout + c * kWords<T>, c == rs ? beta : X[q], (unsigned)j + 1);
+                    put_r(c, c == rs ? beta : X[q], (unsigned)j + 1);
                 }
                 if (part == rs / CPT)
-                    put(rout + B * kWords<T>, fma(-v, qs[rs], fma(-w2, vs[rs], pick(D, rs % CPT))), (unsigned)j + 1);
+                    put_r(B, fma(-v, qs[rs], fma(-w2, vs[rs], pick(D, rs % CPT))), (unsigned)j + 1);
             }
             pin(vd);
             pin(w2);  // D after the row is on its way
@@ -313,6 +336,10 @@ chase_resident_kernel(const T *__restrict__ band, T *v2, T *tau2, double *dout, 
         // the next step's first barrier.
         rs = rs + 1 == B ? 0 : rs + 1;
     }
+    if (CL) {
+        __syncwarp();
+        cluster_sync();  // nobody stores to the shared memory of a CTA that has ended
+    }
 }
 
 template <typename T, int B>
@@ -320,19 +347,49 @@ cudaError_t launch(cudaStream_t st, int n, const T *band, int ldb, double *d, do
                    int *status, unsigned *sync, size_t sync_words, int num_sms)
 {
     const int S = sb2st_steps(n, B);
-    int per_sm = 0;
-    cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chase_resident_kernel<T, B>, 4 * B, 0);
-    if (err != cudaSuccess) return err;
-    const size_t words = (size_t)S * kWords<T> * (B + 2);
-    if (S > per_sm * num_sms || 64 + 4 * words > sync_words) return cudaErrorNotSupported;
     Args a;
     a.n = n; a.ldb = ldb; a.S = S; a.status = status; a.spin_limit = spin_limit();
     a.vmsg = reinterpret_cast<u64 *>(sync + 64);
+    a.rmsg = a.vmsg;
+    void *args[] = {&band, &v2, &tau2, &d, &e, &a};
+    cudaError_t err;
+    // Up to 16 positions (the largest cluster): every hand-over is a store to another SM's shared memory
+    // instead of a store to and a load from L2. One pair that goes through L2 would set the pace of all.
+    if (S <= 16) {
+        auto *kernel = chase_resident_kernel<T, B, true>;
+        static PerDeviceOnce attr;  // per instantiation
+        err = once_per_device(attr, [&] {
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        });
+        if (err != cudaSuccess) return err;
+        unsigned size = 1;
+        while ((int)size < S) size *= 2;
+        cudaLaunchAttribute dim[1];
+        dim[0].id = cudaLaunchAttributeClusterDimension;
+        dim[0].val.clusterDim.x = size;
+        dim[0].val.clusterDim.y = dim[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(size);
+        cfg.blockDim = dim3(4 * B);
+        cfg.stream = st;
+        cfg.attrs = dim;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0) {
+            EGB_COUNT_LAUNCH();
+            return cudaLaunchKernelExC(&cfg, (void *)kernel, args);
+        }
+        cudaGetLastError();
+    }
+    int per_sm = 0;
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chase_resident_kernel<T, B, false>, 4 * B, 0);
+    if (err != cudaSuccess) return err;
+    const size_t words = (size_t)S * kWords<T> * (B + 2);
+    if (S > per_sm * num_sms || 64 + 4 * words > sync_words) return cudaErrorNotSupported;
     a.rmsg = a.vmsg + words;
     if ((err = cudaMemsetAsync(a.vmsg, 0, 2 * words * sizeof(u64), st)) != cudaSuccess) return err;
-    void *args[] = {&band, &v2, &tau2, &d, &e, &a};
     EGB_COUNT_LAUNCH();
-    return cudaLaunchCooperativeKernel((void *)chase_resident_kernel<T, B>, dim3(S), dim3(4 * B), args, 0, st);
+    return cudaLaunchCooperativeKernel((void *)chase_resident_kernel<T, B, false>, dim3(S), dim3(4 * B), args, 0, st);
 }
 
 }  // namespace sys

@@ -67,6 +67,55 @@ __device__ __forceinline__ bool get(const u64 *p, unsigned seq, T &v, long long 
     return true;
 }
 
+// The same between the CTAs of a cluster: the words are in the reader's shared memory, the writer
+// stores to them there (cluster_addr: a shared-memory address of the CTA with this rank).
+__device__ __forceinline__ unsigned cluster_addr(const void *p, int rank)
+{
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void st_cluster(unsigned p, u64 v)
+{
+    asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ u64 ld_own(const u64 *p)
+{
+    u64 v;
+    asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(v) : "r"((unsigned)__cvta_generic_to_shared(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void put_cluster(unsigned p, float v, unsigned seq) { st_cluster(p, word(__float_as_uint(v), seq)); }
+__device__ __forceinline__ void put_cluster(unsigned p, double v, unsigned seq)
+{
+    st_cluster(p, word((unsigned)__double2loint(v), seq));
+    st_cluster(p + 8, word((unsigned)__double2hiint(v), seq));
+}
+__device__ __forceinline__ bool try_get_own(const u64 *p, unsigned seq, float &v)
+{
+    const u64 a = ld_own(p);
+    v = __uint_as_float((unsigned)a);
+    return seq_of(a) == seq;
+}
+__device__ __forceinline__ bool try_get_own(const u64 *p, unsigned seq, double &v)
+{
+    const u64 a = ld_own(p), b = ld_own(p + 1);
+    v = __hiloint2double((int)(unsigned)b, (int)(unsigned)a);
+    return seq_of(a) == seq && seq_of(b) == seq;
+}
+template <typename T>
+__device__ __forceinline__ bool get_own(const u64 *p, unsigned seq, T &v, long long limit, int *status)
+{
+    long long it = 0;
+    while (!try_get_own(p, seq, v))
+        if (!poll_again(it, limit, status, (int)seq)) return false;
+    return true;
+}
+
 }  // namespace pkt
 
 // 1 / x and 1 / sqrt(x) to about an ulp: the hardware's approximation (about 2^-20 in binary64) and
