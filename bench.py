@@ -565,9 +565,9 @@ def batch_workloads(egb, torch, dev, stream, steps: int) -> dict:
 _STAGE_KERNEL = {
     "cholesky": ("potrf_diag_kernel + gemm_tf32x3_kernel", "tf32"),
     "standard_form": ("gemm_tf32x3_kernel (blocked triangular solves)", "tf32"),
-    "full_to_band": ("panel_qr_kernel + w_stage kernels + gemm_tf32x3_kernel", "tf32"),
-    "band_to_tri": ("chase_kernel", None),
-    "tridiag_solve": ("bisect_kernel + twisted_kernel", None),
+    "full_to_band": ("panel_kernel + symm_tall_kernel + w_stage kernels + gemm_tf32x3_kernel", "tf32"),
+    "band_to_tri": ("chase_resident_kernel", None),
+    "tridiag_solve": ("bisect_kernel + twist_factor_kernel + twist_vector_kernel", None),
     "back_q2": ("q2_apply_tc5_kernel (two launches: block ranges) + q2_factor_kernel", "tf32"),
     "back_q1": ("gemm_tf32x3_kernel", "tf32"),
     "back_subst": ("gemm_tf32x3_kernel (blocked triangular solve)", "tf32"),
@@ -603,7 +603,13 @@ def stage_traffic(stage: str, n: int):
     if sha != m["sha256_16"]:
         return None  # the kernel changed since the counters were taken
     return m["bytes"] * (n / m["n"]) ** 3
-OZAKI_PRODUCTS = 28  # bf16 digit products per binary64-accurate product (7 digits, 8 levels)
+
+
+def ozaki_products(stage: str, refine_iters: int) -> float:
+    """bf16 digit products per binary64-accurate product: 21 with six nine-bit digits (P, W and the
+    passes of the refinement from the third on), 10 with four (its first two); the mean over passes."""
+    passes = refine_iters + 1
+    return 21.0 if stage != "refine" or passes <= 0 else (10.0 * min(passes, 2) + 21.0 * max(passes - 2, 0)) / passes
 
 
 def _peaks():
@@ -647,9 +653,10 @@ def roofline_for(stage: str, stage_ms: float, n: int, k: int, prec: int, clocks:
     the stage's device time (CUDA events recorded on the solve stream around the stage).
     Tensor-core stages take the measured sustained bf16 rate of MEASURED_PEAKS.json (times
     the nominal tf32/bf16 ratio for tf32 work; binary64-accurate Ozaki products are
-    counted as their 28 bf16 digit products); the bulge chase takes band bytes against the
-    measured copy bandwidth; binary64 (SIMT) and ALU-bound stages take the binary64 FMA
-    rate derived from unit counts (152 SMs x 2 DFMA/clk x 2070 MHz)."""
+    counted as their bf16 digit products); the bulge chase takes band bytes against the
+    measured copy bandwidth; ALU-bound stages and the binary64 route take the binary64 FMA
+    rate derived from unit counts (152 SMs x 2 DFMA/clk x 2070 MHz; the digit products of
+    that route pass it)."""
     peaks, src = _peaks()
     bf16 = peaks.get("bf16_tflops_sustained") or 1700.0
     hbm = peaks.get("hbm_gbs") or 6800.0
@@ -674,9 +681,10 @@ def roofline_for(stage: str, stage_ms: float, n: int, k: int, prec: int, clocks:
                              ("" if work else "; no dense-flop count for this stage"))
         return out
     if dt == "bf16":
-        tc_work = OZAKI_PRODUCTS * work
+        products = ozaki_products(stage, refine_iters)
+        tc_work = products * work
         peak = bf16
-        note = (f"bf16_tflops_sustained {src}; {OZAKI_PRODUCTS} bf16 digit products per "
+        note = (f"bf16_tflops_sustained {src}; {products:.1f} bf16 digit products per "
                 "binary64-accurate flop")
     else:
         tc_work = work
