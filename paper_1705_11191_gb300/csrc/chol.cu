@@ -125,7 +125,7 @@ static cudaError_t launch_potrf_diag(cudaStream_t st, int jb, T *a, int lda, T *
 // panel's L (right triangular solve by blocks), and the trailing matrix gets one rank-
 // kTriPanel update per panel.
 template <typename T>
-cudaError_t potrf(cudaStream_t st, int n, T *a, int lda, T *inv_diag, T *work, int *status)
+cudaError_t potrf(cudaStream_t st, int n, T *a, int lda, T *inv_diag, int *status)
 {
     const int nb = kTriBlock, np = kTriPanel;
     cudaError_t e;
@@ -208,17 +208,17 @@ static cudaError_t trsm_range(cudaStream_t st, int trans, bool halves, int r0, i
 
 template <typename T>
 cudaError_t trsm_left_lower(cudaStream_t st, int trans, int n, int ncol, const T *L, int ldl,
-                            const T *inv_diag, T *B, int ldb, T *)
+                            const T *inv_diag, T *B, int ldb)
 {
     if (n <= 0 || ncol <= 0) return cudaSuccess;
     return trsm_range<T>(st, trans, n >= 4096, 0, n, ncol, L, ldl, inv_diag, n, B, ldb);
 }
 
-template cudaError_t potrf<double>(cudaStream_t, int, double *, int, double *, double *, int *);
-template cudaError_t potrf<float>(cudaStream_t, int, float *, int, float *, float *, int *);
+template cudaError_t potrf<double>(cudaStream_t, int, double *, int, double *, int *);
+template cudaError_t potrf<float>(cudaStream_t, int, float *, int, float *, int *);
 template cudaError_t trsm_left_lower<double>(cudaStream_t, int, int, int, const double *, int,
-                                             const double *, double *, int, double *);
+                                             const double *, double *, int);
 template cudaError_t trsm_left_lower<float>(cudaStream_t, int, int, int, const float *, int,
-                                            const float *, float *, int, float *);
+                                            const float *, float *, int);
 
 }  // namespace egb

@@ -93,15 +93,15 @@ cudaError_t check_finite(cudaStream_t st, int m, int n, const T *a, int lda, int
 // receives the inverses of the nb x nb diagonal blocks of L (n x nb, block j at rows
 // j*nb). work: n x nb scratch. Status ELSI_ERR_NOT_PD with the pivot on failure.
 template <typename T>
-cudaError_t potrf(cudaStream_t st, int n, T *a, int lda, T *inv_diag, T *work, int *status);
+cudaError_t potrf(cudaStream_t st, int n, T *a, int lda, T *inv_diag, int *status);
 constexpr int kTriBlock = 64;   // nb of potrf / trsm
 constexpr int kTriPanel = 256;  // outer panel of potrf (rank-256 updates), and of trsm below n = 4096
 
 // B (n x ncol) := L^{-1} B (trans = 0) or L^{-T} B (trans = 1), L lower from potrf,
-// inv_diag its diagonal-block inverses. work: kTriBlock x ncol scratch.
+// inv_diag its diagonal-block inverses.
 template <typename T>
 cudaError_t trsm_left_lower(cudaStream_t st, int trans, int n, int ncol, const T *L, int ldl,
-                            const T *inv_diag, T *B, int ldb, T *work);
+                            const T *inv_diag, T *B, int ldb);
 
 // Columns that the refinement of the binary32 route works on for k wanted states: at least
 // 16 more (guard) columns, up to the next multiple of 128, the column tile of its products.

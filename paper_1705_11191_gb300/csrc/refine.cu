@@ -36,23 +36,6 @@ namespace egb {
                              cudaGetErrorString(_e));                                      \
     } while (0)
 
-// out1[j] = x_j . y1_j, out2[j] = x_j . y2_j (binary64), one CTA per column.
-__global__ void col_dots_kernel(int n, const double *x, const double *y1, const double *y2,
-                                double *out1, double *out2)
-{
-    __shared__ double red[32];
-    const int j = blockIdx.x;
-    const double *xc = x + (size_t)j * n, *a = y1 + (size_t)j * n, *b = y2 + (size_t)j * n;
-    double s1 = 0.0, s2 = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        s1 = fma(xc[i], a[i], s1);
-        s2 = fma(xc[i], b[i], s2);
-    }
-    s1 = block_sum(s1, red);
-    s2 = block_sum(s2, red);
-    if (threadIdx.x == 0) { out1[j] = s1; out2[j] = s2; }
-}
-
 // lam_j = g_j / s_j ; R_o = YH - YS diag(lam) (in place in yh), and a binary32 copy.
 __global__ void residual_kernel(int n, int k, const double *g, const double *s, double *lam,
                                 double *yh, const double *ys, float *r32)
@@ -456,7 +439,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
         CKR(check_finite<double>(st, n, n, rq.ovlp, n, w.status));
         CKR(check_finite<double>(st, n, n, rq.ham, n, w.status));
         CKR(copy_matrix<float, double>(st, n, n, rq.ovlp, n, L, n));
-        CKR(potrf<float>(st, n, L, n, INVD, WORK, w.status));
+        CKR(potrf<float>(st, n, L, n, INVD, w.status));
         CKR(cudaMemcpyAsync(w.status_host, w.status, sizeof(int) * ST_WORDS, cudaMemcpyDeviceToHost, st));
         CKR(cudaStreamSynchronize(st));
         if (w.status_host[ST_CODE] == ELSI_ERR_NOT_PD) {
@@ -471,7 +454,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
             CKR(copy_matrix<double, double>(st, n, n, rq.ovlp, n, L64, n));
             set_f64_tc_scratch(cdig, w.oz_cap / sizeof(__nv_bfloat16) - (size_t)4 * n * n, w.ozexp,
                                w.ozexp_cap / sizeof(int));
-            cudaError_t pe = potrf<double>(st, n, L64, n, INV64, w.edm, w.status);
+            cudaError_t pe = potrf<double>(st, n, L64, n, INV64, w.status);
             set_f64_tc_scratch(nullptr, 0, nullptr, 0);
             CKR(pe);
             CKR(copy_matrix<float, double>(st, n, n, L64, n, L, n));
@@ -489,9 +472,9 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     CKR(cudaEventRecord(w.ev[STAGE_STDFORM], st));
     if (!unit) {
         CKR(copy_matrix<float, double>(st, n, n, rq.ham, n, Y, n));
-        CKR(trsm_left_lower<float>(st, 0, n, n, L, n, INVD, Y, n, WORK));
+        CKR(trsm_left_lower<float>(st, 0, n, n, L, n, INVD, Y, n));
         CKR(transpose<float>(st, n, n, Y, n, A, n));
-        CKR(trsm_left_lower<float>(st, 0, n, n, L, n, INVD, A, n, WORK));
+        CKR(trsm_left_lower<float>(st, 0, n, n, L, n, INVD, A, n));
         CKR(symmetrize<float>(st, n, A, n));
     } else {
         CKR(copy_matrix<float, double>(st, n, n, rq.ham, n, A, n));
@@ -526,7 +509,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     if (one_stage) CKR(apply_q_onestage<float>(st, n, n, V1, T1, X32, n, WORK));
     else CKR(apply_q1<float>(st, n, b, n, V1, T1, X32, n, WORK));
     CKR(cudaEventRecord(w.ev[STAGE_BACKSUB], st));
-    if (!unit) CKR(trsm_left_lower<float>(st, 1, n, n, L, n, INVD, X32, n, WORK));
+    if (!unit) CKR(trsm_left_lower<float>(st, 1, n, n, L, n, INVD, X32, n));
     CKR(cudaEventRecord(w.ev[STAGE_REFINE], st));
 
     // ---------------- refinement of the kw wanted eigenpairs (and the guard columns)

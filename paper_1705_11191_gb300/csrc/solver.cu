@@ -166,7 +166,7 @@ static int solve_fp64(elsi_gb_handle_s *h, const SolveRequest &rq)
     if (!unit && !(h->reuse_l && h->have_l && h->have_l_prec == ELSI_PREC_FP64)) {
         CK(check_finite<double>(st, n, n, rq.ovlp, n, w.status));
         CK(copy_matrix<double, double>(st, n, n, rq.ovlp, n, w.l, n));
-        CK(potrf<double>(st, n, w.l, n, w.invd, w.work, w.status));
+        CK(potrf<double>(st, n, w.l, n, w.invd, w.status));
         h->have_l_prec = ELSI_PREC_FP64;
     }
     CK(cudaEventRecord(w.ev[STAGE_STDFORM], st));
@@ -175,9 +175,9 @@ static int solve_fp64(elsi_gb_handle_s *h, const SolveRequest &rq)
     double *A = w.a;
     if (!unit) {
         CK(copy_matrix<double, double>(st, n, n, rq.ham, n, w.edm, n));
-        CK(trsm_left_lower<double>(st, 0, n, n, w.l, n, w.invd, w.edm, n, w.work));  // Y = L^{-1} H
+        CK(trsm_left_lower<double>(st, 0, n, n, w.l, n, w.invd, w.edm, n));  // Y = L^{-1} H
         CK(transpose<double>(st, n, n, w.edm, n, A, n));                             // Y^T
-        CK(trsm_left_lower<double>(st, 0, n, n, w.l, n, w.invd, A, n, w.work));      // L^{-1} Y^T
+        CK(trsm_left_lower<double>(st, 0, n, n, w.l, n, w.invd, A, n));              // L^{-1} Y^T
         CK(symmetrize<double>(st, n, A, n));
     } else {
         CK(copy_matrix<double, double>(st, n, n, rq.ham, n, A, n));
@@ -213,7 +213,7 @@ static int solve_fp64(elsi_gb_handle_s *h, const SolveRequest &rq)
     else CK(apply_q1<double>(st, n, b, k, w.v1, w.t1, w.z, n, w.work));
     CK(cudaEventRecord(w.ev[STAGE_BACKSUB], st));
     // ---- Eq. 9: c = L^{-T} c~
-    if (!unit) CK(trsm_left_lower<double>(st, 1, n, k, w.l, n, w.invd, w.z, n, w.work));
+    if (!unit) CK(trsm_left_lower<double>(st, 1, n, k, w.l, n, w.invd, w.z, n));
     CK(cudaEventRecord(w.ev[STAGE_REFINE], st));
     CK(cudaEventRecord(w.ev[STAGE_OCC], st));
     if (ev_mode) {
