@@ -20,39 +20,40 @@ namespace egb {
 // hold the Schur complement in the columns c > k and, in the columns c <= k, the rows of the
 // unit lower-triangular inverse (row i -= (a_ik / d_k) row k, with the identity understood in
 // the columns already eliminated). L = columns / sqrt(d_k), inverse = rows / sqrt(d_i). Thread
-// (row i, quarter of the columns) keeps its 16 entries in registers; a step publishes the
-// pivot row and 1 / d_k through shared memory and has one block barrier. What bounds it: 64
-// dependent steps, each a reciprocal, a barrier and a rank-1 update (in binary64 up to 4096
-// FMAs at two a clock). Factorising in shared memory with three barriers a step and then
-// inverting column by column took 85 us (binary32) and 210 us (binary64) a block, this 37 and
-// 100 us.
+// (row i, every fourth column) keeps its 16 entries in registers; a step publishes the pivot row
+// and 1 / d_k through shared memory and has one block barrier. The steps are unrolled by register
+// (four steps, one per column of a quad, in a loop), so that column k needs no search through the
+// registers. What bounds it: 64 dependent steps, each a reciprocal, a barrier and a rank-1 update
+// (in binary64 up to 4096 FMAs at two a clock). Factorising in shared memory with three barriers a
+// step and then inverting column by column took 85 us (binary32) and 210 us (binary64) a block, with
+// 16 consecutive columns a thread, picked out by predicated moves, 40 and 96 us, this 23 and 76 us.
 template <typename T>
 __global__ void __launch_bounds__(4 * kTriBlock)
 potrf_diag_kernel(int jb, T *a, int lda, T *inv, int ldi, int *status, int pivot_base)
 {
     constexpr int B = kTriBlock, CPT = B / 4;
-    __shared__ __align__(16) T prow[2][B];  // pivot row
-    __shared__ T prec[2];                   // 1 / d_k
-    __shared__ T piv[B];                    // d_k
-    __shared__ T Ls[B][B + 1];              // a_ik (i > k), by column
+    __shared__ __align__(16) T prow[2][4][CPT];  // pivot row: [part][q] is column 4 q + part
+    __shared__ T prec[2];                        // 1 / d_k
+    __shared__ T piv[B];                         // d_k
+    __shared__ T Ls[B][B + 1];                   // a_ik (i > k), by column
     __shared__ int bad;
     const int tid = threadIdx.x, lane = tid & 31, quad = lane & ~3;
-    const int i = tid >> 2, part = tid & 3, c0 = part * CPT;
+    const int i = tid >> 2, part = tid & 3;
     T E[CPT];
 #pragma unroll
     for (int q = 0; q < CPT; ++q) {
-        const int c = c0 + q, hi = max(i, c), lo = min(i, c);
+        const int c = 4 * q + part, hi = max(i, c), lo = min(i, c);
         E[q] = hi < jb ? a[(size_t)hi + (size_t)lo * lda] : (i == c ? T(1) : T(0));
     }
     if (tid == 0) bad = -1;
-    // the row of the next pivot and its reciprocal, published by the row's four threads
-    auto publish = [&](int k) {
+    // row k of the next pivot and its reciprocal, published by the row's four threads; e is the entry
+    // of the thread's column in the quad of column k
+    auto publish = [&](int k, T e) {
         if (i == k) {
-            const T d0 = pick(E, k % CPT);
 #pragma unroll
-            for (int q = 0; q < CPT; ++q) prow[k & 1][c0 + q] = E[q];
-            if (part == k / CPT) {
-                T d = d0;
+            for (int q = 0; q < CPT; ++q) prow[k & 1][part][q] = E[q];
+            if (part == (k & 3)) {
+                T d = e;
                 if (!(d > T(0)) || !isfinite(d)) {
                     if (bad < 0) bad = k;
                     d = T(1);  // keep going with a harmless pivot; the status reports the failure
@@ -63,40 +64,41 @@ potrf_diag_kernel(int jb, T *a, int lda, T *inv, int ldi, int *status, int pivot
         }
     };
     __syncthreads();
-    publish(0);
+    publish(0, E[0]);
     __syncthreads();
-    for (int k = 0; k < B; ++k) {
-        const T aik = __shfl_sync(0xffffffffu, pick(E, k % CPT), quad | (k / CPT));
-        if (i > k) {
-            const T f = aik * prec[k & 1];
-            if (part == 0) Ls[k][i] = aik;
 #pragma unroll
-            for (int q = 0; q < CPT; ++q) E[q] = fma(-f, prow[k & 1][c0 + q], E[q]);
-            if (part == k / CPT)
+    for (int qk = 0; qk < CPT; ++qk)
+#pragma unroll 1
+        for (int pk = 0; pk < 4; ++pk) {
+            const int k = 4 * qk + pk;
+            const T aik = __shfl_sync(0xffffffffu, E[qk], quad | pk);
+            if (i > k) {
+                const T f = aik * prec[k & 1];
+                if (part == 0) Ls[k][i] = aik;
 #pragma unroll
-                for (int q = 0; q < CPT; ++q) move_if(E[q], -f, k % CPT, q);
-        } else if (i == k && part == k / CPT) {
-            // row k is finished: its entry k of the unit triangular inverse
-#pragma unroll
-            for (int q = 0; q < CPT; ++q) move_if(E[q], T(1), k % CPT, q);
+                for (int q = 0; q < CPT; ++q) E[q] = fma(-f, prow[k & 1][part][q], E[q]);
+                if (part == pk) E[qk] = -f;
+            } else if (i == k && part == pk) {
+                E[qk] = T(1);  // row k is finished: its entry k of the unit triangular inverse
+            }
+            if (k + 1 < B) publish(k + 1, pk < 3 ? E[qk] : E[qk + 1 < CPT ? qk + 1 : qk]);
+            __syncthreads();
+            // row k enters the following steps with a 1 in column k; the others read it here
         }
-        if (k + 1 < B) publish(k + 1);
-        __syncthreads();
-        // row k enters the following steps with a 1 in column k; the others read it here
-    }
     if (tid == 0 && bad >= 0) report_error(status, ELSI_ERR_NOT_PD, pivot_base + bad);
     // L and the inverse; Ls holds a_ik, scaled by 1 / sqrt(d_k)
-    if (tid < B) prow[0][tid] = T(1) / dsqrt(piv[tid]);
+    T *rs = &prow[0][0][0];
+    if (tid < B) rs[tid] = T(1) / dsqrt(piv[tid]);
     __syncthreads();
-    const T ri = prow[0][i];
+    const T ri = rs[i];
 #pragma unroll
     for (int q = 0; q < CPT; ++q) {
-        const int c = c0 + q;
+        const int c = 4 * q + part;
         if (i < jb && c < jb) inv[(size_t)i + (size_t)c * ldi] = c <= i ? ri * E[q] : T(0);
     }
     for (int e = tid; e < jb * jb; e += 4 * B) {
         const int r = e % jb, c = e / jb;
-        a[(size_t)r + (size_t)c * lda] = r > c ? Ls[c][r] * prow[0][c] : (r == c ? dsqrt(piv[c]) : T(0));
+        a[(size_t)r + (size_t)c * lda] = r > c ? Ls[c][r] * rs[c] : (r == c ? dsqrt(piv[c]) : T(0));
     }
 }
 
