@@ -409,7 +409,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
 {
     Workspace &w = h->wk;
     cudaStream_t st = h->stream;
-    const int n = h->n, kw = h->n_state, b = h->band_width;
+    const int n = h->n, kw = h->n_state, b = band_of(h, ELSI_PREC_FP32_REFINE);
     const int k = refine_block(n, kw);  // wanted states and guard columns
     const int kc = kw + 8 < k ? kw + 8 : k;  // columns whose convergence is checked
     const bool unit = h->overlap_is_unit;
