@@ -29,6 +29,16 @@ __device__ __forceinline__ double guard_pivot(double q, double pivmin)
     return (fabs(q) < pivmin) ? -pivmin : q;
 }
 
+// p and pm times the power of two that brings |p| to [1, 2), or |pm| to 2^500 if it would pass that.
+__device__ __forceinline__ void sturm_rescale(double &p, double &pm)
+{
+    const int ep = (__double2hiint(p) >> 20) & 0x7FF, em = (__double2hiint(pm) >> 20) & 0x7FF;
+    const int f = max(min(2046 - max(ep, 1), 2546 - em), 1);
+    const double s = __hiloint2double(f << 20, 0);
+    p *= s;
+    pm *= s;
+}
+
 // number of eigenvalues < sigma: the sign changes of the leading principal minors
 // p_i = det(T[0:i, 0:i] - sigma I), p_0 = 1, p_{i+1} = (d_i - sigma) p_i - e_{i-1}^2 p_{i-1}
 // (Sturm; Givens 1954), e2 = e^2. The ratio q_i = p_{i+1} / p_i is the pivot of the LDL^T
@@ -37,12 +47,17 @@ __device__ __forceinline__ double guard_pivot(double q, double pivmin)
 // operations of the recurrence is done on the bit patterns: on this chip a warp holds its
 // scheduler's binary64 unit for 64 cycles with every addition, product or comparison. Signs
 // come from the sign bits; the test for a tiny pivot is made when the exponent of p_{i+1} is
-// below that of pivmin 2^460 >= pivmin |p_i| (it always is for a zero). The pair (p_i, p_{i-1})
-// is rescaled by an exact power of two when |p_i| leaves [2^-200, 2^200], every 8 steps, which
-// keeps |p| below 2^460 for ||T|| up to 2^31.
+// below that of pivmin 2^460 >= pivmin |p_i| (it always is for a zero; a pivot that this test lets
+// through has the sign of its computed value, which is as good). The pair (p_i, p_{i-1}) is
+// multiplied by the power of two that puts |p_i| next to 1 (sturm_rescale) when one of the two has
+// left [2^-200, 2^200] at the end of eight steps, so that every piece starts there whatever
+// ||T|| is: a fixed factor of 2^200 a piece loses to steps of more than 25 bits, and the counts of
+// ||T|| below 2^-24 or above 2^26 were wrong. Eight steps of up to 100 bits each stay in range; a
+// piece with a value out of range (an infinity or a NaN, or one so small that digits may be lost) is
+// done again step by step, rescaled before each.
 // A warp issues in order, so eight steps are one straight piece without a branch: the next d and
-// e^2 are on their way, the eight d_i - sigma do not wait for the chain, and a piece with a tiny
-// pivot (seen afterwards, from the smallest exponent) is done again step by step.
+// e^2 are on their way, the eight d_i - sigma do not wait for the chain, and what has to be done
+// again is seen afterwards, from the smallest and the largest exponent.
 // Measured against a form with a binary64 product and comparison for the pivot test, sign
 // comparisons and e^2 formed on the way (8 such operations a step, eigenvalues by 8 or 2 lanes
 // at every count), the bisection: n = 1531, 382 values 8.7 -> 4.1 ms; n = 4096, all 15.2 -> 7.1
@@ -58,9 +73,10 @@ __device__ int sturm_count(int n, const double *__restrict__ d, const double *__
     unsigned cnt = 0;
     auto steps = [&](int i0, int i1) {
         for (int i = i0; i < i1; ++i) {
+            sturm_rescale(p, pm);
             double pn = fma(d[i] - sigma, p, -e2[i] * pm);
             // pivot q = pn / p below pivmin in magnitude: q = -pivmin
-            if ((__double2hiint(pn) & 0x7FF00000) <= tiny && fabs(pn) < pivmin * fabs(p)) pn = -pivmin * p;
+            if (fabs(pn) < pivmin * fabs(p)) pn = -pivmin * p;
             cnt += (unsigned)(__double2hiint(pn) ^ __double2hiint(p)) >> 31;
             pm = p;
             p = pn;
@@ -82,25 +98,25 @@ __device__ int sturm_count(int n, const double *__restrict__ d, const double *__
         }
         const double p0 = p, pm0 = pm;
         unsigned c = 0;
-        int least = 0x7FF00000;
+        int least = 0x7FF00000, most = 0;
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             const double pn = fma(x[q], p, -y[q] * pm);
             least = min(least, __double2hiint(pn) & 0x7FF00000);
+            most = max(most, __double2hiint(pn) & 0x7FF00000);
             c += (unsigned)(__double2hiint(pn) ^ __double2hiint(p)) >> 31;
             pm = p;
             p = pn;
         }
-        if (least <= tiny) {
+        if (least <= tiny || most == 0x7FF00000) {
             p = p0;
             pm = pm0;
             steps(i, i + P);
         } else {
             cnt += c;
         }
-        const int ex = __double2hiint(p) & 0x7FF00000;
-        if (ex > ((1023 + 200) << 20)) { p *= 0x1p-200; pm *= 0x1p-200; }
-        else if (ex < ((1023 - 200) << 20)) { p *= 0x1p200; pm *= 0x1p200; }
+        const int ex = __double2hiint(p) & 0x7FF00000, mx = max(ex, __double2hiint(pm) & 0x7FF00000);
+        if (mx > ((1023 + 200) << 20) || ex < ((1023 - 200) << 20)) sturm_rescale(p, pm);
     }
     steps(whole, n);
     return (int)cnt;
