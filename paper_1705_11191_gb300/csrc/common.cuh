@@ -21,7 +21,8 @@ extern std::atomic<long long> g_launches;
 // Device status word layout (one int array per handle, zeroed before each call):
 //   [0] first error code seen by any kernel (ELSI_ERR_*), 0 = none
 //   [1] auxiliary value (e.g. failing Cholesky pivot, 0-based)
-enum { ST_CODE = 0, ST_AUX = 1, ST_WORDS = 8 };
+//   [4] exponent field of the largest |W| of the current panel (sy2sb.cu)
+enum { ST_CODE = 0, ST_AUX = 1, ST_WEXP = 4, ST_WORDS = 8 };
 
 __device__ __forceinline__ void report_error(int *status, int code, int aux)
 {

@@ -322,17 +322,20 @@ static bool digits_pay(int m, int n, int k)
 }
 
 // C -= V W^T + W V^T (lower triangle, m x m, V and W m x b): one product over K = 2 b whose
-// operands' rows are [V_i W_i] and [W_i V_i].
+// operands' rows are [V_i W_i / s] and [W_i / s V_i], times s. A row has one exponent for both halves
+// (72 bits below its largest entry), so s, a power of two, makes W as large as V, which has unit
+// columns: without it the smaller half loses its digits once ||H~|| is beyond 2^+-20 (n = 1500,
+// eigenvalues of 2^40 H: 1.0e-8 of ||H|| off, now 6e-15).
 cudaError_t gemm_f64_two_sided(cudaStream_t st, int m, int b, const double *V, int ldv, const double *W,
-                               int ldw, double *C, int ldc)
+                               int ldw, double *C, int ldc, const int *wexp)
 {
     const size_t pe = ozaki_split_elems(m, 2 * b, kOzWide), xe = (size_t)ceil_div(m, 128) * 128;
     if (!digits_pay(m, m, 2 * b) || 2 * pe > t_oz_elems || 2 * xe > t_oz_exp_elems) return cudaErrorNotSupported;
     __nv_bfloat16 *ad = t_oz_planes, *bd = ad + pe;
     int *ea = t_oz_exps, *eb = ea + xe;
     cudaError_t e;
-    if ((e = ozaki_split(st, m, 2 * b, V, 1, ldv, nullptr, nullptr, ad, ea, kOzWide, W, ldw, b)) != cudaSuccess) return e;
-    if ((e = ozaki_split(st, m, 2 * b, W, 1, ldw, nullptr, nullptr, bd, eb, kOzWide, V, ldv, b)) != cudaSuccess) return e;
+    if ((e = ozaki_split_halves(st, m, b, V, ldv, W, ldw, wexp, false, ad, ea)) != cudaSuccess) return e;
+    if ((e = ozaki_split_halves(st, m, b, W, ldw, V, ldv, wexp, true, bd, eb)) != cudaSuccess) return e;
     return ozaki_gemm(st, m, m, 2 * b, -1.0, ad, ea, bd, eb, 1.0, C, ldc, 1, kOzWide);
 }
 

@@ -49,9 +49,10 @@ void set_tc_scratch(float *work, size_t elems, int *status);
 // of set_tc_scratch for timeouts.
 void set_f64_tc_scratch(__nv_bfloat16 *planes, size_t elems, int *exps, size_t exp_elems);
 // C -= V W^T + W V^T (lower triangle) as one digit product; cudaErrorNotSupported without
-// the scratch or when the product is too small for it.
+// the scratch or when the product is too small for it. wexp: exponent field of the largest |W|
+// (device).
 cudaError_t gemm_f64_two_sided(cudaStream_t st, int m, int b, const double *V, int ldv, const double *W,
-                               int ldw, double *C, int ldc);
+                               int ldw, double *C, int ldc, const int *wexp);
 cudaError_t tc_gemm_f32(cudaStream_t st, int ta, int tb, int m, int n, int k, float alpha,
                         const float *A, int lda, const float *B, int ldb, float beta, float *C,
                         int ldc, int uplo, float *work, size_t work_elems, int *status);
@@ -233,14 +234,18 @@ cudaError_t dup_pairs(cudaStream_t st, int n, const double *f, double *f2);
 // ---- binary64-accurate products on the bf16 tensor cores (ozaki.cu) ----
 // Splits V vectors of length K (element (v, q) at src[v * sv + q * sq], optionally times
 // scale[q] * scale2[q]) into the digit planes consumed by ozaki_gemm; the leading 'digits' of
-// them are written. With src2, element (v, q) for q >= k1 is src2[v * sv + (q - k1) * sq2].
+// them are written.
 constexpr int kOzDigits = 6;  // 9-bit digits of the refinement form: 53 bits below the largest entry
 constexpr int kOzWide = 8;    // of the binary64 route: 71 bits, sums in 128 bits
 size_t ozaki_split_elems(int V, int K, int digits = kOzDigits);  // bf16 elements of the planes
 cudaError_t ozaki_split(cudaStream_t st, int V, int K, const double *src, long long sv,
                         long long sq, const double *scale, const double *scale2,
-                        __nv_bfloat16 *planes, int *exps, int digits = kOzDigits,
-                        const double *src2 = nullptr, long long sq2 = 0, int k1 = 0);
+                        __nv_bfloat16 *planes, int *exps, int digits = kOzDigits);
+// kOzWide digits of vectors of length 2 k1 whose element (v, q) is src[v + q sq] for q < k1, else
+// src2[v + (q - k1) sq2]. One of the two (src if scaled_first, else src2) is of the size 2^e given
+// by the exponent field *wexp and is divided by 2^e, which goes to the exponents if scaled_first.
+cudaError_t ozaki_split_halves(cudaStream_t st, int V, int k1, const double *src, long long sq, const double *src2,
+                               long long sq2, const int *wexp, bool scaled_first, __nv_bfloat16 *planes, int *exps);
 // C (m x n, ldc) = alpha * A B + beta * C with A given by the split of its m rows and B
 // by the split of its n columns (both of length k). uplo = 1: lower triangle only.
 // digits (1..kOzDigits, or kOzWide; that of both splits, or for the refinement form less):

@@ -116,32 +116,60 @@ __device__ __forceinline__ void digits_of(double x, int e, unsigned (&d)[ND])
 
 __device__ __forceinline__ unsigned bf16_pair(unsigned a, unsigned b) { return __byte_perm(a, b, 0x7632); }
 
-// Vector v (0 <= v < V) has elements x(v, q), q < K: src[v * sv + q * sq], or for q >= k1 the
-// second source src2[v * sv + (q - k1) * sq2]; optional per-element factors scale[q],
-// scale2[q] (diagonal matrices multiplied in before splitting). The first nd of its digit
+// Vector v (0 <= v < V) has elements x(v, q) = src.at(v, q), q < K. The first nd of its digit
 // planes go to out[s * plane + v * ldo + q] (bf16, q < Kpad, zero padded), its exponent to
 // exps[v]. Vectors V <= v < Vpad get zero digits.
+//
+// One matrix, with optional per-element factors scale[q], scale2[q] (diagonal matrices multiplied
+// in before splitting)
 struct SplitSrc {
-    const double *src, *src2, *scale, *scale2;
-    long long sv, sq, sq2;
-    int k1;
+    const double *src, *scale, *scale2;
+    long long sv, sq;
+    __device__ __forceinline__ int prepare() { return 0; }  // what exps[v] is raised by
     __device__ __forceinline__ double at(int v, int q) const
     {
-        double x = q < k1 ? src[(size_t)v * sv + (size_t)q * sq] : src2[(size_t)v * sv + (size_t)(q - k1) * sq2];
+        double x = src[(size_t)v * sv + (size_t)q * sq];
         if (scale) x *= scale[q];
         if (scale2) x *= scale2[q];
         return x;
     }
 };
 
+// Two matrices side by side along q, rows consecutive in memory: V and W / 2^e in either order, 2^e
+// the size of W by its exponent field *wexp (e = 0 within 2^+-8, where 64 bits and more are left
+// of either half). A type of its own: the test of every element in SplitSrc took 2 % of a binary64
+// solve of n = 5000.
+struct SplitHalves {
+    const double *src, *src2;
+    long long sq, sq2;
+    int k1;
+    const int *wexp;
+    bool scaled_first;  // src is W: the vectors' exponents take the 2^e
+    double f1, f2;
+    __device__ __forceinline__ int prepare()
+    {
+        const int xf = *wexp;
+        int e = xf == 0 || xf == 2047 ? 0 : xf - 1022;
+        e = abs(e) <= 8 ? 0 : max(-1000, min(e, 1000));
+        const double f = __hiloint2double((1023 - e) << 20, 0);
+        f1 = scaled_first ? f : 1.0;
+        f2 = scaled_first ? 1.0 : f;
+        return scaled_first ? e : 0;
+    }
+    __device__ __forceinline__ double at(int v, int q) const
+    {
+        return q < k1 ? f1 * src[v + (size_t)q * sq] : f2 * src2[v + (size_t)(q - k1) * sq2];
+    }
+};
+
 // Vectors along memory (sq = 1): one CTA per vector.
-template <int ND>
-__global__ void __launch_bounds__(256) ozaki_split_kernel(int V, int K, int Kpad, const SplitSrc s, int nd,
+template <int ND, class Src>
+__global__ void __launch_bounds__(256) ozaki_split_kernel(int V, int K, int Kpad, Src s, int nd,
                                                           __nv_bfloat16 *__restrict__ out, int ldo, size_t plane,
                                                           int *__restrict__ exps)
 {
     __shared__ unsigned long long red[8];
-    const int v = blockIdx.x;
+    const int v = blockIdx.x, raise = s.prepare();
     unsigned long long mb = 0ull;
     if (v < V)
         for (int q = threadIdx.x; q < K; q += 256) {
@@ -157,7 +185,7 @@ __global__ void __launch_bounds__(256) ozaki_split_kernel(int V, int K, int Kpad
 #pragma unroll
     for (int w = 0; w < 8; ++w) mb = red[w] > mb ? red[w] : mb;
     const int e = row_exponent(mb);
-    if (threadIdx.x == 0) exps[v] = e;
+    if (threadIdx.x == 0) exps[v] = e + raise;
     unsigned *o = reinterpret_cast<unsigned *>(out + (size_t)v * ldo);
     for (int q = 2 * threadIdx.x; q < Kpad; q += 512) {
         unsigned a[ND], b[ND];
@@ -174,8 +202,8 @@ __global__ void __launch_bounds__(256) ozaki_split_kernel(int V, int K, int Kpad
 // element per 32-byte sector. Up to 256 elements of a vector are read once and kept in
 // registers; longer ones are read twice. (32 vectors per CTA read whole lines but left two
 // thirds of the SMs idle at n = 1531: 34 us at K = 256.)
-template <int ND>
-__global__ void __launch_bounds__(256) ozaki_split_t_kernel(int V, int K, int Kpad, const SplitSrc s, int nd,
+template <int ND, class Src>
+__global__ void __launch_bounds__(256) ozaki_split_t_kernel(int V, int K, int Kpad, Src s, int nd,
                                                             __nv_bfloat16 *__restrict__ out, int ldo, size_t plane,
                                                             int *__restrict__ exps)
 {
@@ -184,7 +212,7 @@ __global__ void __launch_bounds__(256) ozaki_split_t_kernel(int V, int K, int Kp
     __shared__ double tile[R][C + 2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx = tid & (R - 1), ty = tid / R;  // vector; elements ty, ty + 32, ..
-    const int v0 = blockIdx.x * R, v = v0 + tx;
+    const int v0 = blockIdx.x * R, v = v0 + tx, raise = s.prepare();
     unsigned long long mb = 0ull;
     double x[C / 32];
     for (int q0 = 0; q0 < K; q0 += C) {
@@ -211,7 +239,7 @@ __global__ void __launch_bounds__(256) ozaki_split_t_kernel(int V, int K, int Kp
 #pragma unroll
     for (int w = 0; w < 8; ++w) mb = red[w][warp] > mb ? red[w][warp] : mb;
     const int e = row_exponent(mb);
-    if (lane == 0) exps[v0 + warp] = e;
+    if (lane == 0) exps[v0 + warp] = e + raise;
     unsigned *o = reinterpret_cast<unsigned *>(out + (size_t)(v0 + warp) * ldo);
     for (int q0 = 0; q0 < Kpad; q0 += C) {
         if (K > C) {
@@ -641,15 +669,14 @@ size_t ozaki_split_elems(int V, int K, int digits) { return ozaki_plane_elems(V,
 
 cudaError_t ozaki_split(cudaStream_t st, int V, int K, const double *src, long long sv,
                         long long sq, const double *scale, const double *scale2,
-                        __nv_bfloat16 *planes, int *exps, int digits, const double *src2, long long sq2, int k1)
+                        __nv_bfloat16 *planes, int *exps, int digits)
 {
     if (digits < 1 || (digits > kOzDigits && digits != kOzWide)) return cudaErrorInvalidValue;
     const int Vpad = ceil_div(V, kOzBM) * kOzBM;
     const int Kpad = ceil_div(K, kOzBK) * kOzBK;
     const size_t plane = ozaki_plane_elems(V, K);
     SplitSrc s;
-    s.src = src; s.src2 = src2; s.scale = scale; s.scale2 = scale2;
-    s.sv = sv; s.sq = sq; s.sq2 = sq2; s.k1 = src2 ? k1 : K;
+    s.src = src; s.scale = scale; s.scale2 = scale2; s.sv = sv; s.sq = sq;
     const bool across = sv == 1 && sq != 1;
     EGB_COUNT_LAUNCH();
     if (digits == kOzWide) {
@@ -659,6 +686,18 @@ cudaError_t ozaki_split(cudaStream_t st, int V, int K, const double *src, long l
         if (across) ozaki_split_t_kernel<kOzDigits><<<Vpad / 8, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
         else ozaki_split_kernel<kOzDigits><<<Vpad, 256, 0, st>>>(V, K, Kpad, s, digits, planes, Kpad, plane, exps);
     }
+    return cudaGetLastError();
+}
+
+cudaError_t ozaki_split_halves(cudaStream_t st, int V, int k1, const double *src, long long sq, const double *src2,
+                               long long sq2, const int *wexp, bool scaled_first, __nv_bfloat16 *planes, int *exps)
+{
+    const int K = 2 * k1, Vpad = ceil_div(V, kOzBM) * kOzBM, Kpad = ceil_div(K, kOzBK) * kOzBK;
+    SplitHalves s = {};
+    s.src = src; s.src2 = src2; s.sq = sq; s.sq2 = sq2; s.k1 = k1; s.wexp = wexp; s.scaled_first = scaled_first;
+    EGB_COUNT_LAUNCH();
+    ozaki_split_t_kernel<kOzWide><<<Vpad / 8, 256, 0, st>>>(V, K, Kpad, s, kOzWide, planes, Kpad,
+                                                            ozaki_plane_elems(V, K), exps);
     return cudaGetLastError();
 }
 

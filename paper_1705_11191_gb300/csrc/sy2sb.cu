@@ -74,11 +74,13 @@ __device__ __forceinline__ void load_rows(T *tile, const T *src, int ld, int r0,
                      [&](int i, int c, T x) { tile[i * kWLd + c] = x; });
 }
 
-// X rows = Xa rows T; partial Y (64 x 64 per block, column-major) = V rows^T X rows
+// X rows = Xa rows T; partial Y (64 x 64 per block, column-major) = V rows^T X rows. *wexp = 0 for
+// w_stage3 (binary64: what the two-sided digit product scales W by).
 template <typename T, int CJ>
 __global__ void __launch_bounds__(256) w_stage1_kernel(int m, int bw, const T *xa, const T *V, int ldv,
-                                                       const T *Tm, int ldt, T *X, T *ypart)
+                                                       const T *Tm, int ldt, T *X, T *ypart, int *wexp)
 {
+    if (sizeof(T) == 8 && blockIdx.x == 0 && threadIdx.x == 0) *wexp = 0;
     constexpr int ROWS = WRows<T>, R = ROWS / 16;
     extern __shared__ unsigned char wsm_raw[];
     T *sT = reinterpret_cast<T *>(wsm_raw), *sA = sT + 64 * kWLd, *sX = sA + 64 * kWLd;
@@ -137,10 +139,24 @@ __global__ void __launch_bounds__(256) w_stage2_kernel(int nblk, int bw, const T
     if (q == 0) Y[e] = (part[0][el] + part[1][el]) + (part[2][el] + part[3][el]);
 }
 
+// The exponent field of the largest value of a CTA (256 threads), into *wexp; one atomic a CTA, since
+// those of a launch all go to one address
+__device__ __forceinline__ void block_exponent(int top, int *wexp)
+{
+    __shared__ int tops[8];
+    top = __reduce_max_sync(0xffffffffu, top & 0x7FF00000);
+    if ((threadIdx.x & 31) == 0) tops[threadIdx.x >> 5] = top;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        top = __reduce_max_sync(0xffffffffu, tops[threadIdx.x & 7]);
+        if (threadIdx.x == 0) atomicMax(wexp, top >> 20);
+    }
+}
+
 // W rows = X rows - (1/2) (V rows T^T) Y
 template <typename T, int CJ>
 __global__ void __launch_bounds__(256) w_stage3_kernel(int m, int bw, const T *X, const T *V, int ldv,
-                                                       const T *Tm, int ldt, const T *Y, T *W)
+                                                       const T *Tm, int ldt, const T *Y, T *W, int *wexp)
 {
     constexpr int ROWS = WRows<T>, R = ROWS / 16;
     extern __shared__ unsigned char wsm_raw[];
@@ -162,19 +178,32 @@ __global__ void __launch_bounds__(256) w_stage3_kernel(int m, int bw, const T *X
         for (int j = 0; j < CJ; ++j) sZ[(tr + i) * kWLd + tc + j] = c[i][j];
     __syncthreads();
     tile_mm<T, R, CJ>(sZ, sB, bw, c);
+    int top = 0;
 #pragma unroll
     for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < CJ; ++j)
             if (tr + i < rows && tc + j < bw) {
                 const size_t q = (size_t)(r0 + tr + i) + (size_t)(tc + j) * m;
-                W[q] = X[q] - T(0.5) * c[i][j];
+                const T v = X[q] - T(0.5) * c[i][j];
+                W[q] = v;
+                if (sizeof(T) == 8) top = max(top, __double2hiint((double)v) & 0x7FF00000);
             }
+    if (sizeof(T) == 8) block_exponent(top, wexp);
+}
+
+// The same from W in memory (m x bw, one after the other), *wexp zeroed before
+__global__ void __launch_bounds__(256) w_exponent_kernel(size_t total, const double *__restrict__ W, int *wexp)
+{
+    int top = 0;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x)
+        top = max(top, __double2hiint(W[e]) & 0x7FF00000);
+    block_exponent(top, wexp);
 }
 
 template <typename T, int CJ>
 static cudaError_t form_w(cudaStream_t st, int m, int bw, const T *xa, const T *V, int ldv,
-                          const T *Tm, int ldt, T *X, T *Y, T *W, T *ypart)
+                          const T *Tm, int ldt, T *X, T *Y, T *W, T *ypart, int *wexp)
 {
     const int nblk = ceil_div(m, WRows<T>);
     const size_t smem = (size_t)3 * 64 * kWLd * sizeof(T);
@@ -187,11 +216,11 @@ static cudaError_t form_w(cudaStream_t st, int m, int bw, const T *xa, const T *
     });
     if (e != cudaSuccess) return e;
     EGB_COUNT_LAUNCH();
-    w_stage1_kernel<T, CJ><<<nblk, 256, smem, st>>>(m, bw, xa, V, ldv, Tm, ldt, X, ypart);
+    w_stage1_kernel<T, CJ><<<nblk, 256, smem, st>>>(m, bw, xa, V, ldv, Tm, ldt, X, ypart, wexp);
     EGB_COUNT_LAUNCH();
     w_stage2_kernel<T><<<64, 256, 0, st>>>(nblk, bw, ypart, Y);
     EGB_COUNT_LAUNCH();
-    w_stage3_kernel<T, CJ><<<nblk, 256, smem, st>>>(m, bw, X, V, ldv, Tm, ldt, Y, W);
+    w_stage3_kernel<T, CJ><<<nblk, 256, smem, st>>>(m, bw, X, V, ldv, Tm, ldt, Y, W, wexp);
     return cudaGetLastError();
 }
 
@@ -255,8 +284,8 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
         if (ceil_div(m, WRows<T>) + 1 <= kSyncBlocks) {
             // X = (A22 V) T, W = X - 1/2 V (T^T (V^T X))
             T *ysum = ypart + (size_t)ceil_div(m, WRows<T>) * 64 * 64;
-            e = bw <= 32 ? form_w<T, 2>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart)
-                         : form_w<T, 4>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart);
+            e = bw <= 32 ? form_w<T, 2>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart, status + ST_WEXP)
+                         : form_w<T, 4>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart, status + ST_WEXP);
             if (e != cudaSuccess) return e;
         } else {
             // X = (A22 V) T
@@ -269,6 +298,13 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
             // W = X - 1/2 V Z
             if ((e = cudaMemcpyAsync(W, X, sizeof(T) * (size_t)m * bw, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
             if ((e = gemm<T>(st, 0, 0, m, bw, bw, T(-0.5), V, n, Z, bw, T(1), W, m)) != cudaSuccess) return e;
+            if constexpr (sizeof(T) == 8) {
+                if ((e = cudaMemsetAsync(status + ST_WEXP, 0, sizeof(int), st)) != cudaSuccess) return e;
+                const int grid = ceil_div((long long)m * bw, 256);
+                EGB_COUNT_LAUNCH();
+                w_exponent_kernel<<<grid < 152 * 4 ? grid : 152 * 4, 256, 0, st>>>((size_t)m * bw, W, status + ST_WEXP);
+                if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            }
         }
         // A22 -= V W^T + W V^T   (lower triangle), then mirror. On the tensor-core path the
         // two products are one GEMM over K = 2 bw: [V W] [W V]^T.
@@ -288,7 +324,7 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
             }
         }
         if constexpr (sizeof(T) == 8) {
-            e = gemm_f64_two_sided(st, m, bw, V, n, W, m, A22, lda);
+            e = gemm_f64_two_sided(st, m, bw, V, n, W, m, A22, lda, status + ST_WEXP);
             if (e != cudaErrorNotSupported) {
                 if (e != cudaSuccess) return e;
                 done = true;
