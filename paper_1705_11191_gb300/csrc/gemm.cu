@@ -300,15 +300,15 @@ static cudaError_t gemm_f64_digits(cudaStream_t st, int ta, int tb, int m, int n
     const size_t used = (ea + eb + 7) & ~(size_t)7;
     double *part = reinterpret_cast<double *>(t_oz_planes + used);
     const size_t part_elems = (t_oz_elems > used ? t_oz_elems - used : 0) / 4;
+    // row i of op(A): ta = 0 -> A[i + q lda], ta = 1 -> A[q + i lda]; column j of op(B): tb = 0 ->
+    // B[q + j ldb], tb = 1 -> B[j + q ldb]
+    OzOperands src;
+    src.a = A; src.av = ta ? lda : 1; src.aq = ta ? 1 : lda;
+    src.b = B; src.bv = tb ? 1 : ldb; src.bq = tb ? ldb : 1;
     cudaError_t e;
-    // row i of op(A): ta = 0 -> A[i + q lda], ta = 1 -> A[q + i lda]
-    if ((e = ozaki_split(st, m, k, A, ta ? lda : 1, ta ? 1 : lda, nullptr, nullptr, ad, xe, digits)) != cudaSuccess)
-        return e;
-    // column j of op(B): tb = 0 -> B[q + j ldb], tb = 1 -> B[j + q ldb]
-    if (!same &&
-        (e = ozaki_split(st, n, k, B, tb ? 1 : ldb, tb ? ldb : 1, nullptr, nullptr, bd, ye, digits)) != cudaSuccess)
-        return e;
-    return ozaki_gemm(st, m, n, k, alpha, ad, xe, bd, ye, beta, C, ldc, uplo, digits, part, part_elems);
+    if ((e = ozaki_split(st, m, k, A, src.av, src.aq, nullptr, nullptr, ad, xe, digits)) != cudaSuccess) return e;
+    if (!same && (e = ozaki_split(st, n, k, B, src.bv, src.bq, nullptr, nullptr, bd, ye, digits)) != cudaSuccess) return e;
+    return ozaki_gemm(st, m, n, k, alpha, ad, xe, bd, ye, beta, C, ldc, uplo, digits, part, part_elems, src);
 }
 
 // A binary64 product goes to the digit products when the thread has their scratch and the

@@ -246,6 +246,13 @@ cudaError_t ozaki_split(cudaStream_t st, int V, int K, const double *src, long l
 // by the exponent field *wexp and is divided by 2^e, which goes to the exponents if scaled_first.
 cudaError_t ozaki_split_halves(cudaStream_t st, int V, int k1, const double *src, long long sq, const double *src2,
                                long long sq2, const int *wexp, bool scaled_first, __nv_bfloat16 *planes, int *exps);
+// The operands that were split, element (v, q) of A at a[v av + q aq], of B at b[v bv + q bq]. Rows of
+// A and columns of B with an infinity or a NaN have no digits; their part of C is summed from here,
+// and is NaN without it.
+struct OzOperands {
+    const double *a = nullptr, *b = nullptr;
+    long long av = 0, aq = 0, bv = 0, bq = 0;
+};
 // C (m x n, ldc) = alpha * A B + beta * C with A given by the split of its m rows and B
 // by the split of its n columns (both of length k). uplo = 1: lower triangle only.
 // digits (1..kOzDigits, or kOzWide; that of both splits, or for the refinement form less):
@@ -255,6 +262,7 @@ cudaError_t ozaki_split_halves(cudaStream_t st, int V, int k1, const double *src
 cudaError_t ozaki_gemm(cudaStream_t st, int m, int n, int k, double alpha,
                        const __nv_bfloat16 *Ad, const int *ea, const __nv_bfloat16 *Bd,
                        const int *eb, double beta, double *C, int ldc, int uplo,
-                       int digits = kOzDigits, double *part = nullptr, size_t part_elems = 0);
+                       int digits = kOzDigits, double *part = nullptr, size_t part_elems = 0,
+                       const OzOperands &src = OzOperands());
 
 }  // namespace egb

@@ -65,10 +65,15 @@ __device__ __forceinline__ unsigned long long magnitude(double x)
     return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
 }
 
-// The row exponent from the largest magnitude bit pattern: max |x| = m 2^e, m in [0.25, 0.5).
+// The row exponent from the largest magnitude bit pattern: max |x| = m 2^e, m in [0.25, 0.5). A
+// vector with an infinity or a NaN has kOzNonFinite, and all its digits are zero: the product forms
+// its row or column from the operands instead (see direct_sum).
+constexpr int kOzNonFinite = 1 << 28;
 __device__ __forceinline__ int row_exponent(unsigned long long mb)
 {
     if (mb == 0ull) return 0;
+    // (the field alone: the compiler may take the magnitude by arithmetic, which makes a NaN negative)
+    if (((mb >> 52) & 0x7FFull) == 0x7FFull) return kOzNonFinite;
     const int xf = (int)(mb >> 52);
     return 1 + (xf ? xf - 1022 : (64 - __clzll((long long)(mb & 0xFFFFFFFFFFFFFull))) - 1074);
 }
@@ -185,7 +190,7 @@ __global__ void __launch_bounds__(256) ozaki_split_kernel(int V, int K, int Kpad
 #pragma unroll
     for (int w = 0; w < 8; ++w) mb = red[w] > mb ? red[w] : mb;
     const int e = row_exponent(mb);
-    if (threadIdx.x == 0) exps[v] = e + raise;
+    if (threadIdx.x == 0) exps[v] = e == kOzNonFinite ? e : e + raise;
     unsigned *o = reinterpret_cast<unsigned *>(out + (size_t)v * ldo);
     for (int q = 2 * threadIdx.x; q < Kpad; q += 512) {
         unsigned a[ND], b[ND];
@@ -239,7 +244,7 @@ __global__ void __launch_bounds__(256) ozaki_split_t_kernel(int V, int K, int Kp
 #pragma unroll
     for (int w = 0; w < 8; ++w) mb = red[w][warp] > mb ? red[w][warp] : mb;
     const int e = row_exponent(mb);
-    if (lane == 0) exps[v0 + warp] = e + raise;
+    if (lane == 0) exps[v0 + warp] = e == kOzNonFinite ? e : e + raise;
     unsigned *o = reinterpret_cast<unsigned *>(out + (size_t)(v0 + warp) * ldo);
     for (int q0 = 0; q0 < Kpad; q0 += C) {
         if (K > C) {
@@ -325,6 +330,8 @@ struct Args {
     double *C;
     size_t cstride;     // C of blockIdx.z: C + z cstride
     int *status;
+    OzOperands src;     // for rows and columns that are not finite
+    int k_real;
 };
 constexpr int kNotPow2 = 1 << 20;
 }  // namespace oztc
@@ -372,6 +379,18 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, in
     if (biased >= 1 && biased <= 2045) return pack_double(nrm, sticky, neg, biased);
     const double v = scale_slow((double)(nrm | (sticky ? 1ull : 0ull)), e + 64 - lz);
     return neg ? -v : v;
+}
+
+// An element whose row or column holds an infinity or a NaN: the sum over q0 <= q < q1 of the
+// operands themselves, which has the infinities and NaNs of binary64 arithmetic; a NaN where the
+// operands are not known. Out of line: only input that is not finite gets here.
+__device__ __noinline__ double direct_sum(const OzOperands &o, int row, int col, int q0, int q1)
+{
+    if (!o.a) return __longlong_as_double(0x7FF8000000000000ll);
+    const double *pa = o.a + (size_t)row * o.av, *pb = o.b + (size_t)col * o.bv;
+    double s = 0.0;
+    for (int q = q0; q < q1 && s == s; ++q) s = fma(pa[(size_t)q * o.aq], pb[(size_t)q * o.bq], s);
+    return s;
 }
 
 template <bool WIDE>
@@ -600,6 +619,7 @@ ozaki_gemm_tc_kernel(const __grid_constant__ oztc::Maps maps, const __grid_const
             const bool neg = pow2 && a.alpha < 0.0;
             const int er = (row_in ? a.ea[row] : 0) - kOzBits * (WIDE ? 9 : D + 1) + (WIDE ? 0 : a.eshift) +
                            (pow2 ? a.alpha_exp : 0);
+            const bool row_bad = row_in && a.ea[row] == kOzNonFinite;
             double *crow = a.C + blockIdx.z * a.cstride + (size_t)row;
             // C = beta C + sum, 4 columns at a time (the loads of C first). The sums go through
             // shared memory (the rings are done), each thread reading back its own: a loop over
@@ -628,6 +648,11 @@ ozaki_gemm_tc_kernel(const __grid_constant__ oztc::Maps maps, const __grid_const
                     double val;
                     if (WIDE) val = fixed_to_double(stage[(q + j) * ET], stage[(CW + q + j) * ET], er + ebs[cl]);
                     else val = fixed_to_double(stage[(q + j) * ET], er + ebs[cl]);
+                    if (in[j] && (row_bad || ebs[cl] == kOzNonFinite)) {
+                        const int q0 = (a.kt0 + kz) * BK;
+                        val = direct_sum(a.src, row, col, q0, min(a.k_real, q0 + nkt * BK));
+                        if (pow2) val *= fabs(a.alpha);
+                    }
                     if (neg) val = -val;
                     if (!pow2) val *= a.alpha;
                     if (a.beta == 1.0) val += cv[j];
@@ -736,7 +761,7 @@ static cudaError_t oz_launch(cudaStream_t st, dim3 grid, const oztc::Maps &maps,
 cudaError_t ozaki_gemm(cudaStream_t st, int m, int n, int k, double alpha,
                        const __nv_bfloat16 *Ad, const int *ea, const __nv_bfloat16 *Bd,
                        const int *eb, double beta, double *C, int ldc, int uplo, int digits,
-                       double *part, size_t part_elems)
+                       double *part, size_t part_elems, const OzOperands &src)
 {
     const bool wide = digits == kOzWide;
     if (digits < 1 || (digits > kOzDigits && !wide)) return cudaErrorInvalidValue;
@@ -754,7 +779,7 @@ cudaError_t ozaki_gemm(cudaStream_t st, int m, int n, int k, double alpha,
     Args a;
     a.m_real = m; a.n_real = n; a.mpad = mpad; a.npad = npad; a.uplo = uplo;
     a.ldc = ldc; a.ea = ea; a.eb = eb; a.alpha = alpha; a.beta = beta; a.C = C; a.cstride = 0;
-    a.digits = digits;
+    a.digits = digits; a.src = src; a.k_real = k;
     for (int o = 0; o < 9; ++o) a.order[o] = o + 2;
     if (digits == 6) {  // level 6 (not drained) between 4 and 5: time to drain the two accumulators
         a.order[3] = 6;
