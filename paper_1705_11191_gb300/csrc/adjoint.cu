@@ -91,18 +91,22 @@ int ev_adjoint(elsi_gb_handle_s *h, int n, int k, const double *eps, const doubl
     }
     const size_t nk = (size_t)n * (g ? k : 0), nkk = (size_t)n * kk;
     Workspace &w = h->wk;
-    if (!ensure_buf((void **)&w.adj, &w.adj_cap, sizeof(double) * (nk + 3 * nkk + 16)))
+    if (!ensure_buf((void **)&w.adj, &w.adj_cap, sizeof(double) * (nk + 3 * nkk + 2 * (size_t)n + 16)))
         return set_error(h, ELSI_ERR_NOMEM, "adjoint scratch");
     if (!ensure_digit_scratch(h, n, n)) return set_error(h, ELSI_ERR_NOMEM, "adjoint digit planes");
     const DigitScratch digits(h);
-    double *A = w.adj, *XH = A + nk, *XS = XH + nkk, *Y = XS + nkk;
+    double *A = w.adj, *XH = A + nk, *XS = XH + nkk, *Y = XS + nkk, *scales = Y + nkk;
     cudaStream_t st = h->stream;
     cudaError_t e = cudaMemsetAsync(w.status, 0, sizeof(int) * ST_WORDS, st);
     if (e != cudaSuccess) return set_error(h, ELSI_ERR_CUDA, "eigenpair adjoint: %s", cudaGetErrorString(e));
 #define ACK(x)                                                                             \
     if ((e = (x)) != cudaSuccess)                                                          \
         return set_error(h, ELSI_ERR_CUDA, "eigenpair adjoint: %s", cudaGetErrorString(e));
-    if (g) ACK(gemm<double>(st, 1, 0, n, k, n, 1.0, c, n, g, n, 0.0, A, n));
+    if (g) {
+        const double *ka, *kb;
+        ACK(row_scales(st, n, k, c, n, false, scales, &ka, &kb));
+        ACK(gemm<double>(st, 1, 0, n, k, n, 1.0, c, n, g, n, 0.0, A, n, 0, ka, kb));
+    }
     EGB_COUNT_LAUNCH();
     adjoint_x_kernel<<<grid_for(nkk), 256, 0, st>>>(n, k, kk, eps, eb, g ? A : nullptr, 1e-10, XH, XS);
     ACK(cudaGetLastError());

@@ -287,9 +287,10 @@ void set_f64_tc_scratch(__nv_bfloat16 *planes, size_t elems, int *exps, size_t e
 // rows, op(B) by columns (once for A A^T). cudaErrorNotSupported if the scratch is short.
 static cudaError_t gemm_f64_digits(cudaStream_t st, int ta, int tb, int m, int n, int k, double alpha,
                                    const double *A, int lda, const double *B, int ldb, double beta,
-                                   double *C, int ldc, int uplo, int digits = kOzWide)
+                                   double *C, int ldc, int uplo, int digits = kOzWide,
+                                   const double *ka = nullptr, const double *kb = nullptr)
 {
-    const bool same = A == B && lda == ldb && ta != tb && m == n;
+    const bool same = A == B && lda == ldb && ta != tb && m == n && !ka;
     const size_t ea = ozaki_split_elems(m, k, digits), eb = same ? 0 : ozaki_split_elems(n, k, digits);
     const size_t xa = (size_t)ceil_div(m, 128) * 128, xb = same ? 0 : (size_t)ceil_div(n, 128) * 128;
     if (ea + eb > t_oz_elems || xa + xb > t_oz_exp_elems) return cudaErrorNotSupported;
@@ -306,8 +307,8 @@ static cudaError_t gemm_f64_digits(cudaStream_t st, int ta, int tb, int m, int n
     src.a = A; src.av = ta ? lda : 1; src.aq = ta ? 1 : lda;
     src.b = B; src.bv = tb ? 1 : ldb; src.bq = tb ? ldb : 1;
     cudaError_t e;
-    if ((e = ozaki_split(st, m, k, A, src.av, src.aq, nullptr, nullptr, ad, xe, digits)) != cudaSuccess) return e;
-    if (!same && (e = ozaki_split(st, n, k, B, src.bv, src.bq, nullptr, nullptr, bd, ye, digits)) != cudaSuccess) return e;
+    if ((e = ozaki_split(st, m, k, A, src.av, src.aq, ka, nullptr, ad, xe, digits)) != cudaSuccess) return e;
+    if (!same && (e = ozaki_split(st, n, k, B, src.bv, src.bq, kb, nullptr, bd, ye, digits)) != cudaSuccess) return e;
     return ozaki_gemm(st, m, n, k, alpha, ad, xe, bd, ye, beta, C, ldc, uplo, digits, part, part_elems, src);
 }
 
@@ -319,6 +320,44 @@ static bool digits_pay(int m, int n, int k)
     const double tiles = (double)ceil_div(m, 16) * ceil_div(n, 16);
     const double waves = tiles <= 152.0 ? 1.0 : tiles / 152.0;
     return t_oz_planes && k >= 24 && waves * k >= 450.0;
+}
+
+// Products over the basis functions, L^T x of the back-substitution and C^T G of the eigenpair
+// adjoint: a basis function scaled by s puts s on row q of the one operand and 1 / s on row q of the
+// other, which no row or column exponent takes out. With diag(S) over 10^24 digits down to 2^-72 of
+// the largest entry left P with 10 decimals. So both are divided by the size of row q of the first
+// one, 2^e with e a multiple of 16 (0 within 2^+-8, where nothing changes), exactly.
+__global__ void __launch_bounds__(1024) row_scales_kernel(int n, const double *__restrict__ A, int lda, bool lower,
+                                                          double *__restrict__ ka, double *__restrict__ kb)
+{
+    __shared__ int tops[32][33];
+    const int q = blockIdx.x * 32 + threadIdx.x, cols = q >= n ? 0 : lower ? q + 1 : n;
+    int top = 0;
+#pragma unroll 4
+    for (int j = threadIdx.y; j < cols; j += 32) top = max(top, __double2hiint(A[(size_t)q + (size_t)j * lda]) & 0x7FF00000);
+    tops[threadIdx.y][threadIdx.x] = top >> 20;
+    __syncthreads();
+    const int xf = __reduce_max_sync(0xffffffffu, tops[threadIdx.x][threadIdx.y]);  // of row threadIdx.y
+    const int r = blockIdx.x * 32 + threadIdx.y;
+    if (threadIdx.x == 0 && r < n) {
+        int e = xf == 0 || xf == 2047 ? 0 : xf - 1022;
+        e = (abs(e) + 7) / 16 * (e < 0 ? -16 : 16);
+        e = max(-496, min(e, 496));
+        ka[r] = __hiloint2double((1023 - e) << 20, 0);
+        kb[r] = __hiloint2double((1023 + e) << 20, 0);
+    }
+}
+
+cudaError_t row_scales(cudaStream_t st, int n, int ncol, const double *A, int lda, bool lower, double *scratch,
+                       const double **ka, const double **kb)
+{
+    *ka = *kb = nullptr;
+    if (!scratch || !digits_pay(n, ncol, n)) return cudaSuccess;
+    EGB_COUNT_LAUNCH();
+    row_scales_kernel<<<ceil_div(n, 32), dim3(32, 32), 0, st>>>(n, A, lda, lower, scratch, scratch + n);
+    *ka = scratch;
+    *kb = scratch + n;
+    return cudaGetLastError();
 }
 
 // C -= V W^T + W V^T (lower triangle, m x m, V and W m x b): one product over K = 2 b whose
@@ -341,10 +380,12 @@ cudaError_t gemm_f64_two_sided(cudaStream_t st, int m, int b, const double *V, i
 
 template <typename T>
 cudaError_t gemm(cudaStream_t st, int ta, int tb, int m, int n, int k, T alpha, const T *A,
-                 int lda, const T *B, int ldb, T beta, T *C, int ldc, int uplo)
+                 int lda, const T *B, int ldb, T beta, T *C, int ldc, int uplo, const T *ka, const T *kb)
 {
     if (m <= 0 || n <= 0) return cudaSuccess;
     if constexpr (sizeof(T) == 4) {
+        (void)ka;
+        (void)kb;
         // Large binary32 products go to the tensor cores: two operand passes and the product take
         // 17 us at least, the small-tile kernel about 16 us at this limit (50 us at 64 x 64 x 16384).
         if (t_tc_work && k >= 16 && (double)m * n * k >= 3.0e7) {
@@ -355,7 +396,7 @@ cudaError_t gemm(cudaStream_t st, int ta, int tb, int m, int n, int k, T alpha, 
     } else {
         // binary64 products large enough for the digit products on the tensor cores
         if (digits_pay(m, n, k)) {
-            cudaError_t e = gemm_f64_digits(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, uplo);
+            cudaError_t e = gemm_f64_digits(st, ta, tb, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, uplo, kOzWide, ka, kb);
             if (e != cudaErrorNotSupported) return e;
         }
     }
@@ -435,9 +476,9 @@ template cudaError_t gemm_splitk<float>(cudaStream_t, int, int, int, int, int, f
                                         int, const float *, int, float *, int, float *, size_t);
 
 template cudaError_t gemm<double>(cudaStream_t, int, int, int, int, int, double, const double *,
-                                  int, const double *, int, double, double *, int, int);
+                                  int, const double *, int, double, double *, int, int, const double *, const double *);
 template cudaError_t gemm<float>(cudaStream_t, int, int, int, int, int, float, const float *,
-                                 int, const float *, int, float, float *, int, int);
+                                 int, const float *, int, float, float *, int, int, const float *, const float *);
 
 // ------------------------------------------------------------------ utilities
 template <typename Td, typename Ts>

@@ -10,11 +10,17 @@ namespace egb {
 
 // C = alpha * op(A) * op(B) + beta * C, op(A) m x k, op(B) k x n. ta/tb: 0 = N, 1 = T.
 // uplo = 1: only the lower triangle (row >= col) of C is computed and written.
-// beta == 0 means C is not read.
+// beta == 0 means C is not read. ka, kb (k values each, powers of two, ka[q] kb[q] = 1): factors of
+// op(A)(i, q) and op(B)(q, j) for the digit products of the binary64 route (see row_scales).
 template <typename T>
 cudaError_t gemm(cudaStream_t st, int ta, int tb, int m, int n, int k, T alpha,
                  const T *A, int lda, const T *B, int ldb, T beta, T *C, int ldc,
-                 int uplo = 0);
+                 int uplo = 0, const T *ka = nullptr, const T *kb = nullptr);
+// For products of order up to n x ncol x n with A (n x n) in the place of op(A)^T: *ka = scratch and
+// *kb = scratch + n, formed from the rows of A (the first i + 1 columns of row i if lower), or null
+// where no such product is a digit product. scratch: 2 n values.
+cudaError_t row_scales(cudaStream_t st, int n, int ncol, const double *A, int lda, bool lower, double *scratch,
+                       const double **ka, const double **kb);
 
 // Binary32-accuracy GEMM on the tcgen05 tensor cores (three TF32 products of hi/lo splits;
 // tc_gemm.cu). work: tc_gemm_work_elems(m, n, k) floats, 16-byte aligned. Returns
@@ -99,10 +105,10 @@ constexpr int kTriBlock = 64;   // nb of potrf / trsm
 constexpr int kTriPanel = 256;  // outer panel of potrf (rank-256 updates), and of trsm below n = 4096
 
 // B (n x ncol) := L^{-1} B (trans = 0) or L^{-T} B (trans = 1), L lower from potrf,
-// inv_diag its diagonal-block inverses.
+// inv_diag its diagonal-block inverses. scales: scratch of 2 n values for trans = 1 in binary64.
 template <typename T>
 cudaError_t trsm_left_lower(cudaStream_t st, int trans, int n, int ncol, const T *L, int ldl,
-                            const T *inv_diag, T *B, int ldb);
+                            const T *inv_diag, T *B, int ldb, T *scales = nullptr);
 
 // Columns that the refinement of the binary32 route works on for k wanted states: at least
 // 16 more (guard) columns, up to the next multiple of 128, the column tile of its products.

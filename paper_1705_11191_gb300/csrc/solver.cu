@@ -213,7 +213,7 @@ static int solve_fp64(elsi_gb_handle_s *h, const SolveRequest &rq)
     else CK(apply_q1<double>(st, n, b, k, w.v1, w.t1, w.z, n, w.work));
     CK(cudaEventRecord(w.ev[STAGE_BACKSUB], st));
     // ---- Eq. 9: c = L^{-T} c~
-    if (!unit) CK(trsm_left_lower<double>(st, 1, n, k, w.l, n, w.invd, w.z, n));
+    if (!unit) CK(trsm_left_lower<double>(st, 1, n, k, w.l, n, w.invd, w.z, n, w.stein));  // (stein is free again)
     CK(cudaEventRecord(w.ev[STAGE_REFINE], st));
     CK(cudaEventRecord(w.ev[STAGE_OCC], st));
     if (ev_mode) {
