@@ -91,9 +91,10 @@ int ev_adjoint(elsi_gb_handle_s *h, int n, int k, const double *eps, const doubl
     }
     const size_t nk = (size_t)n * (g ? k : 0), nkk = (size_t)n * kk;
     Workspace &w = h->wk;
-    if (!ensure_buf((void **)&w.adj, &w.adj_cap, sizeof(double) * (nk + 3 * nkk + 2 * (size_t)n + 16)))
+    if (!ensure_or_shed(h, (void **)&w.adj, &w.adj_cap, sizeof(double) * (nk + 3 * nkk + 2 * (size_t)n + 16)) ||
+        !ensure_or_shed(h, (void **)&w.status, &w.status_cap, sizeof(int) * ST_WORDS))
         return set_error(h, ELSI_ERR_NOMEM, "adjoint scratch");
-    if (!ensure_digit_scratch(h, n, n)) return set_error(h, ELSI_ERR_NOMEM, "adjoint digit planes");
+    ensure_digit_scratch(h, n, n);
     const DigitScratch digits(h);
     double *A = w.adj, *XH = A + nk, *XS = XH + nkk, *Y = XS + nkk, *scales = Y + nkk;
     cudaStream_t st = h->stream;

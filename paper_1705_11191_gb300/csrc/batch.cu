@@ -606,8 +606,8 @@ int batch_dm(elsi_gb_handle_s *h, const double *occ, double *const *dm, double *
         planes = e > planes ? e : planes;
         nmax = (size_t)c * it.n > nmax ? (size_t)c * it.n : nmax;
     }
-    BENSURE(dig, __nv_bfloat16, planes);
     BENSURE(digx, int, 2 * nmax + 512);
+    ensure_buf((void **)&b.dig, &b.dig_cap, sizeof(__nv_bfloat16) * planes);  // without it: binary64 sums
     BCK(cudaMemsetAsync(b.status, 0, sizeof(int) * ST_WORDS, st));
     struct Scratch {
         Scratch(BatchState &b)

@@ -45,9 +45,30 @@ bool ensure_buf(void **p, size_t *cap, size_t bytes)
     if (*p) cudaFree(*p);
     *p = nullptr;
     *cap = 0;
-    if (cudaMalloc(p, bytes) != cudaSuccess) { *p = nullptr; return false; }
+    if (cudaMalloc(p, bytes) != cudaSuccess) {
+        (void)cudaGetLastError();  // the next launch check must not see it
+        *p = nullptr;
+        return false;
+    }
     *cap = bytes;
     return true;
+}
+
+void shed_digit_scratch(elsi_gb_handle_s *h)
+{
+    Workspace &w = h->wk;
+    if (h->precision != ELSI_PREC_FP64 || !w.oz) return;  // the binary32 route cannot do without
+    cudaStreamSynchronize(h->stream);
+    cudaFree(w.oz);
+    w.oz = nullptr;
+    w.oz_cap = 0;
+}
+
+bool ensure_or_shed(elsi_gb_handle_s *h, void **p, size_t *cap, size_t bytes)
+{
+    if (ensure_buf(p, cap, bytes)) return true;
+    shed_digit_scratch(h);
+    return ensure_buf(p, cap, bytes);
 }
 
 }  // namespace egb

@@ -48,7 +48,9 @@ struct SingState {
     } while (0)
 
 #define SENSURE(name, count)                                                               \
-    if (!ensure_buf((void **)&g.name, &g.name##_cap, sizeof(double) * (size_t)(count)))   \
+    if (!ensure_buf((void **)&g.name, &g.name##_cap, sizeof(double) * (size_t)(count)) && \
+        (shed_digit_scratch(g.sh), shed_digit_scratch(g.rh),                               \
+         !ensure_or_shed(h, (void **)&g.name, &g.name##_cap, sizeof(double) * (size_t)(count)))) \
         return set_error(h, ELSI_ERR_NOMEM, "cannot allocate singularity-check %s", #name);
 
 static int grid_of(size_t total)
@@ -169,7 +171,7 @@ int solve_singular(elsi_gb_handle_s *h, const SolveRequest &rq)
     const bool ev_mode = rq.evec != nullptr;
     if (k > nn)
         return set_error(h, ELSI_ERR_ARG, "n_state %d exceeds the %d non-singular basis directions", k, nn);
-    int rc = ensure_workspace(h, k);
+    int rc = ensure_workspace(h, k, false);  // its products are not digit products
     if (rc) return rc;
     Workspace &w = h->wk;
     // scratch of the density-matrix products below: n x k binary64 values

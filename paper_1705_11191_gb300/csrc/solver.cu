@@ -35,12 +35,11 @@ static size_t digit_scratch_elems(int n, int k)
     return ozaki_split_elems(n, n, kOzWide) + ozaki_split_elems(n, k > 256 ? k : 256, kOzWide) + 4 * (part < small ? part : small) + 64;
 }
 
-bool ensure_digit_scratch(elsi_gb_handle_s *h, int n, int k)
+void ensure_digit_scratch(elsi_gb_handle_s *h, int n, int k)
 {
     Workspace &w = h->wk;
-    return ensure_buf((void **)&w.oz, &w.oz_cap, sizeof(__nv_bfloat16) * digit_scratch_elems(n, k)) &&
-           ensure_buf((void **)&w.ozexp, &w.ozexp_cap, sizeof(int) * (4 * (size_t)n + 1024)) &&
-           ensure_buf((void **)&w.status, &w.status_cap, sizeof(int) * ST_WORDS);
+    if (!ensure_buf((void **)&w.ozexp, &w.ozexp_cap, sizeof(int) * (4 * (size_t)n + 1024))) shed_digit_scratch(h);
+    else ensure_buf((void **)&w.oz, &w.oz_cap, sizeof(__nv_bfloat16) * digit_scratch_elems(n, k));
 }
 
 DigitScratch::DigitScratch(elsi_gb_handle_s *h)
@@ -57,7 +56,7 @@ DigitScratch::~DigitScratch()
 }
 
 #define ENSURE(name, type, count)                                                          \
-    if (!ensure_buf((void **)&w.name, &w.name##_cap, sizeof(type) * (size_t)(count)))     \
+    if (!ensure_or_shed(h, (void **)&w.name, &w.name##_cap, sizeof(type) * (size_t)(count))) \
         return set_error(h, ELSI_ERR_NOMEM, "cannot allocate %s (%zu bytes)", #name,       \
                          sizeof(type) * (size_t)(count));
 
@@ -66,7 +65,7 @@ DigitScratch::~DigitScratch()
 // the binary64 Cholesky factor live in the digit-plane buffer oz, which is free at those
 // stages (its planes are formed after the back-transformations). A binary64 fallback of a
 // binary32 solve grows the buffers to binary64 sizes first.
-int ensure_workspace(elsi_gb_handle_s *h, int kz)
+int ensure_workspace(elsi_gb_handle_s *h, int kz, bool digits)
 {
     Workspace &w = h->wk;
     const size_t n = h->n;
@@ -102,7 +101,6 @@ int ensure_workspace(elsi_gb_handle_s *h, int kz)
         ENSURE(stein, double, n * kTriBlock + 64);  // binary64 diagonal-block inverses
     } else {
         ENSURE(stein, double, 3 * n * kz + kz + 64);
-        if (!ensure_digit_scratch(h, h->n, kz)) return set_error(h, ELSI_ERR_NOMEM, "cannot allocate the digit planes");
     }
     ENSURE(sync, unsigned, fp32 ? sync_words(h->n, (int)eb) : std::max(sync_words(h->n, (int)eb), q2_f64_sync_words(h->n)));
     ENSURE(status, int, ST_WORDS);
@@ -129,6 +127,7 @@ int ensure_workspace(elsi_gb_handle_s *h, int kz)
             if (cudaEventCreate(&e) != cudaSuccess) return set_error(h, ELSI_ERR_CUDA, "event create");
         w.events_ready = true;
     }
+    if (digits && !fp32) ensure_digit_scratch(h, h->n, kz);
     return ELSI_OK;
 }
 

@@ -136,12 +136,17 @@ inline int band_of(const elsi_gb_handle_s *h, int precision)
 int set_error(elsi_gb_handle_s *h, int code, const char *fmt, ...);
 bool ensure_buf(void **p, size_t *cap, size_t bytes);
 int run_solve(elsi_gb_handle_s *h, const SolveRequest &rq);
-int ensure_workspace(elsi_gb_handle_s *h, int kz);
-// The handle's digit planes, exponents and status word for products of orders up to n x n by
-// n x max(k, 256); false if they cannot be allocated.
-bool ensure_digit_scratch(elsi_gb_handle_s *h, int n, int k);
+// digits: with the scratch below, if there is room for it
+int ensure_workspace(elsi_gb_handle_s *h, int kz, bool digits = true);
+// The handle's digit planes and exponents for products of orders up to n x n by n x max(k, 256):
+// 16 bytes an element of a matrix, as much as two matrices. The binary64 route and the adjoint
+// solve without them (a few times slower) where they do not fit, and give them back
+// for a buffer that cannot be done without (shed_digit_scratch; ensure_or_shed: ensure_buf with that).
+void ensure_digit_scratch(elsi_gb_handle_s *h, int n, int k);
+void shed_digit_scratch(elsi_gb_handle_s *h);
+bool ensure_or_shed(elsi_gb_handle_s *h, void **p, size_t *cap, size_t bytes);
 // While it lives, this thread's large binary64 gemm() calls run as digit products on the
-// tensor cores with the handle's scratch (all on the handle's stream).
+// tensor cores with the handle's scratch (all on the handle's stream), if it has one.
 struct DigitScratch {
     explicit DigitScratch(elsi_gb_handle_s *h);
     ~DigitScratch();
