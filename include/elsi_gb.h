@@ -92,7 +92,9 @@ int elsi_set_precision(elsi_handle h, int precision);      /* ELSI_PREC_* */
 int elsi_set_band_width(elsi_handle h, int band_width);    /* 8..64, multiple of 8 (default 64; 32
                                                               up to n = 19000 in the binary64 route
                                                               and 3500 in the binary32 route, single
-                                                              solves) */
+                                                              solves). The two-stage reduction takes
+                                                              panels of up to 77 312 rows (n less the
+                                                              band width) on 152 SMs */
 /* elsi_customize_elpa, keyword elpa_solver (sec. 4.5): 1 = one-stage tridiagonalisation
  * T = Q^T H~ Q (Eq. 11, first form; blocked Householder with a matrix-vector product per
  * column, memory-bound), 2 = two-stage full -> band -> tridiagonal (default). Applies to

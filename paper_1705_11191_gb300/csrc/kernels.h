@@ -125,7 +125,7 @@ inline int refine_block(int n, int k)
 // Householder QR of the m x bw panel at P (explicit V, compact-WY T), panel.cu. packets:
 // panel_packet_words(m_first, sizeof(T)) words zeroed before the first panel of a reduction
 // (m_first rows); the panel uses the sequence numbers seq0 + 1 .. seq0 + bw, each once per
-// reduction.
+// reduction. work: 2 x 32 x 32 values (panels of bw > 32 with more rows than one launch takes).
 size_t panel_packet_words(int m, int elem);
 
 // Words of the sync scratch: the base (the partials of the W kernels, or the packets of the
@@ -135,7 +135,7 @@ constexpr size_t kSyncWords = 64 + 2 * (size_t)kSyncBlocks * 64 * 64;
 inline size_t sync_words(int n, int elem) { return kSyncWords + 2 * panel_packet_words(n, elem); }
 template <typename T>
 cudaError_t panel_qr(cudaStream_t st, int m, int m_first, int bw, T *P, int lda, T *V, int ldv, T *Tm, int ldt,
-                     unsigned seq0, unsigned long long *packets, int *status, int num_sms);
+                     unsigned seq0, unsigned long long *packets, T *work, int *status, int num_sms);
 template <typename T>
 cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T *work,
                   size_t work_elems, unsigned *sync, int *status, int num_sms);

@@ -339,9 +339,43 @@ cudaError_t choose(cudaStream_t st, T *P, T *V, T *Tm, int ldt, const Args &a, i
     } else {
         if (e == cudaSuccess && !fits) e = launch<T, 8, CPL, 8>(st, P, V, Tm, ldt, a, num_sms, &fits);
         if (e == cudaSuccess && !fits) e = launch<T, 16, CPL, 16>(st, P, V, Tm, ldt, a, num_sms, &fits);
+        // one column a lane leaves registers for 512 rows a CTA: 77 312 rows
+        if constexpr (CPL == 1)
+            if (e == cudaSuccess && !fits) e = launch<T, 32, 1, 16>(st, P, V, Tm, ldt, a, num_sms, &fits);
     }
     if (e != cudaSuccess) return e;
     return fits ? cudaSuccess : cudaErrorInvalidConfiguration;
+}
+
+// A panel with more rows than fit with two columns a lane (binary64: 38 656), as two panels of one
+// column a lane, the reflectors of the first applied to the columns of the second between them.
+// work: 2 x 32 x 32 values.
+template <typename T>
+cudaError_t in_two(cudaStream_t st, T *P, T *V, int ldv, T *Tm, int ldt, const Args &a, T *work, int num_sms)
+{
+    constexpr int b1 = 32;
+    const int m = a.m, b2 = a.bw - b1, lda = a.lda;
+    T *C = P + (size_t)b1 * lda, *V2 = V + (size_t)b1 * ldv, *T2 = Tm + b1 + (size_t)b1 * ldt;
+    T *Y = work, *Z = work + b1 * b1;
+    cudaError_t e;
+    Args s = a;
+    s.bw = b1;
+    if ((e = choose<T, 1>(st, P, V, Tm, ldt, s, num_sms)) != cudaSuccess) return e;
+    // C -= V1 T1^T (V1^T C)
+    if ((e = gemm<T>(st, 1, 0, b1, b2, m, T(1), V, ldv, C, lda, T(0), Y, b1)) != cudaSuccess) return e;
+    if ((e = gemm<T>(st, 1, 0, b1, b2, b1, T(1), Tm, ldt, Y, b1, T(0), Z, b1)) != cudaSuccess) return e;
+    if ((e = gemm<T>(st, 0, 0, m, b2, b1, T(-1), V, ldv, Z, b1, T(1), C, lda)) != cudaSuccess) return e;
+    if ((e = cudaMemset2DAsync(V2, sizeof(T) * ldv, 0, sizeof(T) * b1, b2, st)) != cudaSuccess) return e;
+    s = a;
+    s.m = m - b1;
+    s.bw = b2;
+    s.seq0 = a.seq0 + b1;
+    if ((e = choose<T, 1>(st, C + b1, V2 + b1, T2, ldt, s, num_sms)) != cudaSuccess) return e;
+    // T = [T1, -T1 (V1^T V2) T2; 0, T2]
+    if ((e = gemm<T>(st, 1, 0, b1, b2, m - b1, T(1), V + b1, ldv, V2 + b1, ldv, T(0), Y, b1)) != cudaSuccess) return e;
+    if ((e = gemm<T>(st, 0, 0, b1, b2, b2, T(1), Y, b1, T2, ldt, T(0), Z, b1)) != cudaSuccess) return e;
+    if ((e = gemm<T>(st, 0, 0, b1, b2, b1, T(-1), Tm, ldt, Z, b1, T(0), Tm + (size_t)b1 * ldt, ldt)) != cudaSuccess) return e;
+    return cudaMemset2DAsync(Tm + b1, sizeof(T) * ldt, 0, sizeof(T) * b2, b1, st);
 }
 
 }  // namespace pan
@@ -357,7 +391,7 @@ size_t panel_packet_words(int m, int elem) { return (size_t)64 * 64 * 2 * (max_c
 
 template <typename T>
 cudaError_t panel_qr(cudaStream_t st, int m, int m_first, int bw, T *P, int lda, T *V, int ldv, T *Tm, int ldt,
-                     unsigned seq0, unsigned long long *packets, int *status, int num_sms)
+                     unsigned seq0, unsigned long long *packets, T *work, int *status, int num_sms)
 {
     if (bw < 1 || bw > 64) return cudaErrorInvalidValue;
     pan::Args a;
@@ -365,12 +399,38 @@ cudaError_t panel_qr(cudaStream_t st, int m, int m_first, int bw, T *P, int lda,
     a.gs = max_ctas(m_first, sizeof(T));
     a.seq0 = seq0; a.rpk = packets; a.dpk = packets + 64 * 64 * 2;
     a.status = status; a.spin_limit = spin_limit();
-    return bw <= 32 ? pan::choose<T, 1>(st, P, V, Tm, ldt, a, num_sms)
-                    : pan::choose<T, 2>(st, P, V, Tm, ldt, a, num_sms);
+    if (bw <= 32) return pan::choose<T, 1>(st, P, V, Tm, ldt, a, num_sms);
+    const cudaError_t e = pan::choose<T, 2>(st, P, V, Tm, ldt, a, num_sms);
+    return e == cudaErrorInvalidConfiguration && m > 64 ? pan::in_two<T>(st, P, V, ldv, Tm, ldt, a, work, num_sms) : e;
 }
 template cudaError_t panel_qr<double>(cudaStream_t, int, int, int, double *, int, double *, int, double *, int,
-                                      unsigned, unsigned long long *, int *, int);
+                                      unsigned, unsigned long long *, double *, int *, int);
 template cudaError_t panel_qr<float>(cudaStream_t, int, int, int, float *, int, float *, int, float *, int,
-                                     unsigned, unsigned long long *, int *, int);
+                                     unsigned, unsigned long long *, float *, int *, int);
 
 }  // namespace egb
+
+// Packets, rounded to 16 bytes, then the 2 x 32 x 32 values of work
+extern "C" size_t elsi_gb_panel_qr_f64_work(int m)
+{
+    return m < 1 ? 0 : egb::panel_packet_words(m, sizeof(double)) + 2 * 32 * 32;
+}
+
+extern "C" int elsi_gb_panel_qr_f64(int m, int b, double *P, int lda, double *V, int ldv, double *T, int ldt,
+                                    int num_sms, void *work, size_t work_words, int *status, void *stream)
+{
+    if (m < 1 || b < 1 || b > 64 || !P || !V || !T || !work || !status || lda < m || ldv < m || ldt < b || num_sms < 1 ||
+        (size_t)work % 16 != 0 || work_words < elsi_gb_panel_qr_f64_work(m))
+        return ELSI_ERR_ARG;
+    cudaStream_t st = (cudaStream_t)stream;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    unsigned long long *packets = reinterpret_cast<unsigned long long *>(work);
+    const size_t words = egb::panel_packet_words(m, sizeof(double));
+    cudaError_t e = cudaMemsetAsync(packets, 0, sizeof(unsigned long long) * words, st);
+    if (e == cudaSuccess)
+        e = egb::panel_qr<double>(st, m, m, b, P, lda, V, ldv, T, ldt, 0, packets, reinterpret_cast<double *>(packets + words),
+                                  status, num_sms < sms ? num_sms : sms);
+    return e == cudaSuccess ? ELSI_OK : ELSI_ERR_CUDA;
+}

@@ -254,15 +254,15 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
         T *V = v1 + r0 + (size_t)c0 * n;
         T *Tm = t1 + (size_t)c0 * b;
         int ldt = b;
-        if ((e = panel_qr<T>(st, m, m_first, bw, P, lda, V, n, Tm, ldt, (unsigned)c0, packets, status, num_sms)) != cudaSuccess)
+        T *Y = work + (size_t)2 * n * b;  // b x b
+        T *Z = Y + (size_t)b * b;         // b x b
+        if ((e = panel_qr<T>(st, m, m_first, bw, P, lda, V, n, Tm, ldt, (unsigned)c0, packets, Y, status, num_sms)) != cudaSuccess)
             return e;
 
         // ---- two-sided update of A22 = a[r0:, r0:] (full symmetric storage)
         T *A22 = a + r0 + (size_t)r0 * lda;
         T *X = work;                      // m x b
         T *W = work + (size_t)n * b;      // m x b
-        T *Y = work + (size_t)2 * n * b;  // b x b
-        T *Z = Y + (size_t)b * b;         // b x b
         // X = A22 V (binary32: the symmetric panel product that streams A22 once)
         bool xdone = false;
         if constexpr (sizeof(T) == 4) {
