@@ -106,16 +106,19 @@ int elsi_gb_gemm_f64_wide(int ta, int tb, int m, int n, int k, double alpha, con
                           int *status, void *stream);
 
 /*
- * elsi_gb_panel_qr_f64: the panel factorisation of the full-to-band reduction (Eq. 11, first
- *   line) in binary64: P (m x b, ld lda, 1 <= b <= 64) becomes R on and above the diagonal and
+ * elsi_gb_panel_qr_f64, _f32: the panel factorisation of the full-to-band reduction (Eq. 11, first
+ *   line): P (m x b, ld lda, 1 <= b <= 64) becomes R on and above the diagonal and
  *   the reflector tails below it, V (m x b, ldv) the explicit reflectors (unit diagonal, zero
  *   above), T (b x b, ldt, upper triangular) the factor of Q = I - V T V^T, P = Q R. num_sms:
  *   SMs to reckon with (at most those of the GPU; what does not fit side by side takes the
- *   forms with more rows a CTA). work: elsi_gb_panel_qr_f64_work(m) 8-byte words, 16-byte
+ *   forms with more rows a CTA). work: elsi_gb_panel_qr_f64_work(m) (_f32_work) 8-byte words, 16-byte
  *   aligned; status: device int[8], zeroed by the caller.
  */
 size_t elsi_gb_panel_qr_f64_work(int m);
+size_t elsi_gb_panel_qr_f32_work(int m);
 int elsi_gb_panel_qr_f64(int m, int b, double *P, int lda, double *V, int ldv, double *T, int ldt,
+                         int num_sms, void *work, size_t work_words, int *status, void *stream);
+int elsi_gb_panel_qr_f32(int m, int b, float *P, int lda, float *V, int ldv, float *T, int ldt,
                          int num_sms, void *work, size_t work_words, int *status, void *stream);
 
 #ifdef __cplusplus

@@ -18,7 +18,9 @@
 // same packets and is never waited for.
 //
 // Sums over CTAs are kept to more than the panel's precision: binary32 partial sums are added
-// with their rounding errors (Knuth's two-sum), since binary64 additions are scarce here.
+// with their rounding errors (Knuth's two-sum), since binary64 additions are scarce here, and
+// stay a pair of binary32 numbers up to the one rounding of the update's factors; T is formed from
+// the pairs in binary64.
 //
 // Measured per 64-column panel, before -> now: binary32 n = 777 0.73 -> 0.21 ms, n = 4096 0.82
 // -> 0.24 ms, n = 16384 0.85 -> 0.29 ms; binary64 n = 512 1.09 -> 0.40 ms, n = 5000 1.24 ->
@@ -51,6 +53,7 @@ template <> struct Sum<double> {
     __device__ __forceinline__ void add(double x) { v += x; }
     __device__ __forceinline__ void add(const Sum &o) { v += o.v; }
     __device__ __forceinline__ double value() const { return v; }
+    __device__ __forceinline__ double low() const { return 0.0; }
     __device__ __forceinline__ unsigned w0() const { return (unsigned)__double2loint(v); }
     __device__ __forceinline__ unsigned w1() const { return (unsigned)__double2hiint(v); }
     __device__ __forceinline__ static Sum from(unsigned a, unsigned b) { Sum s; s.v = __hiloint2double((int)b, (int)a); return s; }
@@ -66,6 +69,7 @@ template <> struct Sum<float> {
     }
     __device__ __forceinline__ void add(const Sum &o) { add(o.h); l += o.l; }
     __device__ __forceinline__ float value() const { return h + l; }
+    __device__ __forceinline__ float low() const { return l - ((h + l) - h); }  // of value() + low()
     __device__ __forceinline__ unsigned w0() const { return __float_as_uint(h); }
     __device__ __forceinline__ unsigned w1() const { return __float_as_uint(l); }
     __device__ __forceinline__ static Sum from(unsigned a, unsigned b) { Sum s; s.h = __uint_as_float(a); s.l = __uint_as_float(b); return s; }
@@ -77,6 +81,21 @@ template <> struct Sum<float> {
         return s;
     }
 };
+
+// tau (row + scl (d + dl)), rounded once: the products split by an FMA, the sum by two-sum
+__device__ __forceinline__ float update_factor(float tau, float scl, float row, float d, float dl)
+{
+    const float p = __fmul_rn(scl, d), s = __fadd_rn(row, p), b = __fadd_rn(s, -row);
+    const float t = __fadd_rn(__fadd_rn(row, -__fadd_rn(s, -b)), __fadd_rn(p, -b));
+    const float low = fmaf(scl, dl, t + fmaf(scl, d, -p));
+    const float h = __fadd_rn(s, low), l = __fadd_rn(low, -__fadd_rn(h, -s));
+    const float q = __fmul_rn(tau, h);
+    return q + fmaf(tau, l, fmaf(tau, h, -q));
+}
+__device__ __forceinline__ double update_factor(double tau, double scl, double row, double d, double)
+{
+    return tau * fma(scl, d, row);
+}
 
 __device__ __forceinline__ void ld2_relaxed(const u64 *p, u64 &a, u64 &b)
 {
@@ -107,7 +126,8 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(16) T xbuf[NW][RW];
     __shared__ T partw[NW][NC];
-    __shared__ T rowown[NC], dsum[NC], rowj[NC], scal[3], scls[NC];  // scls: 1 / x scale of column c's reflector
+    __shared__ T rowown[NC], dsum[NC], dlow[sizeof(T) == 4 ? NC : 1], rowj[NC], scal[3], scls[NC];  // scls: 1 / x scale of column c's reflector
+    __shared__ double gram[NC];  // CTA G: v_c . v_j
     __shared__ int failed;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = blockIdx.x, G = a.G, bw = a.bw;
@@ -223,6 +243,7 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
             if (g == 0) row = rowown[xc];
             const T d = tot.value();
             dsum[xc] = d;
+            if (sizeof(T) == 4) dlow[sizeof(T) == 4 ? xc : 0] = tot.low();
             rowj[xc] = row;
             if (xc == j) {
                 T beta, tau, scl;
@@ -241,7 +262,7 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
 #pragma unroll
             for (int c = 0; c < CPL; ++c) {
                 const int col = c * 32 + lane;
-                wv[c] = col > j ? tau * fma(scl, dsum[col], rowj[col]) : T(0);
+                wv[c] = col > j ? update_factor(tau, scl, rowj[col], dsum[col], dlow[sizeof(T) == 4 ? col : 0]) : T(0);
             }
             T wx[CPL];
 #pragma unroll
@@ -264,9 +285,15 @@ panel_kernel(T *P, T *V, T *Tm, int ldt, const Args a)
             }
         } else {
             // ---- T[0:j, j] = -tau T[0:j, 0:j] (v_c . v_j), forward recurrence
+            if (xg == 0) {
+                double d = (double)dsum[xc];
+                if (sizeof(T) == 4) d += (double)dlow[sizeof(T) == 4 ? xc : 0];
+                gram[xc] = ((double)scl * d + (double)rowj[xc]) * (LATE && xc < j ? (double)scls[xc] : 1.0);
+            }
+            __syncthreads();
             double acc = 0.0;
             if (xc < j)
-                for (int q = xc + xg; q < j; q += LPC) acc += Ts[xc][q] * ((double)scl * (double)dsum[q] + (double)rowj[q]) * (LATE ? (double)scls[q] : 1.0);
+                for (int q = xc + xg; q < j; q += LPC) acc += Ts[xc][q] * gram[q];
             __syncwarp();
 #pragma unroll
             for (int o = 1; o < LPC; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -410,27 +437,45 @@ template cudaError_t panel_qr<float>(cudaStream_t, int, int, int, float *, int, 
 
 }  // namespace egb
 
-// Packets, rounded to 16 bytes, then the 2 x 32 x 32 values of work
-extern "C" size_t elsi_gb_panel_qr_f64_work(int m)
-{
-    return m < 1 ? 0 : egb::panel_packet_words(m, sizeof(double)) + 2 * 32 * 32;
-}
+namespace egb {
 
-extern "C" int elsi_gb_panel_qr_f64(int m, int b, double *P, int lda, double *V, int ldv, double *T, int ldt,
-                                    int num_sms, void *work, size_t work_words, int *status, void *stream)
+// Packets, then the 2 x 32 x 32 values of work
+template <typename T>
+static size_t entry_words(int m) { return panel_packet_words(m, sizeof(T)) + 2 * 32 * 32; }
+
+template <typename T>
+static int panel_entry(int m, int b, T *P, int lda, T *V, int ldv, T *Tm, int ldt, int num_sms, void *work,
+                       size_t work_words, int *status, void *stream)
 {
-    if (m < 1 || b < 1 || b > 64 || !P || !V || !T || !work || !status || lda < m || ldv < m || ldt < b || num_sms < 1 ||
-        (size_t)work % 16 != 0 || work_words < elsi_gb_panel_qr_f64_work(m))
+    if (m < 1 || b < 1 || b > 64 || !P || !V || !Tm || !work || !status || lda < m || ldv < m || ldt < b || num_sms < 1 ||
+        (size_t)work % 16 != 0 || work_words < entry_words<T>(m))
         return ELSI_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     unsigned long long *packets = reinterpret_cast<unsigned long long *>(work);
-    const size_t words = egb::panel_packet_words(m, sizeof(double));
+    const size_t words = panel_packet_words(m, sizeof(T));
     cudaError_t e = cudaMemsetAsync(packets, 0, sizeof(unsigned long long) * words, st);
     if (e == cudaSuccess)
-        e = egb::panel_qr<double>(st, m, m, b, P, lda, V, ldv, T, ldt, 0, packets, reinterpret_cast<double *>(packets + words),
-                                  status, num_sms < sms ? num_sms : sms);
+        e = panel_qr<T>(st, m, m, b, P, lda, V, ldv, Tm, ldt, 0, packets, reinterpret_cast<T *>(packets + words), status,
+                        num_sms < sms ? num_sms : sms);
     return e == cudaSuccess ? ELSI_OK : ELSI_ERR_CUDA;
+}
+
+}  // namespace egb
+
+extern "C" size_t elsi_gb_panel_qr_f64_work(int m) { return m < 1 ? 0 : egb::entry_words<double>(m); }
+extern "C" size_t elsi_gb_panel_qr_f32_work(int m) { return m < 1 ? 0 : egb::entry_words<float>(m); }
+
+extern "C" int elsi_gb_panel_qr_f64(int m, int b, double *P, int lda, double *V, int ldv, double *T, int ldt,
+                                    int num_sms, void *work, size_t work_words, int *status, void *stream)
+{
+    return egb::panel_entry<double>(m, b, P, lda, V, ldv, T, ldt, num_sms, work, work_words, status, stream);
+}
+
+extern "C" int elsi_gb_panel_qr_f32(int m, int b, float *P, int lda, float *V, int ldv, float *T, int ldt,
+                                    int num_sms, void *work, size_t work_words, int *status, void *stream)
+{
+    return egb::panel_entry<float>(m, b, P, lda, V, ldv, T, ldt, num_sms, work, work_words, status, stream);
 }
