@@ -121,6 +121,12 @@ int elsi_gb_panel_qr_f64(int m, int b, double *P, int lda, double *V, int ldv, d
 int elsi_gb_panel_qr_f32(int m, int b, float *P, int lda, float *V, int ldv, float *T, int ldt,
                          int num_sms, void *work, size_t work_words, int *status, void *stream);
 
+/*
+ * elsi_gb_recip_rsq: r[i] = 1 / x[i] and s[i] = 1 / sqrt(x[i]) (device arrays of n binary64 or
+ *   binary32 values) as the reflectors, Cholesky pivots and twisted factorisations form them.
+ */
+int elsi_gb_recip_rsq(int n, int binary64, const void *x, void *r, void *s, void *stream);
+
 #ifdef __cplusplus
 }
 #endif

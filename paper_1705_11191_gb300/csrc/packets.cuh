@@ -118,11 +118,15 @@ __device__ __forceinline__ bool get_own(const u64 *p, unsigned seq, T &v, long l
 
 }  // namespace pkt
 
-// 1 / x and 1 / sqrt(x) to about an ulp: the hardware's approximation (about 2^-20 in binary64) and
-// a step of third order (two of Newton's are a longer chain), one of Newton's in binary32. A
+// 1 / x and 1 / sqrt(x), within 1 and 1.25 ulp: the hardware's approximation r (about 2^-20 in
+// binary64) and one of Householder's iterations (A. S. Householder, The Numerical Treatment of
+// a Single Nonlinear Equation, 1970), that of third order in binary64 (two of second order are
+// a longer chain), Newton's in binary32. With h = 1 - x r the value is r / (1 - h) = r (1 + h + h^2 +
+// ..), with h = 1 - x r^2 it is r (1 - h)^(-1/2) = r (1 + h / 2 + 3 h^2 / 8 + ..), cut after h^2. A
 // library division or square root is two to three times as long a chain, and in binary64 two
 // to three times as many operations of the chip's few binary64 units. Arguments whose result
-// or whose approximation would be subnormal or overflow take the library's path.
+// or whose approximation would be subnormal or overflow take the library's path, or in binary32
+// square roots a scaled argument.
 __device__ __forceinline__ double recip(double x)
 {
     const int ex = __double2hiint(x) & 0x7FF00000;
@@ -149,12 +153,19 @@ __device__ __forceinline__ double rsq(double x)
     const double h = fma(-x * r, r, 1.0);  // r (1 + h / 2 + 3 h^2 / 8): a relative error of 5 h^3 / 16
     return fma(h * r, fma(0.375, h, 0.5), r);
 }
-__device__ __forceinline__ float rsq(float x)
+__device__ __forceinline__ float rsq_step(float x)
 {
-    if (!(x > 1e-36f && x < 1e36f)) return 1.0f / sqrtf(x);
     float r;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
+}
+__device__ __forceinline__ float rsq(float x)
+{
+    if (x > 1e-36f && x < 1e36f) return rsq_step(x);
+    // (a square root and a division are two roundings, up to 1.5 ulp)
+    if (x > 0.0f && x <= 1e-36f) return 0x1p32f * rsq_step(0x1p64f * x);
+    if (x >= 1e36f && x < INFINITY) return 0x1p-32f * rsq_step(0x1p-64f * x);
+    return 1.0f / sqrtf(x);
 }
 
 // Householder scalars of x = (alpha, tail) with |tail|^2 = ss: v = (1, scl tail), H = I - tau

@@ -479,3 +479,24 @@ extern "C" int elsi_gb_panel_qr_f32(int m, int b, float *P, int lda, float *V, i
 {
     return egb::panel_entry<float>(m, b, P, lda, V, ldv, T, ldt, num_sms, work, work_words, status, stream);
 }
+
+namespace egb {
+template <typename T>
+__global__ void recip_rsq_kernel(int n, const T *x, T *r, T *s)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    r[i] = recip(x[i]);
+    s[i] = rsq(x[i]);
+}
+}  // namespace egb
+
+extern "C" int elsi_gb_recip_rsq(int n, int binary64, const void *x, void *r, void *s, void *stream)
+{
+    if (n < 1 || !x || !r || !s) return ELSI_ERR_ARG;
+    cudaStream_t st = (cudaStream_t)stream;
+    const int grid = egb::ceil_div(n, 256);
+    if (binary64) egb::recip_rsq_kernel<double><<<grid, 256, 0, st>>>(n, (const double *)x, (double *)r, (double *)s);
+    else egb::recip_rsq_kernel<float><<<grid, 256, 0, st>>>(n, (const float *)x, (float *)r, (float *)s);
+    return cudaGetLastError() == cudaSuccess ? ELSI_OK : ELSI_ERR_CUDA;
+}
