@@ -239,9 +239,9 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
         BCK(cudaMemcpyAsync(b.offs, off.data(), sizeof(int) * (nprob + 1), cudaMemcpyHostToDevice, h->stream));
         BCK(cudaStreamSynchronize(h->stream));
     }
-    // Problem order: largest first (longest-processing-time order), each problem taken by
-    // the next free solver instance (worker: own handle, stream and host thread, since a
-    // solve is synchronous on its host thread).
+    // Problem order: largest first (longest-processing-time order), the first W dealt out, each later
+    // one taken by the next free solver instance (worker: own handle, stream and host thread,
+    // since a solve is synchronous on its host thread).
     std::vector<int> order(nprob);
     for (int i = 0; i < nprob; ++i) order[i] = i;
     const int mult = cplx ? 2 : 1;
@@ -480,30 +480,25 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
     }
     rc = add_workers(W);
     if (rc) return rc;
-    // Every instance has room for the largest problem from the start (W is bounded for that): which
-    // instance takes which problem changes from call to call, and one that has to grow frees and
-    // allocates while the others compute (90 to 130 ms for a batch of 55).
+    // Instance t begins with the t-th largest problem and has room for it before anything runs: what it
+    // takes later is not of a higher order, and an instance that has to grow frees and allocates while the
+    // others compute (90 to 130 ms for a batch of 55). With room for the largest in every instance a
+    // batch of one large and many small problems held W times the memory it needs.
     if (W > 1) {
-        size_t nmax = 0, kmax = 0;
-        int imax = 0;
-        for (int i = 0; i < nprob; ++i) {
-            const size_t N = (size_t)mult * b.items[i].n, K = (size_t)mult * b.items[i].k;
-            if (N > nmax) { nmax = N; imax = i; }
-            if (K > kmax) kmax = K;
-        }
         for (int t = 0; t < W; ++t) {
             elsi_gb_handle_s *s;
             cudaStream_t wst;
             instance(t, W, &s, &wst);
-            configure(s, wst, tv[imax]);
-            s->n = (int)nmax;
-            s->n_state = (int)(kmax < nmax ? kmax : nmax);
+            const BatchItem &it = b.items[order[t]];
+            configure(s, wst, tv[order[t]]);
+            s->n = mult * it.n;
+            s->n_state = mult * it.k;
             const int kz = s->precision == ELSI_PREC_FP32_REFINE ? s->n : s->n_state;
             if (ensure_workspace(s, kz) != ELSI_OK) free_workspace(s);  // the solve asks for what it needs
         }
     }
     std::vector<Result> res(W);
-    std::atomic<int> next{0};
+    std::atomic<int> next{W};
     auto work = [&](int t) {
         cudaSetDevice(dev);
         elsi_gb_handle_s *s;
@@ -511,9 +506,7 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
         instance(t, W, &s, &wst);
         Result &r = res[t];
         ConcurrentSolves share;
-        for (;;) {
-            const int q = next.fetch_add(1);
-            if (q >= nprob) break;
+        for (int q = t; q < nprob; q = next.fetch_add(1)) {
             const int i = order[q];
             const BatchItem &it = b.items[i];
             share.set(W < nprob - q ? W : nprob - q);
