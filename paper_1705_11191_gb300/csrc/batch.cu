@@ -442,7 +442,7 @@ int batch_ev(elsi_gb_handle_s *h, int nprob, const int *n_basis, const int *n_st
         const bool known = tune_get(dev, prec, cplx, size_bucket(N), &v);
         if (!known) {
             // (binary32 route: 64; several solves at a time fill the chip, 8 of n = 2000 69 ms against 72)
-            v.band = prec == ELSI_PREC_FP64 ? band_of(h, prec) : h->band_width;
+            v.band = prec == ELSI_PREC_FP64 ? band_of(h, prec, N) : h->band_width;
             v.solver = h->elpa_solver;
             v.workers = h->batch_workers > 0 ? h->batch_workers : default_workers(N);
             if (h->batch_autotune) {

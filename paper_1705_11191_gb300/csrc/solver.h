@@ -122,16 +122,17 @@ struct SolveRequest {
     bool want_edm = false;         // dm: keep W in the handle
 };
 
-// Band width of a solve in the given route: the one that was set, else 64 and, where the shorter steps
+// Band width of a solve of order n (the handle's, or a batch's problem) in the given route: the one that was set, else 64 and, where the shorter steps
 // of the bulge chase save more than the back-transformation then costs, 32. Binary64 route: a step
 // is 7 b^2 FMAs at two a clock (n = 1531: 35 -> 12 ms, n = 5000: 118 -> 46 ms); with b = 32 the chase holds
 // up to 608 positions on the chip, orders up to 19 400. Binary32 route, whole solves with 64 and 32:
 // n = 500 8.2 and 8.0 ms, 1200 19.0 and 18.3, 2000 32.2 and 31.0, 3000 50.4 and 49.4, 4096 75.9 and 76.0,
 // 6000 141 and 148.
-inline int band_of(const elsi_gb_handle_s *h, int precision)
+inline int band_of(const elsi_gb_handle_s *h, int precision, size_t n)
 {
-    return !h->band_set && h->n <= (precision == ELSI_PREC_FP64 ? 19000 : 3500) ? 32 : h->band_width;
+    return !h->band_set && n <= (precision == ELSI_PREC_FP64 ? 19000 : 3500) ? 32 : h->band_width;
 }
+inline int band_of(const elsi_gb_handle_s *h, int precision) { return band_of(h, precision, (size_t)h->n); }
 
 int set_error(elsi_gb_handle_s *h, int code, const char *fmt, ...);
 bool ensure_buf(void **p, size_t *cap, size_t bytes);

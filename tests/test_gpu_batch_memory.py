@@ -33,3 +33,15 @@ def test_one_large_and_several_small_problems(precision):
     used([1], 1)  # what the context itself takes on a first call
     alone, together = used([1], 1), used([0, 1, 2, 3], 4)
     assert together < 1.6 * alone
+
+
+def test_band_width_goes_by_the_order_of_the_problem():
+    """... and not by that of the handle, which solves none of its own here."""
+    n = 2999  # a size class that no other test tunes
+    a = torch.randn(n, n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    with egb.Handle(25000, 10, 10.0) as hd:
+        hd.use_current_stream()
+        hd.set_overlap_is_unit(True)
+        hd.set_batch_autotune(False)
+        hd.batch_ev([a + a.T], None, [10])
+        assert hd.batch_tuning(n)[0] == 32
