@@ -128,11 +128,17 @@ inline int refine_block(int n, int k)
 // reduction. work: 2 x 32 x 32 values (panels of bw > 32 with more rows than one launch takes).
 size_t panel_packet_words(int m, int elem);
 
-// Words of the sync scratch: the base (the partials of the W kernels, or the packets of the
-// bulge chase), then the packets of the panel factorisations.
-constexpr int kSyncBlocks = 512;
-constexpr size_t kSyncWords = 64 + 2 * (size_t)kSyncBlocks * 64 * 64;
-inline size_t sync_words(int n, int elem) { return kSyncWords + 2 * panel_packet_words(n, elem); }
+// Words of the sync scratch: the base (the packets of the bulge chase, and before that the partials of
+// the W kernels, 64 x 64 values for every kWRows rows), then the packets of the panel factorisations.
+constexpr int kWRows32 = 64, kWRows64 = 16;
+constexpr size_t kSyncWords = 64 + 2 * (size_t)512 * 64 * 64;
+inline size_t sync_base_words(int n, int elem)
+{
+    const size_t blocks = elem == 4 ? n / kWRows32 + 2 : n / kWRows64 + 2;  // and their sum
+    const size_t w = 64 + blocks * 64 * 64 * (elem / 4);
+    return w > kSyncWords ? w : kSyncWords;
+}
+inline size_t sync_words(int n, int elem) { return sync_base_words(n, elem) + 2 * panel_packet_words(n, elem); }
 template <typename T>
 cudaError_t panel_qr(cudaStream_t st, int m, int m_first, int bw, T *P, int lda, T *V, int ldv, T *Tm, int ldt,
                      unsigned seq0, unsigned long long *packets, T *work, int *status, int num_sms);

@@ -20,8 +20,9 @@ namespace egb {
 // two FMAs a clock and SM, so its blocks are 16 rows: four times the CTAs of 64-row blocks
 // (two launches of 135 us at any order), and V (T^T Y) is formed as (V T^T) Y, whose work
 // shrinks with the rows, where T^T Y costs every block 64^3 FMAs: 27 and 20 us at n = 1531,
-// b = 32, and 11 and 13 us with CJ = 2.
-template <typename T> constexpr int WRows = sizeof(T) == 4 ? 64 : 16;
+// b = 32, and 11 and 13 us with CJ = 2. (From 8176 rows on, more than 512 blocks, five general
+// products in their place take as long: full to band of n = 9000 317 and 318 ms, n = 16384 1591 and 1589.)
+template <typename T> constexpr int WRows = sizeof(T) == 4 ? kWRows32 : kWRows64;
 constexpr int kWLd = 65;
 
 // c[R][CJ] = sum_{k < kmax} A[R ty + i][k] B[k][CJ tx + j] for tiles A, B with leading dimension
@@ -192,15 +193,6 @@ __global__ void __launch_bounds__(256) w_stage3_kernel(int m, int bw, const T *X
     if (sizeof(T) == 8) block_exponent(top, wexp);
 }
 
-// The same from W in memory (m x bw, one after the other), *wexp zeroed before
-__global__ void __launch_bounds__(256) w_exponent_kernel(size_t total, const double *__restrict__ W, int *wexp)
-{
-    int top = 0;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x)
-        top = max(top, __double2hiint(W[e]) & 0x7FF00000);
-    block_exponent(top, wexp);
-}
-
 template <typename T, int CJ>
 static cudaError_t form_w(cudaStream_t st, int m, int bw, const T *xa, const T *V, int ldv,
                           const T *Tm, int ldt, T *X, T *Y, T *W, T *ypart, int *wexp)
@@ -226,7 +218,7 @@ static cudaError_t form_w(cudaStream_t st, int m, int bw, const T *xa, const T *
 
 size_t sy2sb_work_elems(int n, int b)
 {
-    // X (n x b), W (n x b), Y (b x b), Z (b x b)
+    // X (n x b), W (n x b), scratch of the panel (2 b x b)
     return (size_t)4 * n * b + 4 * (size_t)b * b;
 }
 
@@ -238,7 +230,7 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
     if (b > 64 || b < 1) return cudaErrorInvalidValue;
     // sync layout: partials of the W kernels, then the packets of the panel factorisation
     T *ypart = reinterpret_cast<T *>(sync + 64);
-    unsigned long long *packets = reinterpret_cast<unsigned long long *>(sync + kSyncWords);
+    unsigned long long *packets = reinterpret_cast<unsigned long long *>(sync + sync_base_words(n, sizeof(T)));
     const int m_first = n - b;
     if (m_first >= 2 &&
         (e = cudaMemsetAsync(packets, 0, sizeof(unsigned long long) * panel_packet_words(m_first, sizeof(T)), st)) != cudaSuccess)
@@ -254,8 +246,7 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
         T *V = v1 + r0 + (size_t)c0 * n;
         T *Tm = t1 + (size_t)c0 * b;
         int ldt = b;
-        T *Y = work + (size_t)2 * n * b;  // b x b
-        T *Z = Y + (size_t)b * b;         // b x b
+        T *Y = work + (size_t)2 * n * b;  // 2 b x b, for panel_qr
         if ((e = panel_qr<T>(st, m, m_first, bw, P, lda, V, n, Tm, ldt, (unsigned)c0, packets, Y, status, num_sms)) != cudaSuccess)
             return e;
 
@@ -281,31 +272,11 @@ cudaError_t sy2sb(cudaStream_t st, int n, int b, T *a, int lda, T *v1, T *t1, T 
         // (A22 is symmetric: transposed, its rows are contiguous for the digit split)
         if (!xdone && (e = gemm<T>(st, 1, 0, m, bw, m, T(1), A22, lda, V, n, T(0), W, m)) != cudaSuccess)
             return e;
-        if (ceil_div(m, WRows<T>) + 1 <= kSyncBlocks) {
-            // X = (A22 V) T, W = X - 1/2 V (T^T (V^T X))
-            T *ysum = ypart + (size_t)ceil_div(m, WRows<T>) * 64 * 64;
-            e = bw <= 32 ? form_w<T, 2>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart, status + ST_WEXP)
-                         : form_w<T, 4>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart, status + ST_WEXP);
-            if (e != cudaSuccess) return e;
-        } else {
-            // X = (A22 V) T
-            if ((e = gemm<T>(st, 0, 0, m, bw, bw, T(1), W, m, Tm, ldt, T(0), X, m)) != cudaSuccess) return e;
-            // Y = V^T X
-            if ((e = gemm_splitk<T>(st, 1, 0, bw, bw, m, T(1), V, n, X, m, Y, bw, W,
-                                    (size_t)n * b)) != cudaSuccess) return e;
-            // Z = T^T Y
-            if ((e = gemm<T>(st, 1, 0, bw, bw, bw, T(1), Tm, ldt, Y, bw, T(0), Z, bw)) != cudaSuccess) return e;
-            // W = X - 1/2 V Z
-            if ((e = cudaMemcpyAsync(W, X, sizeof(T) * (size_t)m * bw, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
-            if ((e = gemm<T>(st, 0, 0, m, bw, bw, T(-0.5), V, n, Z, bw, T(1), W, m)) != cudaSuccess) return e;
-            if constexpr (sizeof(T) == 8) {
-                if ((e = cudaMemsetAsync(status + ST_WEXP, 0, sizeof(int), st)) != cudaSuccess) return e;
-                const int grid = ceil_div((long long)m * bw, 256);
-                EGB_COUNT_LAUNCH();
-                w_exponent_kernel<<<grid < 152 * 4 ? grid : 152 * 4, 256, 0, st>>>((size_t)m * bw, W, status + ST_WEXP);
-                if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            }
-        }
+        // X = (A22 V) T, W = X - 1/2 V (T^T (V^T X))
+        T *ysum = ypart + (size_t)ceil_div(m, WRows<T>) * 64 * 64;
+        e = bw <= 32 ? form_w<T, 2>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart, status + ST_WEXP)
+                     : form_w<T, 4>(st, m, bw, W, V, n, Tm, ldt, X, ysum, W, ypart, status + ST_WEXP);
+        if (e != cudaSuccess) return e;
         // A22 -= V W^T + W V^T   (lower triangle), then mirror. On the tensor-core path the
         // two products are one GEMM over K = 2 bw: [V W] [W V]^T.
         bool done = false;
