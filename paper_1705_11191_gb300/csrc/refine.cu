@@ -578,7 +578,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     const char *venv = getenv("ELSI_GB_VERBOSE");
     const bool verbose = venv && venv[0] == '1';
     int iters = 0;
-    double emax = 1.0;
+    double emax = 1.0, eprev = 1.0;
     for (int it = 0; it < h->refine_max_iter; ++it) {
         // digit planes of this iteration's products: 4 (35 bits) in the first two iterations
         // (binary32 start, errors of about 1e-3), all 6 (53 bits) from the third on. The
@@ -601,6 +601,7 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
         add_f32_to_f64_kernel<<<grid_for(nk), 256, 0, st>>>(nk, R32, XO);
         CKR(cudaMemcpyAsync(w.scal_host + 8, STATS, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
         CKR(cudaStreamSynchronize(st));
+        eprev = emax;
         emax = w.scal_host[8];
         ++iters;
         if (verbose)
@@ -638,9 +639,13 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     h->refine_iters = iters;
     h->orth_err = w.scal_host[8];
     if (verbose) fprintf(stderr, "[elsi-gb] refine final orthonormality defect %.3e\n", h->orth_err);
-    if (!(emax < 1e-8) || !(h->orth_err < 1e-10))
+    // What is left after the last correction is smaller than it by the rate of the last two, 1e-3 and
+    // less where the refinement converges. It stalls where the binary32 vectors of the unwanted
+    // states do not span their space (hundreds of eigenvalues closer than binary64 can tell apart,
+    // as at the end of a graded spectrum), and a small correction then says little about the error.
+    if (!(emax < 1e-8) || !(emax * fmin(1.0, emax / eprev) < 1e-10) || !(h->orth_err < 1e-10))
         return set_error(h, ELSI_ERR_NO_CONVERGENCE,
-                         "refinement did not converge (max|E| %.3g, orthonormality %.3g)", emax,
+                         "refinement did not converge (max|E| %.3g after %.3g, orthonormality %.3g)", emax, eprev,
                          h->orth_err);
     // The refinement converges to the eigenpairs nearest its binary32 start. A start whose
     // error exceeds the gaps (a standard form spoilt by a nearly singular S) can converge to
