@@ -79,12 +79,14 @@ __global__ void occupation_kernel(int k, const double *eps_all, double n_el_all,
         const double rkt = 1.0 / kt;
         // Far from mu an exponential adds nothing to the count (above x = 80 less than 2e-35 a
         // state, below -37 exactly 1): a warp of such states skips the 50 or so operations of the
-        // binary64 unit that are most of the cost of a bisection step.
+        // binary64 unit that are most of the cost of a bisection step. Not without electrons: there every
+        // count is compared with zero.
+        const double far = n_el > 1e-30 ? 80.0 : INFINITY;
         auto count = [&](double mu) {
             double s2 = 0.0;
             for (int l = tid; l < kk; l += nt) {
                 const double x = (eps(l) - mu) * rkt;
-                if (scheme != ELSI_OCC_FERMI || x < 80.0) s2 += g * occ_phi(scheme, x);
+                if (scheme != ELSI_OCC_FERMI || x < far) s2 += g * occ_phi(scheme, x);
             }
             return block_sum(s2, red);
         };
