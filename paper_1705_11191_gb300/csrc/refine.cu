@@ -313,7 +313,8 @@ __global__ void orth_defect_kernel(int kc, int ld, const double *sm, unsigned lo
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < (size_t)kc * kc;
          q += (size_t)gridDim.x * blockDim.x) {
         int i = (int)(q % kc), j = (int)(q / kc);
-        r = fmax(r, fabs((i == j ? 1.0 : 0.0) - sm[(size_t)i + (size_t)j * ld]));
+        const double d = fabs((i == j ? 1.0 : 0.0) - sm[(size_t)i + (size_t)j * ld]);
+        r = d <= DBL_MAX ? fmax(r, d) : INFINITY;  // (fmax drops a NaN)
     }
     for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
     if ((threadIdx.x & 31) == 0) atomicMax(stats, (unsigned long long)__double_as_longlong(r));
