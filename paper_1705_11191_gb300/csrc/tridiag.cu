@@ -423,12 +423,12 @@ twist_factor_kernel(const double *__restrict__ d, const double *__restrict__ e, 
 constexpr int kTwistWarps = 8, kTwistRows = 16;
 
 // z / ||z|| for each of the first kvec eigenvalues (zero outside its block), from the factors;
-// lplus and uminus are overwritten by z.
+// lplus and uminus are overwritten by z. A vector that is lost is zero, and the end of its block negative.
 template <typename T>
 __global__ void __launch_bounds__(32 * kTwistWarps)
 twist_vector_kernel(int n, const double *__restrict__ d, const double *__restrict__ e, int kvec,
-                    const double *__restrict__ w, const double *bounds, const int *__restrict__ blk,
-                    const double *__restrict__ dplus, double *lplus, double *uminus, T *z, int ldz, int *status)
+                    const double *__restrict__ w, const double *bounds, int *blk,
+                    const double *__restrict__ dplus, double *lplus, double *uminus, T *z, int ldz)
 {
     __shared__ T tile[kTwistWarps][32][kTwistRows + 1];
     __shared__ double best_w[kTwistWarps][32], nrm_w[2][32];
@@ -508,8 +508,13 @@ twist_vector_kernel(int n, const double *__restrict__ d, const double *__restric
     }
     __syncthreads();
     const double nrm2 = 1.0 + nrm_w[0][lane] + nrm_w[1][lane];
-    if (warp == 0 && have && !(nrm2 < DBL_MAX)) report_error(status, ELSI_ERR_NO_CONVERGENCE, l);
-    const double s = (nrm2 < DBL_MAX) ? 1.0 / sqrt(nrm2) : 1.0;
+    // No eigenvector: a product out of range, next to pivots of zero in a group of coinciding eigenvalues,
+    // or a residual |gamma| / ||z|| far above the accuracy of the eigenvalue (at most sqrt(n) times
+    // 1e-8 ||T||, or 1e-15): a block that does not hold it, where a group is spread over several. The
+    // vector is left to cluster_orth_kernel.
+    const bool lost = !(nrm2 < DBL_MAX) || !(fabs(best) <= ((sizeof(T) == 8 ? 1e-8 : 1e-4) * bounds[3] + 8.0 * pivmin) * sqrt(nrm2));
+    if (warp == 0 && have && lost) blk[2 * l + 1] = -be;
+    const double s = lost ? 0.0 : 1.0 / sqrt(nrm2);
     // ---- scaled into the columns of z
     for (int i0 = warp * kTwistRows; i0 < n; i0 += kTwistWarps * kTwistRows) {
 #pragma unroll
@@ -518,7 +523,7 @@ twist_vector_kernel(int n, const double *__restrict__ d, const double *__restric
             double x = 0.0;
             if (i >= bs && i < be)
                 x = i < r ? lplus[(size_t)i * kvec + l] : i > r ? uminus[(size_t)(i - 1) * kvec + l] : 1.0;
-            tile[warp][lane][q] = (T)(x * s);
+            tile[warp][lane][q] = lost ? T(0) : (T)(x * s);
         }
         __syncwarp();
         const int q = lane % kTwistRows;
@@ -581,6 +586,7 @@ template <> struct Wide<float> {
 // Measured together with inverse_iteration below, both phases: n = 16384 39 -> 3.6 ms, eight solves of
 // n = 2000 at a time 49 -> 5.3 ms in all (of which this form 2 and 1).
 constexpr int kOrthPiece = 64;  // vectors orthogonalised together (pieces and seams)
+constexpr int kOrthRun = 1024;  // and of a run of coinciding eigenvalues
 
 template <typename T>
 __device__ double cluster_project(int n, int i0, int v, T *z, int ldz, double *red)
@@ -589,31 +595,33 @@ __device__ double cluster_project(int n, int i0, int v, T *z, int ldz, double *r
     __shared__ typename W::Coef coef[kOrthPiece];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     T *zv = z + (size_t)v * ldz;
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int u = i0 + warp; u < v; u += nw) {
-            const T *zu = z + (size_t)u * ldz;
-            W a, b;
-            int i = lane;
-            for (; i + 32 < n; i += 64) {
-                a.fma_(zu[i], zv[i]);
-                b.fma_(zu[i + 32], zv[i + 32]);
-            }
-            if (i < n) a.fma_(zu[i], zv[i]);
-            double s = a.value() + b.value();
+    for (int pass = 0; pass < 2; ++pass)
+        for (int u0 = i0; u0 < v; u0 += kOrthPiece) {  // (once but for the long runs of phase 2)
+            const int u1 = min(v, u0 + kOrthPiece);
+            for (int u = u0 + warp; u < u1; u += nw) {
+                const T *zu = z + (size_t)u * ldz;
+                W a, b;
+                int i = lane;
+                for (; i + 32 < n; i += 64) {
+                    a.fma_(zu[i], zv[i]);
+                    b.fma_(zu[i + 32], zv[i + 32]);
+                }
+                if (i < n) a.fma_(zu[i], zv[i]);
+                double s = a.value() + b.value();
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) coef[u - i0] = W::coef(s);
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            W x(zv[i]);
-            const T *zu = z + (size_t)i0 * ldz + i;
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane == 0) coef[u - u0] = W::coef(s);
+            }
+            __syncthreads();
+            for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                W x(zv[i]);
+                const T *zu = z + (size_t)u0 * ldz + i;
 #pragma unroll 4
-            for (int u = 0; u < v - i0; ++u) x.fms(coef[u], zu[(size_t)u * ldz]);
-            zv[i] = x.rounded();
+                for (int u = 0; u < u1 - u0; ++u) x.fms(coef[u], zu[(size_t)u * ldz]);
+                zv[i] = x.rounded();
+            }
+            __syncthreads();
         }
-        __syncthreads();
-    }
     W s;
     for (int i = threadIdx.x; i < n; i += blockDim.x) s.fma_(zv[i], zv[i]);
     return block_sum(s.value(), red);
@@ -749,10 +757,55 @@ __device__ void inverse_iteration(int n, int bs, int be, int kvec, int v, const 
     for (int i = tid; i < n; i += C) zv[i] = (i >= bs && i < be) ? (T)(x[(size_t)i * kvec] * sc) : T(0);
 }
 
+// D+ of vector v for another shift, by the whole CTA: one thread runs the recurrence over chunks of
+// rows in shared memory (rare: a second attempt below).
+__device__ void shifted_factor(int bs, int be, int kvec, int v, const double *__restrict__ d,
+                               const double *__restrict__ e, double lam, double pivmin, double *dplus)
+{
+    __shared__ double sd[kOrthThreads], se[kOrthThreads];
+    const int tid = threadIdx.x;
+    double dp = 0.0;
+    for (int r0 = bs; r0 < be; r0 += kOrthThreads) {
+        const int i = r0 + tid, cnt = min(kOrthThreads, be - r0);
+        if (i < be) {
+            sd[tid] = d[i] - lam;
+            se[tid] = i > bs ? e[i - 1] : 0.0;
+        }
+        __syncthreads();
+        if (tid == 0)
+            for (int j = 0; j < cnt; ++j) {
+                dp = r0 + j == bs ? sd[j] : fma(-(se[j] / dp), se[j], sd[j]);
+                dp = guard_pivot(dp, pivmin);
+                sd[j] = dp;
+            }
+        __syncthreads();
+        if (i < be) dplus[(size_t)i * kvec + v] = sd[tid];
+        __syncthreads();
+    }
+}
+
+// |(T - lam I) z|^2
+template <typename T>
+__device__ double residual2(int n, const double *__restrict__ d, const double *__restrict__ e, double lam, const T *zv,
+                            double *red)
+{
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        double r = (d[i] - lam) * (double)zv[i];
+        if (i > 0) r = fma(e[i - 1], (double)zv[i - 1], r);
+        if (i + 1 < n) r = fma(e[i], (double)zv[i + 1], r);
+        s = fma(r, r, s);
+    }
+    return block_sum(s, red);
+}
+
 // Gram-Schmidt (two passes) within clusters of eigenvalues closer than tol_rel * ||T||,
 // on ranges of at most kOrthPiece vectors: phase 0 takes the pieces [s + 64p, s + 64p + 64)
 // of a cluster starting at s, phase 1 the seams [s + 64p + 32, s + 64p + 96) that cross a
-// piece boundary; one CTA per range start. A vector that the projection nearly annihilates (its
+// piece boundary; one CTA per range start. Eigenvalues that coincide to working accuracy have vectors
+// that are anything in their space, not orthogonal to eps ||T|| / spacing beyond a seam: phase 2 takes
+// every run of more than 32 of them whole, up to kOrthRun (binary64; one CTA, so time
+// grows with the square of the run: 64-fold at n = 600 10 ms). A vector that the projection nearly annihilates (its
 // eigenvalue coincides with an earlier one to working accuracy, as for the pairs of the
 // real form of a complex Hermitian matrix) is replaced by one step of inverse iteration
 // on its block, x = (T_b - lambda I)^{-1} b for a pseudo-random b orthogonal to the
@@ -760,32 +813,50 @@ __device__ void inverse_iteration(int n, int bs, int be, int kvec, int v, const 
 // dplus (the vector's spent U- column holds the intermediate values), and is then
 // projected and normalised again. When lambda sits much closer to an accepted vector's
 // eigenvalue than to its own, that vector dominates x; what is left after the projection
-// is still accurate as long as it is far above the rounding level.
+// is still accurate as long as it is far above the rounding level. In a group of many eigenvalues
+// that coincide to working accuracy lambda can be one of them to the last bit, and then x is that
+// one vector whatever b is; and where T splits, two of the group can have been given the same place
+// in the same block. So further attempts shift lambda by some roundings of ||T||, from where the
+// members of the group look alike (residuals stay at that size), and take all of T.
 template <typename T>
-__global__ void cluster_orth_kernel(int n, int kvec, const int *cstart, int phase, const double *e,
-                                    const int *blk, const double *dplus, double *work, T *z, int ldz,
-                                    int *status)
+__global__ void cluster_orth_kernel(int n, int kvec, const int *cstart, int phase, const double *d, const double *e,
+                                    const double *w, const double *bounds, int *blk, double *dplus, double *work,
+                                    T *z, int ldz, int *status)
 {
     __shared__ double red[32];
     const int i0 = blockIdx.x;
-    const int s = cstart[i0];
-    const int off = phase == 0 ? 0 : kOrthPiece / 2;
-    if ((i0 - s) % kOrthPiece != off) return;  // not a range start
-    int cend = i0 + 1;  // end of the cluster, looked for up to the end of the range
-    while (cend < kvec && cend < i0 + kOrthPiece && cstart[cend] == s) ++cend;
-    if (phase == 1 && cend <= i0 + kOrthPiece / 2) return;  // no piece boundary inside
+    int cend = i0 + 1;  // end of the range
+    if (phase < 2) {
+        const int s = cstart[i0];
+        const int off = phase == 0 ? 0 : kOrthPiece / 2;
+        if ((i0 - s) % kOrthPiece != off) return;  // not a range start
+        while (cend < kvec && cend < i0 + kOrthPiece && cstart[cend] == s) ++cend;
+        if (phase == 1 && cend <= i0 + kOrthPiece / 2) return;  // no piece boundary inside
+    } else {
+        const double same = 1e-12 * bounds[3];
+        if (i0 > 0 && w[i0] - w[i0 - 1] <= same) return;
+        while (cend < kvec && cend < i0 + kOrthRun && w[cend] - w[cend - 1] <= same) ++cend;
+        if (cend - i0 <= kOrthPiece / 2) return;
+    }
     const int i1 = cend;
-    if (i1 - i0 < 2) return;
-    for (int v = i0 + 1; v < i1; ++v) {
+    for (int v = i0; v < i1; ++v) {
+        const bool lost = blk[2 * v + 1] < 0;  // no vector from the twisted factorisation
+        if (v == i0 && !lost) continue;
         T *zv = z + (size_t)v * ldz;
-        double s = cluster_project(n, i0, v, z, ldz, red);
-        // a regenerated vector is accepted when its part orthogonal to the cluster is far
-        // above the rounding level of T (its direction error is then eps / sqrt(s))
-        const double accept = sizeof(T) == 8 ? 1e-16 : 1e-8;
-        bool regen = false;
-        for (int attempt = 0; attempt < 3 && s < (regen ? accept : 1e-4); ++attempt) {
-            regen = true;
-            const int bs = blk[2 * v], be = blk[2 * v + 1];
+        double s = lost ? 0.0 : cluster_project(n, i0, v, z, ldz, red);
+        // a regenerated vector is accepted when its part orthogonal to the cluster is a good part of
+        // it: what is wrong with the vectors before it enters with the factor 1 / sqrt(s), and adds up
+        // over a large group; after the last attempt, when that part is far above the rounding level
+        // of T (its direction error is then eps / sqrt(s))
+        constexpr int kAttempts = 5;
+        double accept = 1e-4;
+        for (int attempt = lost ? 1 : 0; attempt < kAttempts && !(s >= accept); ++attempt) {
+            accept = attempt + 1 < kAttempts ? 1e-3 : sizeof(T) == 8 ? 1e-16 : 1e-8;
+            const int bs = attempt == 0 ? blk[2 * v] : 0, be = attempt == 0 ? blk[2 * v + 1] : n;
+            if (attempt > 0) {
+                const double roundings = attempt == 1 ? 8.0 : attempt == 2 ? -8.0 : attempt == 3 ? 32.0 : -128.0;
+                shifted_factor(bs, be, kvec, v, d, e, w[v] + roundings * DBL_EPSILON * bounds[3], bounds[2], dplus);
+            }
             // start b: pseudo-random on the block, orthogonal to the cluster's vectors
             for (int i = threadIdx.x; i < n; i += blockDim.x)
                 zv[i] = (i >= bs && i < be) ? (T)hash_unit((unsigned)(v * 7919 + attempt), (unsigned)i) : T(0);
@@ -800,13 +871,17 @@ __global__ void cluster_orth_kernel(int n, int kvec, const int *cstart, int phas
             for (int i = threadIdx.x; i < n; i += blockDim.x) zv[i] = (T)((double)zv[i] * inv);
             __syncthreads();
             s = cluster_project(n, i0, v, z, ldz, red);
+            // with every vector of the group in this block taken, x is of other eigenvalues
+            const double tol = (sizeof(T) == 8 ? 1e-10 : 1e-5) * bounds[3] + 8.0 * bounds[2];
+            if (!(residual2(n, d, e, w[v], zv, red) <= tol * tol * s)) s = 0.0;
         }
-        if (s < (regen ? accept : 1e-4)) {
+        if (!(s >= accept)) {
             if (threadIdx.x == 0) report_error(status, ELSI_ERR_NO_CONVERGENCE, v);
             return;
         }
         const double inv = 1.0 / sqrt(s);
         for (int i = threadIdx.x; i < n; i += blockDim.x) zv[i] = (T)((double)zv[i] * inv);
+        if (lost && threadIdx.x == 0) blk[2 * v + 1] = -blk[2 * v + 1];
         __syncthreads();
     }
 }
@@ -829,15 +904,15 @@ cudaError_t stein(cudaStream_t st, int n, const double *d, const double *e, int 
     twist_factor_kernel<<<dim3(ceil_div(kvec, 32), 2), 32, 0, st>>>(d, e, kvec, w, bounds, blk, dplus, lplus, uminus);
     EGB_COUNT_LAUNCH();
     twist_vector_kernel<T><<<ceil_div(kvec, 32), 32 * kTwistWarps, 0, st>>>(n, d, e, kvec, w, bounds, blk, dplus, lplus,
-                                                                           uminus, z, ldz, status);
+                                                                           uminus, z, ldz);
     // cluster starts (in the L+ scratch, no longer needed), then pieces and seams
     int *cstart = reinterpret_cast<int *>(lplus);
     EGB_COUNT_LAUNCH();
     cluster_start_kernel<<<1, 1024, 0, st>>>(kvec, w, bounds, 1e-5, cstart);
-    for (int phase = 0; phase < 2; ++phase) {
+    for (int phase = 0; phase < (sizeof(T) == 8 && kvec > kOrthPiece / 2 ? 3 : 2); ++phase) {
         EGB_COUNT_LAUNCH();
-        cluster_orth_kernel<T><<<kvec, kOrthThreads, 0, st>>>(n, kvec, cstart, phase, e, blk, dplus, uminus, z,
-                                                     ldz, status);
+        cluster_orth_kernel<T><<<kvec, kOrthThreads, 0, st>>>(n, kvec, cstart, phase, d, e, w, bounds, blk, dplus, uminus,
+                                                              z, ldz, status);
     }
     return cudaGetLastError();
 }
