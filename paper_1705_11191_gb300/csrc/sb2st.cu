@@ -50,8 +50,6 @@ template cudaError_t extract_band<float>(cudaStream_t, int, int, const float *, 
 
 struct ChaseArgs {
     int n, b, ldb, S;
-    long long tmax;
-    unsigned *count, *gen;
     int *status;
     long long spin_limit;  // polls of a progress-flag wait before ELSI_ERR_TIMEOUT
 };
@@ -328,8 +326,7 @@ cudaError_t sb2st(cudaStream_t st, int n, int b, T *band, int ldb, double *d, do
         const int S = sb2st_steps(n, b);
         ChaseArgs a;
         a.n = n; a.b = b; a.ldb = ldb; a.S = S;
-        a.tmax = 3ll * (n - 3) + (S - 1);
-        a.count = sync; a.gen = sync + 1; a.status = status;
+        a.status = status;
         a.spin_limit = spin_limit();
         size_t smem = (2 * (size_t)b * (b + 8) + 3 * b) * sizeof(T);
         static PerDeviceOnce attr_set;  // per instantiation
