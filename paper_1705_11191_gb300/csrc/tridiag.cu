@@ -844,18 +844,20 @@ __global__ void cluster_orth_kernel(int n, int kvec, const int *cstart, int phas
         if (v == i0 && !lost) continue;
         T *zv = z + (size_t)v * ldz;
         double s = lost ? 0.0 : cluster_project(n, i0, v, z, ldz, red);
-        // a regenerated vector is accepted when its part orthogonal to the cluster is a good part of
-        // it: what is wrong with the vectors before it enters with the factor 1 / sqrt(s), and adds up
-        // over a large group; after the last attempt, when that part is far above the rounding level
-        // of T (its direction error is then eps / sqrt(s))
+        // a regenerated vector is accepted when its part orthogonal to the cluster is far above the
+        // rounding level of T (its direction error is then eps / sqrt(s)). In binary64, before the last
+        // attempt, when that is a good part of it: what is wrong with the vectors before it enters
+        // with the factor 1 / sqrt(s), and adds up over a large group. (Binary32 vectors are refined.)
         constexpr int kAttempts = 5;
         double accept = 1e-4;
         for (int attempt = lost ? 1 : 0; attempt < kAttempts && !(s >= accept); ++attempt) {
-            accept = attempt + 1 < kAttempts ? 1e-3 : sizeof(T) == 8 ? 1e-16 : 1e-8;
+            accept = sizeof(T) == 4 ? 1e-8 : attempt + 1 < kAttempts ? 1e-3 : 1e-16;
             const int bs = attempt == 0 ? blk[2 * v] : 0, be = attempt == 0 ? blk[2 * v + 1] : n;
             if (attempt > 0) {
                 const double roundings = attempt == 1 ? 8.0 : attempt == 2 ? -8.0 : attempt == 3 ? 32.0 : -128.0;
-                shifted_factor(bs, be, kvec, v, d, e, w[v] + roundings * DBL_EPSILON * bounds[3], bounds[2], dplus);
+                // in units of the eigenvalues' accuracy (1e-8 ||T|| in the binary32 route)
+                const double unit = (sizeof(T) == 8 ? DBL_EPSILON : 1e-9) * bounds[3];
+                shifted_factor(bs, be, kvec, v, d, e, w[v] + roundings * unit, bounds[2], dplus);
             }
             // start b: pseudo-random on the block, orthogonal to the cluster's vectors
             for (int i = threadIdx.x; i < n; i += blockDim.x)
@@ -871,9 +873,12 @@ __global__ void cluster_orth_kernel(int n, int kvec, const int *cstart, int phas
             for (int i = threadIdx.x; i < n; i += blockDim.x) zv[i] = (T)((double)zv[i] * inv);
             __syncthreads();
             s = cluster_project(n, i0, v, z, ldz, red);
-            // with every vector of the group in this block taken, x is of other eigenvalues
-            const double tol = (sizeof(T) == 8 ? 1e-10 : 1e-5) * bounds[3] + 8.0 * bounds[2];
-            if (!(residual2(n, d, e, w[v], zv, red) <= tol * tol * s)) s = 0.0;
+            // with every vector of the group in this block taken, x is of other eigenvalues (binary64; 1e-14:
+            // the rounding of the projection)
+            if (sizeof(T) == 8) {
+                const double tol = (1e-10 * sqrt(s) + 1e-14) * bounds[3] + 8.0 * bounds[2];
+                if (!(residual2(n, d, e, w[v], zv, red) <= tol * tol)) s = 0.0;
+            }
         }
         if (!(s >= accept)) {
             if (threadIdx.x == 0) report_error(status, ELSI_ERR_NO_CONVERGENCE, v);
