@@ -538,7 +538,10 @@ twist_vector_kernel(int n, const double *__restrict__ d, const double *__restric
 // Sums and updates of the Gram-Schmidt step with at least the precision of binary64 arithmetic
 // rounded to T. A binary32 product and a sum are kept as two binary32 numbers (products split by
 // an FMA, Knuth's two-sum: Ogita, Rump & Oishi 2005), a dozen operations of a unit that has 64
-// times the rate of the binary64 one; a conversion and an FMA there hold it for 128 clocks.
+// times the rate of the binary64 one; a conversion and an FMA there hold it for 128 clocks. What is
+// stored is rounded to binary32 once, so the sums' 48 bits leave what binary64 sums would: of 64
+// vectors the largest |z_u . z_v| is 5.2e-9 at n = 500 and 2.8e-9 at n = 2000 with either, against 1.3e-8
+// and 7.9e-9 with binary64 sums and a rounded update for every pair.
 template <typename T> struct Wide;
 template <> struct Wide<double> {
     double v;
@@ -833,7 +836,8 @@ __global__ void cluster_orth_kernel(int n, int kvec, const int *cstart, int phas
         while (cend < kvec && cend < i0 + kOrthPiece && cstart[cend] == s) ++cend;
         if (phase == 1 && cend <= i0 + kOrthPiece / 2) return;  // no piece boundary inside
     } else {
-        const double same = 1e-12 * bounds[3];
+        // (some hundred roundings; with one huge eigenvalue more would take in the rest of the spectrum)
+        const double same = 1e-13 * bounds[3];
         if (i0 > 0 && w[i0] - w[i0 - 1] <= same) return;
         while (cend < kvec && cend < i0 + kOrthRun && w[cend] - w[cend - 1] <= same) ++cend;
         if (cend - i0 <= kOrthPiece / 2) return;
