@@ -23,8 +23,9 @@ extern "C" {
 
 /*
  * elsi_gb_set_spin_limit: iteration limit of the library's SIMT spin waits (the
- *   packets that the CTAs of the panel factorisation and of the bulge chase exchange and the
- *   progress flags of the general chase; the mbarrier waits of the tensor-core pipelines keep their own limit).
+ *   packets that the CTAs of the panel factorisation and of the bulge chase exchange, the
+ *   progress flags of the general chase and the progress words of both back-transformations
+ *   through Q2; the mbarrier waits of the tensor-core pipelines keep their own limit).
  *   A wait that has polled more than `polls` times records ELSI_ERR_TIMEOUT in the
  *   solve's status word and its kernel returns, so the solve returns ELSI_ERR_TIMEOUT and
  *   the CUDA context stays usable. Process-wide; read at each launch. Default 2^26
@@ -95,7 +96,10 @@ int elsi_gb_gemm_f64_digits(int ta, int tb, int m, int n, int k, double alpha, c
 
 /*
  * elsi_gb_gemm_f64_wide: the same with eight 9-bit digits and 128-bit sums, the products of
- *   the binary64 route (truncation about 2^-72); scratch of elsi_gb_gemm_f64_wide_planes
+ *   the binary64 route: truncation about 2^-72 of max|op(A)_i.| max|op(B)_.j| per term, so that
+ *   an entry more than 2^18 below the largest of its row or column has fewer than 53 bits of its
+ *   own. Rows and columns with an infinity or a NaN give what binary64 sums give (both forms).
+ *   Scratch of elsi_gb_gemm_f64_wide_planes
  *   values and elsi_gb_gemm_f64_digits_exps exponents. Scratch beyond that is used to divide
  *   a long K over CTAs.
  */

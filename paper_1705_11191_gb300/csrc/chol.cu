@@ -180,7 +180,10 @@ cudaError_t potrf(cudaStream_t st, int n, T *a, int lda, T *inv_diag, int *statu
 // in products with a long K. Below, the first part is a panel of 256 rows, then a block: more rows of
 // the products in flight at a time. Standard form and back-substitution by halves against panels:
 // n = 16384 61 and 30 ms against 82 and 40, n = 5000 (binary64) 33.7 and 4.8 against 37.9 and 4.6,
-// n = 4096 4.0 and 1.9 against 4.3 and 2.1; n = 2000 1.55 and 0.82 against 1.38 and 0.75.
+// n = 4096 4.0 and 1.9 against 4.3 and 2.1; n = 2000 1.55 and 0.82 against 1.38 and 0.75. In between, binary32
+// n = 2800 2.52 and 1.23 against 2.46 and 1.20, 3500 3.41 and 1.60 against 3.36 and 1.61, 3800 3.74 and 1.80
+// against 3.96 and 1.91; binary64 n = 2000 4.83 and 1.09 against 5.08 and 1.13, 3200 11.5 and 2.2 against 12.7
+// and 2.1, 4095 19.1 and 3.1 against 22.4 and 3.1 (there halves would pay from 2000 on: 1 % of a solve).
 template <typename T>
 static cudaError_t trsm_range(cudaStream_t st, int trans, bool halves, int r0, int r1, int ncol, const T *L,
                               int ldl, const T *inv_diag, int ldi, T *B, int ldb, const T *ka, const T *kb)

@@ -268,8 +268,9 @@ bool tc_scratch(float **work, size_t *elems, int **status)
 }
 
 // Scratch of the calling thread for binary64-accurate products on the tensor cores (the
-// Ozaki digit planes and row exponents; set around the binary64 Cholesky of the binary32
-// route, absent elsewhere).
+// Ozaki digit planes and row exponents; set around a solve of the binary64 route, the
+// binary64 Cholesky of the binary32 route, the eigenpair adjoint and batched P and W, absent
+// elsewhere and where there is no room for it).
 static thread_local __nv_bfloat16 *t_oz_planes = nullptr;
 static thread_local size_t t_oz_elems = 0;
 static thread_local int *t_oz_exps = nullptr;

@@ -98,7 +98,7 @@ cudaError_t check_finite(cudaStream_t st, int m, int n, const T *a, int lda, int
 // ---- Cholesky and triangular solves (Eqs. 8-9) ----
 // Lower Cholesky of the n x n matrix a in place (upper triangle zeroed). inv_diag
 // receives the inverses of the nb x nb diagonal blocks of L (n x nb, block j at rows
-// j*nb). work: n x nb scratch. Status ELSI_ERR_NOT_PD with the pivot on failure.
+// j*nb). Status ELSI_ERR_NOT_PD with the pivot on failure.
 template <typename T>
 cudaError_t potrf(cudaStream_t st, int n, T *a, int lda, T *inv_diag, int *status);
 constexpr int kTriBlock = 64;   // nb of potrf / trsm
@@ -192,7 +192,9 @@ cudaError_t apply_q2_tc(cudaStream_t st, int n, int b, const float *v2, const fl
                         float *z, int ldz, float *fac, int *status);
 // Z <- Q1 Z in groups of q1_group(n) panels (q1.cu); work: q1_work_elems(n, b, k) elements. Eight panels
 // a group halve the passes over Z, and merging their T takes longer: n = 777 0.77 ms against 0.30 with
-// four, n = 1531 the same, n = 4096 2.35 against 2.54, n = 5000 9.7 against 10.9, n = 16384 62 against 74.
+// four, n = 1531 the same, n = 4096 2.35 against 2.54, n = 5000 9.7 against 10.9, n = 16384 62 against 74;
+// in between, binary64 n = 2800 3.64 against 3.48, 3500 5.07 against 5.14, 4095 6.16 against 6.51, binary32
+// (64-column panels) n = 3800 2.36 against 2.26, 4095 2.69 against 2.60: nothing within 5 % of the limit.
 constexpr int kQ1MaxGroup = 8;
 inline int q1_group(int n) { return n >= 4096 ? kQ1MaxGroup : 4; }
 inline size_t q1_work_elems(int n, int b, int k)

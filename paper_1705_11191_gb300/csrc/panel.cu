@@ -22,6 +22,10 @@
 // stay a pair of binary32 numbers up to the one rounding of the update's factors; T is formed from
 // the pairs in binary64.
 //
+// T is off the row CTAs' path only while its CTA keeps up: with a Gram entry converted to binary64
+// for every row of T it was the slower one (full to band of n = 16384 173 ms, 164 with one conversion
+// an entry and column; whole solves of n = 4096 76.3 -> 72.6 ms).
+//
 // Measured per 64-column panel, before -> now: binary32 n = 777 0.73 -> 0.21 ms, n = 4096 0.82
 // -> 0.24 ms, n = 16384 0.85 -> 0.29 ms; binary64 n = 512 1.09 -> 0.40 ms, n = 5000 1.24 ->
 // 0.51 ms; per 32-column panel, binary64 n = 512 0.152 -> 0.133 ms, n = 5000 0.192 -> 0.169 ms with

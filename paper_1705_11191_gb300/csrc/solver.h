@@ -44,7 +44,7 @@ struct Workspace {
     EGB_BUF(int, ozexp)      // their exponents
     EGB_BUF(float, q2f)      // compact-WY factors of Q2 (binary32 route)
     EGB_BUF(float, tcw)      // TF32 hi/lo operand planes of the tensor-core GEMM
-    EGB_BUF(unsigned, sync)  // grid-barrier words + partial sums
+    EGB_BUF(unsigned, sync)  // packets and partial sums of the reductions, progress words of Q2
     EGB_BUF(int, status)
     EGB_BUF(double, host_h)  // staging for the _host entry points
     EGB_BUF(double, host_s)
@@ -127,7 +127,8 @@ struct SolveRequest {
 // is 7 b^2 FMAs at two a clock (n = 1531: 35 -> 12 ms, n = 5000: 118 -> 46 ms); with b = 32 the chase holds
 // up to 608 positions on the chip, orders up to 19 400. Binary32 route, whole solves with 64 and 32:
 // n = 500 8.2 and 8.0 ms, 1200 19.0 and 18.3, 2000 32.2 and 31.0, 3000 50.4 and 49.4, 4096 75.9 and 76.0,
-// 6000 141 and 148.
+// 6000 141 and 148. Since then panels of 64 columns became 5 % of a solve faster (panel.cu): 2000 29.7 and 29.7,
+// 2400 35.0 and 35.9, 2800 43.2 and 43.9, 3200 50.1 and 52.1, 3500 55.7 and 58.5; the limit has been left.
 inline int band_of(const elsi_gb_handle_s *h, int precision, size_t n)
 {
     return !h->band_set && n <= (precision == ELSI_PREC_FP64 ? 19000 : 3500) ? 32 : h->band_width;
