@@ -579,13 +579,13 @@ TF32_PER_BF16 = 1.1 / 2.25  # nominal dense tf32 / bf16 tensor rates
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of a stage's kernels from one
 # ncu capture, valid while the kernel's source file is unchanged (sha256 prefix). The Q2
-# capture is at n = 8192 (the n = 16384 workspace is too large for a multi-pass capture);
-# its traffic is one read and one write of the remaining rows of Z per block of 64 sweeps,
-# which grows as n^3 once Z exceeds L2 (as it does at 8192 and 16384), so it is scaled by
-# (n / 8192)^3.
+# capture is at n = 6144 (a few GB on the device); its traffic is one read and one write of
+# the remaining rows of Z per block of 64 sweeps, which grows as n^3 once Z exceeds L2, so it
+# is scaled by (n / 6144)^3. At 6144 Z is 151 MB against 129 MB of L2 and part of it hits: a
+# lower bound for larger n (one read and one write of Z each would be half as much again).
 MEASURED_TRAFFIC = {
     "back_q2": {"kernel": "q2_apply_tc5_kernel", "source": "paper_1705_11191_gb300/csrc/q2tc.cu",
-                "sha256_16": "a7bd6373b70be307", "n": 8192, "bytes": 15318903552 + 16249897472},
+                "sha256_16": "3119605bfde227bf", "n": 6144, "bytes": 4931872000 + 5041981696},
 }
 
 
