@@ -496,12 +496,18 @@ int solve_fp32_refine(elsi_gb_handle_s *h, const SolveRequest &rq)
     }
     CKR(cudaEventRecord(w.ev[STAGE_TRIDIAG], st));
     // binary32-route eigenvalues: the wanted ones are recomputed by the refinement and the
-    // rest are reported at the accuracy of this route. T itself carries the binary32
-    // rounding of the reduction (about 6e-8 ||T||), so bisection to 1e-8 ||T|| changes
-    // neither the eigenvalues nor, through the twisted factorisations, the eigenvectors
-    // beyond that level. (At 1e-7 ||T|| the refinement of the 3D-cluster problem at
-    // n = 16384 no longer converges and the solve falls back to the binary64 route.)
-    CKR(stebz(st, n, w.d, w.e, n, w.w, w.status, reinterpret_cast<double *>(w.oz), 1e-8));
+    // rest are reported at the accuracy of this route. The width of the last interval still
+    // matters below the binary32 rounding of T (about 6e-8 ||T||): the vectors of close
+    // eigenvalues come from separate shifts, and their overlap is the defect that the
+    // refinement starts from. Complex k-points of n = 2048, 105 solves: median defect 3.9e-3
+    // at 1e-8, 6.4e-5 at 4e-9 and at 2e-9, 2.0e-5 at 1e-9; 3, 0, 0, 0 of them were repeated in
+    // binary64. 178 other ones (n = 1500 .. 2600), on which the value was not chosen: medians
+    // 8e-4 .. 6e-3 at 1e-8, 3e-5 .. 2e-4 at 2e-9, and 2 against 1 repeated, so a start that
+    // fails is rarer at most, not ruled out. Costs about 0.5 % of a solve (n = 4096, 16384).
+    // The last interval is anywhere between tol / (lanes + 1) and tol, so tol and not the
+    // width that one lane count happens to reach has to be small enough.
+    // (At 1e-7 the 3D-cluster problem at n = 16384 no longer converges either.)
+    CKR(stebz(st, n, w.d, w.e, n, w.w, w.status, reinterpret_cast<double *>(w.oz), 2e-9));
     // eigenvector scratch (3 n^2 + n binary64 values) in the digit-plane buffer, free here
     CKR(stein<float>(st, n, w.d, w.e, n, w.w, X32, n, reinterpret_cast<double *>(w.oz), w.status));
     CKR(cudaEventRecord(w.ev[STAGE_Q2], st));

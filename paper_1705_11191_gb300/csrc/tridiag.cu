@@ -510,7 +510,7 @@ twist_vector_kernel(int n, const double *__restrict__ d, const double *__restric
     const double nrm2 = 1.0 + nrm_w[0][lane] + nrm_w[1][lane];
     // No eigenvector: a product out of range, next to pivots of zero in a group of coinciding eigenvalues,
     // or a residual |gamma| / ||z|| far above the accuracy of the eigenvalue (at most sqrt(n) times
-    // 1e-8 ||T||, or 1e-15): a block that does not hold it, where a group is spread over several. The
+    // 2e-9 ||T||, or 1e-15): a block that does not hold it, where a group is spread over several. The
     // vector is left to cluster_orth_kernel.
     const bool lost = !(nrm2 < DBL_MAX) || !(fabs(best) <= ((sizeof(T) == 8 ? 1e-8 : 1e-4) * bounds[3] + 8.0 * pivmin) * sqrt(nrm2));
     if (warp == 0 && have && lost) blk[2 * l + 1] = -be;
@@ -859,7 +859,7 @@ __global__ void cluster_orth_kernel(int n, int kvec, const int *cstart, int phas
             const int bs = attempt == 0 ? blk[2 * v] : 0, be = attempt == 0 ? blk[2 * v + 1] : n;
             if (attempt > 0) {
                 const double roundings = attempt == 1 ? 8.0 : attempt == 2 ? -8.0 : attempt == 3 ? 32.0 : -128.0;
-                // in units of the eigenvalues' accuracy (1e-8 ||T|| in the binary32 route)
+                // in units of the eigenvalues' accuracy (2e-9 ||T|| at most in the binary32 route)
                 const double unit = (sizeof(T) == 8 ? DBL_EPSILON : 1e-9) * bounds[3];
                 shifted_factor(bs, be, kvec, v, d, e, w[v] + roundings * unit, bounds[2], dplus);
             }
